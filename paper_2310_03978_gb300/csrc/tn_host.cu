@@ -168,12 +168,20 @@ struct Step {
     int out_meta = -1;           // meta block whose per-slice max-abs this step's epilogue records
     int direct_planar = -1;      // planar copy this step writes directly instead of complex64
     int64_t part_off = -1;       // K_GEMM split-K partials (byte offset in the arena)
-    int chain = -1;              // run of small element-wise steps launched together (k_generic_chain)
+    int chain = -1;              // run of small element-wise steps launched together (k_chain)
     bool chain_head = false;     // first step of its run: launches the whole run
+    bool fused_mul = false;      // in a run: products rounded as in k_generic_k1
     // profile mode: recorded (start, stop) event pairs not yet read, and the running totals
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> pending, pending_prep;
     double time_ms = 0, prep_ms = 0;
     int64_t timed = 0;
+};
+
+struct Chain {               // a run of small element-wise steps launched together
+    std::vector<int> steps;
+    int64_t first_level = 0; // its first bound in the plan's level bounds
+    int nlevels = 0;
+    int64_t widest = 0;      // items of its widest level
 };
 
 struct Op {
@@ -205,12 +213,18 @@ struct tn_plan {
     std::vector<tn::BindItem> bind_inv, bind_sl;
     std::vector<tn::BindTiled> tiled_inv, tiled_sl;  // leaves bound by the tiled permutation
     tn::BindItem *bind_inv_dev = nullptr, *bind_sl_dev = nullptr;
-    std::vector<std::vector<int>> chains;  // step indices of each run of chained steps
-    std::vector<int64_t> chain_first;      // first descriptor of each run in chain_dev
-    tn::GenericDesc *chain_dev = nullptr;
+    std::vector<int> exec[2];              // launch order: chain heads and single steps of the
+                                           // slice-independent prologue [0], the slice loop [1]
+    std::vector<Chain> chains;             // runs of small element-wise steps (k_chain)
+    tn::ChainItem *chain_items = nullptr;  // the items of every run (device), and behind them
+    int32_t *chain_levels = nullptr;       // the level bounds of every run
     int max_rank_inv = 0, max_rank_sl = 0;
-    unsigned int *meta = nullptr;  // per meta block: amax[sb] then exps[sb]
-    int nmeta = 0;
+    // per-slice max-abs [nmeta][sb], then the exponents [nmeta][sb]; the first nmeta_inv blocks
+    // belong to slice-independent tensors
+    unsigned int *meta = nullptr;
+    int nmeta = 0, nmeta_inv = 0;
+    unsigned int *amax(int block) const { return meta + sb * block; }
+    int32_t *exps(int block) const { return reinterpret_cast<int32_t *>(meta + sb * (nmeta + block)); }
     double *partial = nullptr;     // readout partials
     double2 *amps_tmp = nullptr;   // tn_contract_host accumulator
     int n_partial = 64;
@@ -821,6 +835,15 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
                     need_meta(pr.b);
                 }
             }
+        // slice-independent blocks first: they are cleared once per call, the others per batch
+        {
+            int next = 0;
+            for (int dep = 0; dep < 2; ++dep) {
+                for (auto &x : p->tensors)
+                    if (x.meta >= 0 && x.dep == (dep == 1)) x.meta = next++;
+                if (dep == 0) p->nmeta_inv = next;
+            }
+        }
         for (auto &q : p->planars) {
             q.meta = p->tensors[q.tensor].meta;
             if (q.direct) {
@@ -832,52 +855,77 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
         for (auto &x : p->tensors)
             if (x.meta >= 0 && x.producer >= 0) p->steps[x.producer].out_meta = x.meta;
     }
-    // runs of consecutive small element-wise steps are launched together, one block per slice
-    // (k_generic_chain): runs of the slice-independent prologue and runs of the slice loop,
-    // each in its own execution order; not in profile mode, which times every step on its own
-    if (!p->opts.profile) {
-        std::vector<int> run[2];  // [0] prologue, [1] slice loop
-        auto close_run = [&](std::vector<int> &r) {
-            if (r.size() >= 2) {
-                const int id = (int)p->chains.size();
-                for (int k : r) p->steps[k].chain = id;
-                p->steps[r[0]].chain_head = true;
-                p->chains.push_back(r);
-            }
-            r.clear();
-        };
-        for (int s = 0; s < path_len; ++s) {
-            const Step &st = p->steps[s];
-            const int rc = p->tensors[st.c].rank(), nk = (int)st.K.size();
-            const bool small = st.kernel == K_GENERIC && st.out_meta < 0 &&
-                               rc <= tn::kChainMaxRankC && nk <= tn::kChainMaxNk &&
-                               rc + nk <= tn::kChainMaxWork;
-            std::vector<int> &r = run[st.dep ? 1 : 0];
-            if (small) r.push_back(s);
-            else close_run(r);
+    // Launch order.  The small element-wise steps run many per launch (k_chain): just before a
+    // larger step that needs one of them, every small step whose operands exist by then joins one
+    // run, wherever the path has it, so a path whose small and large steps alternate still needs
+    // few launches.  The slice-independent prologue and the slice loop are ordered separately.
+    // Profile mode times every step on its own, in path order.
+    for (int cls = 0; cls < 2; ++cls) {
+        std::vector<int> todo;
+        for (int s = 0; s < path_len; ++s)
+            if (p->steps[s].dep == (cls == 1)) todo.push_back(s);
+        if (p->opts.profile) {
+            p->exec[cls] = todo;
+            continue;
         }
-        close_run(run[0]);
-        close_run(run[1]);
+        std::vector<char> done(path_len, 0);
+        for (int s = 0; s < path_len; ++s) done[s] = cls == 1 && !p->steps[s].dep;
+        auto small = [&](const Step &st) {
+            const int rc = p->tensors[st.c].rank(), nk = (int)st.K.size();
+            return st.kernel == K_GENERIC && rc <= tn::kChainMaxRankC && nk <= tn::kChainMaxNk &&
+                   rc + nk <= tn::kChainMaxWork;
+        };
+        // An outer product of 2^10 or more outputs whose max-abs is recorded, or with no small
+        // step beside it in the path, rounds as k_generic_k1 does, the others as k_generic: the
+        // rule looks at the path only, so results do not depend on how steps share launches.
+        auto plain = [&](size_t i) {
+            return i < todo.size() && small(p->steps[todo[i]]) && p->steps[todo[i]].out_meta < 0;
+        };
+        for (size_t i = 0; i < todo.size(); ++i) {
+            Step &st = p->steps[todo[i]];
+            st.fused_mul = st.K.empty() && p->tensors[st.c].rank() >= 10 &&
+                           (st.out_meta >= 0 || !(plain(i - 1) || plain(i + 1)));
+        }
+        auto ready = [&](const Step &st) {
+            const int pa = p->tensors[st.a].producer, pb = p->tensors[st.b].producer;
+            return (pa < 0 || done[pa]) && (pb < 0 || done[pb]);
+        };
+        auto run_small = [&]() {
+            Chain c;
+            for (int s : todo)  // path order, so an operand's producer comes before its reader
+                if (!done[s] && small(p->steps[s]) && ready(p->steps[s])) {
+                    done[s] = 1;
+                    p->steps[s].chain = (int)p->chains.size();
+                    c.steps.push_back(s);
+                }
+            if (c.steps.empty()) return;
+            p->steps[c.steps[0]].chain_head = true;
+            p->exec[cls].push_back(c.steps[0]);
+            p->chains.push_back(std::move(c));
+        };
+        for (int s : todo) {
+            if (small(p->steps[s])) continue;
+            if (!ready(p->steps[s])) run_small();
+            done[s] = 1;
+            p->exec[cls].push_back(s);
+        }
+        run_small();
     }
     // op timeline: invariant leaves, invariant steps, sliced leaves, dependent steps (each
     // tensor-core step preceded by its conversions; a run of chained steps is one op, so every
     // tensor it touches is live at that op and no two of them share memory), accumulate
     std::vector<Op> ops;
     ops.push_back({0, -1});
-    for (int s = 0; s < path_len; ++s)
-        if (!p->steps[s].dep && (p->steps[s].chain < 0 || p->steps[s].chain_head))
-            ops.push_back({1, s});
+    for (int s : p->exec[0]) ops.push_back({1, s});
     ops.push_back({2, -1});
-    for (int s = 0; s < path_len; ++s)
-        if (p->steps[s].dep) {
-            Step &st = p->steps[s];
-            if (st.chain >= 0 && !st.chain_head) continue;  // part of its run's op
-            if (st.kernel == K_TC) {
-                ops.push_back({3, st.pa});
-                ops.push_back({3, st.pb});
-            }
-            ops.push_back({1, s});
+    for (int s : p->exec[1]) {
+        const Step &st = p->steps[s];
+        if (st.kernel == K_TC) {
+            ops.push_back({3, st.pa});
+            ops.push_back({3, st.pb});
         }
+        ops.push_back({1, s});
+    }
     ops.push_back({4, -1});
     const int tend = (int)ops.size() - 1;
     for (int t = 0; t < (int)ops.size(); ++t) {
@@ -888,7 +936,7 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
         } else if (op.kind == 1) {
             const Step &head = p->steps[op.index];
             const std::vector<int> one{op.index};
-            for (int k : head.chain_head ? p->chains[head.chain] : one) {
+            for (int k : head.chain_head ? p->chains[head.chain].steps : one) {
                 Step &st = p->steps[k];
                 st.t = t;
                 p->tensors[st.c].t0 = p->tensors[st.c].t1 = t;
@@ -1065,9 +1113,9 @@ void fill_planar_out(const tn_plan_t *p, const Step &st, tn::PlanarOut &o) {
     o.plane_stride = n * (C.dep ? p->sb : 1);
     o.planes = q.planes;
     o.bf16 = bf16_mode(p->mode);
-    o.exps = reinterpret_cast<int32_t *>(p->meta + 2 * p->sb * q.meta + p->sb);
-    o.amax_a = p->meta + 2 * p->sb * A.meta;
-    o.amax_b = p->meta + 2 * p->sb * B.meta;
+    o.exps = p->exps(q.meta);
+    o.amax_a = p->amax(A.meta);
+    o.amax_b = p->amax(B.meta);
     o.a_sliced = A.dep ? 1 : 0;
     o.b_sliced = B.dep ? 1 : 0;
     o.log2_k = (int)st.K.size();
@@ -1107,10 +1155,10 @@ tn_status make_tc_desc(const tn_plan_t *p, const Step &st, int variant, tn::TcGe
     d.b_sliced = B.dep ? 1 : 0;
     d.slices_a = sa;
     d.slices_b = sbb;
-    d.expA = reinterpret_cast<const int32_t *>(p->meta + 2 * p->sb * qa.meta + p->sb);
-    d.expB = reinterpret_cast<const int32_t *>(p->meta + 2 * p->sb * qb.meta + p->sb);
+    d.expA = p->exps(qa.meta);
+    d.expB = p->exps(qb.meta);
     d.dtype = bf;
-    d.amax_out = st.out_meta >= 0 ? p->meta + 2 * p->sb * st.out_meta : nullptr;
+    d.amax_out = st.out_meta >= 0 ? p->amax(st.out_meta) : nullptr;
     if (st.direct_planar >= 0) {
         d.planar_out = 1;
         fill_planar_out(p, st, d.pout);
@@ -1166,6 +1214,82 @@ tn::GenericDesc make_generic_desc(const tn_plan_t *p, const Step &st, unsigned i
     return d;
 }
 
+// Items of every run of small steps (see tn::ChainItem), sorted by the steps' depth in their run.
+tn_status build_chains(tn_plan_t *p) {
+    if (p->chains.empty()) return TN_OK;
+    std::vector<tn::ChainItem> items;
+    std::vector<int32_t> levels;
+    std::vector<int> depth(p->steps.size(), -1);
+    for (Chain &c : p->chains) {
+        int deepest = 0;
+        for (int k : c.steps) {
+            const Step &st = p->steps[k];
+            int d = 0;
+            for (int x : {st.a, st.b}) {
+                const int pr = p->tensors[x].producer;
+                if (pr >= 0 && p->steps[pr].chain == st.chain) d = std::max(d, depth[pr] + 1);
+            }
+            depth[k] = d;
+            deepest = std::max(deepest, d);
+        }
+        c.first_level = (int64_t)levels.size();
+        c.nlevels = deepest + 1;
+        for (int d = 0; d <= deepest; ++d) {
+            levels.push_back((int32_t)items.size());
+            for (int k : c.steps) {
+                if (depth[k] != d) continue;
+                const Step &st = p->steps[k];
+                const Tensor &A = p->tensors[st.a], &B = p->tensors[st.b], &C = p->tensors[st.c];
+                const int rc = C.rank(), nk = (int)st.K.size(), low = std::min(rc, 5);
+                uint32_t in_a = 0, in_b = 0;  // C's index bits that are labels of A, of B
+                for (int i = 0; i < rc; ++i) {
+                    const int l = C.order[rc - 1 - i];
+                    if (A.pos(l) >= 0) in_a |= 1u << i;
+                    if (B.pos(l) >= 0) in_b |= 1u << i;
+                }
+                auto offset = [&](uint32_t c0, uint32_t in) {
+                    uint32_t r = 0;
+                    int sh = nk;
+                    for (int i = 0; i < rc; ++i)
+                        if ((in >> i) & 1u) r |= ((c0 >> i) & 1u) << sh++;
+                    return (uint16_t)r;
+                };
+                auto stride = [&](const Tensor &X) {
+                    return X.dep ? (uint8_t)X.rank() : tn::kChainShared;
+                };
+                tn::ChainItem it{};
+                it.a = (uint32_t)(A.off >> 5);
+                it.b = (uint32_t)(B.off >> 5);
+                it.c = (uint32_t)(C.off >> 5);
+                it.mask_a = (uint8_t)(in_a & 31u);
+                it.mask_b = (uint8_t)(in_b & 31u);
+                it.ra = stride(A);
+                it.rb = stride(B);
+                it.rc = stride(C);
+                it.lanes_nk = (uint8_t)(low | (nk << 4));
+                it.meta = (uint32_t)(st.out_meta + 1);
+                it.fused_mul = st.fused_mul;
+                for (uint32_t c0 = 0; c0 < (1u << rc); c0 += 32) {
+                    it.ao = offset(c0, in_a);
+                    it.bo = offset(c0, in_b);
+                    it.co = (uint16_t)c0;
+                    items.push_back(it);
+                }
+            }
+            c.widest = std::max(c.widest, (int64_t)items.size() - levels.back());
+        }
+        levels.push_back((int32_t)items.size());
+    }
+    const size_t ib = sizeof(tn::ChainItem) * items.size(), lb = sizeof(int32_t) * levels.size();
+    std::vector<char> host(ib + lb);
+    memcpy(host.data(), items.data(), ib);
+    memcpy(host.data() + ib, levels.data(), lb);
+    TN_CUDA(cudaMalloc(&p->chain_items, ib + lb));
+    TN_CUDA(cudaMemcpy(p->chain_items, host.data(), ib + lb, cudaMemcpyHostToDevice));
+    p->chain_levels = reinterpret_cast<int32_t *>(p->chain_items + items.size());
+    return TN_OK;
+}
+
 tn_status build_descriptors(tn_plan_t *p) {
     for (auto &t : p->tensors) {
         if (t.leaf < 0) continue;
@@ -1203,16 +1327,8 @@ tn_status build_descriptors(tn_plan_t *p) {
     TN_CUDA(cudaMalloc(&p->partial, sizeof(double) * 2 * p->n_partial));
     TN_CUDA(cudaMalloc(&p->amps_tmp, sizeof(double2) << p->net->open.size()));
 
-    if (!p->chains.empty()) {
-        std::vector<tn::GenericDesc> all;
-        for (const auto &run : p->chains) {
-            p->chain_first.push_back((int64_t)all.size());
-            for (int k : run) all.push_back(make_generic_desc(p, p->steps[k], nullptr));
-        }
-        TN_CUDA(cudaMalloc(&p->chain_dev, sizeof(tn::GenericDesc) * all.size()));
-        TN_CUDA(cudaMemcpy(p->chain_dev, all.data(), sizeof(tn::GenericDesc) * all.size(),
-                           cudaMemcpyHostToDevice));
-    }
+    s = build_chains(p);
+    if (s != TN_OK) return s;
     p->tc_desc.resize(p->steps.size());
     for (auto &st : p->steps) {
         if (st.kernel != K_TC) continue;
@@ -1350,11 +1466,18 @@ tn_status tune_tc_step(tn_plan_t *p, Step &st, int64_t slices, cudaStream_t stre
 // conversions) are bracketed by CUDA events on the contraction stream.
 tn_status run_step(tn_plan_t *p, Step &st, int64_t slices, cudaStream_t stream) {
     if (st.chain >= 0) {
-        // the run's first step launches the whole run; the others are part of that launch
-        if (!st.chain_head) return TN_OK;
-        const cudaError_t e = tn::launch_generic_chain(
-            p->chain_dev + p->chain_first[st.chain], (int32_t)p->chains[st.chain].size(), slices,
-            stream);
+        // the run's first step stands for the whole run
+        const Chain &c = p->chains[st.chain];
+        // blocks per slice: one while its 16 warps take at most 2 items each, up to a cluster of
+        // 8; more slices than that fills the GPU with need no second block
+        int cluster = 1;
+        while (cluster < tn::kChainMaxCluster &&
+               (int64_t)cluster * 2 * (tn::kChainThreads / 32) < c.widest &&
+               slices * cluster * 2 <= 304)
+            cluster *= 2;
+        const cudaError_t e = tn::launch_chain(
+            p->chain_items, p->chain_levels + c.first_level, c.nlevels,
+            reinterpret_cast<float2 *>(p->arena), p->meta, p->sb, slices, cluster, stream);
         if (e != cudaSuccess)
             return fail(TN_ERR_CUDA, "step %d chain launch: %s", (int)(&st - &p->steps[0]),
                         cudaGetErrorString(e));
@@ -1384,11 +1507,7 @@ tn_status run_step_inner(tn_plan_t *p, const Step &st, int64_t slices, cudaStrea
     const int64_t sC = C.dep ? ((int64_t)1 << C.rank()) : 0;
     cudaError_t e = cudaSuccess;
     unsigned int *amax_out = nullptr;
-    if (st.out_meta >= 0) {
-        amax_out = p->meta + 2 * p->sb * st.out_meta;
-        TN_CUDA(cudaMemsetAsync(amax_out, 0, sizeof(unsigned int) * (C.dep ? slices : 1),
-                                stream));
-    }
+    if (st.out_meta >= 0) amax_out = p->amax(st.out_meta);
     // a direct CUDA-core or streaming producer bounds its output from its inputs' max-abs;
     // inputs that are leaves (no producer epilogue records it) get an amax pass here
     if ((st.kernel == K_GEMM || st.kernel == K_STREAM) && st.direct_planar >= 0) {
@@ -1399,10 +1518,8 @@ tn_status run_step_inner(tn_plan_t *p, const Step &st, int64_t slices, cudaStrea
             cd.src = arena + X.off;
             cd.n = (int64_t)1 << X.rank();
             cd.src_sstride = X.dep ? cd.n : 0;
-            cd.amax = p->meta + 2 * p->sb * X.meta;
-            const int64_t sx = X.dep ? slices : 1;
-            TN_CUDA(cudaMemsetAsync(cd.amax, 0, sizeof(unsigned int) * sx, stream));
-            TN_CUDA(tn::launch_amax(cd, sx, stream));
+            cd.amax = p->amax(X.meta);
+            TN_CUDA(tn::launch_amax(cd, X.dep ? slices : 1, stream));
             p->launches += 1;
         }
     }
@@ -1421,12 +1538,11 @@ tn_status run_step_inner(tn_plan_t *p, const Step &st, int64_t slices, cudaStrea
             const int64_t sx = X.dep ? slices : 1;
             cd.plane_stride = cd.n * (X.dep ? p->sb : 1);
             cd.dst_sstride = cd.n;
-            cd.amax = p->meta + 2 * p->sb * q.meta;
-            cd.exps = reinterpret_cast<int32_t *>(p->meta + 2 * p->sb * q.meta + p->sb);
+            cd.amax = p->amax(q.meta);
+            cd.exps = p->exps(q.meta);
             cd.dtype = operand_dtype(p->mode);
             cd.planes = q.planes;
             if (X.producer < 0) {  // a leaf: no producer epilogue recorded its max-abs
-                TN_CUDA(cudaMemsetAsync(cd.amax, 0, sizeof(unsigned int) * sx, stream));
                 TN_CUDA(tn::launch_amax(cd, sx, stream));
                 p->launches += 1;
             }
@@ -1704,6 +1820,22 @@ static cudaError_t accumulate(tn_plan_t *p, const Tensor &R, int64_t nout, int64
                                          amps, stream);
 }
 
+// The max-abs of a batch's tensors is gathered by atomicMax, so it starts from zero.
+static tn_status clear_batch_amax(tn_plan_t *p, cudaStream_t stream) {
+    if (p->nmeta > p->nmeta_inv)
+        TN_CUDA(cudaMemsetAsync(p->amax(p->nmeta_inv), 0,
+                                sizeof(unsigned int) * p->sb * (p->nmeta - p->nmeta_inv), stream));
+    return TN_OK;
+}
+
+// The slice-dependent steps of one batch of ns slices.
+static tn_status run_batch(tn_plan_t *p, int64_t ns, cudaStream_t stream) {
+    tn_status s = clear_batch_amax(p, stream);
+    for (size_t i = 0; i < p->exec[1].size() && s == TN_OK; ++i)
+        s = run_step(p, p->steps[p->exec[1][i]], ns, stream);
+    return s;
+}
+
 tn_status tn_contract(tn_plan_t *p, int64_t slice_begin, int64_t slice_end, void *amps_dev,
                       void *stream_) {
     g_err.clear();
@@ -1728,11 +1860,12 @@ tn_status tn_contract(tn_plan_t *p, int64_t slice_begin, int64_t slice_end, void
         tn_status s = bind_leaves(p, false, 0, 1, stream);
         if (s != TN_OK) return s;
     }
-    for (auto &st : p->steps)
-        if (!st.dep) {
-            tn_status s = run_step(p, st, 1, stream);
-            if (s != TN_OK) return s;
-        }
+    if (p->nmeta_inv > 0)
+        TN_CUDA(cudaMemsetAsync(p->amax(0), 0, sizeof(unsigned int) * p->sb * p->nmeta_inv, stream));
+    for (int k : p->exec[0]) {
+        tn_status s = run_step(p, p->steps[k], 1, stream);
+        if (s != TN_OK) return s;
+    }
     const Tensor &R = p->tensors[p->root];
     const int64_t nout = (int64_t)1 << R.rank();
     for (int64_t s0 = slice_begin; s0 < slice_end; s0 += p->sb) {
@@ -1743,12 +1876,14 @@ tn_status tn_contract(tn_plan_t *p, int64_t slice_begin, int64_t slice_end, void
         }
         if (p->opts.autotune && !p->tuned && ns == p->sb) {
             // first full batch: tune the tensor-core steps while running it
-            for (auto &st : p->steps)
-                if (st.dep) {
-                    tn_status s = st.kernel == K_TC ? tune_tc_step(p, st, ns, stream)
-                                                    : run_step(p, st, ns, stream);
-                    if (s != TN_OK) return s;
-                }
+            tn_status s = clear_batch_amax(p, stream);
+            if (s != TN_OK) return s;
+            for (int k : p->exec[1]) {
+                Step &st = p->steps[k];
+                s = st.kernel == K_TC ? tune_tc_step(p, st, ns, stream)
+                                      : run_step(p, st, ns, stream);
+                if (s != TN_OK) return s;
+            }
             p->tuned = true;
             TN_CUDA(accumulate(p, R, nout, ns, s0, amps_dev, stream));
             p->launches++;
@@ -1761,9 +1896,7 @@ tn_status tn_contract(tn_plan_t *p, int64_t slice_begin, int64_t slice_end, void
                 TN_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
             const int64_t l0 = p->launches;
             TN_CUDA(cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal));
-            tn_status cs = TN_OK;
-            for (auto &st : p->steps)
-                if (st.dep && cs == TN_OK) cs = run_step(p, st, ns, p->cap_stream);
+            tn_status cs = run_batch(p, ns, p->cap_stream);
             cudaGraph_t g = nullptr;
             cudaError_t ce = cudaStreamEndCapture(p->cap_stream, &g);
             if (cs != TN_OK) {
@@ -1780,11 +1913,8 @@ tn_status tn_contract(tn_plan_t *p, int64_t slice_begin, int64_t slice_end, void
             TN_CUDA(cudaGraphLaunch(p->graph_exec, stream));
             p->launches += p->graph_launches;
         } else {
-            for (auto &st : p->steps)
-                if (st.dep) {
-                    tn_status s = run_step(p, st, ns, stream);
-                    if (s != TN_OK) return s;
-                }
+            tn_status s = run_batch(p, ns, stream);
+            if (s != TN_OK) return s;
         }
         TN_CUDA(accumulate(p, R, nout, ns, s0, amps_dev, stream));
         p->launches++;
@@ -1861,7 +1991,7 @@ void tn_destroy(void *handle) {
         if (p->own_arena && p->arena) cudaFree(p->arena);
         if (p->bind_inv_dev) cudaFree(p->bind_inv_dev);
         if (p->bind_sl_dev) cudaFree(p->bind_sl_dev);
-        if (p->chain_dev) cudaFree(p->chain_dev);
+        if (p->chain_items) cudaFree(p->chain_items);
         if (p->meta) cudaFree(p->meta);
         if (p->partial) cudaFree(p->partial);
         if (p->amps_tmp) cudaFree(p->amps_tmp);

@@ -77,10 +77,31 @@ struct GenericDesc {
     int8_t posB_k[TN_MAXR];
 };
 
-// Limits of a step run by k_generic_chain: output bits, contracted bits, and their sum.
+// Limits of a step run by k_chain: output bits, contracted bits, and their sum.
 constexpr int kChainMaxRankC = 12;
 constexpr int kChainMaxNk = 10;
 constexpr int kChainMaxWork = 14;
+
+// One warp's work in a run of small element-wise steps (k_chain): up to 32 consecutive outputs of
+// one step.  The layout pass stores every operand as [free labels in the result's order][K], so an
+// operand's offset is the output's index restricted to that operand's labels, shifted by nk, and
+// its K elements are contiguous; the masks say which of the output's five lowest bits (the lane)
+// are labels of A and of B, everything above is in ao / bo.
+struct __align__(16) ChainItem {
+    uint32_t a, b, c;           // arena offsets of the tensors in units of 32 complex64
+    uint16_t ao, bo;            // A's and B's element offset of lane 0
+    uint16_t co;                // C's element offset of lane 0
+    uint8_t mask_a, mask_b;     // lane bits that are labels of A, of B
+    uint8_t ra, rb, rc;         // log2 of the slice stride, kChainShared = shared by all slices
+    uint8_t lanes_nk;           // log2 of the outputs (0..5) | contracted bits << 4
+    uint32_t meta;              // 1 + block of the result's per-slice max-abs; 0 = not recorded
+    uint32_t fused_mul;         // nk = 0: one rounded product and a fused one (k_generic_k1's
+                                //   form) instead of the general loop's
+};
+static_assert(sizeof(ChainItem) == 32, "k_chain loads an item as two 16-byte words");
+constexpr uint8_t kChainShared = 255;
+constexpr int kChainThreads = 512;
+constexpr int kChainMaxCluster = 8;
 
 // Complex GEMM C[m, n] = sum_k A[m, k] * B[n, k] with A = [M][K] and B = [N][K] row-major per
 // slice and C written at pdep(m -> posC_m) | pdep(n -> posC_n), i.e. in the consumer's order.
@@ -224,9 +245,12 @@ cudaError_t launch_sparse_thin(const GenericDesc &d, int32_t ln, const int32_t *
 // amps[i] += root[idx[i]] for the n samples (complex128 accumulation)
 cudaError_t launch_sparse_amps(const float2 *root, const int32_t *idx, int64_t n, double2 *amps,
                                cudaStream_t st);
-// nsteps descriptors in device memory, one block per slice (see k_generic_chain)
-cudaError_t launch_generic_chain(const GenericDesc *steps_dev, int32_t nsteps, int64_t slices,
-                                 cudaStream_t st);
+// A run of small steps: items sorted by level, level l = items [levels[l], levels[l + 1]); every
+// slice is worked by a cluster of `cluster` blocks (a power of two up to kChainMaxCluster).  amax:
+// the plan's max-abs blocks of sb entries each.
+cudaError_t launch_chain(const ChainItem *items, const int32_t *levels, int32_t nlevels,
+                         float2 *arena, unsigned int *amax, int64_t sb, int64_t slices,
+                         int32_t cluster, cudaStream_t st);
 // Set the CUDA-core kernels' shared-memory limits (once per device, outside any stream capture).
 cudaError_t simt_prepare();
 cudaError_t launch_gemm_simt(const GemmDesc &d, int64_t slices, cudaStream_t st);

@@ -1007,6 +1007,40 @@ def test_chained_small_steps_match_single_launches(tn, mode):
     check(res[True], ref, TOL[mode])
 
 
+# (m, n, k, batch) of the first step, slices in flight (log2): one output and less than a warp's 32,
+# whole warps, the largest result, contraction and work of a run, and slices enough for one block
+# each (320 > 304) as for a cluster
+@pytest.mark.parametrize("m,n,k,b,nsl", [(0, 0, 1, 0, 0), (0, 0, 9, 0, 3), (1, 0, 2, 1, 2),
+                                         (2, 2, 1, 0, 9), (3, 1, 0, 1, 0), (2, 3, 4, 1, 1),
+                                         (5, 6, 2, 1, 0), (6, 6, 0, 0, 1), (2, 2, 10, 0, 0)])
+@pytest.mark.parametrize("mode", ["c64", "fp16_scaled"])
+def test_runs_of_small_steps_at_item_edges(tn, mode, m, n, k, b, nsl):
+    # three levels: C0 = A B, C1 = A' B' (the same shape), and their contraction with a leaf each;
+    # the batch labels are shared by four tensors
+    rng = np.random.default_rng(m + 7 * n + 31 * k + 101 * b + 1009 * nsl)
+    M, N, K, B = (list(range(100 * i, 100 * i + r)) for i, r in enumerate((m, n, k, b)))
+    K2, S = [l + 1000 for l in K], list(range(2000, 2000 + nsl))
+    perm = lambda ls: [int(x) for x in rng.permutation(ls)]
+    la, lb = perm(M + K + B + S[::2]), perm(N + K + B + S[1::2])
+    lc, ld = perm(M + K2 + B + S[1::2]), perm(N + K2 + B + S[::2])
+    tensors = [crandn(rng, len(x), 2.0 ** (-len(x) / 2)) for x in (la, lb, lc, ld)]
+    labels, opens, path = [la, lb, lc, ld], B, [(0, 1), (2, 3), (0, 2)]
+    ref = O.contract(tensors, labels, opens, path)
+    net = tn.Network(tensors, labels, opens)
+    got = {}
+    for prof in (False, True):
+        plan = tn.Plan(net, path, S, mode=mode, profile=prof, sync_each_call=True)
+        amps = torch.zeros(1 << len(opens), dtype=torch.complex128, device="cuda")
+        for _ in range(2):  # a second call starts from the first one's workspace
+            amps.zero_()
+            plan.contract(amps)
+        got[prof] = amps.cpu().numpy()
+        plan.close()
+    net.close()
+    check(got[False], ref, TOL["c64"])
+    check(got[True], ref, TOL["c64"])
+
+
 # ------------------------------------------------------------------ sparse-state (Sec. 3.3)
 def sparse_amps(tn, tensors, labels, open_labels, path, samples):
     net = tn.Network(tensors, labels, open_labels)
