@@ -285,7 +285,7 @@ tn_status tn_readout(const tn_plan_t *plan, const void *amps_dev, int32_t n_qubi
  * budget where every allocation must come from its own pool.
  *   - Scratch: a fixed 64 KiB device array inside libtn.so (on every GPU that loads the library,
  *     until the process exits); the call allocates and frees nothing.
- *   - Limit: num_amps <= 2^28 (4096 block sums of 65536 amplitudes); larger -> TN_ERR_INVALID_ARG.
+ *   - Limit: num_amps <= 2^28; larger -> TN_ERR_INVALID_ARG.
  *   - The first call on a device looks up the array's device address (cudaGetSymbolAddress);
  *     make that first call before any stream capture.
  *   - All calls share the array, which keeps the last call's partial sums; calls whose work

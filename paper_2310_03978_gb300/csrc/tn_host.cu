@@ -227,7 +227,6 @@ struct tn_plan {
     int32_t *exps(int block) const { return reinterpret_cast<int32_t *>(meta + sb * (nmeta + block)); }
     double *partial = nullptr;     // readout partials
     double2 *amps_tmp = nullptr;   // tn_contract_host accumulator
-    int n_partial = 64;
     int max_log = 0;
     bool tc_ok = false;
     int single_pass = 0, compensated = 0;  // precision policy: dense steps of each kind
@@ -1324,7 +1323,7 @@ tn_status build_descriptors(tn_plan_t *p) {
     if (s != TN_OK) return s;
     if (p->nmeta > 0)
         TN_CUDA(cudaMalloc(&p->meta, sizeof(unsigned int) * 2 * p->sb * p->nmeta));
-    TN_CUDA(cudaMalloc(&p->partial, sizeof(double) * 2 * p->n_partial));
+    TN_CUDA(cudaMalloc(&p->partial, sizeof(double) * 2 * tn::kReadoutBlocks));
     TN_CUDA(cudaMalloc(&p->amps_tmp, sizeof(double2) << p->net->open.size()));
 
     s = build_chains(p);
@@ -1960,7 +1959,7 @@ tn_status tn_readout(const tn_plan_t *p, const void *amps_dev, int32_t n_qubits,
     cudaStream_t stream = (cudaStream_t)stream_;
     const int64_t m = (int64_t)1 << p->net->open.size();
     TN_CUDA(tn::launch_readout(reinterpret_cast<const double2 *>(amps_dev), m, p->partial,
-                               p->n_partial, stream));
+                               stream));
     double h[2];
     TN_CUDA(cudaMemcpyAsync(h, p->partial, sizeof h, cudaMemcpyDeviceToHost, stream));
     TN_CUDA(cudaStreamSynchronize(stream));

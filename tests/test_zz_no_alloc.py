@@ -59,3 +59,18 @@ def test_noalloc_readout_rejects_vectors_beyond_its_scratch(tn):
     status = tn.lib().tn_readout_noalloc(C.c_void_p(amps.data_ptr()), (1 << 28) + 1, 30,
                                          C.c_void_p(out.ctypes.data), None)
     assert status == 1  # TN_ERR_INVALID_ARG, before any device work
+
+
+# one block and its threads' first, last and second element; just past one and two blocks; past the
+# last block (4 per SM of 1024 amplitudes each); sums of squares of normal values in FP64, all terms
+# positive, so the relative error stays below n 2^-53
+@pytest.mark.parametrize("n", [1, 2, 255, 257, 1024, 1025, 2049, 608 * 1024, 608 * 1024 + 1, 3000001])
+def test_noalloc_readout_at_block_edges(tn, n):
+    g = torch.Generator(device="cuda").manual_seed(n)
+    amps = torch.randn(n, dtype=torch.complex128, device="cuda", generator=g) * 2.0 ** -10
+    p = np.abs(amps.cpu().numpy()) ** 2
+    s1, s2 = float(np.sum(p)), float(np.sum(p * p))
+    got = tn.readout_noalloc(amps, 30)
+    np.testing.assert_allclose(got[:2], [s1, s2], rtol=1e-15 + n * 2.0 ** -53)
+    np.testing.assert_allclose(got[2:], [2.0 ** 30 * s1 / n - 1, 2.0 ** 30 * s2 / s1 - 1],
+                               rtol=1e-9)
