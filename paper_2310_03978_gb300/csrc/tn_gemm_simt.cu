@@ -318,25 +318,81 @@ __global__ void __launch_bounds__(256) k_gemm_skinny(GemmDesc d) {
     }
 }
 
-// Sum of the split-K partials in increasing split order, scattered into C's order.
-__global__ void k_splitk_reduce(GemmDesc d, int64_t slices) {
-    const int64_t MN = 1ll << (d.lm + d.ln);
-    const int64_t total = slices * MN;
-    const uint64_t nmask = (1ull << d.ln) - 1;
-    for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < total;
-         idx += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t s = idx / MN, e = idx % MN;
+// Sum of the split-K partials in increasing split order (one FP32 chain per output, so results do
+// not depend on the kernel), scattered into C's order; grid y = slice.  The max-abs goes out once
+// per block: one atomic per output made a 2^20-output step of two splits wait 700 us for them.
+__device__ __forceinline__ void splitk_store(const GemmDesc &d, int64_t s, uint64_t e, float2 v) {
+    const uint64_t m = e >> d.ln, n = e & ((1ull << d.ln) - 1);
+    d.C[s * d.sC + (int64_t)(deposit(m, d.lm, d.posC_m) | deposit(n, d.ln, d.posC_n))] = v;
+}
+
+__global__ void __launch_bounds__(256) k_splitk_reduce(GemmDesc d, int64_t slices) {
+    const int64_t MN = 1ll << (d.lm + d.ln), s = blockIdx.y;
+    float amx = 0.f;
+    for (int64_t e = blockIdx.x * (int64_t)256 + threadIdx.x; e < MN;
+         e += (int64_t)gridDim.x * 256) {
+        const float2 *P = d.partial + s * MN + e;
         float re = 0.f, im = 0.f;
+#pragma unroll 8
         for (int z = 0; z < d.splits; ++z) {
-            const float2 v = d.partial[((int64_t)z * slices + s) * MN + e];
+            const float2 v = P[(int64_t)z * slices * MN];
             re += v.x;
             im += v.y;
         }
-        const uint64_t m = (uint64_t)e >> d.ln, n = (uint64_t)e & nmask;
-        d.C[s * d.sC + (int64_t)(deposit(m, d.lm, d.posC_m) | deposit(n, d.ln, d.posC_n))] =
-            make_float2(re, im);
-        if (d.amax_out) atomicMax(d.amax_out + s, __float_as_uint(fmaxf(fabsf(re), fabsf(im))));
+        splitk_store(d, s, (uint64_t)e, make_float2(re, im));
+        amx = fmaxf(amx, fmaxf(fabsf(re), fabsf(im)));
     }
+    if (d.amax_out) {
+        __shared__ float warp_max[8];
+        for (int o = 16; o > 0; o >>= 1) amx = fmaxf(amx, __shfl_xor_sync(0xffffffffu, amx, o));
+        if ((threadIdx.x & 31) == 0) warp_max[threadIdx.x >> 5] = amx;
+        __syncthreads();
+        if (threadIdx.x < 32)
+            amax_publish(d.amax_out + s, threadIdx.x < 8 ? warp_max[threadIdx.x] : 0.f);
+    }
+}
+
+// The same for 32 splits or more, which come with few outputs (at most ~19 tiles in all, see
+// gemm_simt_splits): one thread per output would wait for a few loads at a time, thousands of
+// splits long.  A block takes 16 outputs; its threads load 128 splits at once, one tile ahead, and
+// the first 16 add them in order from shared memory.
+constexpr int kDeepSplits = 32, kDeepCols = 16, kDeepRows = 128;
+__global__ void __launch_bounds__(256) k_splitk_reduce_deep(GemmDesc d, int64_t slices) {
+    constexpr int PER = kDeepRows * kDeepCols / 256;
+    __shared__ float2 buf[2][kDeepRows][kDeepCols];
+    const int64_t MN = 1ll << (d.lm + d.ln), s = blockIdx.y;
+    const int col = threadIdx.x % kDeepCols, row = threadIdx.x / kDeepCols;
+    const int64_t e = blockIdx.x * (int64_t)kDeepCols + col;
+    const float2 *P = d.partial + s * MN + e;
+    float2 r[PER];
+    auto load = [&](int z0) {
+#pragma unroll
+        for (int i = 0; i < PER; ++i) {
+            const int z = z0 + row + (256 / kDeepCols) * i;
+            r[i] = z < d.splits && e < MN ? P[(int64_t)z * slices * MN] : make_float2(0.f, 0.f);
+        }
+    };
+    float re = 0.f, im = 0.f;
+    load(0);
+    for (int z0 = 0, b = 0; z0 < d.splits; z0 += kDeepRows, b ^= 1) {
+#pragma unroll
+        for (int i = 0; i < PER; ++i) buf[b][row + (256 / kDeepCols) * i][col] = r[i];
+        __syncthreads();  // also: the sums of the tile two back, in this buffer, are done
+        if (z0 + kDeepRows < d.splits) load(z0 + kDeepRows);
+        if (threadIdx.x < kDeepCols) {
+            const int n = min(kDeepRows, d.splits - z0);
+#pragma unroll 16
+            for (int z = 0; z < n; ++z) {
+                const float2 v = buf[b][z][col];
+                re += v.x;
+                im += v.y;
+            }
+        }
+    }
+    const bool mine = threadIdx.x < kDeepCols && e < MN;
+    if (mine) splitk_store(d, s, (uint64_t)e, make_float2(re, im));
+    if (d.amax_out && threadIdx.x < 32)
+        amax_publish(d.amax_out + s, mine ? fmaxf(fabsf(re), fabsf(im)) : 0.f);
 }
 
 // Thin steps (the low-intensity contractions of App. A.2): C[m, n] = sum_k A[m, k] B[n, k] with
@@ -935,10 +991,16 @@ cudaError_t launch_gemm_simt(const GemmDesc &d, int64_t slices, cudaStream_t st)
         k_gemm_simt<16><<<grid, 256, 0, st>>>(d, tn_);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || d.splits == 1) return e;
-    const int64_t total = slices << (d.lm + d.ln);
-    int64_t blocks = (total + 255) / 256;
-    if (blocks > 152 * 32) blocks = 152 * 32;
-    k_splitk_reduce<<<(unsigned)blocks, 256, 0, st>>>(d, slices);
+    const int64_t MN = 1ll << (d.lm + d.ln);
+    if (d.splits >= kDeepSplits) {
+        const int64_t blocks = (MN + kDeepCols - 1) / kDeepCols;
+        k_splitk_reduce_deep<<<dim3((unsigned)blocks, (unsigned)slices), 256, 0, st>>>(d, slices);
+    } else {
+        int64_t blocks = (MN + 255) / 256;
+        const int64_t most = (152 * 8 + slices - 1) / slices;
+        if (blocks > most) blocks = most;
+        k_splitk_reduce<<<dim3((unsigned)blocks, (unsigned)slices), 256, 0, st>>>(d, slices);
+    }
     return cudaGetLastError();
 }
 

@@ -231,6 +231,29 @@ def test_single_step_cuda_core_kernels(tn, shape, kernel):
     check(got2, ref2, 1e-5)
 
 
+# the sum of split-K partials: 2 and 16 outputs, 64 splits of a 9-bit side, several tiles of 128
+# splits, and few splits of many outputs; then the same result as a tensor-core operand, whose
+# exponent comes from the max-abs that the sum records (result values near 2^-24)
+@pytest.mark.parametrize("shape", [(1, 0, 17), (2, 2, 16), (4, 9, 16), (5, 5, 18), (3, 12, 11)])
+def test_split_k_sums(tn, shape):
+    rng = np.random.default_rng(91 + sum(shape))
+    tensors, labels, out = single_step(rng, *shape)
+    ref = O.contract(tensors, labels, out, [(0, 1)])
+    got, _, kernels = gpu_amps(tn, tensors, labels, out, [(0, 1)])
+    assert kernels == ["gemm_simt"]
+    check(got, ref, 1e-5)
+    if shape[0] + shape[1] < 13:
+        return
+    K = out[:len(out) - 7]  # contracted with a second leaf, leaving 7 of its labels
+    N = list(range(500, 507))
+    T = crandn(rng, len(K) + 7, 2.0 ** -6)
+    t2 = [tensors[0] * 2.0 ** -18, tensors[1], T]
+    l2, o2, path = labels + [K + N], out[len(out) - 7:] + N, [(0, 1), (0, 2)]
+    got, _, kernels = gpu_amps(tn, t2, l2, o2, path, mode="fp16_scaled")
+    assert kernels == ["gemm_simt", "gemm_tc"]
+    check(got, O.contract(t2, l2, o2, path), TOL["fp16_scaled"])
+
+
 def test_long_contraction_with_a_batch_label_on_the_elementwise_kernel(tn):
     # a hyperedge b on three tensors is a batch index of the step that meets two of them; such
     # steps run element-wise, here with k = 2^11 (offsets computed without the shared table)
