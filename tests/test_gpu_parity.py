@@ -989,6 +989,26 @@ def test_sliced_open_labels_give_amplitude_batches(tn, mode):
     tnet.close()
 
 
+# where the open labels stand among the slice id's bits decides which slices in flight share a
+# block: lowest, highest, interleaved, all of them; batches that start and end inside a block
+@pytest.mark.parametrize("order", ["oobb", "bboo", "obob", "boob", "oo"])
+@pytest.mark.parametrize("flight", [1, 3, 16])
+def test_amplitude_batches_for_every_order_of_slice_bits(tn, order, flight):
+    wl = W.small_workload()
+    net = wl.network
+    ref = O.contract_network(net, wl.path)
+    bonds = W.greedy_slices(net.labels, net.open_labels, wl.path, 2)
+    opens = [net.open_labels[4], net.open_labels[1]]
+    sliced = [(opens if c == "o" else bonds).pop(0) for c in order]
+    tnet = tn.Network(net.tensors, net.labels, net.open_labels)
+    plan = tn.Plan(tnet, wl.path, sliced, mode="c64", max_slices_in_flight=flight)
+    total = 1 << len(sliced)
+    check(plan.contract_host(), ref, TOL["c64"])
+    check(plan.contract_host(0, 3) + plan.contract_host(3, total), ref, TOL["c64"])
+    plan.close()
+    tnet.close()
+
+
 def test_all_open_circuit_in_64_amplitude_batches(tn):
     # every qubit of a 12-qubit circuit open, six of them sliced: 64 batches of 64 amplitudes in
     # one call, against the state vector
