@@ -425,7 +425,8 @@ constexpr bool thin_b_in_regs(int nt, int ks) { return ks != 0 && nt * ks <= 16;
 constexpr bool thin_dyn_smem(int nt, int ks) { return ks != 0 && nt == 16; }
 constexpr int thin_dyn_bytes(int nt) { return 2 * kThinRows * (nt + 1) * 8; }
 
-template <int NT, int KS, bool PL>
+// PL: bytes of a planar result's numbers (2 or 4), 0 for a complex64 result
+template <int NT, int KS, int PL>
 __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(GemmDesc d) {
     constexpr int NB = NT < 2 ? 2 : NT;  // row stride of sB (pairs stay 16-byte aligned)
     constexpr int LD = NT + 1;           // row stride of the output stage
@@ -511,7 +512,7 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
         for (int n = 0; n < NT; ++n) stage[tid * LD + n] = make_float2(cr[n], ci[n]);
         __syncthreads();
         float2 *C = d.C + s * d.sC + cbase;
-        if constexpr (PL) {
+        if constexpr (PL != 0) {
 #pragma unroll
             for (int i = 0; i < SPT; ++i) {
                 if (SUBS % 256 != 0 && tid + 256 * i >= SUBS) break;
@@ -521,7 +522,7 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
                     v[j] = stage[ws[i] + w8[j]];
                     amx = fmaxf(amx, fmaxf(fabsf(v[j].x), fabsf(v[j].y)));
                 }
-                planar_out_store4(d.pout, s, cbase | os[i], v, eo);
+                planar_out_store4<PL>(d.pout, s, cbase | os[i], v, eo);
             }
         } else {
 #pragma unroll
@@ -913,9 +914,10 @@ __global__ void __launch_bounds__(256) k_sparse_gemm(GenericDesc d, int32_t ln, 
 
 cudaError_t simt_prepare() {
     cudaError_t e = cudaSuccess;
-    for (auto f : {k_gemm_thin<16, 2, false>, k_gemm_thin<16, 4, false>, k_gemm_thin<16, 8, false>,
-                   k_gemm_thin<16, 16, false>, k_gemm_thin<16, 2, true>, k_gemm_thin<16, 4, true>,
-                   k_gemm_thin<16, 8, true>, k_gemm_thin<16, 16, true>})
+    for (auto f : {k_gemm_thin<16, 2, 0>, k_gemm_thin<16, 4, 0>, k_gemm_thin<16, 8, 0>,
+                   k_gemm_thin<16, 16, 0>, k_gemm_thin<16, 2, 2>, k_gemm_thin<16, 4, 2>,
+                   k_gemm_thin<16, 8, 2>, k_gemm_thin<16, 16, 2>, k_gemm_thin<16, 2, 4>,
+                   k_gemm_thin<16, 4, 4>, k_gemm_thin<16, 8, 4>, k_gemm_thin<16, 16, 4>})
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      thin_dyn_bytes(16));
@@ -1131,14 +1133,16 @@ void launch_thin_walk(const GemmDesc &d, dim3 grid, cudaStream_t st) {
     const int64_t per_slice = (resident + grid.y - 1) / grid.y;
     if (per_slice < (int64_t)grid.x) grid.x = (unsigned)per_slice;
     const int dyn = thin_dyn_smem(NT, KS) ? thin_dyn_bytes(NT) : 0;
-    if (d.planar_out) k_gemm_thin<NT, KS, true><<<grid, 256, dyn, st>>>(d);
-    else k_gemm_thin<NT, KS, false><<<grid, 256, dyn, st>>>(d);
+    if (!d.planar_out) k_gemm_thin<NT, KS, 0><<<grid, 256, dyn, st>>>(d);
+    else if (d.pout.dtype == 2) k_gemm_thin<NT, KS, 4><<<grid, 256, dyn, st>>>(d);
+    else k_gemm_thin<NT, KS, 2><<<grid, 256, dyn, st>>>(d);
 }
 
 template <int NT>
 void launch_thin_long(const GemmDesc &d, dim3 grid, cudaStream_t st) {
-    if (d.planar_out) k_gemm_thin<NT, 0, true><<<grid, 256, 0, st>>>(d);
-    else k_gemm_thin<NT, 0, false><<<grid, 256, 0, st>>>(d);
+    if (!d.planar_out) k_gemm_thin<NT, 0, 0><<<grid, 256, 0, st>>>(d);
+    else if (d.pout.dtype == 2) k_gemm_thin<NT, 0, 4><<<grid, 256, 0, st>>>(d);
+    else k_gemm_thin<NT, 0, 2><<<grid, 256, 0, st>>>(d);
 }
 
 template <int NT>

@@ -547,7 +547,7 @@ __global__ void __launch_bounds__(NPL == 4 ? 192 : 128, MINB)
                     }
                     const uint64_t o = olo | hi_off[it];
                     if (d.planar_out) {
-                        planar_out_store8(d.pout, s, cbase | o, v, eo);
+                        planar_out_store8<ESZ>(d.pout, s, cbase | o, v, eo);
                     } else {
                         float4 *c4 = reinterpret_cast<float4 *>(C + o);
 #pragma unroll
@@ -1159,7 +1159,7 @@ __global__ void __launch_bounds__(PERS_THREADS, 1)
                         }
                         const uint64_t o = olo | hi_off[k];
                         if (d.planar_out) {
-                            planar_out_store8_prescaled(d.pout, c.s, cbase | o, v);
+                            planar_out_store8_prescaled<ESZ>(d.pout, c.s, cbase | o, v);
                         } else {
                             float4 *c4 = reinterpret_cast<float4 *>(C + o);
 #pragma unroll
@@ -1524,7 +1524,10 @@ __global__ void __launch_bounds__(448, 1)
                         w[e] = stg.at(stage, q, e);
                         amx = fmaxf(amx, fmaxf(fabsf(w[e].x), fabsf(w[e].y)));
                     }
-                    planar_out_store8(g.pout, s, cbase | stg.os[q], w, eo);
+                    if (g.pout.dtype == 2)
+                        planar_out_store8<4>(g.pout, s, cbase | stg.os[q], w, eo);
+                    else
+                        planar_out_store8<2>(g.pout, s, cbase | stg.os[q], w, eo);
                 }
             } else {
                 float2 *C = g.C + (int64_t)s * g.sC + cbase;

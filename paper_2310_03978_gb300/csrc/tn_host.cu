@@ -782,7 +782,7 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
     }
     if (path_len == 0) p->tensors[p->root].order = p->root_open;
 
-    // 4. tensor-core operands get planar 16-bit copies.  When the operand's producer is a GEMM
+    // 4. tensor-core operands get planar copies.  When the operand's producer is a GEMM
     //    step of the slice loop (with whole 64 x 64 tiles to spare), that producer writes the
     //    copy directly, with an exponent bounded from its own inputs' max-abs; otherwise a
     //    conversion pass makes it from complex64 just before the step.
@@ -798,13 +798,13 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
             q.bytes_per_slice = (int64_t)((tf32_mode(mode) ? 4 : 2) * q.cap_planes)
                                 << p->tensors[q.tensor].rank();
             const Tensor &X = p->tensors[q.tensor];
-            // TF32 operands (FP32 storage) are always made by the conversion pass
-            if (X.producer >= 0 && st.form != kFormSplit && !tf32_mode(mode)) {
+            if (X.producer >= 0 && (st.form != kFormSplit || operand_dtype(mode) != 0)) {
                 // A producer's direct output takes its exponent from a bound (2 K max|a| max|b|)
                 // that can exceed the true maximum by many binades, which leaves the stored
                 // values low in FP16's range; single-pass operands keep their 11 significant
-                // bits there, but the lo planes of compensated operands would fall into the
+                // bits there, but the lo planes of compensated FP16 operands would fall into the
                 // subnormals, so those are split from complex64 with their measured max-abs.
+                // BF16 and TF32 have FP32's exponents: hi and lo keep their bits at any scale.
                 // A CUDA-core producer writes directly only with whole 64 x 64 tiles, and then
                 // never splits K (its epilogue must hold final sums).
                 // A CUDA-core producer that would split K (judged at one slice in flight, its
@@ -1111,7 +1111,7 @@ void fill_planar_out(const tn_plan_t *p, const Step &st, tn::PlanarOut &o) {
     o.sstride = C.dep ? n : 0;
     o.plane_stride = n * (C.dep ? p->sb : 1);
     o.planes = q.planes;
-    o.bf16 = bf16_mode(p->mode);
+    o.dtype = operand_dtype(p->mode);
     o.exps = p->exps(q.meta);
     o.amax_a = p->amax(A.meta);
     o.amax_b = p->amax(B.meta);

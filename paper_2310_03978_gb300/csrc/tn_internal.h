@@ -30,7 +30,7 @@ constexpr uint32_t kSparseMagic = 0x544e5350u;  // "TNSP": a sparse-state plan
 // Free a sparse-state plan (tn_destroy of a handle with kSparseMagic).
 void sparse_destroy(void *handle);
 
-// Direct planar 16-bit output of a GEMM whose result feeds a tensor-core step: the producer
+// Direct planar output of a GEMM whose result feeds a tensor-core step: the producer
 // writes stored = value * 2^-e into the consumer's planar buffer (re, im, and for the 3M form
 // re + im planes), with e chosen before the GEMM runs from the bound
 //     max(|Re c|, |Im c|) <= 2 K max|a| max|b|,   max|x| = max over x of max(|Re x|, |Im x|),
@@ -41,7 +41,7 @@ struct PlanarOut {
     int64_t plane_stride;           // elements
     int64_t sstride;                // elements
     int32_t planes;                 // 2; 3 with the re + im plane; 4 with re_lo, im_lo planes
-    int32_t bf16;
+    int32_t dtype;                  // 0 = fp16, 1 = bf16, 2 = FP32 rounded to TF32
     int32_t *exps;                  // per slice exponent (written by the producer)
     const unsigned int *amax_a;     // inputs' per-slice max-abs, float bits, true scale
     const unsigned int *amax_b;

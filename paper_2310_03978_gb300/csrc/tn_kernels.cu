@@ -5,6 +5,7 @@
 #include <cuda_bf16.h>
 
 #include "tn_internal.h"
+#include "tn_planar_out.cuh"
 
 namespace tn {
 
@@ -540,13 +541,6 @@ __device__ __forceinline__ __nv_bfloat162 pack2<__nv_bfloat162>(float a, float b
     return __floats2bfloat162_rn(a, b);
 }
 
-// FP32 rounded to the nearest TF32 value (10 fraction bits, ties away from zero), kept in an
-// FP32 container: the tensor core then reads it without further rounding.
-__device__ __forceinline__ float round_tf32(float x) {
-    uint32_t r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
-}
 template <>
 __device__ __forceinline__ float2 pack2<float2>(float a, float b) {
     return make_float2(round_tf32(a), round_tf32(b));

@@ -1,4 +1,4 @@
-// Device store of the direct planar 16-bit output (PlanarOut, declared in tn_internal.h).
+// Device store of the direct planar output (PlanarOut, declared in tn_internal.h).
 #pragma once
 
 #include <cuda_bf16.h>
@@ -8,30 +8,47 @@
 
 namespace tn {
 
-__device__ __forceinline__ void planar_out_store(const PlanarOut &o, int64_t s, uint64_t off,
-                                                 float re, float im, int e) {
+// FP32 rounded to the nearest TF32 value (10 fraction bits, ties away from zero), kept in an
+// FP32 container: the tensor core then reads it without further rounding.
+__device__ __forceinline__ float round_tf32(float x) {
+    uint32_t r;
+    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
+    return __uint_as_float(r);
+}
+
+// N = 2, 4 or 8 consecutive complex values (offset off a multiple of N) into a TF32 planar output:
+// one 8-byte word, or 16-byte words, per plane.  A power-of-two scale does not change TF32's (or
+// BF16's) significand, so the values a tensor core reads are those a conversion pass would write,
+// up to that scale.
+template <int N, bool SCALE>
+__device__ __forceinline__ void planar_out_store_tf32(const PlanarOut &o, int64_t s, uint64_t off,
+                                                      const float2 (&v)[N], int e) {
     const Pow2 pe = pow2_of(-e);
-    const float r = scale_pow2(re, pe), i = scale_pow2(im, pe);
-    const int64_t base = s * o.sstride + (int64_t)off;
-    if (o.bf16) {
-        __nv_bfloat16 *p = static_cast<__nv_bfloat16 *>(o.base) + base;
-        const __nv_bfloat16 rh = __float2bfloat16_rn(r), ih = __float2bfloat16_rn(i);
-        p[0] = rh;
-        p[o.plane_stride] = ih;
-        if (o.planes == 3) p[2 * o.plane_stride] = __float2bfloat16_rn(r + i);
+    float *base = static_cast<float *>(o.base) + s * o.sstride + (int64_t)off;
+    float p[4][N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) {
+        const float r = SCALE ? scale_pow2(v[j].x, pe) : v[j].x;
+        const float i = SCALE ? scale_pow2(v[j].y, pe) : v[j].y;
+        p[0][j] = round_tf32(r);
+        p[1][j] = round_tf32(i);
+        if (o.planes == 3) p[2][j] = round_tf32(r + i);
         if (o.planes == 4) {
-            p[2 * o.plane_stride] = __float2bfloat16_rn(r - __bfloat162float(rh));
-            p[3 * o.plane_stride] = __float2bfloat16_rn(i - __bfloat162float(ih));
+            p[2][j] = round_tf32(r - p[0][j]);
+            p[3][j] = round_tf32(i - p[1][j]);
         }
-    } else {
-        __half *p = static_cast<__half *>(o.base) + base;
-        const __half rh = __float2half_rn(r), ih = __float2half_rn(i);
-        p[0] = rh;
-        p[o.plane_stride] = ih;
-        if (o.planes == 3) p[2 * o.plane_stride] = __float2half_rn(r + i);
-        if (o.planes == 4) {
-            p[2 * o.plane_stride] = __float2half_rn(r - __half2float(rh));
-            p[3 * o.plane_stride] = __float2half_rn(i - __half2float(ih));
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        if (q >= o.planes) break;
+        float *d = base + q * o.plane_stride;
+        if constexpr (N == 2) {
+            *reinterpret_cast<float2 *>(d) = make_float2(p[q][0], p[q][1]);
+        } else {
+#pragma unroll
+            for (int j = 0; j < N; j += 4)
+                *reinterpret_cast<float4 *>(d + j) =
+                    make_float4(p[q][j], p[q][j + 1], p[q][j + 2], p[q][j + 3]);
         }
     }
 }
@@ -40,12 +57,17 @@ __device__ __forceinline__ void planar_out_store(const PlanarOut &o, int64_t s, 
 // as one 2 x 16-bit word per plane.
 __device__ __forceinline__ void planar_out_store2(const PlanarOut &o, int64_t s, uint64_t off,
                                                   float2 v0, float2 v1, int e) {
+    if (o.dtype == 2) {
+        const float2 v[2] = {v0, v1};
+        planar_out_store_tf32<2, true>(o, s, off, v, e);
+        return;
+    }
     const Pow2 pe = pow2_of(-e);
     const float r0 = scale_pow2(v0.x, pe), i0 = scale_pow2(v0.y, pe);
     const float r1 = scale_pow2(v1.x, pe), i1 = scale_pow2(v1.y, pe);
     const int64_t base = s * o.sstride + (int64_t)off;
     const int64_t ps = o.plane_stride / 2;
-    if (o.bf16) {
+    if (o.dtype == 1) {
         __nv_bfloat162 *p =
             reinterpret_cast<__nv_bfloat162 *>(static_cast<__nv_bfloat16 *>(o.base) + base);
         const __nv_bfloat162 rh = __floats2bfloat162_rn(r0, r1), ih = __floats2bfloat162_rn(i0, i1);
@@ -146,22 +168,29 @@ __device__ __forceinline__ void planar_out_store4_t(const PlanarOut &o, int64_t 
     if (o.planes == 4) *reinterpret_cast<uint2 *>(base + 3 * o.plane_stride) = p3.u;
 }
 
+// ESZ: bytes of a stored number, 2 (FP16 or BF16 by o.dtype) or 4 (TF32).
+template <int ESZ>
 __device__ __forceinline__ void planar_out_store4(const PlanarOut &o, int64_t s, uint64_t off,
                                                   const float2 (&v)[4], int e) {
-    if (o.bf16) planar_out_store4_t<__nv_bfloat162>(o, s, off, v, e);
+    if constexpr (ESZ == 4) planar_out_store_tf32<4, true>(o, s, off, v, e);
+    else if (o.dtype == 1) planar_out_store4_t<__nv_bfloat162>(o, s, off, v, e);
     else planar_out_store4_t<__half2>(o, s, off, v, e);
 }
 
+template <int ESZ>
 __device__ __forceinline__ void planar_out_store8(const PlanarOut &o, int64_t s, uint64_t off,
                                                   const float2 (&v)[8], int e) {
-    if (o.bf16) planar_out_store8_t<__nv_bfloat162, true>(o, s, off, v, e);
+    if constexpr (ESZ == 4) planar_out_store_tf32<8, true>(o, s, off, v, e);
+    else if (o.dtype == 1) planar_out_store8_t<__nv_bfloat162, true>(o, s, off, v, e);
     else planar_out_store8_t<__half2, true>(o, s, off, v, e);
 }
 
 // The same for values already multiplied by 2^-e.
+template <int ESZ>
 __device__ __forceinline__ void planar_out_store8_prescaled(const PlanarOut &o, int64_t s,
                                                             uint64_t off, const float2 (&v)[8]) {
-    if (o.bf16) planar_out_store8_t<__nv_bfloat162, false>(o, s, off, v, 0);
+    if constexpr (ESZ == 4) planar_out_store_tf32<8, false>(o, s, off, v, 0);
+    else if (o.dtype == 1) planar_out_store8_t<__nv_bfloat162, false>(o, s, off, v, 0);
     else planar_out_store8_t<__half2, false>(o, s, off, v, 0);
 }
 

@@ -832,6 +832,34 @@ def test_thin_step_feeds_the_tensor_cores(tn, mode, nsl, thin_tc):
     check(got, ref, TOL[mode])
 
 
+# every kind of producer that writes TF32 planes, or the hi and lo planes of a compensated BF16 or
+# TF32 operand, itself: streaming (1 to 16 columns, registers and staged), the same on the tensor
+# cores, CUDA-core GEMM, both tensor-core GEMMs; values near 2^-50 after step 1, and with two slices
+@pytest.mark.parametrize("mode", ["tf32", "split_tf32", "split_bf16"])
+@pytest.mark.parametrize("shape,thin_tc", [((13, 0, 2), -1), ((12, 1, 1), -1), ((12, 2, 3), -1),
+                                           ((11, 3, 4), -1), ((11, 4, 4), -1), ((11, 4, 4), 1),
+                                           ((12, 4, 7), -1), ((8, 8, 2), 0), ((8, 8, 7), 0),
+                                           ((9, 9, 10), 0)])
+def test_producers_write_wide_exponent_planes(tn, mode, shape, thin_tc):
+    lm, ln, lk = shape
+    rng = np.random.default_rng(700 + lm + 20 * ln + 400 * lk)
+    tensors, labels, out = single_step(rng, lm, ln, lk, 2.0 ** -25)
+    K, N = [int(x) for x in rng.permutation(out)[:6]], list(range(500, 507))
+    tensors = tensors + [crandn(rng, 13, 2.0 ** -4)]
+    labels = labels + [K + N]
+    opens = [int(x) for x in rng.permutation([l for l in out if l not in K] + N)]
+    path = [(0, 1), (0, 2)]
+    ref = O.contract(tensors, labels, opens, path)
+    for sliced in ([], [K[0]]):
+        if sliced and lm + ln < 14:
+            continue  # the second step would have too few terms for the tensor cores
+        got, _, kernels = gpu_amps(tn, tensors, labels, opens, path, sliced, mode=mode,
+                                   thin_tc=thin_tc)
+        if not sliced:
+            assert kernels[1] == "gemm_tc"
+        check(got, ref, TOL[mode])
+
+
 @pytest.mark.parametrize("form", ["auto", "4m", "3m"])
 def test_autotuned_plan_matches_oracle(tn, form):
     # the first full batch times every applicable tensor-core variant per step; results before
