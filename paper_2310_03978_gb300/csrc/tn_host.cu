@@ -1827,6 +1827,9 @@ static tn_status clear_batch_amax(tn_plan_t *p, cudaStream_t stream) {
     return TN_OK;
 }
 
+static tn_status contract_range(tn_plan_t *p, int64_t slice_begin, int64_t slice_end,
+                                void *amps_dev, void *stream_);
+
 // The slice-dependent steps of one batch of ns slices.
 static tn_status run_batch(tn_plan_t *p, int64_t ns, cudaStream_t stream) {
     tn_status s = clear_batch_amax(p, stream);
@@ -1840,6 +1843,22 @@ tn_status tn_contract(tn_plan_t *p, int64_t slice_begin, int64_t slice_end, void
     g_err.clear();
     if (check_plan(p) != TN_OK) return TN_ERR_INVALID_ARG;
     if (!amps_dev) return fail(TN_ERR_INVALID_ARG, "amps_dev is NULL");
+    return contract_range(p, slice_begin, slice_end, amps_dev, stream_);
+}
+
+}  // extern "C"
+
+tn_status tn::plan_run_root(tn_plan_t *p, cudaStream_t stream) {
+    return contract_range(p, 0, 1, nullptr, stream);
+}
+
+const float2 *tn::plan_root(const tn_plan_t *p) {
+    return reinterpret_cast<const float2 *>(p->arena) + p->tensors[p->root].off;
+}
+
+// Slices [slice_begin, slice_end) into amps_dev, or without one only into the root tensor.
+static tn_status contract_range(tn_plan_t *p, int64_t slice_begin, int64_t slice_end,
+                                void *amps_dev, void *stream_) {
     if (slice_begin < 0 || slice_end > p->num_slices || slice_begin > slice_end)
         return fail(TN_ERR_INVALID_ARG, "slice range [%lld, %lld) outside [0, %lld)",
                     (long long)slice_begin, (long long)slice_end, (long long)p->num_slices);
@@ -1884,8 +1903,10 @@ tn_status tn_contract(tn_plan_t *p, int64_t slice_begin, int64_t slice_end, void
                 if (s != TN_OK) return s;
             }
             p->tuned = true;
-            TN_CUDA(accumulate(p, R, nout, ns, s0, amps_dev, stream));
-            p->launches++;
+            if (amps_dev) {
+                TN_CUDA(accumulate(p, R, nout, ns, s0, amps_dev, stream));
+                p->launches++;
+            }
             continue;
         }
         const bool graph = p->opts.use_graph && !p->opts.profile && ns == p->sb;
@@ -1915,8 +1936,10 @@ tn_status tn_contract(tn_plan_t *p, int64_t slice_begin, int64_t slice_end, void
             tn_status s = run_batch(p, ns, stream);
             if (s != TN_OK) return s;
         }
-        TN_CUDA(accumulate(p, R, nout, ns, s0, amps_dev, stream));
-        p->launches++;
+        if (amps_dev) {
+            TN_CUDA(accumulate(p, R, nout, ns, s0, amps_dev, stream));
+            p->launches++;
+        }
     }
     if (p->opts.sync_each_call) {
         TN_CUDA(cudaStreamSynchronize(stream));
@@ -1926,6 +1949,8 @@ tn_status tn_contract(tn_plan_t *p, int64_t slice_begin, int64_t slice_end, void
     if (dev != p->device) cudaSetDevice(dev);
     return TN_OK;
 }
+
+extern "C" {
 
 tn_status tn_contract_host(tn_plan_t *p, int64_t slice_begin, int64_t slice_end,
                            double *amps_host, void *stream_) {

@@ -27,6 +27,10 @@ void clear_error();
 
 constexpr uint32_t kNetMagic = 0x544e4e54u;     // "TNNT": a tn_network
 constexpr uint32_t kSparseMagic = 0x544e5350u;  // "TNSP": a sparse-state plan
+// An unsliced plan run only as far as its root tensor, and where that lies: complex64 in the order of
+// the network's open labels, valid until the plan runs again.
+tn_status plan_run_root(tn_plan_t *plan, cudaStream_t stream);
+const float2 *plan_root(const tn_plan_t *plan);
 // Free a sparse-state plan (tn_destroy of a handle with kSparseMagic).
 void sparse_destroy(void *handle);
 

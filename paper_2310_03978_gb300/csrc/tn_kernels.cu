@@ -263,41 +263,75 @@ __global__ void k_sparse_leaves(const SparseLeafDesc *leaves) {
     }
 }
 
-// One sparse-state step: thread per (configuration c, dense output j), summing over the
-// contracted dense bits in increasing order; the operand entries are the configurations gA[c],
-// gB[c] (the projections of c onto each operand's open labels).
+// One sparse-state step, summing over the contracted dense bits in increasing order; the operand
+// entries are the configurations gA[c], gB[c] (the projections of c onto each operand's open
+// labels).  A block walks chunks of 2^LB consecutive outputs (LB <= 10; chunks never leave a
+// configuration, small ones go several at a time), whose operand offsets come from a table built
+// once per block; the bits above LB are deposited by the warp's lanes in parallel.  Bound by the
+// instructions per output: a deposit per output made the 2^24-output steps take 4 times as long.
 __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_t *gA,
                                                      const int32_t *gB, int64_t nconf) {
     __shared__ uint64_t koffA[1024], koffB[1024];
-    const int nk = d.nk;
+    __shared__ uint64_t loA[1024], loB[1024];
+    const int nk = d.nk, lane = threadIdx.x & 31;
     const bool table = nk <= 10;
-    if (table) {
-        for (int k = threadIdx.x; k < (1 << nk); k += blockDim.x) {
+    const int lb = d.rank_c < 10 ? d.rank_c : 10;
+    if (table)
+        for (int k = threadIdx.x; k < (1 << nk); k += 256) {
             koffA[k] = deposit((uint64_t)k, nk, d.posA_k);
             koffB[k] = deposit((uint64_t)k, nk, d.posB_k);
         }
+    for (int j = threadIdx.x; j < (1 << lb); j += 256) {
+        loA[j] = deposit((uint64_t)j, lb, d.posA_c);
+        loB[j] = deposit((uint64_t)j, lb, d.posB_c);
     }
     __syncthreads();
-    const int64_t total = nconf << d.rank_c;
     const int64_t K = 1ll << nk;
-    const uint64_t jmask = (1ull << d.rank_c) - 1;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t c = i >> d.rank_c;
-        const uint64_t j = (uint64_t)i & jmask;
-        const float2 *A = d.A + (int64_t)gA[c] * d.sA + deposit(j, d.rank_c, d.posA_c);
-        const float2 *B = d.B + (int64_t)gB[c] * d.sB + deposit(j, d.rank_c, d.posB_c);
-        float re = 0.f, im = 0.f;
-        for (int64_t k = 0; k < K; ++k) {
-            const uint64_t oa = table ? koffA[k] : deposit((uint64_t)k, nk, d.posA_k);
-            const uint64_t ob = table ? koffB[k] : deposit((uint64_t)k, nk, d.posB_k);
-            const float2 a = A[oa], b = B[ob];
-            re = fmaf(a.x, b.x, re);
-            re = fmaf(-a.y, b.y, re);
-            im = fmaf(a.x, b.y, im);
-            im = fmaf(a.y, b.x, im);
+    const int64_t chunks = nconf << (d.rank_c - lb);
+    const int together = lb < 8 ? 256 >> lb : 1;  // chunks a block takes at once
+    for (int64_t ch0 = (int64_t)blockIdx.x * together; ch0 < chunks;
+         ch0 += (int64_t)gridDim.x * together) {
+        const int64_t ch = ch0 + (together > 1 ? (int)threadIdx.x >> lb : 0);
+        const int64_t c = (ch < chunks ? ch : ch0) >> (d.rank_c - lb);
+        uint64_t ha = 0, hb = 0;
+        if (d.rank_c > lb) {  // one chunk at a time: the same for every thread
+            const uint64_t hi = (uint64_t)ch & ((1ull << (d.rank_c - lb)) - 1);
+            const int i = lb + lane;
+            if (i < d.rank_c && ((hi >> lane) & 1ull)) {
+                if (d.posA_c[i] >= 0) ha = 1ull << d.posA_c[i];
+                if (d.posB_c[i] >= 0) hb = 1ull << d.posB_c[i];
+            }
+            ha = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(ha >> 32)) << 32) |
+                 __reduce_or_sync(0xffffffffu, (uint32_t)ha);
+            hb = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(hb >> 32)) << 32) |
+                 __reduce_or_sync(0xffffffffu, (uint32_t)hb);
+            for (int q = 32; lb + q < d.rank_c; ++q)  // ranks above lb + 32
+                if ((hi >> q) & 1ull) {
+                    if (d.posA_c[lb + q] >= 0) ha |= 1ull << d.posA_c[lb + q];
+                    if (d.posB_c[lb + q] >= 0) hb |= 1ull << d.posB_c[lb + q];
+                }
         }
-        d.C[c * d.sC + (int64_t)j] = make_float2(re, im);
+        if (ch >= chunks) continue;
+        const float2 *Ab = d.A + (int64_t)gA[c] * d.sA + ha;
+        const float2 *Bb = d.B + (int64_t)gB[c] * d.sB + hb;
+        float2 *Cb = d.C + c * d.sC + ((ch & ((1ll << (d.rank_c - lb)) - 1)) << lb);
+        const int j0 = together > 1 ? threadIdx.x & ((1 << lb) - 1) : threadIdx.x;
+        for (int j = j0; j < (1 << lb); j += 256) {
+            const float2 *A = Ab + loA[j];
+            const float2 *B = Bb + loB[j];
+            float re = 0.f, im = 0.f;
+#pragma unroll 4
+            for (int64_t k = 0; k < K; ++k) {
+                const uint64_t oa = table ? koffA[k] : deposit((uint64_t)k, nk, d.posA_k);
+                const uint64_t ob = table ? koffB[k] : deposit((uint64_t)k, nk, d.posB_k);
+                const float2 a = A[oa], b = B[ob];
+                re = fmaf(a.x, b.x, re);
+                re = fmaf(-a.y, b.y, re);
+                im = fmaf(a.x, b.y, im);
+                im = fmaf(a.y, b.x, im);
+            }
+            Cb[j] = make_float2(re, im);
+        }
     }
 }
 
@@ -642,7 +676,11 @@ cudaError_t launch_sparse_leaves(const SparseLeafDesc *leaves_dev, int32_t n, in
 cudaError_t launch_sparse_step(const GenericDesc &d, const int32_t *gA, const int32_t *gB,
                                int64_t nconf, cudaStream_t st) {
     if (nconf <= 0) return cudaSuccess;
-    k_sparse_step<<<grid_for(nconf << d.rank_c, 256), 256, 0, st>>>(d, gA, gB, nconf);
+    const int lb = d.rank_c < 10 ? d.rank_c : 10;
+    const int64_t chunks = nconf << (d.rank_c - lb);
+    int64_t blocks = lb < 8 ? (chunks + (256 >> lb) - 1) >> (8 - lb) : chunks;
+    if (blocks > 152 * 8) blocks = 152 * 8;
+    k_sparse_step<<<(unsigned)blocks, 256, 0, st>>>(d, gA, gB, nconf);
     return cudaGetLastError();
 }
 

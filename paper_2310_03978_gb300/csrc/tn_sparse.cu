@@ -91,24 +91,20 @@ struct tn_sparse_plan {
     };
     std::vector<St> steps;
     // maximal subtrees without open labels, contracted by ordinary dense plans (layout pass,
-    // tensor cores in the low-precision modes); their results are converted into the arena
+    // tensor cores in the low-precision modes); the steps read their root tensors in place
     struct Sub {
         tn_network *net = nullptr;
         tn_plan_t *plan = nullptr;
         int node = -1;               // the sparse tensor the subtree produces
-        double2 *out = nullptr;      // its complex128 result
-        int64_t n = 0;
     };
     std::vector<Sub> subs;
     std::vector<char> skip;          // per step: computed inside a dense subtree
-    std::vector<tn::SparseLeafDesc> convs;
-    tn::SparseLeafDesc *conv_dev = nullptr;
-    int64_t *zero_off = nullptr;
     tn_precision mode = TN_PREC_C64;
     std::vector<tn::SparseLeafDesc> leaves;
     int max_leaf_rank = 0;
     int root = -1;
     float2 *arena = nullptr;
+    std::vector<const float2 *> base;  // per tensor
     int32_t *gather = nullptr;
     int64_t *cfg_off = nullptr;
     int32_t *sample_idx = nullptr;
@@ -123,10 +119,7 @@ void sparse_free(tn_sparse_plan_t *p) {
     for (auto &sb : p->subs) {
         if (sb.plan) tn_destroy(sb.plan);
         if (sb.net) tn_destroy(sb.net);
-        if (sb.out) cudaFree(sb.out);
     }
-    if (p->conv_dev) cudaFree(p->conv_dev);
-    if (p->zero_off) cudaFree(p->zero_off);
     if (p->arena) cudaFree(p->arena);
     if (p->gather) cudaFree(p->gather);
     if (p->cfg_off) cudaFree(p->cfg_off);
@@ -471,8 +464,6 @@ static tn_status sparse_plan_impl(const tn_network_t *net, int32_t path_len,
             e = cudaMemcpy(sb.net->data + sb.net->offset[q], net->data + net->offset[lv[q]],
                            sizeof(double2) * ((size_t)1 << net->labels[lv[q]].size()),
                            cudaMemcpyDeviceToDevice);
-        sb.n = (int64_t)1 << p->ten[c].dense.size();
-        if (e == cudaSuccess) e = cudaMalloc(&sb.out, sizeof(double2) * (size_t)sb.n);
         p->subs.push_back(sb);  // owned by the plan from here on
         if (e != cudaSuccess) {
             sparse_free(p);
@@ -528,24 +519,6 @@ static tn_status sparse_plan_impl(const tn_network_t *net, int32_t path_len,
     if (e == cudaSuccess)
         e = upload(reinterpret_cast<void **>(&p->sample_idx), idx.data(),
                    idx.size() * sizeof(int32_t));
-    if (e == cudaSuccess && !p->subs.empty()) {
-        const int64_t zero = 0;
-        e = upload(reinterpret_cast<void **>(&p->zero_off), &zero, sizeof(int64_t));
-        for (auto &sb : p->subs) {
-            tn::SparseLeafDesc cd{};
-            cd.src = sb.out;
-            cd.dst = p->arena + p->ten[sb.node].off;
-            cd.cfg_off = p->zero_off;
-            cd.nconf = 1;
-            cd.rank_d = (int)p->ten[sb.node].dense.size();
-            fill_pos(cd.pos_d, TN_MAXR, -1);
-            for (int i = 0; i < cd.rank_d; ++i) cd.pos_d[i] = (int8_t)i;
-            p->convs.push_back(cd);
-        }
-        if (e == cudaSuccess)
-            e = upload(reinterpret_cast<void **>(&p->conv_dev), p->convs.data(),
-                       p->convs.size() * sizeof(tn::SparseLeafDesc));
-    }
     if (e == cudaSuccess) {
         for (int t = 0; t < n; ++t) {
             auto &d = p->leaves[t];
@@ -561,6 +534,10 @@ static tn_status sparse_plan_impl(const tn_network_t *net, int32_t path_len,
         return fail(e == cudaErrorMemoryAllocation ? TN_ERR_OOM : TN_ERR_CUDA,
                     "sparse-state plan: %s", cudaGetErrorString(e));
     }
+    // where each tensor lies: its arena range, or its dense plan's root tensor
+    p->base.resize(p->ten.size());
+    for (size_t t = 0; t < p->ten.size(); ++t) p->base[t] = p->arena + p->ten[t].off;
+    for (const auto &sb : p->subs) p->base[(size_t)sb.node] = tn::plan_root(sb.plan);
     for (auto &st : p->steps) {
         if (st.grouped) {
             st.g.gA = p->gather + st.ga;
@@ -570,8 +547,8 @@ static tn_status sparse_plan_impl(const tn_network_t *net, int32_t path_len,
             st.g.grp_len = p->gather + st.g_len;
             st.g.tiles = p->gather + st.g_tiles;
         }
-        st.d.A = p->arena + p->ten[st.a].off;
-        st.d.B = p->arena + p->ten[st.b].off;
+        st.d.A = p->base[(size_t)st.a];
+        st.d.B = p->base[(size_t)st.b];
         st.d.C = p->arena + p->ten[st.c].off;
         st.d.sA = (int64_t)1 << p->ten[st.a].dense.size();
         st.d.sB = (int64_t)1 << p->ten[st.b].dense.size();
@@ -590,19 +567,10 @@ tn_status tn_sparse_contract(tn_sparse_plan_t *p, void *amps_dev, void *stream_)
     int dev = 0;
     TN_CUDA(cudaGetDevice(&dev));
     if (dev != p->device) TN_CUDA(cudaSetDevice(p->device));
-    // dense subtrees first: ordinary plans into their complex128 buffers, then into the arena
-    int max_conv = 0;
+    // dense subtrees first, each an ordinary unsliced plan
     for (auto &sb : p->subs) {
-        TN_CUDA(cudaMemsetAsync(sb.out, 0, sizeof(double2) * (size_t)sb.n, stream));
-        tn_plan_info pi{};
-        tn_status ps = tn_plan_get_info(sb.plan, &pi);
-        if (ps == TN_OK) ps = tn_contract(sb.plan, 0, pi.num_slices, sb.out, stream);
+        tn_status ps = tn::plan_run_root(sb.plan, stream);
         if (ps != TN_OK) return ps;
-        max_conv = std::max(max_conv, (int)(63 - __builtin_clzll((uint64_t)sb.n)));
-    }
-    if (!p->subs.empty()) {
-        TN_CUDA(tn::launch_sparse_leaves(p->conv_dev, (int32_t)p->convs.size(), max_conv, stream));
-        p->launches += 1;
     }
     TN_CUDA(tn::launch_sparse_leaves(p->leaves_dev, (int32_t)p->leaves.size(), p->max_leaf_rank,
                                      stream));
@@ -624,7 +592,7 @@ tn_status tn_sparse_contract(tn_sparse_plan_t *p, void *amps_dev, void *stream_)
                                            stream));
         p->launches += 1;
     }
-    TN_CUDA(tn::launch_sparse_amps(p->arena + p->ten[p->root].off, p->sample_idx,
+    TN_CUDA(tn::launch_sparse_amps(p->base[(size_t)p->root], p->sample_idx,
                                    p->num_samples, reinterpret_cast<double2 *>(amps_dev), stream));
     p->launches += 1;
     if (dev != p->device) cudaSetDevice(dev);
