@@ -640,41 +640,60 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
 
 // Thin sparse-state step (at most 16 columns): thread per (configuration c, row m) holding all
 // NN outputs of its row; B[gB[c]] is staged in shared memory 64 values of k at a time, so each
-// element of A is read once.  Block = 256 rows of one configuration.
+// element of A is read once.  A block takes `per` consecutive 256-row chunks of one
+// configuration: the offsets of k, the row's low eight bits and, up to 64 terms, B are set up once
+// for all of them (set up per chunk they took longer than the rows of a short contraction).
+constexpr int kSparseThinKC = 64;
 template <int NN>
 __global__ void __launch_bounds__(256) k_sparse_thin(GenericDesc d, const int32_t *gA,
-                                                     const int32_t *gB, int64_t mblocks) {
-    constexpr int KC = 64;
-    __shared__ float2 Bs[KC][NN];
+                                                     const int32_t *gB, int64_t chunks, int32_t per,
+                                                     int64_t blocks_per_conf) {
+    constexpr int KC = kSparseThinKC;
+    __shared__ __align__(16) float2 Bs[KC][NN];
     __shared__ uint64_t offak[KC], offbk[KC];
     constexpr int ln = NN == 1 ? 0 : NN == 2 ? 1 : NN == 4 ? 2 : NN == 8 ? 3 : 4;  // NN = 2^ln
-    const int lm = d.rank_c - ln, nk = d.nk;
-    const int64_t c = (int64_t)blockIdx.x / mblocks;
-    const int64_t m = ((int64_t)blockIdx.x % mblocks) * 256 + threadIdx.x;
+    const int lm = d.rank_c - ln, nk = d.nk, tid = threadIdx.x, lane = tid & 31;
+    const int64_t c = (int64_t)blockIdx.x / blocks_per_conf;
+    const int64_t first = ((int64_t)blockIdx.x % blocks_per_conf) * per;
+    const int64_t last = first + per < chunks ? first + per : chunks;
     const int64_t M = 1ll << lm, K = 1ll << nk;
     const float2 *A = d.A + (int64_t)gA[c] * d.sA;
     const float2 *B = d.B + (int64_t)gB[c] * d.sB;
-    const bool row_ok = m < M;
-    const uint64_t offm = row_ok ? deposit((uint64_t)m, lm, d.posA_c + ln) : 0;
-    float cr[NN], ci[NN];
-#pragma unroll
-    for (int n = 0; n < NN; ++n) cr[n] = ci[n] = 0.f;
-    for (int64_t k0 = 0; k0 < K; k0 += KC) {
-        const int kc = (int)(K - k0 < KC ? K - k0 : KC);
-        __syncthreads();  // the previous chunk is consumed
-        if (threadIdx.x < kc) {
-            offak[threadIdx.x] = deposit((uint64_t)(k0 + threadIdx.x), nk, d.posA_k);
-            offbk[threadIdx.x] = deposit((uint64_t)(k0 + threadIdx.x), nk, d.posB_k);
+    const int8_t *pm = d.posA_c + ln;
+    const uint64_t row_lo = deposit((uint64_t)tid & (uint64_t)(M - 1), lm < 8 ? lm : 8, pm);
+    auto stage = [&](int64_t k0, int kc) {
+        __syncthreads();  // the previous values are consumed
+        if (tid < kc) {
+            offak[tid] = deposit((uint64_t)(k0 + tid), nk, d.posA_k);
+            offbk[tid] = deposit((uint64_t)(k0 + tid), nk, d.posB_k);
         }
         __syncthreads();
-        for (int e = threadIdx.x; e < kc * NN; e += blockDim.x) {
+        for (int e = tid; e < kc * NN; e += 256) {
             const int kk = e / NN, n = e % NN;
             Bs[kk][n] = B[deposit((uint64_t)n, ln, d.posB_c) | offbk[kk]];
         }
         __syncthreads();
-        if (row_ok)
+    };
+    if (K <= KC) stage(0, (int)K);
+    for (int64_t ch = first; ch < last; ++ch) {
+        uint64_t hi = 0;  // offset of the chunk's row bits 8 and up, one bit per lane
+        for (int i = 8 + lane; i < lm; i += 32)
+            if (((uint64_t)ch >> (i - 8)) & 1ull) hi |= 1ull << pm[i];
+        hi = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(hi >> 32)) << 32) |
+             __reduce_or_sync(0xffffffffu, (uint32_t)hi);
+        const int64_t m = ch * 256 + tid;
+        const bool row_ok = m < M;
+        const float2 *Am = A + (hi | row_lo);
+        float cr[NN], ci[NN];
+#pragma unroll
+        for (int n = 0; n < NN; ++n) cr[n] = ci[n] = 0.f;
+        for (int64_t k0 = 0; k0 < K; k0 += KC) {
+            const int kc = (int)(K - k0 < KC ? K - k0 : KC);
+            if (K > KC) stage(k0, kc);
+            if (!row_ok) continue;
+#pragma unroll 4
             for (int kk = 0; kk < kc; ++kk) {
-                const float2 a = A[offm | offak[kk]];
+                const float2 a = Am[offak[kk]];
 #pragma unroll
                 for (int n = 0; n < NN; ++n) {
                     const float2 b = Bs[kk][n];
@@ -684,11 +703,18 @@ __global__ void __launch_bounds__(256) k_sparse_thin(GenericDesc d, const int32_
                     ci[n] = fmaf(a.y, b.x, ci[n]);
                 }
             }
-    }
-    if (row_ok) {
-        float2 *Cc = d.C + c * d.sC + m * NN;
+        }
+        if (row_ok) {
+            float2 *Cc = d.C + c * d.sC + m * NN;
+            if constexpr (NN == 1) {
+                Cc[0] = make_float2(cr[0], ci[0]);
+            } else {
 #pragma unroll
-        for (int n = 0; n < NN; ++n) Cc[n] = make_float2(cr[n], ci[n]);
+                for (int n = 0; n < NN; n += 2)
+                    *reinterpret_cast<float4 *>(Cc + n) =
+                        make_float4(cr[n], ci[n], cr[n + 1], ci[n + 1]);
+            }
+        }
     }
 }
 
@@ -945,15 +971,22 @@ cudaError_t launch_sparse_thin(const GenericDesc &d, int32_t ln, const int32_t *
     if (nconf <= 0) return cudaSuccess;
     const int lm = d.rank_c - ln;
     if (lm < 0 || ln < 0 || ln > 4) return cudaErrorInvalidValue;
-    const int64_t mblocks = ((1ll << lm) + 255) / 256;
-    const int64_t blocks = mblocks * nconf;
+    // chunks a block, fewer while that leaves under 8 blocks per SM: setting a block up costs as
+    // much as ~2 of its chunks, but blocks in flight then cover fewer configurations and share
+    // less of A in L2.  The 24-qubit batch's 8 one-column steps take 557 / 355 / 328 us with
+    // 1 / 4 / 8 chunks, its 4 four-column steps 567 / 511 / 595 us.
+    const int64_t chunks = ((1ll << lm) + 255) / 256;
+    int32_t per = ln == 0 ? 8 : 4;
+    while (per > 1 && (chunks + per - 1) / per * nconf < 8 * 152) per /= 2;
+    const int64_t bpc = (chunks + per - 1) / per, blocks = bpc * nconf;
     if (blocks > 0x7fffffffll) return cudaErrorInvalidValue;
+    const unsigned g = (unsigned)blocks;
     switch (ln) {
-    case 0: k_sparse_thin<1><<<(unsigned)blocks, 256, 0, st>>>(d, gA, gB, mblocks); break;
-    case 1: k_sparse_thin<2><<<(unsigned)blocks, 256, 0, st>>>(d, gA, gB, mblocks); break;
-    case 2: k_sparse_thin<4><<<(unsigned)blocks, 256, 0, st>>>(d, gA, gB, mblocks); break;
-    case 3: k_sparse_thin<8><<<(unsigned)blocks, 256, 0, st>>>(d, gA, gB, mblocks); break;
-    default: k_sparse_thin<16><<<(unsigned)blocks, 256, 0, st>>>(d, gA, gB, mblocks); break;
+    case 0: k_sparse_thin<1><<<g, 256, 0, st>>>(d, gA, gB, chunks, per, bpc); break;
+    case 1: k_sparse_thin<2><<<g, 256, 0, st>>>(d, gA, gB, chunks, per, bpc); break;
+    case 2: k_sparse_thin<4><<<g, 256, 0, st>>>(d, gA, gB, chunks, per, bpc); break;
+    case 3: k_sparse_thin<8><<<g, 256, 0, st>>>(d, gA, gB, chunks, per, bpc); break;
+    default: k_sparse_thin<16><<<g, 256, 0, st>>>(d, gA, gB, chunks, per, bpc); break;
     }
     return cudaGetLastError();
 }
