@@ -111,6 +111,14 @@ struct tn_sparse_plan {
     tn::SparseLeafDesc *leaves_dev = nullptr;
     double tcc = 0;
     int64_t arena_elems = 0, total_configs = 0, distinct = 0, launches = 0;
+    // CUDA graph of everything but the addition into the caller's amplitudes, and the streams it is
+    // captured on.  It is made at the second call: making it costs more than one call's launches.
+    bool called = false;
+    static constexpr int kLanes = 8;
+    cudaStream_t lanes[kLanes] = {};
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t graph_exec = nullptr;
+    int64_t graph_launches = 0;
 };
 
 namespace {
@@ -120,6 +128,10 @@ void sparse_free(tn_sparse_plan_t *p) {
         if (sb.plan) tn_destroy(sb.plan);
         if (sb.net) tn_destroy(sb.net);
     }
+    if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
+    if (p->graph) cudaGraphDestroy(p->graph);
+    for (cudaStream_t st : p->lanes)
+        if (st) cudaStreamDestroy(st);
     if (p->arena) cudaFree(p->arena);
     if (p->gather) cudaFree(p->gather);
     if (p->cfg_off) cudaFree(p->cfg_off);
@@ -558,6 +570,130 @@ static tn_status sparse_plan_impl(const tn_network_t *net, int32_t path_len,
     return TN_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+tn_status sparse_launch_step(tn_sparse_plan_t *p, size_t k, cudaStream_t stream) {
+    const auto &st = p->steps[k];
+    const int64_t nconf = (int64_t)p->ten[st.c].cfg.size();
+    const int32_t *ga = p->gather + st.ga, *gb = p->gather + st.gb;
+    if (st.grouped) TN_CUDA(tn::launch_sparse_group(st.d, st.ln, st.g, stream));
+    else if (st.gemm) TN_CUDA(tn::launch_sparse_gemm(st.d, st.ln, ga, gb, nconf, stream));
+    else if (st.thin) TN_CUDA(tn::launch_sparse_thin(st.d, st.ln, ga, gb, nconf, stream));
+    else TN_CUDA(tn::launch_sparse_step(st.d, ga, gb, nconf, stream));
+    p->launches += 1;
+    return TN_OK;
+}
+
+// Dense subtrees, leaves and steps, one after the other on one stream.
+tn_status sparse_run(tn_sparse_plan_t *p, cudaStream_t stream) {
+    for (auto &sb : p->subs) {  // each an ordinary unsliced plan
+        tn_status ps = tn::plan_run_root(sb.plan, stream);
+        if (ps != TN_OK) return ps;
+    }
+    TN_CUDA(tn::launch_sparse_leaves(p->leaves_dev, (int32_t)p->leaves.size(), p->max_leaf_rank,
+                                     stream));
+    p->launches += 1;
+    for (size_t k = 0; k < p->steps.size(); ++k) {
+        if (p->skip[k]) continue;
+        tn_status s = sparse_launch_step(p, k, stream);
+        if (s != TN_OK) return s;
+    }
+    return TN_OK;
+}
+
+// The same on the capturing stream lanes[0] and branches of it: every tensor has memory of its
+// own, so only the contraction tree orders the work.  A step goes on in the branch of its first
+// computed operand and waits for the other's; a step of two leaves takes the branches in turn, the
+// dense subtrees too.
+tn_status sparse_capture(tn_sparse_plan_t *p, std::vector<cudaEvent_t> &events) {
+    constexpr int L = tn_sparse_plan::kLanes;
+    auto record = [&](int lane, cudaEvent_t *out) -> cudaError_t {
+        cudaEvent_t ev = nullptr;
+        cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+        if (e != cudaSuccess) return e;
+        events.push_back(ev);
+        *out = ev;
+        return cudaEventRecord(ev, p->lanes[lane]);
+    };
+    std::vector<int> lane_of(p->ten.size(), -1);            // -1: a leaf
+    std::vector<cudaEvent_t> done(p->ten.size(), nullptr);
+    cudaEvent_t ev = nullptr;
+    TN_CUDA(record(0, &ev));
+    for (int i = 1; i < L; ++i) TN_CUDA(cudaStreamWaitEvent(p->lanes[i], ev, 0));
+    int next = 0;
+    // the subtrees first (the leaves' launch does not hold them up)
+    for (auto &sb : p->subs) {
+        next = next % (L - 1) + 1;  // lanes 1 .. L - 1
+        tn_status ps = tn::plan_run_root(sb.plan, p->lanes[next]);
+        if (ps != TN_OK) return ps;
+        lane_of[(size_t)sb.node] = next;
+        TN_CUDA(record(next, &done[(size_t)sb.node]));
+    }
+    TN_CUDA(tn::launch_sparse_leaves(p->leaves_dev, (int32_t)p->leaves.size(), p->max_leaf_rank,
+                                     p->lanes[0]));
+    p->launches += 1;
+    cudaEvent_t leaves = nullptr;
+    TN_CUDA(record(0, &leaves));
+    std::vector<char> has_leaves(L, 0);
+    has_leaves[0] = 1;
+    next = 0;
+    for (size_t k = 0; k < p->steps.size(); ++k) {
+        if (p->skip[k]) continue;
+        const auto &st = p->steps[k];
+        int lane = lane_of[(size_t)st.a] >= 0 ? lane_of[(size_t)st.a] : lane_of[(size_t)st.b];
+        if (lane < 0) {
+            lane = next;
+            next = (next + 1) % L;
+        }
+        if (!has_leaves[lane]) {
+            TN_CUDA(cudaStreamWaitEvent(p->lanes[lane], leaves, 0));
+            has_leaves[lane] = 1;
+        }
+        for (int x : {st.a, st.b})
+            if (lane_of[(size_t)x] >= 0 && lane_of[(size_t)x] != lane)
+                TN_CUDA(cudaStreamWaitEvent(p->lanes[lane], done[(size_t)x], 0));
+        tn_status s = sparse_launch_step(p, k, p->lanes[lane]);
+        if (s != TN_OK) return s;
+        lane_of[(size_t)st.c] = lane;
+        TN_CUDA(record(lane, &done[(size_t)st.c]));
+    }
+    for (int i = 1; i < L; ++i) {  // join
+        TN_CUDA(record(i, &ev));
+        TN_CUDA(cudaStreamWaitEvent(p->lanes[0], ev, 0));
+    }
+    return TN_OK;
+}
+
+// One launch for ~110 and the steps of independent branches at once, for the 24-qubit batch
+// 5.3 -> 4.4 ms.
+tn_status sparse_make_graph(tn_sparse_plan_t *p) {
+    for (auto &st : p->lanes)
+        if (!st) TN_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+    std::vector<cudaEvent_t> events;
+    const int64_t l0 = p->launches;
+    TN_CUDA(cudaStreamBeginCapture(p->lanes[0], cudaStreamCaptureModeThreadLocal));
+    tn_status s = sparse_capture(p, events);
+    cudaGraph_t g = nullptr;
+    cudaError_t e = cudaStreamEndCapture(p->lanes[0], &g);
+    for (cudaEvent_t ev : events) cudaEventDestroy(ev);
+    p->graph_launches = p->launches - l0;
+    p->launches = l0;
+    if (s != TN_OK || e != cudaSuccess) {
+        if (g) cudaGraphDestroy(g);
+        return s != TN_OK ? s : fail(TN_ERR_CUDA, "sparse-state graph capture: %s",
+                                     cudaGetErrorString(e));
+    }
+    p->graph = g;
+    TN_CUDA(cudaGraphInstantiate(&p->graph_exec, p->graph, 0));
+    return TN_OK;
+}
+
+}  // namespace
+
+extern "C" {
+
 tn_status tn_sparse_contract(tn_sparse_plan_t *p, void *amps_dev, void *stream_) {
     tn::clear_error();
     if (!p || p->magic != kSparseMagic)
@@ -567,31 +703,21 @@ tn_status tn_sparse_contract(tn_sparse_plan_t *p, void *amps_dev, void *stream_)
     int dev = 0;
     TN_CUDA(cudaGetDevice(&dev));
     if (dev != p->device) TN_CUDA(cudaSetDevice(p->device));
-    // dense subtrees first, each an ordinary unsliced plan
-    for (auto &sb : p->subs) {
-        tn_status ps = tn::plan_run_root(sb.plan, stream);
-        if (ps != TN_OK) return ps;
+    // a caller that captures this stream gets the launches themselves
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    TN_CUDA(cudaStreamIsCapturing(stream, &capturing));
+    tn_status s = TN_OK;
+    if (capturing != cudaStreamCaptureStatusNone || !p->called) {
+        s = sparse_run(p, stream);
+        p->called = true;
+    } else {
+        if (!p->graph_exec) s = sparse_make_graph(p);
+        if (s == TN_OK) {
+            TN_CUDA(cudaGraphLaunch(p->graph_exec, stream));
+            p->launches += p->graph_launches;
+        }
     }
-    TN_CUDA(tn::launch_sparse_leaves(p->leaves_dev, (int32_t)p->leaves.size(), p->max_leaf_rank,
-                                     stream));
-    p->launches += 1;
-    for (size_t k = 0; k < p->steps.size(); ++k) {
-        const auto &st = p->steps[k];
-        if (p->skip[k]) continue;
-        const int64_t nconf = (int64_t)p->ten[st.c].cfg.size();
-        if (st.grouped)
-            TN_CUDA(tn::launch_sparse_group(st.d, st.ln, st.g, stream));
-        else if (st.gemm)
-            TN_CUDA(tn::launch_sparse_gemm(st.d, st.ln, p->gather + st.ga, p->gather + st.gb,
-                                           nconf, stream));
-        else if (st.thin)
-            TN_CUDA(tn::launch_sparse_thin(st.d, st.ln, p->gather + st.ga, p->gather + st.gb,
-                                           nconf, stream));
-        else
-            TN_CUDA(tn::launch_sparse_step(st.d, p->gather + st.ga, p->gather + st.gb, nconf,
-                                           stream));
-        p->launches += 1;
-    }
+    if (s != TN_OK) return s;
     TN_CUDA(tn::launch_sparse_amps(p->base[(size_t)p->root], p->sample_idx,
                                    p->num_samples, reinterpret_cast<double2 *>(amps_dev), stream));
     p->launches += 1;

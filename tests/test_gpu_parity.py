@@ -1211,3 +1211,36 @@ def test_sparse_state_dense_subtrees_on_ordinary_plans(tn, mode):
     assert info["grouped_steps"] > 0
     sv = O.statevector(circ.n_qubits, circ.gates)
     check(amps.cpu().numpy(), sv[[sv_index(r) for r in smp]], TOL[mode])
+
+
+def test_sparse_state_graph_replay_and_capture(tn):
+    # the first call launches directly, later ones replay a graph of parallel branches, a call on a
+    # capturing stream is recorded: all add the same amplitudes (dense subtree on a plan included)
+    circ = W.random_circuit(3, 4, 8, 5)
+    net = W.build_network(circ, [0, 1, 10, 11], {q: q & 1 for q in range(2, 10)})
+    path = W.greedy_path(net.labels, net.open_labels)
+    rng = np.random.default_rng(9)
+    smp = rng.integers(0, 2, (9, 4), dtype=np.uint8)
+    ref = O.contract_sparse(net.tensors, net.labels, net.open_labels, path, smp)
+    tnet = tn.Network(net.tensors, net.labels, net.open_labels)
+    plan = tn.SparsePlan(tnet, path, smp)
+    amps = torch.zeros(len(smp), dtype=torch.complex128, device="cuda")
+    first = None
+    for _ in range(3):
+        amps.zero_()
+        plan.contract(amps)
+        got = amps.cpu().numpy()
+        check(got, ref, TOL["c64"])
+        assert first is None or np.array_equal(first, got)
+        first = got
+    stream = torch.cuda.Stream()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        with torch.cuda.graph(graph, stream=stream):
+            plan.contract(amps, stream=stream)
+        amps.zero_()
+        graph.replay()
+    torch.cuda.synchronize()
+    assert np.array_equal(first, amps.cpu().numpy())
+    plan.close()
+    tnet.close()
