@@ -184,6 +184,12 @@ struct Chain {               // a run of small element-wise steps launched toget
     int64_t widest = 0;      // items of its widest level
 };
 
+struct Graph {
+    cudaGraph_t graph = nullptr;
+    cudaGraphExec_t exec = nullptr;
+    int64_t launches = 0;    // kernels inside one replay
+};
+
 struct Op {
     int kind;   // 0 bind invariant, 1 step, 2 bind sliced, 3 convert, 4 accumulate
     int index;  // step or planar index
@@ -235,11 +241,11 @@ struct tn_plan {
     int64_t launches = 0;                 // kernels launched by this plan
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> event_pool;
     bool tuned = false;                   // autotune done (first full batch)
-    // CUDA graph of the slice-dependent steps of one full batch (use_graph)
+    // CUDA graphs (use_graph): the slice-independent prologue, the slice-dependent steps of one
+    // full batch, and, when one batch holds every slice, the whole call over all of them (leaf
+    // binding included: its slice ids are then fixed)
     cudaStream_t cap_stream = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t graph_exec = nullptr;
-    int64_t graph_launches = 0;           // kernels inside one replay
+    Graph g_prologue, g_batch, g_call;
     // profile mode: leaf-binding launches bracketed by events, and their running total
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> pending_bind;
     double bind_ms = 0;
@@ -1865,6 +1871,42 @@ const float2 *tn::plan_root(const tn_plan_t *p) {
     return reinterpret_cast<const float2 *>(p->arena) + p->tensors[p->root].off;
 }
 
+// Slice-independent leaves and steps, once per call.
+static tn_status run_prologue(tn_plan_t *p, cudaStream_t stream) {
+    tn_status s = bind_leaves(p, false, 0, 1, stream);
+    if (s != TN_OK) return s;
+    if (p->nmeta_inv > 0)
+        TN_CUDA(cudaMemsetAsync(p->amax(0), 0, sizeof(unsigned int) * p->sb * p->nmeta_inv, stream));
+    for (size_t i = 0; i < p->exec[0].size() && s == TN_OK; ++i)
+        s = run_step(p, p->steps[p->exec[0][i]], 1, stream);
+    return s;
+}
+
+// Replay `g` on `stream`; the first time it is captured from body(stream) on a plan-owned stream.
+template <class F>
+static tn_status replay(tn_plan_t *p, Graph &g, cudaStream_t stream, F body) {
+    if (!g.exec) {
+        if (!p->cap_stream)
+            TN_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
+        const int64_t l0 = p->launches;
+        TN_CUDA(cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal));
+        const tn_status s = body(p->cap_stream);
+        cudaGraph_t graph = nullptr;
+        const cudaError_t e = cudaStreamEndCapture(p->cap_stream, &graph);
+        g.launches = p->launches - l0;
+        p->launches = l0;
+        if (s != TN_OK || e != cudaSuccess) {
+            if (graph) cudaGraphDestroy(graph);
+            return s != TN_OK ? s : fail(TN_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
+        }
+        g.graph = graph;
+        TN_CUDA(cudaGraphInstantiate(&g.exec, g.graph, 0));
+    }
+    TN_CUDA(cudaGraphLaunch(g.exec, stream));
+    p->launches += g.launches;
+    return TN_OK;
+}
+
 // Slices [slice_begin, slice_end) into amps_dev, or without one only into the root tensor.
 static tn_status contract_range(tn_plan_t *p, int64_t slice_begin, int64_t slice_end,
                                 void *amps_dev, void *stream_) {
@@ -1881,73 +1923,56 @@ static tn_status contract_range(tn_plan_t *p, int64_t slice_begin, int64_t slice
     int dev = 0;
     TN_CUDA(cudaGetDevice(&dev));
     if (dev != p->device) TN_CUDA(cudaSetDevice(p->device));
-    float2 *arena = reinterpret_cast<float2 *>(p->arena);
-    // prologue: slice-independent leaves and steps, once per call
-    {
-        tn_status s = bind_leaves(p, false, 0, 1, stream);
-        if (s != TN_OK) return s;
-    }
-    if (p->nmeta_inv > 0)
-        TN_CUDA(cudaMemsetAsync(p->amax(0), 0, sizeof(unsigned int) * p->sb * p->nmeta_inv, stream));
-    for (int k : p->exec[0]) {
-        tn_status s = run_step(p, p->steps[k], 1, stream);
-        if (s != TN_OK) return s;
-    }
     const Tensor &R = p->tensors[p->root];
     const int64_t nout = (int64_t)1 << R.rank();
-    for (int64_t s0 = slice_begin; s0 < slice_end; s0 += p->sb) {
-        const int64_t ns = std::min(p->sb, slice_end - s0);
-        {
-            tn_status s = bind_leaves(p, true, s0, ns, stream);
+    const bool graphs = p->opts.use_graph && !p->opts.profile;
+    auto add = [&](int64_t s0, int64_t ns) -> tn_status {
+        if (!amps_dev) return TN_OK;
+        TN_CUDA(accumulate(p, R, nout, ns, s0, amps_dev, stream));
+        p->launches++;
+        return TN_OK;
+    };
+    tn_status s = TN_OK;
+    if (graphs && (!p->opts.autotune || p->tuned) && slice_begin == 0 &&
+        slice_end == p->num_slices && p->num_slices == p->sb) {
+        s = replay(p, p->g_call, stream, [&](cudaStream_t st) {
+            tn_status e = run_prologue(p, st);
+            if (e == TN_OK) e = bind_leaves(p, true, 0, p->sb, st);
+            return e == TN_OK ? run_batch(p, p->sb, st) : e;
+        });
+        if (s == TN_OK) s = add(0, p->sb);
+        if (s != TN_OK) return s;
+    } else {
+        // the slice-independent leaves and steps, once per call
+        const bool prologue = !p->exec[0].empty() || !p->bind_inv.empty() || !p->tiled_inv.empty();
+        if (prologue)
+            s = graphs ? replay(p, p->g_prologue, stream,
+                                [&](cudaStream_t st) { return run_prologue(p, st); })
+                       : run_prologue(p, stream);
+        if (s != TN_OK) return s;
+        for (int64_t s0 = slice_begin; s0 < slice_end; s0 += p->sb) {
+            const int64_t ns = std::min(p->sb, slice_end - s0);
+            s = bind_leaves(p, true, s0, ns, stream);
             if (s != TN_OK) return s;
-        }
-        if (p->opts.autotune && !p->tuned && ns == p->sb) {
-            // first full batch: tune the tensor-core steps while running it
-            tn_status s = clear_batch_amax(p, stream);
-            if (s != TN_OK) return s;
-            for (int k : p->exec[1]) {
-                Step &st = p->steps[k];
-                s = st.kernel == K_TC ? tune_tc_step(p, st, ns, stream)
-                                      : run_step(p, st, ns, stream);
+            if (p->opts.autotune && !p->tuned && ns == p->sb) {
+                // first full batch: tune the tensor-core steps while running it
+                s = clear_batch_amax(p, stream);
                 if (s != TN_OK) return s;
+                for (int k : p->exec[1]) {
+                    Step &st = p->steps[k];
+                    s = st.kernel == K_TC ? tune_tc_step(p, st, ns, stream)
+                                          : run_step(p, st, ns, stream);
+                    if (s != TN_OK) return s;
+                }
+                p->tuned = true;
+            } else if (graphs && ns == p->sb) {
+                s = replay(p, p->g_batch, stream,
+                           [&](cudaStream_t st) { return run_batch(p, p->sb, st); });
+            } else {
+                s = run_batch(p, ns, stream);
             }
-            p->tuned = true;
-            if (amps_dev) {
-                TN_CUDA(accumulate(p, R, nout, ns, s0, amps_dev, stream));
-                p->launches++;
-            }
-            continue;
-        }
-        const bool graph = p->opts.use_graph && !p->opts.profile && ns == p->sb;
-        if (graph && !p->graph_exec) {
-            // capture the dependent steps once, on a plan-owned stream
-            if (!p->cap_stream)
-                TN_CUDA(cudaStreamCreateWithFlags(&p->cap_stream, cudaStreamNonBlocking));
-            const int64_t l0 = p->launches;
-            TN_CUDA(cudaStreamBeginCapture(p->cap_stream, cudaStreamCaptureModeThreadLocal));
-            tn_status cs = run_batch(p, ns, p->cap_stream);
-            cudaGraph_t g = nullptr;
-            cudaError_t ce = cudaStreamEndCapture(p->cap_stream, &g);
-            if (cs != TN_OK) {
-                if (g) cudaGraphDestroy(g);
-                return cs;
-            }
-            if (ce != cudaSuccess) return fail(TN_ERR_CUDA, "graph capture: %s", cudaGetErrorString(ce));
-            p->graph = g;
-            TN_CUDA(cudaGraphInstantiate(&p->graph_exec, p->graph, 0));
-            p->graph_launches = p->launches - l0;
-            p->launches = l0;
-        }
-        if (graph) {
-            TN_CUDA(cudaGraphLaunch(p->graph_exec, stream));
-            p->launches += p->graph_launches;
-        } else {
-            tn_status s = run_batch(p, ns, stream);
+            if (s == TN_OK) s = add(s0, ns);
             if (s != TN_OK) return s;
-        }
-        if (amps_dev) {
-            TN_CUDA(accumulate(p, R, nout, ns, s0, amps_dev, stream));
-            p->launches++;
         }
     }
     if (p->opts.sync_each_call) {
@@ -2037,8 +2062,10 @@ void tn_destroy(void *handle) {
             cudaEventDestroy(ev.first);
             cudaEventDestroy(ev.second);
         }
-        if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
-        if (p->graph) cudaGraphDestroy(p->graph);
+        for (Graph *g : {&p->g_prologue, &p->g_batch, &p->g_call}) {
+            if (g->exec) cudaGraphExecDestroy(g->exec);
+            if (g->graph) cudaGraphDestroy(g->graph);
+        }
         if (p->cap_stream) cudaStreamDestroy(p->cap_stream);
         p->magic = 0;
         delete p;
