@@ -125,7 +125,9 @@ struct Tensor {
     int64_t off = -1;        // complex64 element offset in the arena
     int t0 = 0, t1 = 0;      // lifetime on the op timeline
     int meta = -1;           // block of per-slice (max-abs, exponent) if some step needs them
-    bool direct = false;     // produced directly as a planar 16-bit copy (no complex64 storage)
+    bool direct = false;     // produced directly as a planar copy (no complex64 storage)
+    bool operand = false;    // a tensor-core operand, or one of a CUDA-core step that writes a
+                             // single-pass 16-bit one directly
     int rank() const { return (int)order.size(); }
     int pos(int label) const {  // bit position of a label in this tensor's memory index
         for (int i = 0; i < rank(); ++i)
@@ -171,6 +173,7 @@ struct Step {
     int chain = -1;              // run of small element-wise steps launched together (k_chain)
     bool chain_head = false;     // first step of its run: launches the whole run
     bool fused_mul = false;      // in a run: products rounded as in k_generic_k1
+    bool stored = true;          // in a run: its result is read outside the run
     // profile mode: recorded (start, stop) event pairs not yet read, and the running totals
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> pending, pending_prep;
     double time_ms = 0, prep_ms = 0;
@@ -179,9 +182,12 @@ struct Step {
 
 struct Chain {               // a run of small element-wise steps launched together
     std::vector<int> steps;
-    int64_t first_level = 0; // its first bound in the plan's level bounds
+    int64_t first_level = 0; // its first bound in the plan's level bounds (global-memory form)
     int nlevels = 0;
     int64_t widest = 0;      // items of its widest level
+    int64_t first_group = 0; // shared-memory form: its groups, and the most elements of one
+    int ngroups = 0;
+    int64_t elems = 0;
 };
 
 struct Graph {
@@ -222,8 +228,12 @@ struct tn_plan {
     std::vector<int> exec[2];              // launch order: chain heads and single steps of the
                                            // slice-independent prologue [0], the slice loop [1]
     std::vector<Chain> chains;             // runs of small element-wise steps (k_chain)
-    tn::ChainItem *chain_items = nullptr;  // the items of every run (device), and behind them
-    int32_t *chain_levels = nullptr;       // the level bounds of every run
+    // the runs' work (device, one allocation): items, copies, records, groups, level bounds
+    tn::ChainItem *chain_items = nullptr;
+    tn::ChainCopy *chain_copies = nullptr;
+    tn::ChainRec *chain_recs = nullptr;
+    tn::ChainGroup *chain_groups = nullptr;
+    int32_t *chain_levels = nullptr;
     int max_rank_inv = 0, max_rank_sl = 0;
     // per-slice max-abs [nmeta][sb], then the exponents [nmeta][sb]; the first nmeta_inv blocks
     // belong to slice-independent tensors
@@ -529,6 +539,57 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
                            int32_t num_sliced, const int32_t *sliced_labels, tn_precision mode,
                            const tn_plan_options *opts, tn_plan_t **out);
 
+// The connected parts of a run (steps joined through tensors made in it), and what each one takes in
+// shared memory: its tensors (whole pairs, so that two elements of K are one 16-byte load), one
+// record per output, and levels.
+struct ChainPart {
+    std::vector<int> steps;  // path order
+    int64_t elems = 0, recs = 0;
+    int depth = 0;
+    int64_t total() const { return elems + recs + 1; }  // records are padded to pairs
+    bool fits() const { return total() <= tn::kChainShmElems && depth <= tn::kChainShmLevels; }
+};
+static int64_t chain_elems(const Tensor &t) { return (int64_t)1 << std::max(1, t.rank()); }
+// whether tensor x is made by a step of run `id`
+static bool made_in_run(const tn_plan_t *p, int id, int x) {
+    const int pr = p->tensors[x].producer;
+    return pr >= 0 && p->steps[pr].chain == id;
+}
+static std::vector<ChainPart> chain_parts(const tn_plan_t *p, const Chain &c) {
+    const int id = p->steps[c.steps[0]].chain;
+    std::unordered_map<int, int> top, part, depth;  // per step: the step that reads its result, if
+                                                    // in the run; its part; its level
+    for (int k : c.steps)
+        for (int x : {p->steps[k].a, p->steps[k].b})
+            if (made_in_run(p, id, x)) top[p->tensors[x].producer] = k;
+    std::vector<ChainPart> parts;
+    for (size_t i = c.steps.size(); i-- > 0;) {  // readers before the steps they read
+        const int k = c.steps[i];
+        const auto t = top.find(k);
+        if (t == top.end()) {
+            part[k] = (int)parts.size();
+            parts.emplace_back();
+        } else {
+            part[k] = part[t->second];
+        }
+    }
+    for (int k : c.steps) {
+        const Step &st = p->steps[k];
+        ChainPart &q = parts[part[k]];
+        q.steps.push_back(k);
+        q.elems += chain_elems(p->tensors[st.c]);
+        q.recs += (int64_t)1 << p->tensors[st.c].rank();
+        int d = 1;
+        for (int x : {st.a, st.b}) {
+            if (made_in_run(p, id, x)) d = std::max(d, depth[p->tensors[x].producer] + 1);
+            else q.elems += chain_elems(p->tensors[x]);
+        }
+        depth[k] = d;
+        q.depth = std::max(q.depth, d);
+    }
+    return parts;
+}
+
 // host allocations of the planners may throw; nothing crosses the C ABI
 extern "C" tn_status tn_plan(const tn_network_t *net, int32_t path_len, const int32_t *path,
                              int32_t num_sliced, const int32_t *sliced_labels, tn_precision mode,
@@ -563,7 +624,7 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
     p->device = net->device;
     if (opts) p->opts = *opts;
     p->tc_ok = tn::tc_available() && tn::tc_prepare() == cudaSuccess;
-    if (tn::simt_prepare() != cudaSuccess) {
+    if (tn::simt_prepare() != cudaSuccess || tn::chain_prepare() != cudaSuccess) {
         delete p;
         return fail(TN_ERR_CUDA, "setting the CUDA-core kernels' shared-memory limit failed");
     }
@@ -840,14 +901,18 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
         auto need_meta = [&](int ti) {
             if (p->tensors[ti].meta < 0) p->tensors[ti].meta = p->nmeta++;
         };
-        for (auto &q : p->planars) need_meta(q.tensor);
+        for (auto &q : p->planars) {
+            need_meta(q.tensor);
+            p->tensors[q.tensor].operand = true;
+        }
         for (auto &q : p->planars)
             if (q.direct) {
                 const Step &pr = p->steps[p->tensors[q.tensor].producer];
-                if (pr.kernel == K_GEMM || pr.kernel == K_STREAM) {
-                    need_meta(pr.a);
-                    need_meta(pr.b);
-                }
+                if (pr.kernel == K_GEMM || pr.kernel == K_STREAM)
+                    for (int x : {pr.a, pr.b}) {
+                        need_meta(x);
+                        if (q.planes != 4 && !tf32_mode(mode)) p->tensors[x].operand = true;
+                    }
             }
         // slice-independent blocks first: they are cleared once per call, the others per batch
         {
@@ -869,10 +934,10 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
         for (auto &x : p->tensors)
             if (x.meta >= 0 && x.producer >= 0) p->steps[x.producer].out_meta = x.meta;
     }
-    // Launch order.  The small element-wise steps run many per launch (k_chain): just before a
-    // larger step that needs one of them, every small step whose operands exist by then joins one
-    // run, wherever the path has it, so a path whose small and large steps alternate still needs
-    // few launches.  The slice-independent prologue and the slice loop are ordered separately.
+    // Launch order.  The small steps run many per launch (k_chain, k_chain_shm): just before a larger
+    // step that needs one of them, every small step whose operands exist by then joins one run,
+    // wherever the path has it, so a path whose small and large steps alternate still needs few
+    // launches.  The slice-independent prologue and the slice loop are ordered separately.
     // Profile mode times every step on its own, in path order.
     for (int cls = 0; cls < 2; ++cls) {
         std::vector<int> todo;
@@ -882,48 +947,78 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
             p->exec[cls] = todo;
             continue;
         }
-        std::vector<char> done(path_len, 0);
-        for (int s = 0; s < path_len; ++s) done[s] = cls == 1 && !p->steps[s].dep;
-        auto small = [&](const Step &st) {
-            const int rc = p->tensors[st.c].rank(), nk = (int)st.K.size();
+        auto rank_c = [&](const Step &st) { return p->tensors[st.c].rank(); };
+        auto tiny = [&](const Step &st) {
+            const int rc = rank_c(st), nk = (int)st.K.size();
             return st.kernel == K_GENERIC && rc <= tn::kChainMaxRankC && nk <= tn::kChainMaxNk &&
                    rc + nk <= tn::kChainMaxWork;
         };
-        // An outer product of 2^10 or more outputs whose max-abs is recorded, or with no small
-        // step beside it in the path, rounds as k_generic_k1 does, the others as k_generic: the
-        // rule looks at the path only, so results do not depend on how steps share launches.
+        // In shared memory a run also takes streaming and GEMM steps of up to 2^16
+        // multiply-adds: a launch of their own costs 4-10 us, the block less than 1.  The sums
+        // are the same bits: one chain over k, or (GEMM, K > 16, too short to be split) blocks of
+        // 16 terms.
+        auto small_shm = [&](const Step &st) {
+            const int rc = rank_c(st), nk = (int)st.K.size();
+            return tiny(st) || ((st.kernel == K_STREAM || st.kernel == K_GEMM) && !st.thin_tc &&
+                                st.direct_planar < 0 && rc <= tn::kChainMaxRankC && nk <= 8 &&
+                                rc + nk <= 16);
+        };
+        // An outer product of 2^10 or more outputs that makes an operand (see Tensor), or with no
+        // other tiny step beside it in the path, rounds as k_generic_k1 does, the others as
+        // k_generic: the rule looks at path and precision only, so results do not depend on how
+        // steps share launches.
         auto plain = [&](size_t i) {
-            return i < todo.size() && small(p->steps[todo[i]]) && p->steps[todo[i]].out_meta < 0;
+            return i < todo.size() && tiny(p->steps[todo[i]]) &&
+                   !p->tensors[p->steps[todo[i]].c].operand;
         };
         for (size_t i = 0; i < todo.size(); ++i) {
             Step &st = p->steps[todo[i]];
-            st.fused_mul = st.K.empty() && p->tensors[st.c].rank() >= 10 &&
-                           (st.out_meta >= 0 || !(plain(i - 1) || plain(i + 1)));
+            st.fused_mul = st.K.empty() && rank_c(st) >= 10 &&
+                           (p->tensors[st.c].operand || !(plain(i - 1) || plain(i + 1)));
         }
-        auto ready = [&](const Step &st) {
-            const int pa = p->tensors[st.a].producer, pb = p->tensors[st.b].producer;
-            return (pa < 0 || done[pa]) && (pb < 0 || done[pb]);
+        const size_t chains0 = p->chains.size();
+        auto schedule = [&](auto small) {
+            std::vector<char> done(path_len, 0);
+            for (int s = 0; s < path_len; ++s) done[s] = cls == 1 && !p->steps[s].dep;
+            auto ready = [&](const Step &st) {
+                const int pa = p->tensors[st.a].producer, pb = p->tensors[st.b].producer;
+                return (pa < 0 || done[pa]) && (pb < 0 || done[pb]);
+            };
+            auto run_small = [&]() {
+                Chain c;
+                for (int s : todo)  // path order, so an operand's producer comes before its reader
+                    if (!done[s] && small(p->steps[s]) && ready(p->steps[s])) {
+                        done[s] = 1;
+                        p->steps[s].chain = (int)p->chains.size();
+                        c.steps.push_back(s);
+                    }
+                if (c.steps.empty()) return;
+                p->steps[c.steps[0]].chain_head = true;
+                p->exec[cls].push_back(c.steps[0]);
+                p->chains.push_back(std::move(c));
+            };
+            for (int s : todo) {
+                if (small(p->steps[s])) continue;
+                if (!ready(p->steps[s])) run_small();
+                done[s] = 1;
+                p->exec[cls].push_back(s);
+            }
+            run_small();
         };
-        auto run_small = [&]() {
-            Chain c;
-            for (int s : todo)  // path order, so an operand's producer comes before its reader
-                if (!done[s] && small(p->steps[s]) && ready(p->steps[s])) {
-                    done[s] = 1;
-                    p->steps[s].chain = (int)p->chains.size();
-                    c.steps.push_back(s);
-                }
-            if (c.steps.empty()) return;
-            p->steps[c.steps[0]].chain_head = true;
-            p->exec[cls].push_back(c.steps[0]);
-            p->chains.push_back(std::move(c));
-        };
-        for (int s : todo) {
-            if (small(p->steps[s])) continue;
-            if (!ready(p->steps[s])) run_small();
-            done[s] = 1;
-            p->exec[cls].push_back(s);
+        schedule(small_shm);
+        bool fits = true;
+        for (size_t c = chains0; c < p->chains.size(); ++c)
+            for (const auto &part : chain_parts(p, p->chains[c]))
+                fits = fits && part.fits();
+        if (!fits) {  // the streaming and GEMM steps need the whole run in shared memory
+            for (int s : todo) {
+                p->steps[s].chain = -1;
+                p->steps[s].chain_head = false;
+            }
+            p->exec[cls].clear();
+            p->chains.resize(chains0);
+            schedule(tiny);
         }
-        run_small();
     }
     // op timeline: invariant leaves, invariant steps, sliced leaves, dependent steps (each
     // tensor-core step preceded by its conversions; a run of chained steps is one op, so every
@@ -1228,79 +1323,217 @@ tn::GenericDesc make_generic_desc(const tn_plan_t *p, const Step &st, unsigned i
     return d;
 }
 
-// Items of every run of small steps (see tn::ChainItem), sorted by the steps' depth in their run.
+// Steps of a run by depth in it.
+std::vector<std::vector<int>> by_depth(const tn_plan_t *p, const std::vector<int> &steps) {
+    const int id = p->steps[steps[0]].chain;
+    std::vector<std::vector<int>> levels;
+    std::unordered_map<int, int> depth;
+    for (int k : steps) {
+        int d = 0;
+        for (int x : {p->steps[k].a, p->steps[k].b})
+            if (made_in_run(p, id, x)) d = std::max(d, depth[p->tensors[x].producer] + 1);
+        depth[k] = d;
+        if ((int)levels.size() <= d) levels.resize(d + 1);
+        levels[d].push_back(k);
+    }
+    return levels;
+}
+
+// How a step of a run addresses its operands: their tensors in the order they are multiplied, and which
+// bits of the result's index are labels of each.
+struct ChainStep {
+    int ta, tb, rc, nk;
+    uint32_t in_a = 0, in_b = 0;
+    uint16_t flags = 0;
+    ChainStep(const tn_plan_t *p, const Step &st) {
+        // the streaming kernels multiply (larger operand) x (smaller): the same order here
+        const bool swap = st.kernel == K_STREAM && st.N.size() > st.M.size();
+        ta = swap ? st.b : st.a;
+        tb = swap ? st.a : st.b;
+        const Tensor &A = p->tensors[ta], &B = p->tensors[tb], &C = p->tensors[st.c];
+        rc = C.rank();
+        nk = (int)st.K.size();
+        for (int i = 0; i < rc; ++i) {
+            const int l = C.order[rc - 1 - i];
+            if (A.pos(l) >= 0) in_a |= 1u << i;
+            if (B.pos(l) >= 0) in_b |= 1u << i;
+        }
+        if (st.fused_mul) flags |= tn::kChainFused;
+        if (st.kernel == K_GEMM && nk > 4) flags |= tn::kChainBlocked;
+    }
+    uint32_t offset(uint32_t c, uint32_t in) const {  // an operand's element for output c
+        uint32_t r = 0;
+        int sh = nk;
+        for (int i = 0; i < rc; ++i)
+            if ((in >> i) & 1u) r |= ((c >> i) & 1u) << sh++;
+        return r;
+    }
+};
+
+uint8_t chain_stride(const Tensor &X) { return X.dep ? (uint8_t)X.rank() : tn::kChainShared; }
+
+// A run in the global-memory form: its level-sorted items.
+void chain_items(const tn_plan_t *p, Chain &c, std::vector<tn::ChainItem> &items,
+                 std::vector<int32_t> &levels) {
+    const int lanes = tn::kChainItemLanes;
+    const auto depth = by_depth(p, c.steps);
+    c.first_level = (int64_t)levels.size();
+    c.nlevels = (int)depth.size();
+    for (const auto &level : depth) {
+        levels.push_back((int32_t)items.size());
+        for (int k : level) {
+            const Step &st = p->steps[k];
+            const ChainStep cs(p, st);
+            const Tensor &A = p->tensors[cs.ta], &B = p->tensors[cs.tb], &C = p->tensors[st.c];
+            tn::ChainItem it{};
+            it.a = (uint32_t)(A.off >> 5);
+            it.b = (uint32_t)(B.off >> 5);
+            it.c = (uint32_t)(C.off >> 5);
+            it.mask_a = (uint8_t)(cs.in_a & (lanes - 1));
+            it.mask_b = (uint8_t)(cs.in_b & (lanes - 1));
+            it.ra = chain_stride(A);
+            it.rb = chain_stride(B);
+            it.rc = chain_stride(C);
+            it.lanes_nk = (uint8_t)(std::min(cs.rc, tn::kChainItemBits) | (cs.nk << 4));
+            it.meta = (uint32_t)(st.out_meta + 1);
+            it.flags = cs.flags;
+            for (uint32_t c0 = 0; c0 < (1u << cs.rc); c0 += lanes) {
+                it.ao = (uint16_t)cs.offset(c0, cs.in_a);
+                it.bo = (uint16_t)cs.offset(c0, cs.in_b);
+                it.co = (uint16_t)c0;
+                items.push_back(it);
+            }
+        }
+        c.widest = std::max(c.widest, (int64_t)items.size() - levels.back());
+    }
+    levels.push_back((int32_t)items.size());
+}
+
+// A group of a run in the shared-memory form.
+tn::ChainGroup chain_group(const tn_plan_t *p, const std::vector<int> &steps,
+                           std::vector<tn::ChainCopy> &copies, std::vector<tn::ChainRec> &recs,
+                           std::vector<int32_t> &levels) {
+    const int id = p->steps[steps[0]].chain;
+    tn::ChainGroup g{};
+    std::unordered_map<int, int> shm;  // tensor -> offset
+    auto take = [&](int x) {
+        shm[x] = g.elems;
+        g.elems += (int32_t)chain_elems(p->tensors[x]);
+    };
+    auto copy = [&](int x, uint32_t meta) {
+        const Tensor &X = p->tensors[x];
+        tn::ChainCopy c{};
+        c.base = (uint32_t)(X.off >> 5);
+        c.meta = meta;
+        c.r = chain_stride(X);
+        c.lanes = (uint8_t)std::min(X.rank(), tn::kChainItemBits);
+        for (uint32_t e = 0; e < (1u << X.rank()); e += tn::kChainItemLanes) {
+            c.off = (uint16_t)e;
+            c.shm = (uint16_t)(shm.at(x) + (int)e);
+            copies.push_back(c);
+        }
+    };
+    g.copies = (int32_t)copies.size();
+    for (int k : steps) {
+        for (int x : {p->steps[k].a, p->steps[k].b})
+            if (!made_in_run(p, id, x)) {
+                take(x);
+                copy(x, 0);
+            }
+        take(p->steps[k].c);
+    }
+    g.n_in = (int32_t)copies.size() - g.copies;
+    for (int k : steps)
+        if (p->steps[k].stored) copy(p->steps[k].c, (uint32_t)(p->steps[k].out_meta + 1));
+    g.n_out = (int32_t)copies.size() - g.copies - g.n_in;
+    g.recs = (int32_t)recs.size();
+    g.levels = (int32_t)levels.size();
+    const auto depth = by_depth(p, steps);
+    g.n_levels = (int32_t)depth.size();
+    for (const auto &level : depth) {
+        levels.push_back((int32_t)recs.size() - g.recs);
+        for (int k : level) {
+            const ChainStep cs(p, p->steps[k]);
+            const int a = shm.at(cs.ta), b = shm.at(cs.tb), c = shm.at(p->steps[k].c);
+            for (uint32_t o = 0; o < (1u << cs.rc); ++o)
+                recs.push_back({(uint16_t)(a + cs.offset(o, cs.in_a)),
+                                (uint16_t)(b + cs.offset(o, cs.in_b)), (uint16_t)(c + o),
+                                (uint16_t)(cs.nk | cs.flags)});
+        }
+    }
+    levels.push_back((int32_t)recs.size() - g.recs);
+    if (recs.size() & 1) recs.push_back({});
+    g.n_recs = (int32_t)recs.size() - g.recs;
+    return g;
+}
+
 tn_status build_chains(tn_plan_t *p) {
     if (p->chains.empty()) return TN_OK;
     std::vector<tn::ChainItem> items;
+    std::vector<tn::ChainCopy> copies;
+    std::vector<tn::ChainRec> recs;
+    std::vector<tn::ChainGroup> groups;
     std::vector<int32_t> levels;
-    std::vector<int> depth(p->steps.size(), -1);
+    // results read outside their run (or by nobody: the root) are stored in the arena
+    for (auto &st : p->steps) st.stored = true;
+    for (const auto &st : p->steps)
+        for (int x : {st.a, st.b})
+            if (st.chain >= 0 && made_in_run(p, st.chain, x))
+                p->steps[p->tensors[x].producer].stored = false;
     for (Chain &c : p->chains) {
-        int deepest = 0;
-        for (int k : c.steps) {
-            const Step &st = p->steps[k];
-            int d = 0;
-            for (int x : {st.a, st.b}) {
-                const int pr = p->tensors[x].producer;
-                if (pr >= 0 && p->steps[pr].chain == st.chain) d = std::max(d, depth[pr] + 1);
-            }
-            depth[k] = d;
-            deepest = std::max(deepest, d);
+        std::vector<ChainPart> parts = chain_parts(p, c);
+        bool fits = true;
+        for (const auto &q : parts) fits = fits && q.fits();
+        if (!fits) {
+            chain_items(p, c, items, levels);
+            continue;
         }
-        c.first_level = (int64_t)levels.size();
-        c.nlevels = deepest + 1;
-        for (int d = 0; d <= deepest; ++d) {
-            levels.push_back((int32_t)items.size());
-            for (int k : c.steps) {
-                if (depth[k] != d) continue;
-                const Step &st = p->steps[k];
-                const Tensor &A = p->tensors[st.a], &B = p->tensors[st.b], &C = p->tensors[st.c];
-                const int rc = C.rank(), nk = (int)st.K.size(), low = std::min(rc, 5);
-                uint32_t in_a = 0, in_b = 0;  // C's index bits that are labels of A, of B
-                for (int i = 0; i < rc; ++i) {
-                    const int l = C.order[rc - 1 - i];
-                    if (A.pos(l) >= 0) in_a |= 1u << i;
-                    if (B.pos(l) >= 0) in_b |= 1u << i;
-                }
-                auto offset = [&](uint32_t c0, uint32_t in) {
-                    uint32_t r = 0;
-                    int sh = nk;
-                    for (int i = 0; i < rc; ++i)
-                        if ((in >> i) & 1u) r |= ((c0 >> i) & 1u) << sh++;
-                    return (uint16_t)r;
-                };
-                auto stride = [&](const Tensor &X) {
-                    return X.dep ? (uint8_t)X.rank() : tn::kChainShared;
-                };
-                tn::ChainItem it{};
-                it.a = (uint32_t)(A.off >> 5);
-                it.b = (uint32_t)(B.off >> 5);
-                it.c = (uint32_t)(C.off >> 5);
-                it.mask_a = (uint8_t)(in_a & 31u);
-                it.mask_b = (uint8_t)(in_b & 31u);
-                it.ra = stride(A);
-                it.rb = stride(B);
-                it.rc = stride(C);
-                it.lanes_nk = (uint8_t)(low | (nk << 4));
-                it.meta = (uint32_t)(st.out_meta + 1);
-                it.fused_mul = st.fused_mul;
-                for (uint32_t c0 = 0; c0 < (1u << rc); c0 += 32) {
-                    it.ao = offset(c0, in_a);
-                    it.bo = offset(c0, in_b);
-                    it.co = (uint16_t)c0;
-                    items.push_back(it);
-                }
+        // Independent parts share blocks: as many groups as fill the GPU with all slices in
+        // flight, each part to the emptiest group, largest part first.
+        std::stable_sort(parts.begin(), parts.end(), [](const ChainPart &x, const ChainPart &y) {
+            return x.total() > y.total();
+        });
+        const int64_t sl = p->steps[c.steps[0]].dep ? p->sb : 1;
+        const int64_t want =
+            std::max<int64_t>(1, std::min<int64_t>((int64_t)parts.size(), 152 / sl));
+        std::vector<ChainPart> gs((size_t)want);
+        for (const auto &q : parts) {
+            size_t best = 0;
+            for (size_t g = 1; g < gs.size(); ++g)
+                if (gs[g].total() < gs[best].total()) best = g;
+            if (gs[best].total() + q.total() > tn::kChainShmElems) {
+                best = gs.size();
+                gs.emplace_back();
             }
-            c.widest = std::max(c.widest, (int64_t)items.size() - levels.back());
+            gs[best].elems += q.elems;
+            gs[best].recs += q.recs;
+            gs[best].steps.insert(gs[best].steps.end(), q.steps.begin(), q.steps.end());
         }
-        levels.push_back((int32_t)items.size());
+        c.first_group = (int64_t)groups.size();
+        c.ngroups = (int)gs.size();
+        for (const auto &g : gs) {
+            groups.push_back(chain_group(p, g.steps, copies, recs, levels));
+            c.elems = std::max<int64_t>(c.elems, groups.back().elems + groups.back().n_recs);
+        }
     }
-    const size_t ib = sizeof(tn::ChainItem) * items.size(), lb = sizeof(int32_t) * levels.size();
-    std::vector<char> host(ib + lb);
-    memcpy(host.data(), items.data(), ib);
-    memcpy(host.data() + ib, levels.data(), lb);
-    TN_CUDA(cudaMalloc(&p->chain_items, ib + lb));
-    TN_CUDA(cudaMemcpy(p->chain_items, host.data(), ib + lb, cudaMemcpyHostToDevice));
-    p->chain_levels = reinterpret_cast<int32_t *>(p->chain_items + items.size());
+    auto bytes = [](const auto &v) { return sizeof(v[0]) * v.size(); };
+    std::vector<char> host;
+    auto add = [&](const auto &v) {  // 16-byte aligned: the sizes of what precedes are multiples
+        const size_t at = host.size();
+        host.resize(at + (bytes(v) + 15) / 16 * 16);
+        if (!v.empty()) memcpy(host.data() + at, v.data(), bytes(v));
+        return at;
+    };
+    const size_t oi = add(items), oc = add(copies), orr = add(recs), og = add(groups),
+                 ol = add(levels);
+    char *dev = nullptr;
+    TN_CUDA(cudaMalloc(&dev, host.size()));
+    p->chain_items = reinterpret_cast<tn::ChainItem *>(dev + oi);
+    p->chain_copies = reinterpret_cast<tn::ChainCopy *>(dev + oc);
+    p->chain_recs = reinterpret_cast<tn::ChainRec *>(dev + orr);
+    p->chain_groups = reinterpret_cast<tn::ChainGroup *>(dev + og);
+    p->chain_levels = reinterpret_cast<int32_t *>(dev + ol);
+    TN_CUDA(cudaMemcpy(dev, host.data(), host.size(), cudaMemcpyHostToDevice));
     return TN_OK;
 }
 
@@ -1482,16 +1715,23 @@ tn_status run_step(tn_plan_t *p, Step &st, int64_t slices, cudaStream_t stream) 
     if (st.chain >= 0) {
         // the run's first step stands for the whole run
         const Chain &c = p->chains[st.chain];
-        // blocks per slice: one while its 16 warps take at most 2 items each, up to a cluster of
-        // 8; more slices than that fills the GPU with need no second block
-        int cluster = 1;
-        while (cluster < tn::kChainMaxCluster &&
-               (int64_t)cluster * 2 * (tn::kChainThreads / 32) < c.widest &&
-               slices * cluster * 2 <= 304)
-            cluster *= 2;
-        const cudaError_t e = tn::launch_chain(
-            p->chain_items, p->chain_levels + c.first_level, c.nlevels,
-            reinterpret_cast<float2 *>(p->arena), p->meta, p->sb, slices, cluster, stream);
+        float2 *arena = reinterpret_cast<float2 *>(p->arena);
+        cudaError_t e;
+        if (c.ngroups > 0) {
+            e = tn::launch_chain_shm(p->chain_groups + c.first_group, c.ngroups, p->chain_copies,
+                                     p->chain_recs, p->chain_levels, c.elems, arena, p->meta,
+                                     p->sb, slices, stream);
+        } else {
+            // blocks per slice: one while its quarter warps take at most 2 items each, up to a
+            // cluster of 8; more slices than that fills the GPU with need no second block
+            int cluster = 1;
+            while (cluster < tn::kChainMaxCluster &&
+                   (int64_t)cluster * 2 * (tn::kChainThreads / tn::kChainItemLanes) < c.widest &&
+                   slices * cluster * 2 <= 304)
+                cluster *= 2;
+            e = tn::launch_chain(p->chain_items, p->chain_levels + c.first_level, c.nlevels, arena,
+                                 p->meta, p->sb, slices, cluster, stream);
+        }
         if (e != cudaSuccess)
             return fail(TN_ERR_CUDA, "step %d chain launch: %s", (int)(&st - &p->steps[0]),
                         cudaGetErrorString(e));

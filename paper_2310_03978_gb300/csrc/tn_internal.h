@@ -86,26 +86,54 @@ constexpr int kChainMaxRankC = 12;
 constexpr int kChainMaxNk = 10;
 constexpr int kChainMaxWork = 14;
 
-// One warp's work in a run of small element-wise steps (k_chain): up to 32 consecutive outputs of
-// one step.  The layout pass stores every operand as [free labels in the result's order][K], so an
-// operand's offset is the output's index restricted to that operand's labels, shifted by nk, and
-// its K elements are contiguous; the masks say which of the output's five lowest bits (the lane)
-// are labels of A and of B, everything above is in ao / bo.
+// Work of a run of small steps.  The layout pass stores every operand as [free labels in the result's
+// order][K], so an operand's offset is the output's index restricted to that operand's labels,
+// shifted by nk, and its K elements are contiguous.
+//
+// Global-memory form (k_chain): an item is up to 8 consecutive outputs of one step, one per lane of
+// a quarter warp; the masks say which of the output's three lowest bits (the lane) are labels of A
+// and of B, everything above is in ao / bo.
 struct __align__(16) ChainItem {
     uint32_t a, b, c;           // arena offsets of the tensors in units of 32 complex64
     uint16_t ao, bo;            // A's and B's element offset of lane 0
     uint16_t co;                // C's element offset of lane 0
     uint8_t mask_a, mask_b;     // lane bits that are labels of A, of B
     uint8_t ra, rb, rc;         // log2 of the slice stride, kChainShared = shared by all slices
-    uint8_t lanes_nk;           // log2 of the outputs (0..5) | contracted bits << 4
+    uint8_t lanes_nk;           // log2 of the outputs (0..3) | contracted bits << 4
     uint32_t meta;              // 1 + block of the result's per-slice max-abs; 0 = not recorded
-    uint32_t fused_mul;         // nk = 0: one rounded product and a fused one (k_generic_k1's
-                                //   form) instead of the general loop's
+    uint32_t flags;             // kChainFused, kChainBlocked
 };
 static_assert(sizeof(ChainItem) == 32, "k_chain loads an item as two 16-byte words");
 constexpr uint8_t kChainShared = 255;
+constexpr uint16_t kChainFused = 16;    // nk = 0: one rounded product and a fused one, as
+                                        //   k_generic_k1, instead of the general loop's
+constexpr uint16_t kChainBlocked = 32;  // sums of 16 terms added up, as k_gemm_simt
 constexpr int kChainThreads = 512;
+constexpr int kChainItemBits = 3, kChainItemLanes = 1 << kChainItemBits;
 constexpr int kChainMaxCluster = 8;
+
+// Shared-memory form (k_chain_shm): every output has a record of its offsets (in complex64) in the
+// block's shared memory, which holds the tensors and, behind them, the records.  Copies bring in
+// the operands made elsewhere and store the results read elsewhere.
+struct __align__(8) ChainRec {
+    uint16_t a, b, c;
+    uint16_t nk_flags;          // contracted bits | kChainFused | kChainBlocked
+};
+struct __align__(16) ChainCopy {  // up to 8 consecutive elements
+    uint32_t base;              // arena offset of the tensor in units of 32 complex64
+    uint16_t off, shm;          // first element in the tensor, and its place in shared memory
+    uint32_t meta;              // results: as in ChainItem
+    uint8_t r, lanes;           // log2 of the slice stride (or kChainShared), log2 of the elements
+    uint16_t pad_;
+};
+struct ChainGroup {             // the work of one block
+    int32_t copies, n_in, n_out;  // first copy; operands, then results
+    int32_t recs, n_recs;         // first record (n_recs is even)
+    int32_t levels, n_levels;     // level l: records [levels[l], levels[l + 1]) from `recs`
+    int32_t elems;                // complex64 of the tensors (even)
+};
+constexpr int kChainShmThreads = 1024, kChainShmLevels = 256;
+constexpr int kChainShmElems = 27 * 1024;  // complex64 that tensors and records may take (216 KB)
 
 // Complex GEMM C[m, n] = sum_k A[m, k] * B[n, k] with A = [M][K] and B = [N][K] row-major per
 // slice and C written at pdep(m -> posC_m) | pdep(n -> posC_n), i.e. in the consumer's order.
@@ -249,7 +277,15 @@ cudaError_t launch_sparse_thin(const GenericDesc &d, int32_t ln, const int32_t *
 // amps[i] += root[idx[i]] for the n samples (complex128 accumulation)
 cudaError_t launch_sparse_amps(const float2 *root, const int32_t *idx, int64_t n, double2 *amps,
                                cudaStream_t st);
-// A run of small steps: items sorted by level, level l = items [levels[l], levels[l + 1]); every
+// Set the chain kernels' shared-memory limit (once per device, outside any stream capture).
+cudaError_t chain_prepare();
+// A run of small steps in shared memory: every slice is worked by `ngroups` independent blocks;
+// `elems`: the most complex64 a group's tensors and records take.
+cudaError_t launch_chain_shm(const ChainGroup *groups, int32_t ngroups, const ChainCopy *copies,
+                             const ChainRec *recs, const int32_t *levels, int64_t elems,
+                             float2 *arena, unsigned int *amax, int64_t sb, int64_t slices,
+                             cudaStream_t st);
+// A run of small steps in global memory: items sorted by level, level l = items [levels[l], levels[l + 1]); every
 // slice is worked by a cluster of `cluster` blocks (a power of two up to kChainMaxCluster).  amax:
 // the plan's max-abs blocks of sb entries each.
 cudaError_t launch_chain(const ChainItem *items, const int32_t *levels, int32_t nlevels,

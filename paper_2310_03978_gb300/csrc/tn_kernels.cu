@@ -18,20 +18,39 @@ __device__ __forceinline__ uint64_t deposit(uint64_t x, int n, const int8_t *pos
     return r;
 }
 
+// Operand offsets of output bits.  An element-wise kernel's thread takes outputs tid + 256 t of a
+// chunk of 2^LB (LB <= 10) consecutive ones: an offset is the OR of the thread's part (bits 0-7,
+// set up once), of t's (bits 8, 9) and of the chunk's (bits LB and up, one bit per lane of the
+// warp).  A block's set-up is then a few dozen instructions; tables of all 2^LB offsets in shared
+// memory took longer to build than a small step's outputs.
+struct LowOffsets {
+    uint64_t own, bit8, bit9;
+    __device__ __forceinline__ LowOffsets(const int8_t *pos, int lb)
+        : own(deposit((uint64_t)(threadIdx.x & ((1 << (lb < 8 ? lb : 8)) - 1)), lb < 8 ? lb : 8, pos)),
+          bit8(lb > 8 && pos[8] >= 0 ? 1ull << pos[8] : 0),
+          bit9(lb > 9 && pos[9] >= 0 ? 1ull << pos[9] : 0) {}
+    __device__ __forceinline__ uint64_t at(int t) const {
+        return own | ((t & 1) ? bit8 : 0) | ((t & 2) ? bit9 : 0);
+    }
+};
+// of bits lb and up of x (n bits in all), the same x in every lane of the warp
+__device__ __forceinline__ uint64_t high_offset(uint64_t x, int lb, int n, const int8_t *pos) {
+    uint64_t r = 0;
+    for (int i = lb + (threadIdx.x & 31); i < n; i += 32)
+        if (((x >> i) & 1ull) && pos[i] >= 0) r |= 1ull << pos[i];
+    return ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(r >> 32)) << 32) |
+           __reduce_or_sync(0xffffffffu, (uint32_t)r);
+}
+
 // One thread per output element of C (in C's own memory order, so stores are coalesced),
-// summing over the contracted bits in increasing order.  A block walks chunks of 2^LB
-// consecutive outputs; the operand offsets of the chunk's low LB bits come from shared-memory
-// tables built once per block, those of the high bits are computed once per chunk.
+// summing over the contracted bits in increasing order; a block walks chunks of 2^LB consecutive
+// outputs (see LowOffsets).
 __global__ void __launch_bounds__(256) k_generic(GenericDesc d, int64_t total) {
     __shared__ uint64_t koffA[1024], koffB[1024];
-    __shared__ uint64_t loA[1024], loB[1024];
     const int nk = d.nk;
     const bool table = nk <= 10;
     const int lb = d.rank_c < 10 ? d.rank_c : 10;
-    for (int j = threadIdx.x; j < (1 << lb); j += blockDim.x) {
-        loA[j] = deposit((uint64_t)j, lb, d.posA_c);
-        loB[j] = deposit((uint64_t)j, lb, d.posB_c);
-    }
+    const LowOffsets la(d.posA_c, lb), lob(d.posB_c, lb);
     if (table) {
         for (int k = threadIdx.x; k < (1 << nk); k += blockDim.x) {
             koffA[k] = deposit((uint64_t)k, nk, d.posA_k);
@@ -46,15 +65,13 @@ __global__ void __launch_bounds__(256) k_generic(GenericDesc d, int64_t total) {
         const int64_t base = ch << lb;
         const int64_t s = base >> d.rank_c;
         const uint64_t c0 = (uint64_t)base & cmask;
-        const uint64_t hA = deposit(c0 >> lb, d.rank_c - lb, d.posA_c + lb);
-        const uint64_t hB = deposit(c0 >> lb, d.rank_c - lb, d.posB_c + lb);
-        const float2 *Ab = d.A + s * d.sA + hA;
-        const float2 *Bb = d.B + s * d.sB + hB;
+        const float2 *Ab = d.A + s * d.sA + high_offset(c0, lb, d.rank_c, d.posA_c);
+        const float2 *Bb = d.B + s * d.sB + high_offset(c0, lb, d.rank_c, d.posB_c);
         float2 *Cb = d.C + s * d.sC + (int64_t)c0;
         float amx = 0.f;
-        for (int j = threadIdx.x; j < (1 << lb); j += blockDim.x) {
-            const float2 *A = Ab + loA[j];
-            const float2 *B = Bb + loB[j];
+        for (int t = 0; (t << 8) + (int)threadIdx.x < (1 << lb); ++t) {
+            const float2 *A = Ab + la.at(t);
+            const float2 *B = Bb + lob.at(t);
             float re = 0.f, im = 0.f;
             for (int64_t k = 0; k < K; ++k) {
                 uint64_t oa, ob;
@@ -71,7 +88,7 @@ __global__ void __launch_bounds__(256) k_generic(GenericDesc d, int64_t total) {
                 im = fmaf(a.x, b.y, im);
                 im = fmaf(a.y, b.x, im);
             }
-            Cb[j] = make_float2(re, im);
+            Cb[(t << 8) + threadIdx.x] = make_float2(re, im);
             amx = fmaxf(amx, fmaxf(fabsf(re), fabsf(im)));
         }
         if (d.amax_out) amax_publish(d.amax_out + s, amx);
@@ -131,16 +148,62 @@ __global__ void __launch_bounds__(256) k_generic_k1(GenericDesc d, int64_t total
     if (cur_s >= 0 && d.amax_out) amax_publish(d.amax_out + cur_s, amx);
 }
 
-// A run of small element-wise steps in one launch.  The steps are sorted by their depth in the
-// run (level 0 reads only what earlier launches wrote), so all steps of a level are independent:
-// the warps of a slice's blocks share out the level's items (32 outputs of one step each), and a
-// barrier separates the levels: the block's own, or the cluster's when several blocks work on one
-// slice.  The plan gives all tensors a run touches pairwise disjoint memory, so nothing else
-// orders the items.  Bound by latency: a level costs one round trip of operand loads and one
-// barrier, so the item of a warp's next level is fetched before the barrier.
-// Measured on GB300, against one block that walked the steps one after the other: 402 steps of a
-// 20-qubit circuit, 16 levels, 1205 -> 25 us; the 12-qubit circuit's call, 366 -> 51 us; 77 runs
-// of a 30-qubit annealed path, 1651 us, are 2 runs, 48 us.
+// Runs of small steps in one launch.  The steps are sorted by their depth in the run (level 0 reads
+// only what earlier launches wrote), so all outputs of a level are independent: the threads of a
+// slice's blocks share them out, and a barrier separates the levels.  The plan gives all tensors
+// a run touches pairwise disjoint memory, so nothing else orders the work.  Bound by the latency
+// of a level, not by its work.
+
+// One output: the sum over 2^nk consecutive elements of A and B.
+__device__ __forceinline__ float2 chain_sum(const float2 *A, const float2 *B, int nk,
+                                            uint32_t flags) {
+    float re = 0.f, im = 0.f;
+    auto mac = [&](float ax, float ay, float bx, float by) {
+        re = fmaf(ax, bx, re);
+        re = fmaf(-ay, by, re);
+        im = fmaf(ax, by, im);
+        im = fmaf(ay, bx, im);
+    };
+    if (nk == 0) {
+        const float2 a = *A, b = *B;
+        if (flags & kChainFused) {
+            re = fmaf(a.x, b.x, -a.y * b.y);
+            im = fmaf(a.x, b.y, a.y * b.x);
+        } else {
+            mac(a.x, a.y, b.x, b.y);
+        }
+        return make_float2(re, im);
+    }
+    const float4 *A4 = reinterpret_cast<const float4 *>(A);
+    const float4 *B4 = reinterpret_cast<const float4 *>(B);
+    if (flags & kChainBlocked) {
+        float2 sum = make_float2(0.f, 0.f);
+        for (int k = 0; k < (1 << (nk - 1)); k += 8) {
+            re = im = 0.f;
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const float4 a = A4[k + q], b = B4[k + q];
+                mac(a.x, a.y, b.x, b.y);
+                mac(a.z, a.w, b.z, b.w);
+            }
+            sum.x += re;
+            sum.y += im;
+        }
+        return sum;
+    }
+#pragma unroll 4
+    for (int k = 0; k < (1 << (nk - 1)); ++k) {
+        const float4 a = A4[k], b = B4[k];
+        mac(a.x, a.y, b.x, b.y);
+        mac(a.z, a.w, b.z, b.w);
+    }
+    return make_float2(re, im);
+}
+
+// Global-memory form, for runs with a connected part too large for shared memory: quarter warps take
+// items of 8 outputs; a cluster of blocks per slice with a cluster barrier per level, or one
+// block.  ~1.1 us a level: 402 steps of a 20-qubit circuit, 16 levels, take 25 us (1205 us by one
+// block, step after step).
 __device__ __forceinline__ uint4 ldg_item(const uint4 *p) {
     uint4 v;
     asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
@@ -149,11 +212,11 @@ __device__ __forceinline__ uint4 ldg_item(const uint4 *p) {
     return v;
 }
 
-// bits of x at the set positions of the 5-bit mask m, packed
-__device__ __forceinline__ uint32_t pack5(uint32_t x, uint32_t m) {
+// bits of x at the set positions of the mask m of an item's lanes, packed
+__device__ __forceinline__ uint32_t pack_lane(uint32_t x, uint32_t m) {
     uint32_t r = 0, sh = 0;
 #pragma unroll
-    for (int i = 0; i < 5; ++i) {
+    for (int i = 0; i < kChainItemBits; ++i) {
         const uint32_t in = (m >> i) & 1u;
         r |= ((x >> i) & in) << sh;
         sh += in;
@@ -161,90 +224,126 @@ __device__ __forceinline__ uint32_t pack5(uint32_t x, uint32_t m) {
     return r;
 }
 
+// max of v over the item's lanes into amax[block][slice], for the items that record it
+__device__ __forceinline__ void chain_amax(unsigned int *amax, int64_t sb, int64_t s, uint32_t meta,
+                                           int lane, float v) {
+    if (!__any_sync(0xffffffffu, meta != 0)) return;
+    for (int o = kChainItemLanes / 2; o > 0; o >>= 1)
+        v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if (meta != 0 && lane == 0)
+        atomicMax(amax + (int64_t)(meta - 1) * sb + s, __float_as_uint(v));
+}
+
 __global__ void __launch_bounds__(kChainThreads)
     k_chain(const ChainItem *items, const int32_t *levels, int32_t nlevels, float2 *arena,
             unsigned int *amax, int64_t sb, int32_t cluster) {
-    constexpr int kWarps = kChainThreads / 32;
+    constexpr int kTeams = kChainThreads / kChainItemLanes;
     const int64_t s = blockIdx.x / cluster;
-    const int rank = blockIdx.x % cluster;
-    const int lane = threadIdx.x & 31, w = rank * kWarps + (threadIdx.x >> 5);
-    const int stride = cluster * kWarps;
+    const int lane = threadIdx.x % kChainItemLanes;
+    const int team = (blockIdx.x % cluster) * kTeams + threadIdx.x / kChainItemLanes;
+    const int stride = cluster * kTeams;
     auto load = [&](int i, uint4 &x, uint4 &y) {
         const uint4 *p = reinterpret_cast<const uint4 *>(items + i);
         x = ldg_item(p);
         y = ldg_item(p + 1);
     };
     int hi = levels[1];
-    int i = levels[0] + w;
-    bool have = i < hi;
+    int i = levels[0] + team;
     uint4 x = make_uint4(0, 0, 0, 0), y = x;
-    if (have) load(i, x, y);
+    if (i < hi) load(i, x, y);
     for (int l = 0; l < nlevels; ++l) {
         const int nhi = l + 1 < nlevels ? levels[l + 2] : hi;
-        while (have) {
-            const bool more = i + stride < hi;
+        while (__any_sync(0xffffffffu, i < hi)) {  // the warp's teams go on together
             uint4 nx = x, ny = y;
-            if (more) load(i + stride, nx, ny);
-            const uint32_t ao = x.w & 0xffffu, bo = x.w >> 16, co = y.x & 0xffffu;
-            const uint32_t ma = (y.x >> 16) & 0xffu, mb = y.x >> 24;
+            if (i + stride < hi) load(i + stride, nx, ny);
             const uint32_t ra = y.y & 0xffu, rb = (y.y >> 8) & 0xffu, rc = (y.y >> 16) & 0xffu;
             const int lanes = (y.y >> 24) & 15, nk = y.y >> 28;
             float amx = 0.f;
-            if (lane < (1 << lanes)) {
-                const float2 *A = arena + ((int64_t)x.x << 5) + ao + (pack5(lane, ma) << nk) +
-                                  (ra == kChainShared ? 0 : s << ra);
-                const float2 *B = arena + ((int64_t)x.y << 5) + bo + (pack5(lane, mb) << nk) +
-                                  (rb == kChainShared ? 0 : s << rb);
-                float2 *C = arena + ((int64_t)x.z << 5) + co + lane +
-                            (rc == kChainShared ? 0 : s << rc);
-                float re = 0.f, im = 0.f;
-                auto mac = [&](float ax, float ay, float bx, float by) {
-                    re = fmaf(ax, bx, re);
-                    re = fmaf(-ay, by, re);
-                    im = fmaf(ax, by, im);
-                    im = fmaf(ay, bx, im);
+            if (i < hi && lane < (1 << lanes)) {
+                auto at = [&](uint32_t base, uint32_t off, uint32_t r) {
+                    return arena + ((int64_t)base << 5) + off + (r == kChainShared ? 0 : s << r);
                 };
-                if (nk == 0) {
-                    const float2 a = *A, b = *B;
-                    if (y.w) {
-                        re = fmaf(a.x, b.x, -a.y * b.y);
-                        im = fmaf(a.x, b.y, a.y * b.x);
-                    } else {
-                        mac(a.x, a.y, b.x, b.y);
-                    }
-                } else {
-                    const float4 *A4 = reinterpret_cast<const float4 *>(A);
-                    const float4 *B4 = reinterpret_cast<const float4 *>(B);
-#pragma unroll 4
-                    for (int k = 0; k < (1 << (nk - 1)); ++k) {
-                        const float4 a = A4[k], b = B4[k];
-                        mac(a.x, a.y, b.x, b.y);
-                        mac(a.z, a.w, b.z, b.w);
-                    }
-                }
-                *C = make_float2(re, im);
-                amx = fmaxf(fabsf(re), fabsf(im));
+                const uint32_t oa = (x.w & 0xffffu) + (pack_lane(lane, (y.x >> 16) & 0xffu) << nk);
+                const uint32_t ob = (x.w >> 16) + (pack_lane(lane, y.x >> 24) << nk);
+                const float2 v = chain_sum(at(x.x, oa, ra), at(x.y, ob, rb), nk, y.w);
+                *at(x.z, (y.x & 0xffffu) + lane, rc) = v;
+                amx = fmaxf(fabsf(v.x), fabsf(v.y));
             }
-            if (y.z) amax_publish(amax + (int64_t)(y.z - 1) * sb + (rc == kChainShared ? 0 : s), amx);
+            chain_amax(amax, sb, rc == kChainShared ? 0 : s, i < hi ? y.z : 0, lane, amx);
             i += stride;
-            have = more;
             x = nx;
             y = ny;
         }
         if (l + 1 < nlevels) {
-            i = hi + w;
-            have = i < nhi;
+            i = hi + team;
             hi = nhi;
-            if (have) load(i, x, y);
+            if (i < hi) load(i, x, y);
             // both barriers make the level's results visible to every warp of the slice
-            if (cluster == 1) {
+            if (cluster == 1)
                 __syncthreads();
-            } else {
+            else
                 asm volatile("barrier.cluster.arrive.release.aligned;\n\t"
                              "barrier.cluster.wait.acquire.aligned;" ::
                                  : "memory");
+        }
+    }
+}
+
+// Shared-memory form: each block works one group of connected steps of one slice.  Everything a level
+// touches (operands, records, results) is in shared memory, so a level is a record load, the
+// operand loads, the sum and a block barrier.  Measured: the 12-qubit circuit (146 steps, 24 levels)
+// in one launch of 20 us, 340 us by one block step after step, ~29 us in the global-memory form
+// with two launches for its GEMM steps; 402 steps of the 20-qubit circuit 8.8 us (25 us global).
+__global__ void __launch_bounds__(kChainShmThreads)
+    k_chain_shm(const ChainGroup *groups, int32_t ngroups, const ChainCopy *copies,
+                const ChainRec *recs, const int32_t *levels, float2 *arena, unsigned int *amax,
+                int64_t sb) {
+    extern __shared__ __align__(16) float2 chain_mem[];
+    __shared__ int32_t bounds[kChainShmLevels + 1];
+    const int64_t s = blockIdx.x / ngroups;
+    const ChainGroup g = groups[blockIdx.x % ngroups];
+    const int tid = threadIdx.x, lane = tid % kChainItemLanes;
+    constexpr int kTeams = kChainShmThreads / kChainItemLanes;
+    float2 *rec_mem = chain_mem + g.elems;
+    auto place = [&](const ChainCopy &c) {
+        return arena + ((int64_t)c.base << 5) + c.off + lane + (c.r == kChainShared ? 0 : s << c.r);
+    };
+    for (int i = tid; i <= g.n_levels; i += kChainShmThreads) bounds[i] = levels[g.levels + i];
+    {
+        const uint4 *src = reinterpret_cast<const uint4 *>(recs + g.recs);
+        uint4 *dst = reinterpret_cast<uint4 *>(rec_mem);
+        for (int i = tid; i < g.n_recs / 2; i += kChainShmThreads) dst[i] = src[i];
+    }
+    for (int i = tid / kChainItemLanes; i < g.n_in; i += kTeams) {
+        const ChainCopy c = copies[g.copies + i];
+        if (lane < (1 << c.lanes)) chain_mem[c.shm + lane] = *place(c);
+    }
+    __syncthreads();
+    for (int l = 0; l < g.n_levels; ++l) {
+        const int hi = bounds[l + 1];
+        for (int i = bounds[l] + tid; i < hi; i += kChainShmThreads) {
+            const ChainRec r = reinterpret_cast<const ChainRec *>(rec_mem)[i];
+            chain_mem[r.c] = chain_sum(chain_mem + r.a, chain_mem + r.b, r.nk_flags & 15,
+                                       r.nk_flags);
+        }
+        __syncthreads();
+    }
+    const int i0 = tid / kChainItemLanes;
+    for (int i = i0; __any_sync(0xffffffffu, i < g.n_out); i += kTeams) {
+        uint32_t meta = 0;
+        int64_t ms = 0;
+        float amx = 0.f;
+        if (i < g.n_out) {
+            const ChainCopy c = copies[g.copies + g.n_in + i];
+            meta = c.meta;
+            ms = c.r == kChainShared ? 0 : s;
+            if (lane < (1 << c.lanes)) {
+                const float2 v = chain_mem[c.shm + lane];
+                *place(c) = v;
+                amx = fmaxf(fabsf(v.x), fabsf(v.y));
             }
         }
+        chain_amax(amax, sb, ms, meta, lane, amx);
     }
 }
 
@@ -265,60 +364,43 @@ __global__ void k_sparse_leaves(const SparseLeafDesc *leaves) {
 
 // One sparse-state step, summing over the contracted dense bits in increasing order; the operand
 // entries are the configurations gA[c], gB[c] (the projections of c onto each operand's open
-// labels).  A block walks chunks of 2^LB consecutive outputs (LB <= 10; chunks never leave a
-// configuration, small ones go several at a time), whose operand offsets come from a table built
-// once per block; the bits above LB are deposited by the warp's lanes in parallel.  Bound by the
+// labels).  A block walks chunks of 2^LB consecutive outputs (see LowOffsets; chunks never leave a
+// configuration, those of less than 256 outputs go several at a time).  Bound by the
 // instructions per output: a deposit per output made the 2^24-output steps take 4 times as long.
 __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_t *gA,
                                                      const int32_t *gB, int64_t nconf) {
     __shared__ uint64_t koffA[1024], koffB[1024];
-    __shared__ uint64_t loA[1024], loB[1024];
-    const int nk = d.nk, lane = threadIdx.x & 31;
+    const int nk = d.nk;
     const bool table = nk <= 10;
     const int lb = d.rank_c < 10 ? d.rank_c : 10;
+    const LowOffsets la(d.posA_c, lb), lob(d.posB_c, lb);
     if (table)
         for (int k = threadIdx.x; k < (1 << nk); k += 256) {
             koffA[k] = deposit((uint64_t)k, nk, d.posA_k);
             koffB[k] = deposit((uint64_t)k, nk, d.posB_k);
         }
-    for (int j = threadIdx.x; j < (1 << lb); j += 256) {
-        loA[j] = deposit((uint64_t)j, lb, d.posA_c);
-        loB[j] = deposit((uint64_t)j, lb, d.posB_c);
-    }
     __syncthreads();
     const int64_t K = 1ll << nk;
     const int64_t chunks = nconf << (d.rank_c - lb);
     const int together = lb < 8 ? 256 >> lb : 1;  // chunks a block takes at once
+    const int j0 = together > 1 ? threadIdx.x & ((1 << lb) - 1) : threadIdx.x;
     for (int64_t ch0 = (int64_t)blockIdx.x * together; ch0 < chunks;
          ch0 += (int64_t)gridDim.x * together) {
         const int64_t ch = ch0 + (together > 1 ? (int)threadIdx.x >> lb : 0);
-        const int64_t c = (ch < chunks ? ch : ch0) >> (d.rank_c - lb);
         uint64_t ha = 0, hb = 0;
+        const uint64_t hi = ((uint64_t)ch << lb) & ((1ull << d.rank_c) - 1);
         if (d.rank_c > lb) {  // one chunk at a time: the same for every thread
-            const uint64_t hi = (uint64_t)ch & ((1ull << (d.rank_c - lb)) - 1);
-            const int i = lb + lane;
-            if (i < d.rank_c && ((hi >> lane) & 1ull)) {
-                if (d.posA_c[i] >= 0) ha = 1ull << d.posA_c[i];
-                if (d.posB_c[i] >= 0) hb = 1ull << d.posB_c[i];
-            }
-            ha = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(ha >> 32)) << 32) |
-                 __reduce_or_sync(0xffffffffu, (uint32_t)ha);
-            hb = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(hb >> 32)) << 32) |
-                 __reduce_or_sync(0xffffffffu, (uint32_t)hb);
-            for (int q = 32; lb + q < d.rank_c; ++q)  // ranks above lb + 32
-                if ((hi >> q) & 1ull) {
-                    if (d.posA_c[lb + q] >= 0) ha |= 1ull << d.posA_c[lb + q];
-                    if (d.posB_c[lb + q] >= 0) hb |= 1ull << d.posB_c[lb + q];
-                }
+            ha = high_offset(hi, lb, d.rank_c, d.posA_c);
+            hb = high_offset(hi, lb, d.rank_c, d.posB_c);
         }
         if (ch >= chunks) continue;
+        const int64_t c = ch >> (d.rank_c - lb);
         const float2 *Ab = d.A + (int64_t)gA[c] * d.sA + ha;
         const float2 *Bb = d.B + (int64_t)gB[c] * d.sB + hb;
-        float2 *Cb = d.C + c * d.sC + ((ch & ((1ll << (d.rank_c - lb)) - 1)) << lb);
-        const int j0 = together > 1 ? threadIdx.x & ((1 << lb) - 1) : threadIdx.x;
-        for (int j = j0; j < (1 << lb); j += 256) {
-            const float2 *A = Ab + loA[j];
-            const float2 *B = Bb + loB[j];
+        float2 *Cb = d.C + c * d.sC + (int64_t)hi;
+        for (int t = 0; (t << 8) + j0 < (1 << lb); ++t) {
+            const float2 *A = Ab + la.at(t);
+            const float2 *B = Bb + lob.at(t);
             float re = 0.f, im = 0.f;
 #pragma unroll 4
             for (int64_t k = 0; k < K; ++k) {
@@ -330,7 +412,7 @@ __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_
                 im = fmaf(a.x, b.y, im);
                 im = fmaf(a.y, b.x, im);
             }
-            Cb[j] = make_float2(re, im);
+            Cb[(t << 8) + j0] = make_float2(re, im);
         }
     }
 }
@@ -641,6 +723,22 @@ cudaError_t launch_generic(const GenericDesc &d, int64_t slices, cudaStream_t st
         k_generic_k1<<<(unsigned)blocks, 256, 0, st>>>(d, total);
     else
         k_generic<<<(unsigned)blocks, 256, 0, st>>>(d, total);
+    return cudaGetLastError();
+}
+
+cudaError_t chain_prepare() {
+    return cudaFuncSetAttribute(k_chain_shm, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kChainShmElems * 8);
+}
+
+cudaError_t launch_chain_shm(const ChainGroup *groups, int32_t ngroups, const ChainCopy *copies,
+                             const ChainRec *recs, const int32_t *levels, int64_t elems,
+                             float2 *arena, unsigned int *amax, int64_t sb, int64_t slices,
+                             cudaStream_t st) {
+    if (ngroups <= 0 || slices <= 0) return cudaSuccess;
+    if (elems > kChainShmElems || slices * ngroups > 0x7fffffff) return cudaErrorInvalidValue;
+    k_chain_shm<<<(unsigned)(slices * ngroups), kChainShmThreads, (size_t)elems * 8, st>>>(
+        groups, ngroups, copies, recs, levels, arena, amax, sb);
     return cudaGetLastError();
 }
 

@@ -1112,6 +1112,38 @@ def test_runs_of_small_steps_at_item_edges(tn, mode, m, n, k, b, nsl):
     check(got[True], ref, TOL["c64"])
 
 
+# seven connected steps of 2^12 outputs take more than a block's shared memory, so the run works in global
+# memory: alone (a cluster of blocks), two slices, and 256 (one block each).  The last result feeds a
+# tensor-core step, whose exponent comes from the max-abs the run records (values near 2^-40).
+@pytest.mark.parametrize("nsl", [0, 1, 8])
+@pytest.mark.parametrize("mode", ["c64", "fp16_scaled"])
+def test_large_connected_run_of_small_steps(tn, mode, nsl):
+    rng = np.random.default_rng(60 + nsl)
+    wires, S = list(range(12)), list(range(900, 900 + nsl))
+    tensors, labels, path = [crandn(rng, 12 + nsl, 2.0 ** -46)], [wires + S], []
+    if S:
+        tensors.append(crandn(rng, nsl))
+        labels.append(S)
+        path.append((0, 1))
+    for g in range(7):  # one-qubit gates on seven wires
+        tensors.append(crandn(rng, 2))
+        labels.append([100 + g, wires[g]])
+        wires[g] = 100 + g
+        path.append((0, len(tensors) - 1))
+    opens = list(wires)
+    if mode != "c64":
+        K, N = wires[3:9], list(range(500, 513))
+        tensors.append(crandn(rng, 19, 2.0 ** -6))
+        labels.append(K + N)
+        path.append((0, len(tensors) - 1))
+        opens = [l for l in wires if l not in K] + N
+    ref = O.contract(tensors, labels, opens, path)
+    got, info, kernels = gpu_amps(tn, tensors, labels, opens, path, S, mode=mode)
+    assert info["slices_in_flight"] == 1 << nsl
+    assert (kernels[-1] == "gemm_tc") == (mode != "c64")
+    check(got, ref, TOL[mode])
+
+
 # ------------------------------------------------------------------ sparse-state (Sec. 3.3)
 def sparse_amps(tn, tensors, labels, open_labels, path, samples):
     net = tn.Network(tensors, labels, open_labels)
