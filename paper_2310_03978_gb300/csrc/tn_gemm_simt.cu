@@ -1077,7 +1077,7 @@ int rank4(const int *v, int n) {
 }
 }  // namespace
 
-int thin_choose_swizzle(const int8_t *tb_src, int lnt, bool planar, int8_t *phi) {
+int thin_choose_swizzle(const int8_t *tb_src, int lnt, int planar, int8_t *phi) {
     // the 8-byte bank pair (0..15) of element (r, c) is ((r << lnt) & 15) | (c ^ phi(r)): a row
     // bit i adds bit lnt + i (when below 4) and phi[i]; a column bit k adds bit k
     const int nt = 1 << lnt;
@@ -1091,8 +1091,10 @@ int thin_choose_swizzle(const int8_t *tb_src, int lnt, bool planar, int8_t *phi)
         return 1 << sq;
     };
     const int rbits[4] = {128, 129, 130, 131};
-    const int rd[4] = {planar ? tb_src[3] : tb_src[1], tb_src[planar ? 4 : 3],
-                       tb_src[planar ? 5 : 4], tb_src[planar ? 6 : 5]};
+    // sorted tile bits that a half-warp's lanes span in a read
+    const int lanes[3][4] = {{1, 3, 4, 5}, {3, 4, 5, 6}, {2, 3, 4, 5}};
+    int rd[4];
+    for (int q = 0; q < 4; ++q) rd[q] = tb_src[lanes[planar / 2][q]];
     auto score = [&](const int *f) {
         int w[4], r[4];
         for (int q = 0; q < 4; ++q) {

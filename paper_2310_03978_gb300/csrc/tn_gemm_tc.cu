@@ -1276,11 +1276,13 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[N]) {
     }
 }
 
-template <int NT, int KC>
+// PL as for ThinStage: with one body for all results the complex64 and 16-bit ones spilled and ran up
+// to a third slower.
+template <int NT, int KC, int PL>
 __global__ void __launch_bounds__(448, 1)
     k_gemm_thin_tc(const __grid_constant__ ThinTcDesc d, int64_t slices) {
     using F = ThinTcCfg<NT, KC>;
-    constexpr int RS = F::RS, CS = F::CS, NB = F::NB, ROWS = ThinStage<NT>::ROWS;
+    constexpr int RS = F::RS, CS = F::CS, NB = F::NB, ROWS = ThinStage<NT, PL>::ROWS;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(
         (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -1466,23 +1468,22 @@ __global__ void __launch_bounds__(448, 1)
         // gt of a group holds row gt of its tile (TMEM lane 32 (warp % 4) + lane)
         const int grp = warp >> 2, gt = threadIdx.x - ROWS * grp;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
-        ThinStage<NT> stg;
+        ThinStage<NT, PL> stg;
         stg.init(g, gt);
-        constexpr int TASKS = ThinStage<NT>::TASKS, SUBS = ThinStage<NT>::SUBS;
-        constexpr int SPT = ThinStage<NT>::SPT, SPTP = ThinStage<NT>::SPTP;
+        constexpr int SUBS = ThinStage<NT, PL>::SUBS, SPT = ThinStage<NT, PL>::SPT;
         // C offset of tile t of a slice: deposit(t * ROWS); the warp's lanes take one bit each
         auto tile_base = [&](uint32_t t) {
             uint64_t r = 0;
-            for (int b = ThinStage<NT>::LR + lane; b < g.lm; b += 32)
-                if ((t >> (b - ThinStage<NT>::LR)) & 1u) r |= 1ull << g.posC_m[b];
+            for (int b = ThinStage<NT, PL>::LR + lane; b < g.lm; b += 32)
+                if ((t >> (b - ThinStage<NT, PL>::LR)) & 1u) r |= 1ull << g.posC_m[b];
             const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)r);
             const uint32_t hi = __reduce_or_sync(0xffffffffu, (uint32_t)(r >> 32));
             return ((uint64_t)hi << 32) | lo;
         };
         float cr[NT], ci[NT];
         float amx = 0.f;
-        const int eo = g.planar_out ? planar_out_exponent(g.pout, s) : 0;
-        if (g.planar_out && blockIdx.x == 0 && threadIdx.x == 0) g.pout.exps[s] = eo;
+        const int eo = PL ? planar_out_exponent(g.pout, s) : 0;
+        if (PL && blockIdx.x == 0 && threadIdx.x == 0) g.pout.exps[s] = eo;
         int j = 0;  // tiles this group has drained
         for (uint32_t tile = blockIdx.x + grp * gridDim.x; tile < tps;
              tile += 2 * gridDim.x, ++j) {
@@ -1514,18 +1515,19 @@ __global__ void __launch_bounds__(448, 1)
             stg.put(stage, gt, cr, ci);
             named_sync(3 + grp, ROWS);
             const uint64_t cbase = tile_base(tile);
-            if (g.planar_out) {
+            if constexpr (PL != 0) {
+                constexpr int N = PL == 4 ? 4 : 8;  // elements of a task
 #pragma unroll
-                for (int q = 0; q < SPTP; ++q) {
-                    if (TASKS % ROWS != 0 && gt + ROWS * q >= TASKS) break;
-                    float2 w[8];
+                for (int q = 0; q < SPT; ++q) {
+                    if (SUBS % ROWS != 0 && gt + ROWS * q >= SUBS) break;
+                    float2 w[N];
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
+                    for (int e = 0; e < N; ++e) {
                         w[e] = stg.at(stage, q, e);
                         amx = fmaxf(amx, fmaxf(fabsf(w[e].x), fabsf(w[e].y)));
                     }
-                    if (g.pout.dtype == 2)
-                        planar_out_store8<4>(g.pout, s, cbase | stg.os[q], w, eo);
+                    if constexpr (PL == 4)
+                        planar_out_store4<4>(g.pout, s, cbase | stg.os[q], w, eo);
                     else
                         planar_out_store8<2>(g.pout, s, cbase | stg.os[q], w, eo);
                 }
@@ -1720,8 +1722,12 @@ cudaError_t launch_pers(const TcGemmDesc &d, int64_t slices, cudaStream_t st) {
 
 template <int NT, int KC>
 cudaError_t configure_thin_tc() {
-    return cudaFuncSetAttribute(k_gemm_thin_tc<NT, KC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                ThinTcCfg<NT, KC>::SMEM_BYTES);
+    cudaError_t e = cudaSuccess;
+    for (auto f : {k_gemm_thin_tc<NT, KC, 0>, k_gemm_thin_tc<NT, KC, 2>, k_gemm_thin_tc<NT, KC, 4>})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     ThinTcCfg<NT, KC>::SMEM_BYTES);
+    return e;
 }
 
 template <int NT, int KC>
@@ -1732,8 +1738,13 @@ cudaError_t launch_thin_tc_t(const ThinTcDesc &d, int64_t slices, cudaStream_t s
     int64_t per_slice = sm_count() / slices;
     if (per_slice < 1) per_slice = 1;
     if (per_slice > tps) per_slice = tps;
-    k_gemm_thin_tc<NT, KC><<<dim3((unsigned)per_slice, (unsigned)slices), F::THREADS,
-                             F::SMEM_BYTES, st>>>(d, slices);
+    const dim3 grid((unsigned)per_slice, (unsigned)slices);
+    if (!d.g.planar_out)
+        k_gemm_thin_tc<NT, KC, 0><<<grid, F::THREADS, F::SMEM_BYTES, st>>>(d, slices);
+    else if (d.g.pout.dtype == 2)
+        k_gemm_thin_tc<NT, KC, 4><<<grid, F::THREADS, F::SMEM_BYTES, st>>>(d, slices);
+    else
+        k_gemm_thin_tc<NT, KC, 2><<<grid, F::THREADS, F::SMEM_BYTES, st>>>(d, slices);
     return cudaGetLastError();
 }
 

@@ -1853,7 +1853,8 @@ tn_status run_step_inner(tn_plan_t *p, const Step &st, int64_t slices, cudaStrea
                             (int)(&st - &p->steps[0]));
         }
         if (on_tc && !st.thin_phi_set) {
-            tn::thin_choose_swizzle(d.tb_src, d.ln, d.planar_out != 0, st.thin_phi);
+            const int planar = !d.planar_out ? 0 : (d.pout.dtype == 2 ? 4 : 2);
+            tn::thin_choose_swizzle(d.tb_src, d.ln, planar, st.thin_phi);
             st.thin_phi_set = true;
         }
         memcpy(d.phi, st.thin_phi, sizeof d.phi);

@@ -202,9 +202,9 @@ struct BindTiled {
 // (each below NT).  Chosen so that the staging writes (a half-warp: 16 consecutive rows, one
 // column) and the reads in C's order (tile bits sorted by position in C, tb_src as
 // sort_tile_bits writes them with row tag 128; a half-warp spans tile bits 1, 3, 4, 5 for
-// complex64 results, 3-6 for planar ones) each touch 16 distinct 8-byte bank pairs where the
+// complex64 results, 3-6 for planar 16-bit (planar = 2) and 2-5 for TF32 ones (4)) each touch 16 distinct 8-byte bank pairs where the
 // layout allows; returns how many of the two patterns are conflict-free.
-int thin_choose_swizzle(const int8_t *tb_src, int lnt, bool planar, int8_t *phi);
+int thin_choose_swizzle(const int8_t *tb_src, int lnt, int planar, int8_t *phi);
 void sort_tile_bits(int tm, int tn, const int8_t *posC_m, const int8_t *posC_n, int row_tag,
                     int8_t *src, int8_t *pos);
 

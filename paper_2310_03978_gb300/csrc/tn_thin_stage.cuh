@@ -18,15 +18,17 @@
 
 namespace tn {
 
-template <int NT>
+// PL: bytes of a planar result's numbers (2 or 4), 0 for a complex64 result.
+template <int NT, int PL>
 struct ThinStage {
     static constexpr int LR = 7, ROWS = 1 << LR;  // rows of a tile (= threads of a group)
     // a tile has ROWS * NT elements: ROWS * NT / 8 runs of 8.  Complex64 results: two lanes
     // share each run (lane half h writes elements 4j + 2h and 4j + 2h + 1 in its store j, so
-    // each store fills whole 32-byte sectors); planar 16-bit results (16 bytes per plane and
-    // run): a lane writes whole runs, consecutive lanes consecutive runs
-    static constexpr int TASKS = ROWS * NT / 8, SUBS = 2 * TASKS;
-    static constexpr int SPT = (SUBS + ROWS - 1) / ROWS, SPTP = (TASKS + ROWS - 1) / ROWS;
+    // each store fills whole 32-byte sectors); planar TF32 results (32 bytes per plane and run):
+    // lane half h writes elements 4h .. 4h + 3; planar 16-bit results (16 bytes): a lane writes
+    // whole runs.  Consecutive lanes write consecutive pieces.
+    static constexpr int SUBS = ROWS * NT / 8 * (PL == 2 ? 1 : 2);
+    static constexpr int SPT = (SUBS + ROWS - 1) / ROWS;
     int phr;                  // column XOR of this thread's own row
     int r0, r1, r2, x0, x1, x2;  // tile bits 0-2: row part * NT, column part ^ phi(row part)
     int qr[SPT], qx[SPT];     // task q of this thread: the same for its run bits
@@ -55,9 +57,9 @@ struct ThinStage {
 #pragma unroll
         for (int i = 0; i < SPT; ++i) {
             const int u = tid + ROWS * i;
-            const int r = d.planar_out ? u : u >> 1, h = d.planar_out ? 0 : u & 1;
+            const int r = PL == 2 ? u : u >> 1, h = PL == 2 ? 0 : u & 1;
             int R = 0, Cc = 0;
-            uint64_t o = h ? 2 : 0;
+            uint64_t o = h ? (PL == 4 ? 4 : 2) : 0;
             for (int q = 3; q < d.tile_bits; ++q)
                 if ((r >> (q - 3)) & 1) {
                     const int sq = d.tb_src[q];
@@ -65,8 +67,8 @@ struct ThinStage {
                     else Cc |= 1 << sq;
                     o |= 1ull << d.tb_pos[q];
                 }
-            qr[i] = R * NT + (h ? r1 : 0);
-            qx[i] = (Cc ^ phi_of(d, R)) ^ (h ? x1 : 0);
+            qr[i] = R * NT + (h ? (PL == 4 ? r2 : r1) : 0);
+            qx[i] = (Cc ^ phi_of(d, R)) ^ (h ? (PL == 4 ? x2 : x1) : 0);
             os[i] = o;
         }
     }
