@@ -1959,7 +1959,8 @@ bool tc_variant_fits(int variant, int lk, int ln) {
 
 // bk_pref / bn_pref: 0 or the K / N tile the caller asks for (K tile in 16-bit elements of a
 // shared-memory row: 32 = 64-byte rows, 64 = 128-byte rows, for both operand types).
-int tc_pick_variant(int form, int lk, int ln, int bk_pref, int bn_pref, bool tf32) {
+int tc_pick_variant(int form, int lk, int lm, int ln, int64_t slices, int bk_pref, int bn_pref,
+                    bool tf32) {
     // short 4M or compensated contractions: the persistent kernel with a 128-, 64- or 32-column
     // tile, unless a tile shape was asked for
     if ((form == 1 || form == 3) && lk >= 3 && lk <= 9 && bk_pref == 0 && bn_pref == 0 &&
@@ -1979,13 +1980,23 @@ int tc_pick_variant(int form, int lk, int ln, int bk_pref, int bn_pref, bool tf3
         if (form == 2) return tf32 ? 22 : 21;
         return tf32 ? 18 : 17;
     }
+    // Longer contractions, results of 128 columns or more.  128 x 128 tiles in all: while they fit
+    // the SMs at once, twice as many SMs as with 128 x 256 tiles share the work (2^9 x 2^9, K =
+    // 2^11: 37 against 60 us); at K = 2^10 and two tiles per SM or more the persistent kernel,
+    // which hides the epilogue, beats 128 x 256 tiles (2^13 x 2^13: 0.44 against 0.56 ms, 2^20 x
+    // 2^10 12.3 against 13.1), from K = 2^11 on their smaller operand traffic counts as much
+    // (2^13 x 2^13: 0.80 ms each).
+    const int64_t tiles = ((int64_t)1 << (lm + ln - 14)) * slices;
+    if (form == 1 && !tf32 && lk == 10 && bk_pref == 0 && bn_pref == 0 && tiles >= 2 * 152)
+        return pers_variant(kPersFp16, 128, false);
+    const bool one_wave = tiles <= 152 && bn_pref != 256;
     if (tf32) {
         if (form == 3) return 11;
         if (form == 2) return 10;
         if (bn_pref == 256 && ln >= 8) return 7;
         if (bk_pref == 64) return 9;
         if (lk <= 9) return 8;
-        return ln >= 8 && bn_pref != 128 ? 7 : 9;
+        return ln >= 8 && bn_pref != 128 && !one_wave ? 7 : 9;
     }
     if (form == 3) return 6;
     if (form == 2) return bk_pref == 64 ? 4 : 3;
@@ -1993,7 +2004,7 @@ int tc_pick_variant(int form, int lk, int ln, int bk_pref, int bn_pref, bool tf3
     if (bk_pref == 32) return lk <= 9 ? 2 : 5;
     if (bk_pref == 64 || bn_pref == 128) return lk <= 9 && bk_pref != 64 ? 2 : 0;
     if (lk <= 9) return 2;
-    return ln >= 8 ? 1 : 0;
+    return ln >= 8 && !one_wave ? 1 : 0;
 }
 
 cudaError_t launch_gemm_tc(const TcGemmDesc &d, int64_t slices, cudaStream_t st) {

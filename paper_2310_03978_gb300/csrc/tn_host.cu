@@ -1580,7 +1580,8 @@ tn_status build_descriptors(tn_plan_t *p) {
     for (auto &st : p->steps) {
         if (st.kernel != K_TC) continue;
         st.variant = tn::tc_pick_variant(st.form == TN_GEMM_3M ? 2 : (st.form == kFormSplit ? 3 : 1),
-                                         (int)st.K.size(), (int)st.N.size(), p->opts.tc_bk,
+                                         (int)st.K.size(), (int)st.M.size(), (int)st.N.size(),
+                                         st.dep ? p->sb : 1, p->opts.tc_bk,
                                          p->opts.tc_bn, tf32_mode(p->mode));
         tn_status s = make_tc_desc(p, st, st.variant, p->tc_desc[&st - &p->steps[0]]);
         if (s != TN_OK) return s;

@@ -382,7 +382,8 @@ int encode_tmap_planar(void *tmap_host, const void *base, int64_t K, int64_t row
                        int64_t depth, int dtype, int bk, int box_rows);
 // Tensor-core kernel variants: pick one for a step (form 1 = 4M, 2 = 3M, 3 = split; preferences
 // 0 = any), and read its K tile (elements per stage), N tile and operand type.
-int tc_pick_variant(int form, int lk, int ln, int bk_pref, int bn_pref, bool tf32);
+int tc_pick_variant(int form, int lk, int lm, int ln, int64_t slices, int bk_pref, int bn_pref,
+                    bool tf32);
 bool tc_variant_tf32(int variant);
 int tc_variant_bk(int variant);
 int tc_variant_bn(int variant);
