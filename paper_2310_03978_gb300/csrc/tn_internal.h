@@ -412,6 +412,77 @@ bool thin_tc_fits(int lm, int ln, int lk);  // 2^8 <= M <= 2^30 rows, 4-16 colum
 int encode_tmap_thin(void *tmap_host, const void *A, int lm, int lk, int64_t depth);
 cudaError_t launch_gemm_thin_tc(const ThinTcDesc &d, int64_t slices, cudaStream_t st);
 
+// Captures launches of a dependency graph as parallel branches of a CUDA graph: `lanes` are streams, the
+// first of them capturing.  A node goes on in the branch that ends with an operand of its own, else
+// takes the branches in turn, and waits for its operands in other branches.
+class Branches {
+public:
+    static constexpr int kLanes = 8;
+    Branches(cudaStream_t *lanes, size_t nodes) : lanes_(lanes), lane_(nodes, -1), done_(nodes) {}
+    ~Branches() {
+        for (cudaEvent_t e : events_) cudaEventDestroy(e);
+    }
+    Branches(const Branches &) = delete;
+    Branches &operator=(const Branches &) = delete;
+    // what is on lanes[0] so far precedes every branch
+    cudaError_t fork() {
+        cudaEvent_t e = nullptr;
+        cudaError_t r = record(0, &e);
+        for (int i = 1; i < kLanes && r == cudaSuccess; ++i)
+            r = cudaStreamWaitEvent(lanes_[i], e, 0);
+        return r;
+    }
+    // the stream of a node that needs the given nodes (negative or unknown ones are ignored)
+    cudaError_t begin(const int *needs, int n, cudaStream_t *stream) {
+        cur_ = -1;
+        for (int i = 0; i < n && cur_ < 0; ++i) {
+            const int l = needs[i] >= 0 ? lane_[(size_t)needs[i]] : -1;
+            if (l >= 0 && last_[l] == needs[i]) cur_ = l;
+        }
+        if (cur_ < 0) {
+            cur_ = next_;
+            next_ = (next_ + 1) % kLanes;
+        }
+        *stream = lanes_[cur_];
+        for (int i = 0; i < n; ++i) {
+            const int l = needs[i] >= 0 ? lane_[(size_t)needs[i]] : -1;
+            if (l < 0 || l == cur_) continue;
+            cudaError_t r = cudaStreamWaitEvent(lanes_[cur_], done_[(size_t)needs[i]], 0);
+            if (r != cudaSuccess) return r;
+        }
+        return cudaSuccess;
+    }
+    // the node whose launches followed begin()
+    cudaError_t end(int node) {
+        lane_[(size_t)node] = cur_;
+        last_[cur_] = node;
+        return record(cur_, &done_[(size_t)node]);
+    }
+    // lanes[0] waits for every branch
+    cudaError_t join() {
+        cudaError_t r = cudaSuccess;
+        for (int i = 1; i < kLanes && r == cudaSuccess; ++i) {
+            cudaEvent_t e = nullptr;
+            r = record(i, &e);
+            if (r == cudaSuccess) r = cudaStreamWaitEvent(lanes_[0], e, 0);
+        }
+        return r;
+    }
+
+private:
+    cudaError_t record(int lane, cudaEvent_t *out) {
+        cudaError_t r = cudaEventCreateWithFlags(out, cudaEventDisableTiming);
+        if (r != cudaSuccess) return r;
+        events_.push_back(*out);
+        return cudaEventRecord(*out, lanes_[lane]);
+    }
+    cudaStream_t *lanes_;
+    std::vector<int> lane_;
+    std::vector<cudaEvent_t> done_, events_;
+    int last_[kLanes] = {-1, -1, -1, -1, -1, -1, -1, -1};
+    int cur_ = 0, next_ = 0;
+};
+
 }  // namespace tn
 
 // A loaded network (tn_network_load): labels and offsets on the host, the complex128 data on the

@@ -114,8 +114,7 @@ struct tn_sparse_plan {
     // CUDA graph of everything but the addition into the caller's amplitudes, and the streams it is
     // captured on.  It is made at the second call: making it costs more than one call's launches.
     bool called = false;
-    static constexpr int kLanes = 8;
-    cudaStream_t lanes[kLanes] = {};
+    cudaStream_t lanes[tn::Branches::kLanes] = {};
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t graph_exec = nullptr;
     int64_t graph_launches = 0;
@@ -604,65 +603,29 @@ tn_status sparse_run(tn_sparse_plan_t *p, cudaStream_t stream) {
 }
 
 // The same on the capturing stream lanes[0] and branches of it: every tensor has memory of its
-// own, so only the contraction tree orders the work.  A step goes on in the branch of its first
-// computed operand and waits for the other's; a step of two leaves takes the branches in turn, the
-// dense subtrees too.
-tn_status sparse_capture(tn_sparse_plan_t *p, std::vector<cudaEvent_t> &events) {
-    constexpr int L = tn_sparse_plan::kLanes;
-    auto record = [&](int lane, cudaEvent_t *out) -> cudaError_t {
-        cudaEvent_t ev = nullptr;
-        cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
-        if (e != cudaSuccess) return e;
-        events.push_back(ev);
-        *out = ev;
-        return cudaEventRecord(ev, p->lanes[lane]);
-    };
-    std::vector<int> lane_of(p->ten.size(), -1);            // -1: a leaf
-    std::vector<cudaEvent_t> done(p->ten.size(), nullptr);
-    cudaEvent_t ev = nullptr;
-    TN_CUDA(record(0, &ev));
-    for (int i = 1; i < L; ++i) TN_CUDA(cudaStreamWaitEvent(p->lanes[i], ev, 0));
-    int next = 0;
-    // the subtrees first (the leaves' launch does not hold them up)
-    for (auto &sb : p->subs) {
-        next = next % (L - 1) + 1;  // lanes 1 .. L - 1
-        tn_status ps = tn::plan_run_root(sb.plan, p->lanes[next]);
-        if (ps != TN_OK) return ps;
-        lane_of[(size_t)sb.node] = next;
-        TN_CUDA(record(next, &done[(size_t)sb.node]));
-    }
+// own, so only the contraction tree orders the work.
+tn_status sparse_capture(tn_sparse_plan_t *p) {
+    tn::Branches br(p->lanes, p->ten.size());
     TN_CUDA(tn::launch_sparse_leaves(p->leaves_dev, (int32_t)p->leaves.size(), p->max_leaf_rank,
                                      p->lanes[0]));
     p->launches += 1;
-    cudaEvent_t leaves = nullptr;
-    TN_CUDA(record(0, &leaves));
-    std::vector<char> has_leaves(L, 0);
-    has_leaves[0] = 1;
-    next = 0;
+    TN_CUDA(br.fork());
+    cudaStream_t stream = nullptr;
+    for (auto &sb : p->subs) {
+        TN_CUDA(br.begin(nullptr, 0, &stream));
+        tn_status ps = tn::plan_run_root(sb.plan, stream);
+        if (ps != TN_OK) return ps;
+        TN_CUDA(br.end(sb.node));
+    }
     for (size_t k = 0; k < p->steps.size(); ++k) {
         if (p->skip[k]) continue;
-        const auto &st = p->steps[k];
-        int lane = lane_of[(size_t)st.a] >= 0 ? lane_of[(size_t)st.a] : lane_of[(size_t)st.b];
-        if (lane < 0) {
-            lane = next;
-            next = (next + 1) % L;
-        }
-        if (!has_leaves[lane]) {
-            TN_CUDA(cudaStreamWaitEvent(p->lanes[lane], leaves, 0));
-            has_leaves[lane] = 1;
-        }
-        for (int x : {st.a, st.b})
-            if (lane_of[(size_t)x] >= 0 && lane_of[(size_t)x] != lane)
-                TN_CUDA(cudaStreamWaitEvent(p->lanes[lane], done[(size_t)x], 0));
-        tn_status s = sparse_launch_step(p, k, p->lanes[lane]);
+        const int needs[2] = {p->steps[k].a, p->steps[k].b};
+        TN_CUDA(br.begin(needs, 2, &stream));
+        tn_status s = sparse_launch_step(p, k, stream);
         if (s != TN_OK) return s;
-        lane_of[(size_t)st.c] = lane;
-        TN_CUDA(record(lane, &done[(size_t)st.c]));
+        TN_CUDA(br.end(p->steps[k].c));
     }
-    for (int i = 1; i < L; ++i) {  // join
-        TN_CUDA(record(i, &ev));
-        TN_CUDA(cudaStreamWaitEvent(p->lanes[0], ev, 0));
-    }
+    TN_CUDA(br.join());
     return TN_OK;
 }
 
@@ -671,13 +634,11 @@ tn_status sparse_capture(tn_sparse_plan_t *p, std::vector<cudaEvent_t> &events) 
 tn_status sparse_make_graph(tn_sparse_plan_t *p) {
     for (auto &st : p->lanes)
         if (!st) TN_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-    std::vector<cudaEvent_t> events;
     const int64_t l0 = p->launches;
     TN_CUDA(cudaStreamBeginCapture(p->lanes[0], cudaStreamCaptureModeThreadLocal));
-    tn_status s = sparse_capture(p, events);
+    tn_status s = sparse_capture(p);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(p->lanes[0], &g);
-    for (cudaEvent_t ev : events) cudaEventDestroy(ev);
     p->graph_launches = p->launches - l0;
     p->launches = l0;
     if (s != TN_OK || e != cudaSuccess) {
