@@ -1938,6 +1938,10 @@ tn_status run_step_inner(tn_plan_t *p, const Step &st, int64_t slices, cudaStrea
         p->launches += 1;
     } else {
         const tn::GenericDesc d = make_generic_desc(p, st, amax_out);
+        for (int j = 0; j < d.nk; ++j)  // the layout pass puts K last, in one order
+            if (d.posA_k[j] != j || d.posB_k[j] != j)
+                return fail(TN_ERR_UNSUPPORTED, "step %d: contracted labels are not the last",
+                            (int)(&st - &p->steps[0]));
         if (ev) TN_CUDA(cudaEventRecord(ev->first, stream));
         e = tn::launch_generic(d, slices, stream);
         if (ev) TN_CUDA(cudaEventRecord(ev->second, stream));

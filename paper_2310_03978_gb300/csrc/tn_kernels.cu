@@ -23,138 +23,77 @@ __device__ __forceinline__ uint64_t deposit(uint64_t x, int n, const int8_t *pos
 // set up once), of t's (bits 8, 9) and of the chunk's (bits LB and up, one bit per lane of the
 // warp).  A block's set-up is then a few dozen instructions; tables of all 2^LB offsets in shared
 // memory took longer to build than a small step's outputs.
+struct Offsets {  // of A and of B
+    uint64_t a, b;
+};
+// bits 0 .. n - 1 of x, both operands in one pass (unrolled: a step's set-up waits for these loads)
+__device__ __forceinline__ Offsets deposit2(uint32_t x, int n, const int8_t *pa, const int8_t *pb) {
+    Offsets r{0, 0};
+#pragma unroll 4
+    for (int i = 0; i < n; ++i) {
+        const int qa = pa[i], qb = pb[i];
+        const uint64_t bit = (x >> i) & 1u;
+        r.a |= qa >= 0 ? bit << qa : 0;
+        r.b |= qb >= 0 ? bit << qb : 0;
+    }
+    return r;
+}
 struct LowOffsets {
-    uint64_t own, bit8, bit9;
-    __device__ __forceinline__ LowOffsets(const int8_t *pos, int lb)
-        : own(deposit((uint64_t)(threadIdx.x & ((1 << (lb < 8 ? lb : 8)) - 1)), lb < 8 ? lb : 8, pos)),
-          bit8(lb > 8 && pos[8] >= 0 ? 1ull << pos[8] : 0),
-          bit9(lb > 9 && pos[9] >= 0 ? 1ull << pos[9] : 0) {}
-    __device__ __forceinline__ uint64_t at(int t) const {
-        return own | ((t & 1) ? bit8 : 0) | ((t & 2) ? bit9 : 0);
+    Offsets own, bit8{0, 0}, bit9{0, 0};
+    __device__ __forceinline__ LowOffsets(const GenericDesc &d, int lb)
+        : own(deposit2(threadIdx.x & ((1u << (lb < 8 ? lb : 8)) - 1), lb < 8 ? lb : 8, d.posA_c,
+                       d.posB_c)) {
+        if (lb > 8) bit8 = deposit2(1, 1, d.posA_c + 8, d.posB_c + 8);
+        if (lb > 9) bit9 = deposit2(1, 1, d.posA_c + 9, d.posB_c + 9);
+    }
+    __device__ __forceinline__ uint64_t a(int t) const {
+        return own.a | ((t & 1) ? bit8.a : 0) | ((t & 2) ? bit9.a : 0);
+    }
+    __device__ __forceinline__ uint64_t b(int t) const {
+        return own.b | ((t & 1) ? bit8.b : 0) | ((t & 2) ? bit9.b : 0);
     }
 };
-// of bits lb and up of x (n bits in all), the same x in every lane of the warp
-__device__ __forceinline__ uint64_t high_offset(uint64_t x, int lb, int n, const int8_t *pos) {
-    uint64_t r = 0;
-    for (int i = lb + (threadIdx.x & 31); i < n; i += 32)
-        if (((x >> i) & 1ull) && pos[i] >= 0) r |= 1ull << pos[i];
-    return ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(r >> 32)) << 32) |
-           __reduce_or_sync(0xffffffffu, (uint32_t)r);
-}
-
-// One thread per output element of C (in C's own memory order, so stores are coalesced),
-// summing over the contracted bits in increasing order; a block walks chunks of 2^LB consecutive
-// outputs (see LowOffsets).
-__global__ void __launch_bounds__(256) k_generic(GenericDesc d, int64_t total) {
-    __shared__ uint64_t koffA[1024], koffB[1024];
-    const int nk = d.nk;
-    const bool table = nk <= 10;
-    const int lb = d.rank_c < 10 ? d.rank_c : 10;
-    const LowOffsets la(d.posA_c, lb), lob(d.posB_c, lb);
-    if (table) {
-        for (int k = threadIdx.x; k < (1 << nk); k += blockDim.x) {
-            koffA[k] = deposit((uint64_t)k, nk, d.posA_k);
-            koffB[k] = deposit((uint64_t)k, nk, d.posB_k);
-        }
-    }
-    __syncthreads();
-    const uint64_t cmask = (d.rank_c >= 63) ? ~0ull : ((1ull << d.rank_c) - 1);
-    const int64_t nchunks = total >> lb;
-    const int64_t K = 1ll << nk;
-    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t base = ch << lb;
-        const int64_t s = base >> d.rank_c;
-        const uint64_t c0 = (uint64_t)base & cmask;
-        const float2 *Ab = d.A + s * d.sA + high_offset(c0, lb, d.rank_c, d.posA_c);
-        const float2 *Bb = d.B + s * d.sB + high_offset(c0, lb, d.rank_c, d.posB_c);
-        float2 *Cb = d.C + s * d.sC + (int64_t)c0;
-        float amx = 0.f;
-        for (int t = 0; (t << 8) + (int)threadIdx.x < (1 << lb); ++t) {
-            const float2 *A = Ab + la.at(t);
-            const float2 *B = Bb + lob.at(t);
-            float re = 0.f, im = 0.f;
-            for (int64_t k = 0; k < K; ++k) {
-                uint64_t oa, ob;
-                if (table) {
-                    oa = koffA[k];
-                    ob = koffB[k];
-                } else {
-                    oa = deposit((uint64_t)k, nk, d.posA_k);
-                    ob = deposit((uint64_t)k, nk, d.posB_k);
-                }
-                const float2 a = A[oa], b = B[ob];
-                re = fmaf(a.x, b.x, re);
-                re = fmaf(-a.y, b.y, re);
-                im = fmaf(a.x, b.y, im);
-                im = fmaf(a.y, b.x, im);
-            }
-            Cb[(t << 8) + threadIdx.x] = make_float2(re, im);
-            amx = fmaxf(amx, fmaxf(fabsf(re), fabsf(im)));
-        }
-        if (d.amax_out) amax_publish(d.amax_out + s, amx);
+// the offsets of the contracted index, up to 10 bits, in shared memory
+__device__ __forceinline__ void k_offsets(const GenericDesc &d, uint64_t *ka, uint64_t *kb) {
+    for (int k = threadIdx.x; k < (1 << d.nk); k += 256) {
+        const Offsets o = deposit2((uint32_t)k, d.nk, d.posA_k, d.posB_k);
+        ka[k] = o.a;
+        kb[k] = o.b;
     }
 }
-
-// Steps with nothing contracted (outer products, with or without batch labels): C[c] = A[a(c)]
-// B[b(c)].  Pure streams of stores, so the per-output work is cut to the bone: a thread keeps
-// the operand offsets of its 4 outputs in each 1024-output chunk in registers (the same in every
-// chunk), the chunk's high-bit offsets come from a warp-parallel deposit (lane i takes output
-// bit 10 + i), and the max-abs is published once per slice a block touches rather than per
-// chunk.
-__global__ void __launch_bounds__(256) k_generic_k1(GenericDesc d, int64_t total) {
-    constexpr int LB = 10, PER = (1 << LB) / 256;
-    const int lane = threadIdx.x & 31;
-    uint64_t oa[PER], ob[PER];
+// of bits lb .. n - 1 of x, the same x in every lane of the warp: lane i keeps the places of bits
+// lb + i and lb + i + 32 (kernel parameters indexed by the lane are read one lane at a time, so
+// not once per chunk)
+struct HighOffsets {
+    int shift, qa[2], qb[2];
+    __device__ __forceinline__ HighOffsets(const GenericDesc &d, int lb)
+        : shift(lb + (threadIdx.x & 31)) {
 #pragma unroll
-    for (int t = 0; t < PER; ++t) {
-        const uint64_t j = (uint64_t)threadIdx.x + 256 * t;
-        oa[t] = deposit(j, LB, d.posA_c);
-        ob[t] = deposit(j, LB, d.posB_c);
-    }
-    const uint64_t cmask = (d.rank_c >= 63) ? ~0ull : ((1ull << d.rank_c) - 1);
-    const int64_t nchunks = total >> LB;
-    int64_t cur_s = -1;
-    float amx = 0.f;
-    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
-        const int64_t base = ch << LB;
-        const int64_t s = base >> d.rank_c;
-        const uint64_t c0 = (uint64_t)base & cmask;
-        if (s != cur_s) {
-            if (cur_s >= 0 && d.amax_out) amax_publish(d.amax_out + cur_s, amx);
-            amx = 0.f;
-            cur_s = s;
+        for (int h = 0; h < 2; ++h) {
+            const int i = shift + 32 * h;
+            qa[h] = i < d.rank_c ? d.posA_c[i] : -1;
+            qb[h] = i < d.rank_c ? d.posB_c[i] : -1;
         }
-        uint64_t ha = 0, hb = 0;
-        for (int i = LB + lane; i < d.rank_c; i += 32)
-            if ((c0 >> i) & 1ull) {
-                if (d.posA_c[i] >= 0) ha |= 1ull << d.posA_c[i];
-                if (d.posB_c[i] >= 0) hb |= 1ull << d.posB_c[i];
-            }
-        ha = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(ha >> 32)) << 32) |
-             __reduce_or_sync(0xffffffffu, (uint32_t)ha);
-        hb = ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(hb >> 32)) << 32) |
-             __reduce_or_sync(0xffffffffu, (uint32_t)hb);
-        const float2 *Ab = d.A + s * d.sA + ha;
-        const float2 *Bb = d.B + s * d.sB + hb;
-        float2 *Cb = d.C + s * d.sC + (int64_t)c0;
+    }
+    __device__ __forceinline__ Offsets at(uint64_t x) const {
+        uint64_t a = 0, b = 0;
 #pragma unroll
-        for (int t = 0; t < PER; ++t) {
-            const float2 a = Ab[oa[t]], b = Bb[ob[t]];
-            const float re = fmaf(a.x, b.x, -a.y * b.y), im = fmaf(a.x, b.y, a.y * b.x);
-            Cb[threadIdx.x + 256 * t] = make_float2(re, im);
-            amx = fmaxf(amx, fmaxf(fabsf(re), fabsf(im)));
+        for (int h = 0; h < 2; ++h) {
+            const uint64_t bit = shift + 32 * h < 64 ? (x >> (shift + 32 * h)) & 1ull : 0;
+            a |= qa[h] >= 0 ? bit << qa[h] : 0;
+            b |= qb[h] >= 0 ? bit << qb[h] : 0;
         }
+        auto all = [](uint64_t v) {
+            return ((uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(v >> 32)) << 32) |
+                   __reduce_or_sync(0xffffffffu, (uint32_t)v);
+        };
+        return Offsets{all(a), all(b)};
     }
-    if (cur_s >= 0 && d.amax_out) amax_publish(d.amax_out + cur_s, amx);
-}
-
-// Runs of small steps in one launch.  The steps are sorted by their depth in the run (level 0 reads
-// only what earlier launches wrote), so all outputs of a level are independent: the threads of a
-// slice's blocks share them out, and a barrier separates the levels.  The plan gives all tensors
-// a run touches pairwise disjoint memory, so nothing else orders the work.  Bound by the latency
-// of a level, not by its work.
+};
 
 // One output: the sum over 2^nk consecutive elements of A and B.
+// UNROLL: pairs of k whose loads are in flight at once; INDEX counts them.
+template <int UNROLL, class INDEX = int>
 __device__ __forceinline__ float2 chain_sum(const float2 *A, const float2 *B, int nk,
                                             uint32_t flags) {
     float re = 0.f, im = 0.f;
@@ -191,14 +130,110 @@ __device__ __forceinline__ float2 chain_sum(const float2 *A, const float2 *B, in
         }
         return sum;
     }
-#pragma unroll 4
-    for (int k = 0; k < (1 << (nk - 1)); ++k) {
+#pragma unroll UNROLL
+    for (INDEX k = 0; k < (INDEX)1 << (nk - 1); ++k) {
         const float4 a = A4[k], b = B4[k];
         mac(a.x, a.y, b.x, b.y);
         mac(a.z, a.w, b.z, b.w);
     }
     return make_float2(re, im);
 }
+
+// One thread per output element of C (in C's own memory order, so stores are coalesced),
+// summing over the contracted elements, which the layout pass puts last and in one order in both
+// operands (16-byte loads of two); a block walks chunks of 2^LB consecutive outputs (see
+// LowOffsets).  2^22 outputs of 2 terms: 57 -> 32 us against tables of K and of the chunk.
+__global__ void __launch_bounds__(256) k_generic(GenericDesc d, int64_t total) {
+    const int lb = d.rank_c < 10 ? d.rank_c : 10;
+    const LowOffsets low(d, lb);
+    const HighOffsets high(d, lb);
+    const uint64_t cmask = (d.rank_c >= 63) ? ~0ull : ((1ull << d.rank_c) - 1);
+    const int64_t nchunks = total >> lb;
+    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
+        const int64_t base = ch << lb;
+        const int64_t s = base >> d.rank_c;
+        const uint64_t c0 = (uint64_t)base & cmask;
+        const Offsets h = high.at(c0);
+        const float2 *Ab = d.A + s * d.sA + h.a;
+        const float2 *Bb = d.B + s * d.sB + h.b;
+        float2 *Cb = d.C + s * d.sC + (int64_t)c0;
+        float amx = 0.f;
+#pragma unroll 2
+        for (int t = 0; (t << 8) + (int)threadIdx.x < (1 << lb); ++t) {
+            const float2 v = chain_sum<4, int64_t>(Ab + low.a(t), Bb + low.b(t), d.nk, 0);
+            Cb[(t << 8) + threadIdx.x] = v;
+            amx = fmaxf(amx, fmaxf(fabsf(v.x), fabsf(v.y)));
+        }
+        if (d.amax_out) amax_publish(d.amax_out + s, amx);
+    }
+}
+
+// Steps with nothing contracted (outer products, with or without batch labels): C[c] = A[a(c)]
+// B[b(c)].  Pure streams of stores, so the per-output work is cut to the bone: a thread takes pairs
+// of consecutive outputs (16-byte stores), PER of them in each chunk of 512 PER outputs, whose
+// operand offsets it keeps in registers (the same in every chunk); the chunk's high-bit offsets come
+// from a warp-parallel deposit, and the max-abs is published once per slice a block touches.
+// 2^26 x 2^2 outputs: 1.07 -> 0.50 ms (5.4 TB/s) against 8-byte stores in 1024-output chunks.
+template <int PER>
+__global__ void __launch_bounds__(256) k_generic_k1(GenericDesc d, int64_t total) {
+    constexpr int LB = PER == 1 ? 9 : (PER == 2 ? 10 : 12);
+    static_assert((1 << LB) == 512 * PER, "outputs of a chunk");
+    // bit 0 (the pair), then the thread's bits 1-8, then t's
+    const Offsets own = deposit2(2 * threadIdx.x, 9, d.posA_c, d.posB_c);
+    const Offsets pair = deposit2(1, 1, d.posA_c, d.posB_c);
+    const HighOffsets high(d, LB);
+    uint64_t oa[PER], ob[PER];
+#pragma unroll
+    for (int t = 0; t < PER; ++t) {
+        const Offsets o = deposit2(t, LB - 9, d.posA_c + 9, d.posB_c + 9);
+        oa[t] = own.a | o.a;
+        ob[t] = own.b | o.b;
+    }
+    const uint64_t cmask = (d.rank_c >= 63) ? ~0ull : ((1ull << d.rank_c) - 1);
+    const int64_t nchunks = total >> LB;
+    int64_t cur_s = -1;
+    float amx = 0.f;
+    for (int64_t ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
+        const int64_t base = ch << LB;
+        const int64_t s = base >> d.rank_c;
+        const uint64_t c0 = (uint64_t)base & cmask;
+        if (s != cur_s) {
+            if (cur_s >= 0 && d.amax_out) amax_publish(d.amax_out + cur_s, amx);
+            amx = 0.f;
+            cur_s = s;
+        }
+        const Offsets h = high.at(c0);
+        const float2 *Ab = d.A + s * d.sA + h.a;
+        const float2 *Bb = d.B + s * d.sB + h.b;
+        float4 *Cb = reinterpret_cast<float4 *>(d.C + s * d.sC + (int64_t)c0) + threadIdx.x;
+        float2 a[PER][2], b[PER][2];
+#pragma unroll
+        for (int t = 0; t < PER; ++t) {
+            a[t][0] = Ab[oa[t]];
+            a[t][1] = Ab[oa[t] | pair.a];
+            b[t][0] = Bb[ob[t]];
+            b[t][1] = Bb[ob[t] | pair.b];
+        }
+#pragma unroll
+        for (int t = 0; t < PER; ++t) {
+            float2 v[2];
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                v[q].x = fmaf(a[t][q].x, b[t][q].x, -a[t][q].y * b[t][q].y);
+                v[q].y = fmaf(a[t][q].x, b[t][q].y, a[t][q].y * b[t][q].x);
+                amx = fmaxf(amx, fmaxf(fabsf(v[q].x), fabsf(v[q].y)));
+            }
+            Cb[256 * t] = make_float4(v[0].x, v[0].y, v[1].x, v[1].y);
+        }
+    }
+    if (cur_s >= 0 && d.amax_out) amax_publish(d.amax_out + cur_s, amx);
+}
+
+// Runs of small steps in one launch.  The steps are sorted by their depth in the run (level 0 reads
+// only what earlier launches wrote), so all outputs of a level are independent: the threads of a
+// slice's blocks share them out, and a barrier separates the levels.  The plan gives all tensors
+// a run touches pairwise disjoint memory, so nothing else orders the work.  Bound by the latency
+// of a level, not by its work.
 
 // Global-memory form, for runs with a connected part too large for shared memory: quarter warps take
 // items of 8 outputs; a cluster of blocks per slice with a cluster barrier per level, or one
@@ -265,7 +300,7 @@ __global__ void __launch_bounds__(kChainThreads)
                 };
                 const uint32_t oa = (x.w & 0xffffu) + (pack_lane(lane, (y.x >> 16) & 0xffu) << nk);
                 const uint32_t ob = (x.w >> 16) + (pack_lane(lane, y.x >> 24) << nk);
-                const float2 v = chain_sum(at(x.x, oa, ra), at(x.y, ob, rb), nk, y.w);
+                const float2 v = chain_sum<8>(at(x.x, oa, ra), at(x.y, ob, rb), nk, y.w);
                 *at(x.z, (y.x & 0xffffu) + lane, rc) = v;
                 amx = fmaxf(fabsf(v.x), fabsf(v.y));
             }
@@ -323,8 +358,8 @@ __global__ void __launch_bounds__(kChainShmThreads)
         const int hi = bounds[l + 1];
         for (int i = bounds[l] + tid; i < hi; i += kChainShmThreads) {
             const ChainRec r = reinterpret_cast<const ChainRec *>(rec_mem)[i];
-            chain_mem[r.c] = chain_sum(chain_mem + r.a, chain_mem + r.b, r.nk_flags & 15,
-                                       r.nk_flags);
+            chain_mem[r.c] = chain_sum<4>(chain_mem + r.a, chain_mem + r.b, r.nk_flags & 15,
+                                          r.nk_flags);
         }
         __syncthreads();
     }
@@ -373,12 +408,9 @@ __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_
     const int nk = d.nk;
     const bool table = nk <= 10;
     const int lb = d.rank_c < 10 ? d.rank_c : 10;
-    const LowOffsets la(d.posA_c, lb), lob(d.posB_c, lb);
-    if (table)
-        for (int k = threadIdx.x; k < (1 << nk); k += 256) {
-            koffA[k] = deposit((uint64_t)k, nk, d.posA_k);
-            koffB[k] = deposit((uint64_t)k, nk, d.posB_k);
-        }
+    const LowOffsets low(d, lb);
+    const HighOffsets high(d, lb);
+    if (table) k_offsets(d, koffA, koffB);
     __syncthreads();
     const int64_t K = 1ll << nk;
     const int64_t chunks = nconf << (d.rank_c - lb);
@@ -387,20 +419,17 @@ __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_
     for (int64_t ch0 = (int64_t)blockIdx.x * together; ch0 < chunks;
          ch0 += (int64_t)gridDim.x * together) {
         const int64_t ch = ch0 + (together > 1 ? (int)threadIdx.x >> lb : 0);
-        uint64_t ha = 0, hb = 0;
         const uint64_t hi = ((uint64_t)ch << lb) & ((1ull << d.rank_c) - 1);
-        if (d.rank_c > lb) {  // one chunk at a time: the same for every thread
-            ha = high_offset(hi, lb, d.rank_c, d.posA_c);
-            hb = high_offset(hi, lb, d.rank_c, d.posB_c);
-        }
+        Offsets h{0, 0};
+        if (d.rank_c > lb) h = high.at(hi);  // one chunk at a time: the same for every thread
         if (ch >= chunks) continue;
         const int64_t c = ch >> (d.rank_c - lb);
-        const float2 *Ab = d.A + (int64_t)gA[c] * d.sA + ha;
-        const float2 *Bb = d.B + (int64_t)gB[c] * d.sB + hb;
+        const float2 *Ab = d.A + (int64_t)gA[c] * d.sA + h.a;
+        const float2 *Bb = d.B + (int64_t)gB[c] * d.sB + h.b;
         float2 *Cb = d.C + c * d.sC + (int64_t)hi;
         for (int t = 0; (t << 8) + j0 < (1 << lb); ++t) {
-            const float2 *A = Ab + la.at(t);
-            const float2 *B = Bb + lob.at(t);
+            const float2 *A = Ab + low.a(t);
+            const float2 *B = Bb + low.b(t);
             float re = 0.f, im = 0.f;
 #pragma unroll 4
             for (int64_t k = 0; k < K; ++k) {
@@ -719,10 +748,18 @@ cudaError_t launch_generic(const GenericDesc &d, int64_t slices, cudaStream_t st
     const int lb = d.rank_c < 10 ? d.rank_c : 10;
     int64_t blocks = total >> lb;
     if (blocks > 152 * 16) blocks = 152 * 16;
-    if (d.nk == 0 && d.rank_c >= 10)
-        k_generic_k1<<<(unsigned)blocks, 256, 0, st>>>(d, total);
-    else
+    if (d.nk == 0 && d.rank_c >= 10) {
+        // large products: chunks of 4096 outputs; small ones keep more blocks busy with 1024
+        if (d.rank_c >= 12 && total >= (int64_t)1 << 23) {
+            blocks = total >> 12;
+            if (blocks > 152 * 8) blocks = 152 * 8;
+            k_generic_k1<8><<<(unsigned)blocks, 256, 0, st>>>(d, total);
+        } else {
+            k_generic_k1<2><<<(unsigned)blocks, 256, 0, st>>>(d, total);
+        }
+    } else {
         k_generic<<<(unsigned)blocks, 256, 0, st>>>(d, total);
+    }
     return cudaGetLastError();
 }
 
