@@ -1384,12 +1384,16 @@ struct ChainStep {
         if (st.fused_mul) flags |= tn::kChainFused;
         if (st.kernel == K_GEMM && nk > 4) flags |= tn::kChainBlocked;
     }
-    uint32_t offset(uint32_t c, uint32_t in) const {  // an operand's element for output c
-        uint32_t r = 0;
+    // an operand's element for every output (those without the operand's labels repeat)
+    std::vector<uint16_t> offsets(uint32_t in) const {
+        std::vector<uint16_t> off((size_t)1 << rc, 0);
         int sh = nk;
-        for (int i = 0; i < rc; ++i)
-            if ((in >> i) & 1u) r |= ((c >> i) & 1u) << sh++;
-        return r;
+        for (int i = 0; i < rc; ++i) {
+            const uint32_t w = (in >> i) & 1u ? 1u << sh++ : 0;
+            for (uint32_t j = 0; j < (1u << i); ++j)
+                off[j | (1u << i)] = (uint16_t)(off[j] + w);
+        }
+        return off;
     }
 };
 
@@ -1420,9 +1424,10 @@ void chain_items(const tn_plan_t *p, Chain &c, std::vector<tn::ChainItem> &items
             it.lanes_nk = (uint8_t)(std::min(cs.rc, tn::kChainItemBits) | (cs.nk << 4));
             it.meta = (uint32_t)(st.out_meta + 1);
             it.flags = cs.flags;
+            const std::vector<uint16_t> oa = cs.offsets(cs.in_a), ob = cs.offsets(cs.in_b);
             for (uint32_t c0 = 0; c0 < (1u << cs.rc); c0 += lanes) {
-                it.ao = (uint16_t)cs.offset(c0, cs.in_a);
-                it.bo = (uint16_t)cs.offset(c0, cs.in_b);
+                it.ao = oa[c0];
+                it.bo = ob[c0];
                 it.co = (uint16_t)c0;
                 items.push_back(it);
             }
@@ -1478,9 +1483,9 @@ tn::ChainGroup chain_group(const tn_plan_t *p, const std::vector<int> &steps,
         for (int k : level) {
             const ChainStep cs(p, p->steps[k]);
             const int a = shm.at(cs.ta), b = shm.at(cs.tb), c = shm.at(p->steps[k].c);
+            const std::vector<uint16_t> oa = cs.offsets(cs.in_a), ob = cs.offsets(cs.in_b);
             for (uint32_t o = 0; o < (1u << cs.rc); ++o)
-                recs.push_back({(uint16_t)(a + cs.offset(o, cs.in_a)),
-                                (uint16_t)(b + cs.offset(o, cs.in_b)), (uint16_t)(c + o),
+                recs.push_back({(uint16_t)(a + oa[o]), (uint16_t)(b + ob[o]), (uint16_t)(c + o),
                                 (uint16_t)(cs.nk | cs.flags)});
         }
     }
