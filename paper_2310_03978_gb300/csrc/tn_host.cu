@@ -125,6 +125,7 @@ struct Tensor {
     int64_t off = -1;        // complex64 element offset in the arena
     int t0 = 0, t1 = 0;      // lifetime on the op timeline
     int meta = -1;           // block of per-slice (max-abs, exponent) if some step needs them
+    bool bound_amax = false;  // a leaf whose max-abs its binding records (k_bind_tiled)
     bool direct = false;     // produced directly as a planar copy (no complex64 storage)
     bool operand = false;    // a tensor-core operand, or one of a CUDA-core step that writes a
                              // single-pass 16-bit one directly
@@ -225,6 +226,7 @@ struct tn_plan {
     bool own_arena = false;
     std::vector<tn::BindItem> bind_inv, bind_sl;
     std::vector<tn::BindTiled> tiled_inv, tiled_sl;  // leaves bound by the tiled permutation
+    bool bind_sl_amax = false;  // some of tiled_sl record their max-abs
     tn::BindItem *bind_inv_dev = nullptr, *bind_sl_dev = nullptr;
     std::vector<int> exec[2];              // launch order: chain heads and single steps of the
                                            // slice-independent prologue [0], the slice loop [1]
@@ -1575,7 +1577,11 @@ tn_status build_descriptors(tn_plan_t *p) {
         if (nsl > 8) return fail(TN_ERR_UNSUPPORTED, "a leaf carries more than 8 sliced labels");
         tn::BindItem it = make_bind(p, t);
         if (t.rank() >= kTiledBindMinRank) {
-            (t.dep ? p->tiled_sl : p->tiled_inv).push_back(make_bind_tiled(it));
+            auto &tiled = t.dep ? p->tiled_sl : p->tiled_inv;
+            tiled.push_back(make_bind_tiled(it));
+            tiled.back().meta = t.meta;
+            t.bound_amax = t.meta >= 0;
+            if (t.dep && t.bound_amax) p->bind_sl_amax = true;
             continue;
         }
         if (t.dep) {
@@ -1635,6 +1641,16 @@ tn_status take_events(tn_plan_t *p, EventPair &ev) {
 
 tn_status make_tc_desc(const tn_plan_t *p, const Step &st, int variant, tn::TcGemmDesc &d);
 
+// The max-abs of tensors is gathered by atomicMax, so it starts from zero: before a call's
+// invariant leaves are bound, and before the first kernel of a batch that gathers one.
+tn_status clear_amax(tn_plan_t *p, bool sliced, cudaStream_t stream) {
+    const int first = sliced ? p->nmeta_inv : 0, end = sliced ? p->nmeta : p->nmeta_inv;
+    if (end > first)
+        TN_CUDA(cudaMemsetAsync(p->amax(first), 0, sizeof(unsigned int) * p->sb * (end - first),
+                                stream));
+    return TN_OK;
+}
+
 // Bind the invariant leaves (sliced = false, once per call) or the sliced leaves of slices
 // [s0, s0 + ns): small leaves in one gather launch, each large leaf by the tiled permutation.
 // Profile mode brackets them with one event pair.
@@ -1642,6 +1658,10 @@ tn_status bind_leaves(tn_plan_t *p, bool sliced, int64_t s0, int64_t ns, cudaStr
     const auto &items = sliced ? p->bind_sl : p->bind_inv;
     const auto &tiled = sliced ? p->tiled_sl : p->tiled_inv;
     if (items.empty() && tiled.empty()) return TN_OK;
+    if (sliced && p->bind_sl_amax) {
+        tn_status s = clear_amax(p, true, stream);
+        if (s != TN_OK) return s;
+    }
     float2 *arena = reinterpret_cast<float2 *>(p->arena);
     const double2 *src = p->net->data;
     EventPair ev{};
@@ -1657,7 +1677,8 @@ tn_status bind_leaves(tn_plan_t *p, bool sliced, int64_t s0, int64_t ns, cudaStr
         p->launches++;
     }
     for (const auto &b : tiled) {
-        TN_CUDA(tn::launch_bind_tiled(b, src, arena, s0, ns, stream));
+        TN_CUDA(tn::launch_bind_tiled(b, src, arena, b.meta >= 0 ? p->amax(b.meta) : nullptr, s0,
+                                      ns, stream));
         p->launches++;
     }
     if (p->opts.profile) {
@@ -1796,7 +1817,7 @@ tn_status run_step_inner(tn_plan_t *p, const Step &st, int64_t slices, cudaStrea
     if ((st.kernel == K_GEMM || st.kernel == K_STREAM) && st.direct_planar >= 0) {
         for (int side = 0; side < 2; ++side) {
             const Tensor &X = side ? B : A;
-            if (X.producer >= 0) continue;
+            if (X.producer >= 0 || X.bound_amax) continue;
             tn::ConvertDesc cd{};
             cd.src = arena + X.off;
             cd.n = (int64_t)1 << X.rank();
@@ -1825,7 +1846,7 @@ tn_status run_step_inner(tn_plan_t *p, const Step &st, int64_t slices, cudaStrea
             cd.exps = p->exps(q.meta);
             cd.dtype = operand_dtype(p->mode);
             cd.planes = q.planes;
-            if (X.producer < 0) {  // a leaf: no producer epilogue recorded its max-abs
+            if (X.producer < 0 && !X.bound_amax) {  // a small leaf: nothing recorded its max-abs
                 TN_CUDA(tn::launch_amax(cd, sx, stream));
                 p->launches += 1;
             }
@@ -2108,20 +2129,12 @@ static cudaError_t accumulate(tn_plan_t *p, const Tensor &R, int64_t nout, int64
                                          amps, stream);
 }
 
-// The max-abs of a batch's tensors is gathered by atomicMax, so it starts from zero.
-static tn_status clear_batch_amax(tn_plan_t *p, cudaStream_t stream) {
-    if (p->nmeta > p->nmeta_inv)
-        TN_CUDA(cudaMemsetAsync(p->amax(p->nmeta_inv), 0,
-                                sizeof(unsigned int) * p->sb * (p->nmeta - p->nmeta_inv), stream));
-    return TN_OK;
-}
-
 static tn_status contract_range(tn_plan_t *p, int64_t slice_begin, int64_t slice_end,
                                 void *amps_dev, void *stream_);
 
 // The slice-dependent steps of one batch of ns slices.
 static tn_status run_batch(tn_plan_t *p, int64_t ns, cudaStream_t stream) {
-    tn_status s = clear_batch_amax(p, stream);
+    tn_status s = p->bind_sl_amax ? TN_OK : clear_amax(p, true, stream);
     for (size_t i = 0; i < p->exec[1].size() && s == TN_OK; ++i)
         s = run_step(p, p->steps[p->exec[1][i]], ns, stream);
     return s;
@@ -2147,10 +2160,9 @@ const float2 *tn::plan_root(const tn_plan_t *p) {
 
 // Slice-independent leaves and steps, once per call.
 static tn_status run_prologue(tn_plan_t *p, cudaStream_t stream) {
-    tn_status s = bind_leaves(p, false, 0, 1, stream);
+    tn_status s = clear_amax(p, false, stream);
+    if (s == TN_OK) s = bind_leaves(p, false, 0, 1, stream);
     if (s != TN_OK) return s;
-    if (p->nmeta_inv > 0)
-        TN_CUDA(cudaMemsetAsync(p->amax(0), 0, sizeof(unsigned int) * p->sb * p->nmeta_inv, stream));
     if (!p->prologue_branches || stream != p->lanes[0]) {
         for (size_t i = 0; i < p->exec[0].size() && s == TN_OK; ++i)
             s = run_step(p, p->steps[p->exec[0][i]], 1, stream);
@@ -2268,7 +2280,7 @@ static tn_status contract_range(tn_plan_t *p, int64_t slice_begin, int64_t slice
             if (s != TN_OK) return s;
             if (p->opts.autotune && !p->tuned && ns == p->sb) {
                 // first full batch: tune the tensor-core steps while running it
-                s = clear_batch_amax(p, stream);
+                if (!p->bind_sl_amax) s = clear_amax(p, true, stream);
                 if (s != TN_OK) return s;
                 for (int k : p->exec[1]) {
                     Step &st = p->steps[k];

@@ -176,7 +176,8 @@ struct BindItem {
 // destination bits of the leaf's six lowest unsliced source bits (contiguous in the source).
 // A block reads a tile in source order (a warp reads 32 consecutive complex128, 512 bytes,
 // 16 bytes per lane), stages it in shared memory and writes it in destination order (16 bytes
-// of two adjacent complex64 per lane).  The remaining destination bits number the tiles.
+// of two adjacent complex64 per lane).  The remaining destination bits number the tiles.  For a
+// leaf that a later kernel scales, the blocks record its max-abs per slice.
 struct BindTiled {
     int64_t dst_off;            // element offset of the destination (complex64) in the arena
     int64_t dst_sstride;        // slice stride of the destination (0 = invariant leaf)
@@ -185,7 +186,7 @@ struct BindTiled {
     int32_t t;                  // tile bits (11..12, fewer only for ranks below 11)
     int32_t nrest;              // rank - t
     int32_t nsl;                // sliced labels of this leaf
-    int32_t pad_;
+    int32_t meta;               // meta block that takes the leaf's max-abs (-1 = none)
     int8_t e2t[12];             // read-order bit q -> tile bit
     int8_t e2s[12];             // read-order bit q -> source bit
     int8_t t2d[12];             // tile bit -> destination bit (bits 0-5 map to themselves)
@@ -303,7 +304,8 @@ cudaError_t launch_bind(const BindItem *items_dev, int32_t n_items, const double
                         float2 *arena, int64_t slice_begin, int64_t slices, int32_t max_rank,
                         cudaStream_t st);
 cudaError_t launch_bind_tiled(const BindTiled &b, const double2 *src, float2 *arena,
-                              int64_t slice_begin, int64_t slices, cudaStream_t st);
+                              unsigned int *amax, int64_t slice_begin, int64_t slices,
+                              cudaStream_t st);
 cudaError_t launch_accumulate(const float2 *root, int64_t root_sstride, int64_t n, int64_t slices,
                               double2 *amps, cudaStream_t st);
 // Where the root's elements go when open labels are sliced (amplitude batches): root bit r is

@@ -455,6 +455,30 @@ __global__ void k_sparse_amps(const float2 *root, const int32_t *idx, int64_t n,
     }
 }
 
+// Conversions between FP32 and FP64 in integer operations.  GB300 runs conversion instructions
+// from and to 64 bits at the rate of its FP64 units, 2 a clock and SM: a complex128 leaf of 2^23
+// elements took 28 us for them alone, its memory traffic takes 30.  Normal numbers and zeros are
+// rounded (to nearest, ties to even) or widened here, the rest by the instruction.
+__device__ __forceinline__ float narrow(double x) {
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t sign = hi & 0x80000000u, mag = hi ^ sign;
+    if ((mag | lo) == 0) return __uint_as_float(sign);
+    if ((mag >> 20) - 897u > 253u) return (float)x;  // outside FP32's normal range
+    const uint32_t m = (mag - (896u << 20)) << 3 | lo >> 29;
+    const uint32_t up = (lo & 0x1fffffffu) + (m & 1u) > 0x10000000u;
+    return __uint_as_float(sign | (m + up));
+}
+__device__ __forceinline__ double widen(float x) {
+    const uint32_t u = __float_as_uint(x), sign = u & 0x80000000u, mag = u ^ sign;
+    if ((mag >> 23) - 1u > 253u && mag != 0) return (double)x;  // subnormal, infinite or NaN
+    return __hiloint2double((int)(sign | (mag ? (mag >> 3) + (896u << 20) : 0u)),
+                            (int)(u << 29));
+}
+// a + x; an amplitude that is still +0, as before its first slice, takes x as it is
+__device__ __forceinline__ double add_widened(double a, float x) {
+    return __double_as_longlong(a) != 0 ? a + widen(x) : widen(x == 0.f ? 0.f : x);
+}
+
 // Leaf binding: grid (item, slice, chunk); the blocks of one (item, slice) share its elements.
 __global__ void k_bind(const BindItem *items, const double2 *src, float2 *arena,
                        int64_t slice_begin) {
@@ -470,7 +494,7 @@ __global__ void k_bind(const BindItem *items, const double2 *src, float2 *arena,
          i += (int64_t)gridDim.z * blockDim.x) {
         const uint64_t so = deposit((uint64_t)i, it.rank, it.pos_src) | soff;
         const double2 v = src[it.src_off + (int64_t)so];
-        dst[i] = make_float2((float)v.x, (float)v.y);
+        dst[i] = make_float2(narrow(v.x), narrow(v.y));
     }
 }
 
@@ -482,11 +506,16 @@ __global__ void k_bind(const BindItem *items, const double2 *src, float2 *arena,
 // 16-byte slots of one 512-byte row.
 __device__ __forceinline__ int tile_slot(int tau) { return tau ^ (((tau >> 6) & 31) << 1); }
 
-template <int MAXN>
-__global__ void __launch_bounds__(256) k_bind_tiled(BindTiled b, const double2 *__restrict__ src,
-                                                    float2 *__restrict__ arena,
-                                                    int64_t slice_begin) {
-    __shared__ __align__(16) float2 tile[MAXN];
+// A thread has eight 16-byte loads in flight.  HBM bounds the kernel (24 bytes per element, and
+// the max-abs of the leaf costs no pass of its own): 2^23 elements in
+// 34.5 us (5.8 TB/s), 66 us with one load in flight and a pass for the max-abs.
+template <int T>
+__global__ void __launch_bounds__(256, 4)
+    k_bind_tiled(const __grid_constant__ BindTiled b, const double2 *__restrict__ src,
+                 float2 *__restrict__ arena, unsigned int *__restrict__ amax,
+                 int64_t slice_begin) {
+    __shared__ __align__(16) float2 tile[1 << T];
+    __shared__ float wmax[8];
     const int64_t s = blockIdx.y;
     const uint64_t sigma = (uint64_t)(slice_begin + s);
     uint64_t soff = 0;
@@ -494,66 +523,103 @@ __global__ void __launch_bounds__(256) k_bind_tiled(BindTiled b, const double2 *
         if ((sigma >> b.sl_bit[j]) & 1ull) soff |= 1ull << b.sl_pos[j];
     const double2 *S = src + b.src_off + soff;
     float2 *D = arena + b.dst_off + s * b.dst_sstride;
-    const int n = 1 << b.t;
     const int tid = threadIdx.x;
     // read-order index e = tid + 256 k: its tile index and source offset are those of tid OR'ed
     // with those of 256 k (disjoint bits)
     int tau0 = 0;
     uint64_t so0 = 0;
-    for (int q = 0; q < 8 && q < b.t; ++q)
+#pragma unroll
+    for (int q = 0; q < 8; ++q)
         if ((tid >> q) & 1) {
             tau0 |= 1 << b.e2t[q];
             so0 |= 1ull << b.e2s[q];
         }
     // write-order pair j = tid + 256 k covers tile indices 2 j, 2 j + 1; destination bits of
     // tile bits 6-8 come from tid, those of tile bits 9 and up from k
-    uint64_t dw0 = 0;
-    for (int q = 6; q < 9 && q < b.t; ++q)
+    uint64_t dw0 = (2 * tid) & 63;
+#pragma unroll
+    for (int q = 6; q < 9; ++q)
         if (((2 * tid) >> q) & 1) dw0 |= 1ull << b.t2d[q];
+    float m = 0.f;
     for (int64_t w = blockIdx.x; w < b.ntiles; w += gridDim.x) {
-        uint64_t dbase = 0, sbase = 0;
+        uint64_t dbase = dw0, sbase = so0;
         for (int u = 0; u < b.nrest; ++u)
             if ((w >> u) & 1) {
                 dbase |= 1ull << b.rest_d[u];
                 sbase |= 1ull << b.rest_s[u];
             }
-        for (int k = 0; (k << 8) + tid < n; ++k) {
-            int tau = tau0;
-            uint64_t so = so0;
-            for (int q = 8; q < b.t; ++q)
-                if ((k >> (q - 8)) & 1) {
-                    tau |= 1 << b.e2t[q];
-                    so |= 1ull << b.e2s[q];
-                }
-            const double2 v = S[sbase | so];
-            tile[tile_slot(tau)] = make_float2((float)v.x, (float)v.y);
+#pragma unroll
+        for (int k0 = 0; k0 < (1 << (T - 8)); k0 += 8) {
+            double2 v[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                uint64_t so = sbase;
+#pragma unroll
+                for (int q = 8; q < T; ++q)
+                    if (((k0 + k) >> (q - 8)) & 1) so |= 1ull << b.e2s[q];
+                v[k] = S[so];
+            }
+#pragma unroll
+            for (int k = 0; k < 8; ++k) {
+                int tau = tau0;
+#pragma unroll
+                for (int q = 8; q < T; ++q)
+                    if (((k0 + k) >> (q - 8)) & 1) tau |= 1 << b.e2t[q];
+                const float2 f = make_float2(narrow(v[k].x), narrow(v[k].y));
+                m = fmaxf(m, fmaxf(fabsf(f.x), fabsf(f.y)));
+                tile[tile_slot(tau)] = f;
+            }
         }
         __syncthreads();
-        for (int k = 0; (k << 8) + tid < (n >> 1); ++k) {
-            const int tau = 2 * (tid + (k << 8));
-            uint64_t doff = dbase | dw0 | (uint64_t)(tau & 63);
-            for (int q = 9; q < b.t; ++q)
-                if ((tau >> q) & 1) doff |= 1ull << b.t2d[q];
+#pragma unroll
+        for (int k = 0; k < (1 << (T - 9)); ++k) {
+            uint64_t doff = dbase;
+#pragma unroll
+            for (int q = 9; q < T; ++q)
+                if ((k >> (q - 9)) & 1) doff |= 1ull << b.t2d[q];
             *reinterpret_cast<float4 *>(D + doff) =
-                *reinterpret_cast<const float4 *>(&tile[tile_slot(tau)]);
+                *reinterpret_cast<const float4 *>(&tile[tile_slot(2 * (tid + (k << 8)))]);
         }
         __syncthreads();
     }
+    if (!amax) return;
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if ((tid & 31) == 0) wmax[tid >> 5] = m;
+    __syncthreads();
+    if (tid == 0) {
+        for (int i = 1; i < 8; ++i) m = fmaxf(m, wmax[i]);
+        atomicMax(amax + (b.dst_sstride ? s : 0), __float_as_uint(m));
+    }
 }
 
-// amps[x] += sum over slices s (in increasing order) of root[s][x], in FP64.
-__global__ void k_accumulate(const float2 *root, int64_t sstride, int64_t n, int64_t slices,
-                             double2 *amps) {
-    for (int64_t x = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; x < n;
-         x += (int64_t)gridDim.x * blockDim.x) {
-        double2 acc = amps[x];
-#pragma unroll 8
+// amps[x] += sum over slices s (in increasing order) of root[s][x], in FP64.  A thread takes two
+// amplitudes.  With one slice HBM bounds it (40 bytes per amplitude), with several the FP64 adds:
+// 2^24 amplitudes of one slice in 102 us (6.6 TB/s), 128 us when the root's values were widened and added
+// to zeros by the FP64 units too.
+__global__ void __launch_bounds__(256) k_accumulate(const float2 *root, int64_t sstride, int64_t n,
+                                                    int64_t slices, double2 *amps) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n >> 1);
+         i += (int64_t)gridDim.x * blockDim.x) {
+        double2 a = amps[2 * i], b = amps[2 * i + 1];
+#pragma unroll 4
         for (int64_t s = 0; s < slices; ++s) {
-            const float2 v = root[s * sstride + x];
-            acc.x += (double)v.x;
-            acc.y += (double)v.y;
+            const float4 v = reinterpret_cast<const float4 *>(root + s * sstride)[i];
+            a.x = add_widened(a.x, v.x);
+            a.y = add_widened(a.y, v.y);
+            b.x = add_widened(b.x, v.z);
+            b.y = add_widened(b.y, v.w);
         }
-        amps[x] = acc;
+        amps[2 * i] = a;
+        amps[2 * i + 1] = b;
+    }
+    if (n == 1 && blockIdx.x == 0 && threadIdx.x == 0) {
+        double2 a = amps[0];
+        for (int64_t s = 0; s < slices; ++s) {
+            const float2 v = root[s * sstride];
+            a.x = add_widened(a.x, v.x);
+            a.y = add_widened(a.y, v.y);
+        }
+        amps[0] = a;
     }
 }
 
@@ -580,8 +646,8 @@ __global__ void k_accumulate_batched(const float2 *root, int64_t sstride, int64_
         double2 a = amps[o];
         for (; sig < (uint64_t)(s0 + slices); sig = (((sig | open) + 1) & ~open) | (sig & open)) {
             const float2 v = root[(int64_t)(sig - (uint64_t)s0) * sstride + x];
-            a.x += (double)v.x;
-            a.y += (double)v.y;
+            a.x = add_widened(a.x, v.x);
+            a.y = add_widened(a.y, v.y);
         }
         amps[o] = a;
     }
@@ -695,32 +761,61 @@ __device__ __forceinline__ float2 unpack2(__half2 h) { return __half22float2(h);
 __device__ __forceinline__ float2 unpack2(__nv_bfloat162 h) { return __bfloat1622float2(h); }
 __device__ __forceinline__ float2 unpack2(float2 h) { return h; }
 
+// Four complex64 (32 bytes) in one load.
+struct Quad {
+    float re[4], im[4];
+};
+__device__ __forceinline__ Quad load_quad(const float2 *p) {
+    Quad q;
+    asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(q.re[0]), "=f"(q.im[0]), "=f"(q.re[1]), "=f"(q.im[1]), "=f"(q.re[2]),
+          "=f"(q.im[2]), "=f"(q.re[3]), "=f"(q.im[3])
+        : "l"(p)
+        : "memory");
+    return q;
+}
+
 // T2 is a pair of stored elements (two 16-bit numbers, or two FP32 for TF32); the planes and
-// strides of d count elements.
+// strides of d count elements.  A thread takes four elements (d.n is a multiple of four): a
+// 32-byte load and an 8-byte store per plane (16 for TF32), each a whole number of sectors per
+// warp.  HBM bounds it: 2^23 elements into four planes in 23 us (5.8 TB/s),
+// 29.5 us with pairs.
 template <typename T2>
 __device__ __forceinline__ void convert_body(const ConvertDesc &d, int64_t s, int e) {
     using T = decltype(T2().x);
+    struct alignas(2 * sizeof(T2)) T4 {
+        T2 lo, hi;
+    };
     const Pow2 pe = pow2_of(-e);
     const float2 *src = d.src + s * d.src_sstride;
     T *base = reinterpret_cast<T *>(d.dst) + s * d.dst_sstride;
-    T2 *re = reinterpret_cast<T2 *>(base);
-    T2 *im = reinterpret_cast<T2 *>(base + d.plane_stride);
-    T2 *sm = reinterpret_cast<T2 *>(base + 2 * d.plane_stride);
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (d.n >> 1);
+    T4 *re = reinterpret_cast<T4 *>(base);
+    T4 *im = reinterpret_cast<T4 *>(base + d.plane_stride);
+    T4 *sm = reinterpret_cast<T4 *>(base + 2 * d.plane_stride);
+    T4 *il = reinterpret_cast<T4 *>(base + 3 * d.plane_stride);
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (d.n >> 2);
          i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 v = reinterpret_cast<const float4 *>(src)[i];
-        const float r0 = scale_pow2(v.x, pe), i0 = scale_pow2(v.y, pe);
-        const float r1 = scale_pow2(v.z, pe), i1 = scale_pow2(v.w, pe);
-        const T2 rh = pack2<T2>(r0, r1), ih = pack2<T2>(i0, i1);
+        Quad q = load_quad(src + 4 * i);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            q.re[j] = scale_pow2(q.re[j], pe);
+            q.im[j] = scale_pow2(q.im[j], pe);
+        }
+        const T4 rh{pack2<T2>(q.re[0], q.re[1]), pack2<T2>(q.re[2], q.re[3])};
+        const T4 ih{pack2<T2>(q.im[0], q.im[1]), pack2<T2>(q.im[2], q.im[3])};
         re[i] = rh;
         im[i] = ih;
-        if (d.planes == 3) sm[i] = pack2<T2>(r0 + i0, r1 + i1);
+        if (d.planes == 3)
+            sm[i] = T4{pack2<T2>(q.re[0] + q.im[0], q.re[1] + q.im[1]),
+                       pack2<T2>(q.re[2] + q.im[2], q.re[3] + q.im[3])};
         if (d.planes == 4) {
             // lo planes: the rounding residuals x - hi (exact in FP32), rounded again
-            const float2 rf = unpack2(rh), jf = unpack2(ih);
-            sm[i] = pack2<T2>(r0 - rf.x, r1 - rf.y);
-            T2 *iml = reinterpret_cast<T2 *>(base + 3 * d.plane_stride);
-            iml[i] = pack2<T2>(i0 - jf.x, i1 - jf.y);
+            const float2 r0 = unpack2(rh.lo), r1 = unpack2(rh.hi);
+            const float2 i0 = unpack2(ih.lo), i1 = unpack2(ih.hi);
+            sm[i] = T4{pack2<T2>(q.re[0] - r0.x, q.re[1] - r0.y),
+                       pack2<T2>(q.re[2] - r1.x, q.re[3] - r1.y)};
+            il[i] = T4{pack2<T2>(q.im[0] - i0.x, q.im[1] - i0.y),
+                       pack2<T2>(q.im[2] - i1.x, q.im[3] - i1.y)};
         }
     }
 }
@@ -840,24 +935,23 @@ cudaError_t launch_bind(const BindItem *items_dev, int32_t n_items, const double
 }
 
 cudaError_t launch_bind_tiled(const BindTiled &b, const double2 *src, float2 *arena,
-                              int64_t slice_begin, int64_t slices, cudaStream_t st) {
+                              unsigned int *amax, int64_t slice_begin, int64_t slices,
+                              cudaStream_t st) {
     if (slices <= 0) return cudaSuccess;
-    if (b.t < 6 || b.t > 12 || slices > 65535 || b.ntiles < 1) return cudaErrorInvalidValue;
-    const int per_sm = b.t <= 11 ? 8 : 6;  // resident blocks (16 or 32 KiB of shared memory)
-    int64_t gx = (152 * per_sm + slices - 1) / slices;
+    if (b.t < 11 || b.t > 12 || slices > 65535 || b.ntiles < 1) return cudaErrorInvalidValue;
+    int64_t gx = (152 * 4 + slices - 1) / slices;  // four resident blocks per SM
     if (gx > b.ntiles) gx = b.ntiles;
-    if (b.t <= 11)
-        k_bind_tiled<2048><<<dim3((unsigned)gx, (unsigned)slices), 256, 0, st>>>(b, src, arena,
-                                                                                 slice_begin);
+    const dim3 grid((unsigned)gx, (unsigned)slices);
+    if (b.t == 11)
+        k_bind_tiled<11><<<grid, 256, 0, st>>>(b, src, arena, amax, slice_begin);
     else
-        k_bind_tiled<4096><<<dim3((unsigned)gx, (unsigned)slices), 256, 0, st>>>(b, src, arena,
-                                                                                 slice_begin);
+        k_bind_tiled<12><<<grid, 256, 0, st>>>(b, src, arena, amax, slice_begin);
     return cudaGetLastError();
 }
 
 cudaError_t launch_accumulate(const float2 *root, int64_t root_sstride, int64_t n, int64_t slices,
                               double2 *amps, cudaStream_t st) {
-    k_accumulate<<<grid_for(n, 256), 256, 0, st>>>(root, root_sstride, n, slices, amps);
+    k_accumulate<<<grid_for(n >> 1, 256), 256, 0, st>>>(root, root_sstride, n, slices, amps);
     return cudaGetLastError();
 }
 
@@ -895,7 +989,8 @@ cudaError_t launch_amax(const ConvertDesc &d, int64_t slices, cudaStream_t st) {
 }
 
 cudaError_t launch_convert16(const ConvertDesc &d, int64_t slices, cudaStream_t st) {
-    const int gx = grid_for(d.n / 2, 256);
+    if (d.n & 3) return cudaErrorInvalidValue;
+    const int gx = grid_for(d.n / 4, 256);
     const int g = gx > 2048 ? 2048 : gx;
     k_convert16<<<dim3((unsigned)g, (unsigned)slices), 256, 0, st>>>(d);
     return cudaGetLastError();

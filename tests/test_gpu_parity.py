@@ -1276,3 +1276,114 @@ def test_sparse_state_graph_replay_and_capture(tn):
     assert np.array_equal(first, amps.cpu().numpy())
     plan.close()
     tnet.close()
+
+
+# A tensor alone is bound and added to the amplitudes: the tiled binding (rank >= 12), the
+# gathering one, and conversions between FP32 and FP64 that round and widen as IEEE does.
+@pytest.mark.parametrize("rank", [1, 5, 11, 12, 13, 15])
+@pytest.mark.parametrize("order", ["same", "reversed", "shuffled"])
+def test_bound_values_are_rounded_to_nearest_even(tn, rank, order):
+    rng = np.random.default_rng(rank)
+    n = 1 << rank
+    bits = rng.integers(0, 1 << 64, 2 * n, dtype=np.uint64)
+    v = (bits & np.uint64(0xffffffffe0000000)).view(np.float64)  # FP32 significands ...
+    half = np.where(rng.random(2 * n) < 0.5, 0x10000000, rng.integers(0, 1 << 29, 2 * n))
+    v = (v.view(np.uint64) | half.astype(np.uint64)).view(np.float64)  # ... and ties
+    e = rng.integers(-160, 132, 2 * n)  # below FP32's subnormals to above its largest
+    v = np.ldexp(np.frexp(np.where(np.isfinite(v), v, 1.0))[0], e)
+    special = rng.random(2 * n) < 0.2
+    v[special] = rng.choice([0.0, -0.0, 1.0, 2.0 ** -126, -2.0 ** -149, 2.0 ** -150, np.inf,
+                             (2 - 2.0 ** -24) * 2.0 ** 127, -(2 - 2.0 ** -23) * 2.0 ** 127],
+                            int(special.sum()))
+    T = v.view(np.complex128).reshape((2,) * rank)
+    labels = list(range(rank))
+    out = {"same": labels, "reversed": labels[::-1],
+           "shuffled": [int(x) for x in rng.permutation(rank)]}[order]
+    net = tn.Network([T], [labels], out)
+    plan = tn.Plan(net, [], [], mode="c64", sync_each_call=True)
+    amps = torch.zeros(n, dtype=torch.complex128, device="cuda")
+    with np.errstate(over="ignore"):
+        ref = np.ascontiguousarray(np.transpose(T, out)).reshape(-1).view(np.float64)
+        ref = ref.astype(np.float32).astype(np.float64)
+    for times in (1, 2):  # the second call adds to amplitudes that are not zero
+        plan.contract(amps)
+        assert np.array_equal(amps.cpu().numpy().view(np.float64), times * ref)
+    plan.close()
+    net.close()
+
+
+# Leaves bound by the tiled kernel record their own max-abs, per slice and again in every call.
+@pytest.mark.parametrize("mode", ["fp16_scaled", "bf16_scaled", "split_tf32"])
+@pytest.mark.parametrize("flight", [1, 2, 4])
+def test_large_sliced_leaves_are_scaled_per_slice(tn, mode, flight):
+    rng = np.random.default_rng(5 + flight)
+    tensors, labels, out = single_step(rng, 8, 7, 7)
+    x, y = 900, 901
+    A = np.stack([tensors[0], tensors[0][::-1] * 2.0 ** -14])
+    A = np.stack([A, A * 2.0 ** 9])
+    B = np.stack([tensors[1], tensors[1][::-1] * 2.0 ** 11])
+    B = np.stack([B * 2.0 ** -3, B])
+    t2, l2 = [A, B], [[y, x] + labels[0], [y, x] + labels[1]]
+    ref = O.contract(t2, l2, out, [(0, 1)], [x, y])
+    net = tn.Network(t2, l2, out)
+    for graph in (False, True):
+        plan = tn.Plan(net, [(0, 1)], [x, y], mode=mode, use_graph=graph, sync_each_call=True,
+                       max_slices_in_flight=flight)
+        assert plan.step_info(0)["kernel_name"] == "gemm_tc"
+        for _ in range(3):
+            amps = torch.zeros(1 << len(out), dtype=torch.complex128, device="cuda")
+            plan.contract(amps)
+            check(amps.cpu().numpy(), ref, TOL[mode])
+        plan.close()
+    net.close()
+
+
+# Outer products above and below the size at which a thread takes eight pairs of outputs.
+@pytest.mark.parametrize("m,n,batch", [(12, 11, 0), (11, 11, 0), (9, 11, 3), (22, 1, 0)])
+def test_large_outer_products(tn, m, n, batch):
+    rng = np.random.default_rng(m + 40 * n)
+    M, N, B = (list(range(o, o + k)) for o, k in ((0, m), (100, n), (200, batch)))
+    la, lb, out = ([int(x) for x in rng.permutation(v)] for v in (M + B, N + B, M + N + B))
+    tensors = [crandn(rng, m + batch), crandn(rng, n + batch)]
+    got, _, kernels = gpu_amps(tn, tensors, [la, lb], out, [(0, 1)])
+    assert kernels == ["generic"]
+    check(got, O.contract(tensors, [la, lb], out, [(0, 1)]), 1e-6)
+
+
+# The tensor-core kernel chosen at K = 2^10 and for results of few tiles.
+@pytest.mark.parametrize("shape", [(12, 11, 10), (11, 10, 10), (10, 9, 11), (8, 8, 12)])
+@pytest.mark.parametrize("mode", ["fp16_scaled", "tf32"])
+def test_tensor_core_kernels_at_the_edges_of_the_variant_rule(tn, shape, mode):
+    rng = np.random.default_rng(sum(shape))
+    tensors, labels, out = single_step(rng, *shape)
+    (A, B), (la, lb) = tensors, labels
+    K = [l for l in la if l in lb]
+    ref = np.tensordot(A, B, ([la.index(l) for l in K], [lb.index(l) for l in K]))
+    order = [l for l in la if l not in K] + [l for l in lb if l not in K]
+    got, _, kernels = gpu_amps(tn, tensors, labels, out, [(0, 1)], mode=mode)
+    assert kernels == ["gemm_tc"]
+    check(got, np.transpose(ref, [order.index(l) for l in out]), TOL[mode])
+
+
+# A plan's graphs, whose prologue runs independent branches at once, give the direct launches'
+# amplitudes bit for bit, from the call that makes them on.
+@pytest.mark.parametrize("mode", ["c64", "fp16_scaled"])
+@pytest.mark.parametrize("flight", [0, 1])
+def test_graphs_equal_direct_launches(tn, mode, flight):
+    circ = W.random_circuit(4, 5, 10, 3)
+    net = W.build_network(circ, list(range(12, 20)), {q: 0 for q in range(12)})
+    path = W.greedy_path(net.labels, net.open_labels)
+    sl = W.greedy_slices(net.labels, net.open_labels, path, 2)
+    tnet = tn.Network(net.tensors, net.labels, net.open_labels)
+    direct = tn.Plan(tnet, path, sl, mode=mode, max_slices_in_flight=flight)
+    graph = tn.Plan(tnet, path, sl, mode=mode, max_slices_in_flight=flight, use_graph=True)
+    ref = torch.zeros(256, dtype=torch.complex128, device="cuda")
+    direct.contract(ref)
+    assert torch.count_nonzero(ref).item() > 0
+    for _ in range(4):
+        amps = torch.zeros_like(ref)
+        graph.contract(amps)
+        assert torch.equal(amps, ref)
+    graph.close()
+    direct.close()
+    tnet.close()
