@@ -29,6 +29,11 @@ __device__ __forceinline__ uint64_t deposit(uint64_t x, int n, const int8_t *pos
     return r;
 }
 
+// Where index bit p of a staged output tile puts an element: C's order differs from the order the
+// threads hold the tile in, and without the swizzle (GemmDesc::bank) up to 16 lanes of a half-warp
+// met in one bank on the way out.
+__device__ __forceinline__ int stage_off(const GemmDesc &d, int p) { return (1 << p) ^ d.bank[p]; }
+
 // 256 threads as 16 x 16; each thread owns rows ty + 16*i and columns tx + 16*j (i, j < 4).
 // BK is the K tile (16, or 8 for contractions of at most 8 elements, which would otherwise
 // multiply half a tile of zero padding).
@@ -131,24 +136,32 @@ __global__ void __launch_bounds__(256) k_gemm_simt(GemmDesc d, int64_t tiles_n) 
         }
         return;
     }
-    // stage the tile (row-major 64 x 64) and write it out in C's memory order
+    // stage the tile (row-major 64 x 64, swizzled: stage_off) and write it out in C's memory order
     float2 *stage = sbuf;
+    {
+        int w0 = tx;
 #pragma unroll
-    for (int i = 0; i < TM; ++i)
+        for (int b = 0; b < 4; ++b)
+            if ((ty >> b) & 1) w0 ^= stage_off(d, 6 + b);
 #pragma unroll
-        for (int j = 0; j < TN; ++j)
-            stage[(ty + 16 * i) * BN + tx + 16 * j] = make_float2(cr[i][j], ci[i][j]);
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; ++j)
+                stage[w0 ^ ((i & 1) ? stage_off(d, 10) : 0) ^ ((i & 2) ? stage_off(d, 11) : 0) ^
+                      ((j & 1) ? stage_off(d, 4) : 0) ^ ((j & 2) ? stage_off(d, 5) : 0)] =
+                    make_float2(cr[i][j], ci[i][j]);
+    }
     // element pairs of the tile in C order: sorted tile bit 0 is C's position 0 (the pair),
     // bits 1..8 come from the thread index and the rest from the iteration; the sorted tile bits
     // were computed on the host
     const int nb = d.tile_bits;
     __syncthreads();
-    const int dpair = 1 << d.tb_src[0];
+    const int dpair = stage_off(d, d.tb_src[0]);
     int wlo = 0;
     uint64_t olo = 0;
     for (int q = 1; q < 9 && q < nb; ++q)
         if ((threadIdx.x >> (q - 1)) & 1) {
-            wlo |= 1 << d.tb_src[q];
+            wlo ^= stage_off(d, d.tb_src[q]);
             olo |= 1ull << d.tb_pos[q];
         }
     const uint64_t cbase =
@@ -159,7 +172,7 @@ __global__ void __launch_bounds__(256) k_gemm_simt(GemmDesc d, int64_t tiles_n) 
         d.pout.exps[s] = eo;
     float amx = 0.f;
     auto put = [&](uint64_t off, int w) {
-        const float2 v0 = stage[w], v1 = stage[w + dpair];
+        const float2 v0 = stage[w], v1 = stage[w ^ dpair];
         if (d.planar_out) {
             planar_out_store2(d.pout, s, cbase | off, v0, v1, eo);
         } else {
@@ -175,7 +188,7 @@ __global__ void __launch_bounds__(256) k_gemm_simt(GemmDesc d, int64_t tiles_n) 
             uint64_t off = olo;
             for (int q = 9; q < nb; ++q)
                 if ((it >> (q - 9)) & 1) {
-                    w |= 1 << d.tb_src[q];
+                    w ^= stage_off(d, d.tb_src[q]);
                     off |= 1ull << d.tb_pos[q];
                 }
             put(off, w);
@@ -409,8 +422,12 @@ __global__ void __launch_bounds__(256) k_splitk_reduce_deep(GemmDesc d, int64_t 
 // turn leave one block barrier per tile.  For longer K (KS = 0) a block
 // takes one tile and stages its rows through shared memory in chunks of 16 of K with coalesced
 // 16-byte loads.  A step whose small operand is A runs with the roles swapped (the complex
-// product commutes).  Each tile (256 x NT) is staged and written in C's order with 8 consecutive
-// elements per thread, as in the other epilogues.
+// product commutes).  Each tile (256 x NT) is staged and written in C's order, 32 bytes per
+// thread and store.  HBM should bound these steps, but the L1 / shared-memory pipe did (86% busy at
+// half the HBM rate): bank conflicts of the stage's reads (row stride NT + 1) and 16-byte accesses
+// that used half of each sector.  With the swizzle and 32-byte accesses 2^27 x 4 with K = 4
+// went from 2.73 to 2.53 ms (5.1 TB/s), 2^26 x 8 with K = 8 from 2.97 to 2.67 ms, and five steps of
+// 4 columns with planar results from 7.93 to 6.84 ms.
 constexpr int kThinRows = 256, kThinKC = 16, kThinLd = kThinKC + 1;
 // blocks per SM the launch bounds guarantee: the walking form keeps its rows of A in registers
 // (two tiles' worth), so 16 columns with it fit 2 blocks
@@ -423,17 +440,31 @@ constexpr int thin_min_blocks(int nt, int ks) {
 constexpr bool thin_b_in_regs(int nt, int ks) { return ks != 0 && nt * ks <= 16; }
 // the walking form with 16 columns stages its two output tiles in dynamic shared memory
 constexpr bool thin_dyn_smem(int nt, int ks) { return ks != 0 && nt == 16; }
-constexpr int thin_dyn_bytes(int nt) { return 2 * kThinRows * (nt + 1) * 8; }
+constexpr int thin_dyn_bytes(int nt) { return 2 * kThinRows * nt * 8; }
+// four complex64 (32 bytes) in one load or store
+__device__ __forceinline__ void load32(const float2 *p, float2 *v) {
+    asm("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+        : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y),
+          "=f"(v[3].x), "=f"(v[3].y)
+        : "l"(p)
+        : "memory");
+}
+__device__ __forceinline__ void store32(float2 *p, const float2 (&v)[4]) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(p), "f"(v[0].x),
+                 "f"(v[0].y), "f"(v[1].x), "f"(v[1].y), "f"(v[2].x), "f"(v[2].y), "f"(v[3].x),
+                 "f"(v[3].y)
+                 : "memory");
+}
 
 // PL: bytes of a planar result's numbers (2 or 4), 0 for a complex64 result
 template <int NT, int KS, int PL>
 __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(GemmDesc d) {
     constexpr int NB = NT < 2 ? 2 : NT;  // row stride of sB (pairs stay 16-byte aligned)
-    constexpr int LD = NT + 1;           // row stride of the output stage
+    constexpr int LNT = NT == 1 ? 0 : NT == 2 ? 1 : NT == 4 ? 2 : NT == 8 ? 3 : 4;  // NT = 2^LNT
     // KS > 0: two output stages used in turn (one barrier per tile); KS = 0: rows of A, then
     // the stage
     constexpr bool DYN = thin_dyn_smem(NT, KS);
-    __shared__ __align__(16) float2 sA_st[DYN ? 2 : (KS ? 2 * kThinRows * LD : kThinRows * kThinLd)];
+    __shared__ __align__(16) float2 sA_st[DYN ? 2 : (KS ? 2 * kThinRows * NT : kThinRows * kThinLd)];
     extern __shared__ __align__(16) float2 sA_dyn[];
     float2 *sA = DYN ? sA_dyn : sA_st;
     constexpr bool BREG = thin_b_in_regs(NT, KS);
@@ -468,35 +499,31 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
             }
         }
     };
-    // output: stage rows with stride NT + 1, then write 8 consecutive elements of C per task
-    auto soff = [&](int sq) { return (sq & 128) ? (LD << (sq & 127)) : (1 << sq); };
-    int w8[8];
-    {
-        const int d0 = soff(d.tb_src[0]), d1 = soff(d.tb_src[1]), d2 = soff(d.tb_src[2]);
+    // output: element (r, n) of the tile has stage index r * NT + n (swizzled: stage_off); written
+    // as runs of 8 consecutive elements of C
+    int own = 0;  // this thread's row
 #pragma unroll
-        for (int j = 0; j < 8; ++j)
-            w8[j] = ((j & 1) ? d0 : 0) + ((j & 2) ? d1 : 0) + ((j & 4) ? d2 : 0);
-    }
+    for (int b = 0; b < 8; ++b)
+        if ((tid >> b) & 1) own ^= stage_off(d, LNT + b);
+    const int d0 = stage_off(d, d.tb_src[0]), d1 = stage_off(d, d.tb_src[1]),
+              d2 = stage_off(d, d.tb_src[2]);
+    const int w4[4] = {0, d0, d1, d0 ^ d1};
     // a tile has 256 * NT elements (tile_bits = 8 + log2 NT): 32 * NT runs of 8 consecutive
     // elements of C; their stage and C offsets are the same for every tile, so they are set once
     constexpr int TASKS = kThinRows * NT / 8;
-    // two lanes share each run of 8, so every thread has stores to make: for complex64 results
-    // lane half h writes elements 4j + 2h and 4j + 2h + 1 in its store j (each store instruction
-    // fills whole 32-byte sectors); for planar 16-bit results (PL, a separate instantiation)
-    // lane half h writes elements 4h .. 4h + 3, 8 bytes per plane (a warp's stores cover 256
-    // contiguous bytes of each plane)
+    // two lanes share each run of 8: lane half h writes elements 4h .. 4h + 3, 32 bytes of
+    // complex64 in one store, or 8 (16) bytes per plane of a planar result of 16-bit (32-bit) numbers
     constexpr int SUBS = TASKS * 2, SPT = (SUBS + 255) / 256;
     int ws[SPT];
     uint64_t os[SPT];
-    const int d0 = w8[1], d1 = w8[2], d2 = w8[4];
 #pragma unroll
     for (int i = 0; i < SPT; ++i) {
         const int u = tid + 256 * i, r = u >> 1, h = u & 1;
-        ws[i] = h ? (PL ? d2 : d1) : 0;
-        os[i] = h ? (PL ? 4 : 2) : 0;
+        ws[i] = h ? d2 : 0;
+        os[i] = h ? 4 : 0;
         for (int q = 3; q < d.tile_bits; ++q)
             if ((r >> (q - 3)) & 1) {
-                ws[i] += soff(d.tb_src[q]);
+                ws[i] ^= stage_off(d, d.tb_src[q]);
                 os[i] |= 1ull << d.tb_pos[q];
             }
     }
@@ -509,48 +536,34 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
     // sure no thread still reads `stage` from an earlier tile
     auto emit = [&](float2 *stage, uint64_t cbase) {
 #pragma unroll
-        for (int n = 0; n < NT; ++n) stage[tid * LD + n] = make_float2(cr[n], ci[n]);
+        for (int n = 0; n < NT; ++n) stage[own ^ n] = make_float2(cr[n], ci[n]);
         __syncthreads();
         float2 *C = d.C + s * d.sC + cbase;
-        if constexpr (PL != 0) {
 #pragma unroll
-            for (int i = 0; i < SPT; ++i) {
-                if (SUBS % 256 != 0 && tid + 256 * i >= SUBS) break;
-                float2 v[4];
+        for (int i = 0; i < SPT; ++i) {
+            if (SUBS % 256 != 0 && tid + 256 * i >= SUBS) break;
+            float2 v[4];
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    v[j] = stage[ws[i] + w8[j]];
-                    amx = fmaxf(amx, fmaxf(fabsf(v[j].x), fabsf(v[j].y)));
-                }
-                planar_out_store4<PL>(d.pout, s, cbase | os[i], v, eo);
+            for (int j = 0; j < 4; ++j) {
+                v[j] = stage[ws[i] ^ w4[j]];
+                amx = fmaxf(amx, fmaxf(fabsf(v[j].x), fabsf(v[j].y)));
             }
-        } else {
-#pragma unroll
-            for (int i = 0; i < SPT; ++i) {
-                if (SUBS % 256 != 0 && tid + 256 * i >= SUBS) break;
-#pragma unroll
-                for (int j = 0; j < 2; ++j) {
-                    const int w = ws[i] + (j ? d2 : 0);
-                    const float2 v0 = stage[w], v1 = stage[w + d0];
-                    amx = fmaxf(amx, fmaxf(fmaxf(fabsf(v0.x), fabsf(v0.y)),
-                                           fmaxf(fabsf(v1.x), fabsf(v1.y))));
-                    *reinterpret_cast<float4 *>(C + (os[i] + 4 * j)) =
-                        make_float4(v0.x, v0.y, v1.x, v1.y);
-                }
-            }
+            if constexpr (PL != 0) planar_out_store4<PL>(d.pout, s, cbase | os[i], v, eo);
+            else store32(C + os[i], v);
         }
     };
     if constexpr (KS != 0) {
         const int64_t tiles = (1ll << d.lm) / kThinRows;
         float2 a[KS], an[KS];
         auto fetch = [&](float2 *dst, int64_t t) {
-            const float4 *Ar =
-                reinterpret_cast<const float4 *>(As + (t * kThinRows + tid) * KS);
+            const float2 *Ar = As + (t * kThinRows + tid) * KS;
+            if constexpr (KS >= 4) {
 #pragma unroll
-            for (int q = 0; q < KS / 2; ++q) {
-                const float4 v = Ar[q];
-                dst[2 * q] = make_float2(v.x, v.y);
-                dst[2 * q + 1] = make_float2(v.z, v.w);
+                for (int q = 0; q < KS; q += 4) load32(Ar + q, dst + q);
+            } else {
+                const float4 v = *reinterpret_cast<const float4 *>(Ar);
+                dst[0] = make_float2(v.x, v.y);
+                dst[1] = make_float2(v.z, v.w);
             }
         };
         // C offset of tile t: deposit(t * 256), its 8 low bits zero; the warp's lanes take one
@@ -598,7 +611,7 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
             }
             // stage `buf` was last read two tiles ago, before every thread passed the barrier
             // inside the previous tile's emit
-            emit(sA + buf * kThinRows * LD, tile_base(t));
+            emit(sA + buf * kThinRows * NT, tile_base(t));
             buf ^= 1;
 #pragma unroll
             for (int k = 0; k < KS; ++k) a[k] = an[k];
@@ -1076,6 +1089,35 @@ int rank4(const int *v, int n) {
     return r;
 }
 }  // namespace
+
+void stage_choose_banks(const int *write, const int *read, int nread, int8_t *bank) {
+    for (int p = 0; p < 12; ++p) bank[p] = 0;
+    bool set[12];
+    for (int p = 0; p < 12; ++p) set[p] = p < 4;
+    auto vec = [&](int p) { return p < 4 ? 1 << p : (int)bank[p]; };
+    // every vector of a list is the smallest one outside the span of the others set so far, of
+    // both lists: two spans of at most 8 vectors share 0, so one of 16 is always left
+    auto in_span = [&](const int *list, int n, int p, int x) {
+        int others[5], k = 0;
+        bool member = false;
+        for (int q = 0; q < n; ++q) {
+            member |= list[q] == p;
+            if (list[q] != p && set[list[q]]) others[k++] = vec(list[q]);
+        }
+        if (!member) return false;
+        const int r = rank4(others, k);
+        others[k] = x;
+        return rank4(others, k + 1) == r;
+    };
+    for (int i = 0; i < 4 + nread; ++i) {
+        const int p = i < 4 ? write[i] : read[i - 4];
+        if (set[p]) continue;
+        int x = 1;
+        while (x < 15 && (in_span(write, 4, p, x) || in_span(read, nread, p, x))) ++x;
+        bank[p] = (int8_t)x;
+        set[p] = true;
+    }
+}
 
 int thin_choose_swizzle(const int8_t *tb_src, int lnt, int planar, int8_t *phi) {
     // the 8-byte bank pair (0..15) of element (r, c) is ((r << lnt) & 15) | (c ^ phi(r)): a row

@@ -1901,6 +1901,12 @@ tn_status run_step_inner(tn_plan_t *p, const Step &st, int64_t slices, cudaStrea
             if (d.tb_pos[0] != 0 || d.tb_pos[1] != 1 || d.tb_pos[2] != 2)
                 return fail(TN_ERR_UNSUPPORTED, "step %d: result bits 0-2 outside the thin tile",
                             (int)(&st - &p->steps[0]));
+            // index bits of the stage: columns first, row bit i is bit ln + i
+            for (int q = 0; q < d.tile_bits; ++q)
+                if (d.tb_src[q] & 128) d.tb_src[q] = (int8_t)(d.ln + (d.tb_src[q] & 127));
+            const int write[4] = {d.ln, d.ln + 1, d.ln + 2, d.ln + 3};
+            const int read[4] = {d.tb_src[2], d.tb_src[3], d.tb_src[4], d.tb_src[5]};
+            tn::stage_choose_banks(write, read, 4, d.bank);
         }
         if (on_tc && !st.thin_phi_set) {
             const int planar = !d.planar_out ? 0 : (d.pout.dtype == 2 ? 4 : 2);
@@ -1956,6 +1962,10 @@ tn_status run_step_inner(tn_plan_t *p, const Step &st, int64_t slices, cudaStrea
             if (d.tb_pos[0] != 0)
                 return fail(TN_ERR_UNSUPPORTED, "step %d: result bit 0 outside the GEMM tile",
                             (int)(&st - &p->steps[0]));
+            const int write[4] = {0, 1, 2, 3};
+            int read[4], nread = 0;
+            for (int q = 1; q <= 4 && q < d.tile_bits; ++q) read[nread++] = d.tb_src[q];
+            tn::stage_choose_banks(write, read, nread, d.bank);
         }
         if (ev) TN_CUDA(cudaEventRecord(ev->first, stream));
         e = tn::launch_gemm_simt(d, slices, stream);

@@ -153,6 +153,8 @@ struct GemmDesc {
     int8_t tb_pos[16];         //   (n: 0..5, m: 6..11) and its position in C
     int8_t posC_m[TN_MAXR];    // bit i of m (0 = least significant) -> bit of C's index
     int8_t posC_n[TN_MAXR];
+    int8_t bank[12];           // CUDA-core kernels: what index bit p of the output stage adds to an
+                               //   element's place by XOR (stage_choose_banks)
     int8_t phi[8];             // tensor-core thin kernel: XOR swizzle of the output stage by
                                //   row bit (thin_choose_swizzle)
 };
@@ -206,6 +208,11 @@ struct BindTiled {
 // complex64 results, 3-6 for planar 16-bit (planar = 2) and 2-5 for TF32 ones (4)) each touch 16 distinct 8-byte bank pairs where the
 // layout allows; returns how many of the two patterns are conflict-free.
 int thin_choose_swizzle(const int8_t *tb_src, int lnt, int planar, int8_t *phi);
+// Output stage of the CUDA-core GEMM kernels: an element whose stage index has the bits p sits at
+// the index XOR bank[p] of those bits (bank[p] < 16, 0 for p < 4).  Chosen so that a half-warp,
+// whose lanes span the four index bits `write` when the tile is staged and the bits `read`
+// (nread <= 4) when it is read in C's order, meets 16 different 8-byte bank pairs either way.
+void stage_choose_banks(const int *write, const int *read, int nread, int8_t *bank);
 void sort_tile_bits(int tm, int tn, const int8_t *posC_m, const int8_t *posC_n, int row_tag,
                     int8_t *src, int8_t *pos);
 
