@@ -35,10 +35,12 @@ __device__ __forceinline__ uint64_t deposit(uint64_t x, int n, const int8_t *pos
 __device__ __forceinline__ int stage_off(const GemmDesc &d, int p) { return (1 << p) ^ d.bank[p]; }
 
 // 256 threads as 16 x 16; each thread owns rows ty + 16*i and columns tx + 16*j (i, j < 4).
-// BK is the K tile (16, or 8 for contractions of at most 8 elements, which would otherwise
-// multiply half a tile of zero padding).
-template <int BK>
-__global__ void __launch_bounds__(256) k_gemm_simt(GemmDesc d, int64_t tiles_n) {
+// BK is the K tile, 16.  ONE: a contraction of at most BK terms (8 or 16) in one tile: no second
+// set of sums and no loads ahead, so that four blocks fit an SM instead of two; these steps wait
+// for their loads and stores, not for the FMA units.  2^17 x 64, K = 4: 24 us, 40 us in the general
+// form (67 MB written: 10 us); 2^12 x 2^12, K = 8: 55 us, 76 us; K = 16: 77 us, 94 us.
+template <int BK, bool ONE>
+__global__ void __launch_bounds__(256, ONE ? 4 : 2) k_gemm_simt(GemmDesc d, int64_t tiles_n) {
     constexpr int AS = 2 * 16 * (BM + 1), BS = 2 * 16 * (BN + 1);
     static_assert(AS + BS >= BM * BN, "staging tile must fit in the operand buffers");
     __shared__ __align__(16) float2 sbuf[AS + BS];
@@ -85,7 +87,27 @@ __global__ void __launch_bounds__(256) k_gemm_simt(GemmDesc d, int64_t tiles_n) 
     load(0);
     store(0);
     __syncthreads();
-    const int64_t ktiles = (K + BK - 1) / BK;
+    auto mac = [&](float (&r)[TM][TN], float (&im)[TM][TN], int buf, int kk) {
+        float2 a[TM], b[TN];
+#pragma unroll
+        for (int i = 0; i < TM; ++i) a[i] = As[buf][kk][ty + 16 * i];
+#pragma unroll
+        for (int j = 0; j < TN; ++j) b[j] = Bs[buf][kk][tx + 16 * j];
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+            for (int j = 0; j < TN; ++j) {
+                r[i][j] = fmaf(a[i].x, b[j].x, r[i][j]);
+                r[i][j] = fmaf(-a[i].y, b[j].y, r[i][j]);
+                im[i][j] = fmaf(a[i].x, b[j].y, im[i][j]);
+                im[i][j] = fmaf(a[i].y, b[j].x, im[i][j]);
+            }
+    };
+    const int64_t ktiles = ONE ? 0 : (K + BK - 1) / BK;
+    if constexpr (ONE) {
+        for (int kk = 0; kk < (int)K; ++kk) mac(cr, ci, 0, kk);
+        __syncthreads();
+    }
     for (int64_t kt = 0; kt < ktiles; ++kt) {
         const int buf = kt & 1;
         if (kt + 1 < ktiles) load((kt + 1) * BK);
@@ -95,22 +117,7 @@ __global__ void __launch_bounds__(256) k_gemm_simt(GemmDesc d, int64_t tiles_n) 
 #pragma unroll
             for (int j = 0; j < TN; ++j) tr[i][j] = ti[i][j] = 0.f;
 #pragma unroll
-        for (int kk = 0; kk < BK; ++kk) {
-            float2 a[TM], b[TN];
-#pragma unroll
-            for (int i = 0; i < TM; ++i) a[i] = As[buf][kk][ty + 16 * i];
-#pragma unroll
-            for (int j = 0; j < TN; ++j) b[j] = Bs[buf][kk][tx + 16 * j];
-#pragma unroll
-            for (int i = 0; i < TM; ++i)
-#pragma unroll
-                for (int j = 0; j < TN; ++j) {
-                    tr[i][j] = fmaf(a[i].x, b[j].x, tr[i][j]);
-                    tr[i][j] = fmaf(-a[i].y, b[j].y, tr[i][j]);
-                    ti[i][j] = fmaf(a[i].x, b[j].y, ti[i][j]);
-                    ti[i][j] = fmaf(a[i].y, b[j].x, ti[i][j]);
-                }
-        }
+        for (int kk = 0; kk < BK; ++kk) mac(tr, ti, buf, kk);
 #pragma unroll
         for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -164,8 +171,14 @@ __global__ void __launch_bounds__(256) k_gemm_simt(GemmDesc d, int64_t tiles_n) 
             wlo ^= stage_off(d, d.tb_src[q]);
             olo |= 1ull << d.tb_pos[q];
         }
-    const uint64_t cbase =
-        deposit((uint64_t)m0, d.lm, d.posC_m) | deposit((uint64_t)n0, d.ln, d.posC_n);
+    // C offset of the tile: the warp's lanes take a bit each
+    uint64_t cbase = 0;
+    for (int i = 6 + (tid & 31); i < d.lm; i += 32)
+        if ((m0 >> i) & 1) cbase |= 1ull << d.posC_m[i];
+    for (int i = 6 + (tid & 31); i < d.ln; i += 32)
+        if ((n0 >> i) & 1) cbase |= 1ull << d.posC_n[i];
+    cbase = (uint64_t)__reduce_or_sync(0xffffffffu, (uint32_t)(cbase >> 32)) << 32 |
+            __reduce_or_sync(0xffffffffu, (uint32_t)cbase);
     float2 *C = d.C + s * d.sC + cbase;
     const int eo = d.planar_out ? planar_out_exponent(d.pout, s) : 0;
     if (d.planar_out && blockIdx.x == 0 && blockIdx.z == 0 && threadIdx.x == 0)
@@ -1033,10 +1046,12 @@ cudaError_t launch_gemm_simt(const GemmDesc &d, int64_t slices, cudaStream_t st)
         k_gemm_skinny<16><<<dim3(1, (unsigned)slices, (unsigned)d.splits), 256, kSkSmem, st>>>(d);
     else if (skinny)
         k_gemm_skinny<32><<<dim3(1, (unsigned)slices, (unsigned)d.splits), 256, kSkSmem, st>>>(d);
-    else if (d.lk - (d.splits > 1 ? __builtin_ctz((unsigned)d.splits) : 0) <= 3)
-        k_gemm_simt<8><<<grid, 256, 0, st>>>(d, tn_);
+    else if (((1ll << d.lk) / d.splits) <= 8)
+        k_gemm_simt<8, true><<<grid, 256, 0, st>>>(d, tn_);
+    else if (((1ll << d.lk) / d.splits) == 16)
+        k_gemm_simt<16, true><<<grid, 256, 0, st>>>(d, tn_);
     else
-        k_gemm_simt<16><<<grid, 256, 0, st>>>(d, tn_);
+        k_gemm_simt<16, false><<<grid, 256, 0, st>>>(d, tn_);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || d.splits == 1) return e;
     const int64_t MN = 1ll << (d.lm + d.ln);
