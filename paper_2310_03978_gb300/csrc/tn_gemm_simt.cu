@@ -433,19 +433,20 @@ __global__ void __launch_bounds__(256) k_splitk_reduce_deep(GemmDesc d, int64_t 
 // bytes; a warp reads one contiguous span) and fetches its row of the next tile before it stores
 // the current one, so loads stay in flight during the store phase; two output stages taken in
 // turn leave one block barrier per tile.  For longer K (KS = 0) a block
-// takes one tile and stages its rows through shared memory in chunks of 16 of K with coalesced
-// 16-byte loads.  A step whose small operand is A runs with the roles swapped (the complex
+// takes one tile and a thread reads its row 8 of K ahead, two 32-byte sectors that only it needs:
+// no barrier stands between the loads and the sums (2^13 x 8, K = 1024: 102 us, 199 us when
+// chunks of 16 were staged in shared memory; 2^17 x 16, K = 32: 26 us, 33 us).  A step whose small operand is A runs with the roles swapped (the complex
 // product commutes).  Each tile (256 x NT) is staged and written in C's order, 32 bytes per
 // thread and store.  HBM should bound these steps, but the L1 / shared-memory pipe did (86% busy at
 // half the HBM rate): bank conflicts of the stage's reads (row stride NT + 1) and 16-byte accesses
 // that used half of each sector.  With the swizzle and 32-byte accesses 2^27 x 4 with K = 4
 // went from 2.73 to 2.53 ms (5.1 TB/s), 2^26 x 8 with K = 8 from 2.97 to 2.67 ms, and five steps of
 // 4 columns with planar results from 7.93 to 6.84 ms.
-constexpr int kThinRows = 256, kThinKC = 16, kThinLd = kThinKC + 1;
-// blocks per SM the launch bounds guarantee: the walking form keeps its rows of A in registers
-// (two tiles' worth), so 16 columns with it fit 2 blocks
+constexpr int kThinRows = 256;
+// blocks per SM the launch bounds guarantee: rows of A are kept in registers (the walking form:
+// two tiles' worth), so 16 columns fit 2 blocks
 constexpr int thin_min_blocks(int nt, int ks) {
-    return ks && nt == 16 ? 2 : ((ks && nt < 8) ? 4 : 3);
+    return nt == 16 ? 2 : (nt < 8 ? 4 : 3);
 }
 // the walking form holds a small operand of at most 16 complex values in registers (every
 // thread the same values), so the inner loop reads no shared memory at all; larger ones stay
@@ -474,10 +475,9 @@ template <int NT, int KS, int PL>
 __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(GemmDesc d) {
     constexpr int NB = NT < 2 ? 2 : NT;  // row stride of sB (pairs stay 16-byte aligned)
     constexpr int LNT = NT == 1 ? 0 : NT == 2 ? 1 : NT == 4 ? 2 : NT == 8 ? 3 : 4;  // NT = 2^LNT
-    // KS > 0: two output stages used in turn (one barrier per tile); KS = 0: rows of A, then
-    // the stage
+    // KS > 0: two output stages used in turn (one barrier per tile); KS = 0: one
     constexpr bool DYN = thin_dyn_smem(NT, KS);
-    __shared__ __align__(16) float2 sA_st[DYN ? 2 : (KS ? 2 * kThinRows * NT : kThinRows * kThinLd)];
+    __shared__ __align__(16) float2 sA_st[DYN ? 2 : (KS ? 2 : 1) * kThinRows * NT];
     extern __shared__ __align__(16) float2 sA_dyn[];
     float2 *sA = DYN ? sA_dyn : sA_st;
     constexpr bool BREG = thin_b_in_regs(NT, KS);
@@ -529,17 +529,19 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
     constexpr int SUBS = TASKS * 2, SPT = (SUBS + 255) / 256;
     int ws[SPT];
     uint64_t os[SPT];
+    auto set_offsets = [&] {
 #pragma unroll
-    for (int i = 0; i < SPT; ++i) {
-        const int u = tid + 256 * i, r = u >> 1, h = u & 1;
-        ws[i] = h ? d2 : 0;
-        os[i] = h ? 4 : 0;
-        for (int q = 3; q < d.tile_bits; ++q)
-            if ((r >> (q - 3)) & 1) {
-                ws[i] ^= stage_off(d, d.tb_src[q]);
-                os[i] |= 1ull << d.tb_pos[q];
-            }
-    }
+        for (int i = 0; i < SPT; ++i) {
+            const int u = tid + 256 * i, r = u >> 1, h = u & 1;
+            ws[i] = h ? d2 : 0;
+            os[i] = h ? 4 : 0;
+            for (int q = 3; q < d.tile_bits; ++q)
+                if ((r >> (q - 3)) & 1) {
+                    ws[i] ^= stage_off(d, d.tb_src[q]);
+                    os[i] |= 1ull << d.tb_pos[q];
+                }
+        }
+    };
     float amx = 0.f;
     // a result that feeds a tensor-core step is written as its scaled planar 16-bit copy, with
     // the exponent bounded from the inputs' max-abs (as in the other epilogues)
@@ -566,6 +568,7 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
         }
     };
     if constexpr (KS != 0) {
+        set_offsets();
         const int64_t tiles = (1ll << d.lm) / kThinRows;
         float2 a[KS], an[KS];
         auto fetch = [&](float2 *dst, int64_t t) {
@@ -631,10 +634,16 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
         }
     } else {
         const int64_t m0 = (int64_t)blockIdx.x * kThinRows;
-        const float2 *A = As + m0 * K;
+        const float2 *A = As + (m0 + tid) * K;
+        float2 a[8], an[8];
+        auto fetch = [&](float2 *dst, int k) {
+            load32(A + k, dst);
+            load32(A + k + 4, dst + 4);
+        };
+        fetch(an, 0);
 #pragma unroll
         for (int n = 0; n < NT; ++n) cr[n] = ci[n] = 0.f;
-        // the small operand 64 of K at a time (K up to 1024), the rows of A 16 of K at a time
+        // the small operand 64 of K at a time (K up to 1024), the row of A 8 of K ahead
         for (int kb = 0; kb < K; kb += 64) {
             const int kbw = K - kb < 64 ? K - kb : 64;
             __syncthreads();  // every thread is done with the previous part of sB
@@ -642,23 +651,16 @@ __global__ void __launch_bounds__(256, thin_min_blocks(NT, KS)) k_gemm_thin(Gemm
                 const int n = e / kbw, k = e % kbw;
                 sB[k * NB + n] = B[(int64_t)n * K + kb + k];
             }
-            for (int kc = kb; kc < kb + kbw; kc += kThinKC) {
-                const int kw = kb + kbw - kc < kThinKC ? kb + kbw - kc : kThinKC;  // 2^j >= 2
-                const int hp = kw >> 1;  // 16-byte pairs per row
-                __syncthreads();
-                for (int e = tid; e < kThinRows * hp; e += 256) {
-                    const int r = e / hp, q = e % hp;
-                    const float4 v =
-                        *reinterpret_cast<const float4 *>(A + (int64_t)r * K + kc + 2 * q);
-                    sA[r * kThinLd + 2 * q] = make_float2(v.x, v.y);
-                    sA[r * kThinLd + 2 * q + 1] = make_float2(v.z, v.w);
-                }
-                __syncthreads();
-                for (int k = 0; k < kw; ++k)
-                    mac(sA[tid * kThinLd + k], sB + (kc - kb + k) * NB);
+            __syncthreads();
+            for (int kc = 0; kc < kbw; kc += 8) {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) a[k] = an[k];
+                if (kb + kc + 8 < K) fetch(an, kb + kc + 8);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) mac(a[k], sB + (kc + k) * NB);
             }
         }
-        __syncthreads();  // the stage reuses sA
+        set_offsets();
         emit(sA, deposit((uint64_t)m0, d.lm, d.posC_m));
     }
     if (d.amax_out) amax_publish(d.amax_out + s, amx);
