@@ -1531,7 +1531,8 @@ tn_status build_chains(tn_plan_t *p) {
             size_t best = 0;
             for (size_t g = 1; g < gs.size(); ++g)
                 if (gs[g].total() < gs[best].total()) best = g;
-            if (gs[best].total() + q.total() > tn::kChainShmElems) {
+            // total() counts a record of padding; two parts in one group share it
+            if (gs[best].total() + q.total() - 1 > tn::kChainShmElems) {
                 best = gs.size();
                 gs.emplace_back();
             }

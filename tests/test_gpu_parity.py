@@ -1387,3 +1387,22 @@ def test_graphs_equal_direct_launches(tn, mode, flight):
     graph.close()
     direct.close()
     tnet.close()
+
+
+# Connected small steps that just fit a block's shared memory, and that just do not (the networks of
+# test_host_runtime.py), with their numbers.
+@pytest.mark.parametrize("ops", ["ggvvpvvvppvo", "ggvvpvvpgpvvov", "ggvvpvvvpvvv", "ggvvpvvvpvg",
+                                 "ggvvpvvvpvpo"])
+def test_runs_of_small_steps_at_the_shared_memory_limit(tn, ops):
+    rng = np.random.default_rng(len(ops))
+    wires, labels, path = list(range(12)), [list(range(12))], []
+    for i, op in enumerate(ops):
+        k, n = {"g": (1, 1), "v": (1, 0), "p": (2, 0), "o": (0, 1)}[op]
+        cut, new = wires[:k], [100 + i] * n
+        wires = wires[k:] + new
+        labels.append(cut + new)
+        path.append((0, len(labels) - 1))
+    tensors = [crandn(rng, len(ls)) for ls in labels]
+    ref = O.contract(tensors, labels, wires, path)
+    got, _, _ = gpu_amps(tn, tensors, labels, wires, path)
+    check(got, ref, TOL["c64"])

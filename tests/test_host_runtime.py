@@ -1,0 +1,86 @@
+"""The library's host code (planning, graphs, the small-step schedule) without a GPU: libtn.so's
+object files linked against a stand-in for the CUDA runtime (fake_cudart.c), whose kernels do
+nothing.  Each test runs in a process of its own."""
+import os
+import shutil
+import subprocess
+import sys
+import textwrap
+
+import pytest
+
+from paper_2310_03978_gb300 import build as B
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes as C, sys, types
+import numpy as np
+from paper_2310_03978_gb300 import tn, workload as W
+tn.LIB_PATH = sys.argv[1]
+L = tn.lib()
+L.fake_calls.restype = L.fake_alive.restype = C.c_long
+calls = lambda name: L.fake_calls(name.encode())
+NULL = types.SimpleNamespace(cuda_stream=0)
+MINE = types.SimpleNamespace(cuda_stream=64)
+
+def net_of(labels, opens):
+    return tn.Network([np.zeros((2,) * len(l), complex) for l in labels], labels, opens)
+"""
+
+
+@pytest.fixture(scope="module")
+def fake(tmp_path_factory):
+    cc = shutil.which("gcc")
+    if cc is None or os.uname().sysname != "Linux":
+        pytest.skip("needs gcc")
+    B.build()
+    out = str(tmp_path_factory.mktemp("fake") / "libtn_fake.so")
+    objs = [os.path.join(B.BUILD, os.path.splitext(s)[0] + ".o") for s in B.SOURCES]
+    # -Bsymbolic: the stand-in serves this library only, whatever else the process has loaded
+    subprocess.run([cc.replace("gcc", "g++"), "-shared", "-fPIC", "-Wl,-Bsymbolic", "-o", out,
+                    "-x", "c", os.path.join(HERE, "fake_cudart.c"), "-x", "none", *objs],
+                   check=True)
+
+    def run(code):
+        r = subprocess.run([sys.executable, "-c", PRELUDE + textwrap.dedent(code), out], cwd=ROOT,
+                           capture_output=True, text=True, timeout=300)
+        assert r.returncode == 0, "exit %d\n%s%s" % (r.returncode, r.stdout, r.stderr)
+        return r.stdout
+
+    return run
+
+
+# Connected steps on one rank-12 leaf (g: one-qubit gate, v: vector, p: a tensor of two of its labels,
+# o: outer product with a vector).  Tensors, records and padding take as many complex64 as the key
+# says; a block's shared memory holds 27648, so the last two work in global memory.
+RUNS = {27646: "ggvvpvvvppvo", 27647: "ggvvpvvpgpvvov", 27648: "ggvvpvvvpvvv",
+        27649: "ggvvpvvvpvg", 27650: "ggvvpvvvpvpo"}
+
+
+def run_network(ops):
+    """(labels, open labels, path) of the run."""
+    wires, fresh = list(range(12)), 100
+    labels, path = [list(wires)], []
+    for op in ops:
+        k, n = {"g": (1, 1), "v": (1, 0), "p": (2, 0), "o": (0, 1)}[op]
+        cut, wires = wires[:k], wires[k:]
+        new = list(range(fresh, fresh + n))
+        fresh += n
+        labels.append(cut + new)
+        wires += new
+        path.append((0, len(labels) - 1))
+    return labels, wires, path
+
+
+@pytest.mark.parametrize("size", RUNS)
+def test_runs_of_small_steps_that_just_fit_shared_memory(fake, size):
+    labels, opens, path = run_network(RUNS[size])
+    fake("""
+    net = net_of(%r, %r)
+    plan = tn.Plan(net, %r)
+    plan.contract_host(stream=NULL)
+    assert calls("launch") > 0
+    plan.close(); net.close()
+    """ % (labels, opens, path))
