@@ -597,6 +597,308 @@ static std::vector<ChainPart> chain_parts(const tn_plan_t *p, const Chain &c) {
     return parts;
 }
 
+// How a plan's steps are launched and how long its tensors live: the planar copies, the launch order
+// with its runs of small steps, and the lifetimes on the op timeline.  What saves launches keeps
+// more tensors alive at once, so when the workspace limit costs slices in flight (or the plan) the
+// next way down is tried: without branches in the prologue, then in path order, with runs of
+// neighbouring steps only and planes wider than the complex64 values made just before their use.
+// The amplitudes are the same bits in all of them.
+enum { kBranches, kMerged, kFrugal };
+
+static void arrange(tn_plan_t *p, int level) {
+    const int path_len = (int)p->steps.size();
+    const tn_precision mode = p->mode;
+    p->planars.clear();
+    p->chains.clear();
+    p->nmeta = p->nmeta_inv = 0;
+    p->prologue_branches = false;
+    for (auto &x : p->tensors) {
+        x.meta = -1;
+        x.direct = x.operand = false;
+    }
+    for (auto &st : p->steps) {
+        st.out_meta = st.direct_planar = st.chain = -1;
+        st.chain_head = false;
+    }
+    const auto wide = [&](const Planar &q) { return q.planes == 4 || tf32_mode(mode); };
+
+    // Tensor-core operands get planar copies.  When the operand's producer is a GEMM
+    // step of the slice loop (with whole 64 x 64 tiles to spare), that producer writes the
+    // copy directly, with an exponent bounded from its own inputs' max-abs; otherwise a
+    // conversion pass makes it from complex64 just before the step.
+    for (int s = 0; s < path_len; ++s) {
+        Step &st = p->steps[s];
+        if (!st.dep || st.kernel != K_TC) continue;
+        for (int side = 0; side < 2; ++side) {
+            Planar q;
+            q.tensor = side ? st.b : st.a;
+            q.planes = st.form == TN_GEMM_3M ? 3 : (st.form == kFormSplit ? 4 : 2);
+            if (st.tune_form) q.planes = 3;  // the tuner may pick 3M for this step
+            q.cap_planes = q.planes;
+            q.bytes_per_slice = (int64_t)((tf32_mode(mode) ? 4 : 2) * q.cap_planes)
+                                << p->tensors[q.tensor].rank();
+            const Tensor &X = p->tensors[q.tensor];
+            if (X.producer >= 0 && (st.form != kFormSplit || operand_dtype(mode) != 0) &&
+                (level != kFrugal || !wide(q))) {
+                // A producer's direct output takes its exponent from a bound (2 K max|a| max|b|)
+                // that can exceed the true maximum by many binades, which leaves the stored
+                // values low in FP16's range; single-pass operands keep their 11 significant
+                // bits there, but the lo planes of compensated FP16 operands would fall into the
+                // subnormals, so those are split from complex64 with their measured max-abs.
+                // BF16 and TF32 have FP32's exponents: hi and lo keep their bits at any scale.
+                // A CUDA-core producer writes directly only with whole 64 x 64 tiles, and then
+                // never splits K (its epilogue must hold final sums).
+                // A CUDA-core producer that would split K (judged at one slice in flight, its
+                // fewest tiles) writes complex64 instead: a long contraction over few tiles
+                // needs the split more than the saved conversion pass.
+                const Step &pr = p->steps[X.producer];
+                q.direct = pr.dep && (pr.kernel == K_TC || pr.kernel == K_STREAM ||
+                                      (pr.kernel == K_GEMM && pr.M.size() >= 6 &&
+                                       pr.N.size() >= 6 &&
+                                       tn::gemm_simt_splits((int)pr.M.size(), (int)pr.N.size(),
+                                                            (int)pr.K.size(), 1) == 1));
+            }
+            (side ? st.pb : st.pa) = (int)p->planars.size();
+            p->planars.push_back(q);
+        }
+    }
+    {
+        auto need_meta = [&](int ti) {
+            if (p->tensors[ti].meta < 0) p->tensors[ti].meta = p->nmeta++;
+        };
+        for (auto &q : p->planars) {
+            need_meta(q.tensor);
+            p->tensors[q.tensor].operand = true;
+        }
+        for (auto &q : p->planars)
+            if (q.direct) {
+                const Step &pr = p->steps[p->tensors[q.tensor].producer];
+                if (pr.kernel == K_GEMM || pr.kernel == K_STREAM)
+                    for (int x : {pr.a, pr.b}) {
+                        need_meta(x);
+                        if (!wide(q)) p->tensors[x].operand = true;
+                    }
+            }
+        // slice-independent blocks first: they are cleared once per call, the others per batch
+        {
+            int next = 0;
+            for (int dep = 0; dep < 2; ++dep) {
+                for (auto &x : p->tensors)
+                    if (x.meta >= 0 && x.dep == (dep == 1)) x.meta = next++;
+                if (dep == 0) p->nmeta_inv = next;
+            }
+        }
+        for (auto &q : p->planars) {
+            q.meta = p->tensors[q.tensor].meta;
+            if (q.direct) {
+                p->tensors[q.tensor].direct = true;
+                p->steps[p->tensors[q.tensor].producer].direct_planar = (int)(&q - &p->planars[0]);
+            }
+        }
+        // a tensor's max-abs is recorded by its producer's epilogue; leaves get an amax pass
+        for (auto &x : p->tensors)
+            if (x.meta >= 0 && x.producer >= 0) p->steps[x.producer].out_meta = x.meta;
+    }
+    // Launch order.  The small steps run many per launch (k_chain, k_chain_shm): just before a larger
+    // step that needs one of them, every small step whose operands exist by then joins one run,
+    // wherever the path has it, so a path whose small and large steps alternate still needs few
+    // launches.  The slice-independent prologue and the slice loop are ordered separately.
+    // Profile mode times every step on its own, in path order.
+    for (int cls = 0; cls < 2; ++cls) {
+        std::vector<int> todo;
+        for (int s = 0; s < path_len; ++s)
+            if (p->steps[s].dep == (cls == 1)) todo.push_back(s);
+        if (p->opts.profile) {
+            p->exec[cls] = todo;
+            continue;
+        }
+        auto rank_c = [&](const Step &st) { return p->tensors[st.c].rank(); };
+        auto tiny = [&](const Step &st) {
+            const int rc = rank_c(st), nk = (int)st.K.size();
+            return st.kernel == K_GENERIC && rc <= tn::kChainMaxRankC && nk <= tn::kChainMaxNk &&
+                   rc + nk <= tn::kChainMaxWork;
+        };
+        // In shared memory a run also takes streaming and GEMM steps of up to 2^16
+        // multiply-adds: a launch of their own costs 4-10 us, the block less than 1.  The sums
+        // are the same bits: one chain over k, or (GEMM, K > 16, too short to be split) blocks of
+        // 16 terms.
+        auto small_shm = [&](const Step &st) {
+            const int rc = rank_c(st), nk = (int)st.K.size();
+            return tiny(st) || ((st.kernel == K_STREAM || st.kernel == K_GEMM) && !st.thin_tc &&
+                                st.direct_planar < 0 && rc <= tn::kChainMaxRankC && nk <= 8 &&
+                                rc + nk <= 16);
+        };
+        // An outer product of 2^10 or more outputs that makes an operand (see Tensor), or with no
+        // other tiny step beside it in the path, rounds as k_generic_k1 does, the others as
+        // k_generic: the rule looks at path and precision only, so results do not depend on how
+        // steps share launches.
+        auto plain = [&](size_t i) {
+            return i < todo.size() && tiny(p->steps[todo[i]]) &&
+                   !p->tensors[p->steps[todo[i]].c].operand;
+        };
+        for (size_t i = 0; i < todo.size(); ++i) {
+            Step &st = p->steps[todo[i]];
+            st.fused_mul = st.K.empty() && rank_c(st) >= 10 &&
+                           (p->tensors[st.c].operand || !(plain(i - 1) || plain(i + 1)));
+        }
+        const size_t chains0 = p->chains.size();
+        auto schedule = [&](auto small) {
+            std::vector<char> done(path_len, 0);
+            for (int s = 0; s < path_len; ++s) done[s] = cls == 1 && !p->steps[s].dep;
+            auto ready = [&](const Step &st) {
+                const int pa = p->tensors[st.a].producer, pb = p->tensors[st.b].producer;
+                return (pa < 0 || done[pa]) && (pb < 0 || done[pb]);
+            };
+            auto run_small = [&]() {
+                Chain c;
+                for (int s : todo)  // path order, so an operand's producer comes before its reader
+                    if (!done[s] && small(p->steps[s]) && ready(p->steps[s])) {
+                        done[s] = 1;
+                        p->steps[s].chain = (int)p->chains.size();
+                        c.steps.push_back(s);
+                    }
+                if (c.steps.empty()) return;
+                p->steps[c.steps[0]].chain_head = true;
+                p->exec[cls].push_back(c.steps[0]);
+                p->chains.push_back(std::move(c));
+            };
+            for (int s : todo) {
+                if (small(p->steps[s])) continue;
+                if (!ready(p->steps[s])) run_small();
+                done[s] = 1;
+                p->exec[cls].push_back(s);
+            }
+            run_small();
+        };
+        if (level == kFrugal) {  // runs of neighbours in the path only
+            int last = -1;
+            for (size_t i = 0; i < todo.size(); ++i) {
+                Step &st = p->steps[todo[i]];
+                const auto in_run = [&](size_t j) { return plain(j) && p->steps[todo[j]].out_meta < 0; };
+                if (!in_run(i) || !(in_run(i - 1) || in_run(i + 1))) {
+                    p->exec[cls].push_back(todo[i]);
+                    continue;
+                }
+                if (!in_run(i - 1)) {
+                    last = (int)p->chains.size();
+                    p->chains.emplace_back();
+                    st.chain_head = true;
+                    p->exec[cls].push_back(todo[i]);
+                }
+                st.chain = last;
+                p->chains[last].steps.push_back(todo[i]);
+            }
+            continue;
+        }
+        schedule(small_shm);
+        bool fits = true;
+        for (size_t c = chains0; c < p->chains.size(); ++c)
+            for (const auto &part : chain_parts(p, p->chains[c]))
+                fits = fits && part.fits();
+        if (!fits) {  // the streaming and GEMM steps need the whole run in shared memory
+            for (int s : todo) {
+                p->steps[s].chain = -1;
+                p->steps[s].chain_head = false;
+            }
+            p->exec[cls].clear();
+            p->chains.resize(chains0);
+            schedule(tiny);
+        }
+    }
+    // op timeline: invariant leaves, invariant steps, sliced leaves, dependent steps (each
+    // tensor-core step preceded by its conversions; a run of chained steps is one op, so every
+    // tensor it touches is live at that op and no two of them share memory), accumulate
+    std::vector<Op> ops;
+    ops.push_back({0, -1});
+    for (int s : p->exec[0]) ops.push_back({1, s});
+    ops.push_back({2, -1});
+    for (int s : p->exec[1]) {
+        const Step &st = p->steps[s];
+        if (st.kernel == K_TC) {
+            ops.push_back({3, st.pa});
+            ops.push_back({3, st.pb});
+        }
+        ops.push_back({1, s});
+    }
+    ops.push_back({4, -1});
+    const int tend = (int)ops.size() - 1;
+    for (int t = 0; t < (int)ops.size(); ++t) {
+        const Op &op = ops[t];
+        if (op.kind == 0 || op.kind == 2) {
+            for (auto &x : p->tensors)
+                if (x.producer < 0 && x.dep == (op.kind == 2)) x.t0 = x.t1 = t;
+        } else if (op.kind == 1) {
+            const Step &head = p->steps[op.index];
+            const std::vector<int> one{op.index};
+            for (int k : head.chain_head ? p->chains[head.chain].steps : one) {
+                Step &st = p->steps[k];
+                st.t = t;
+                p->tensors[st.c].t0 = p->tensors[st.c].t1 = t;
+                p->tensors[st.a].t1 = t;
+                p->tensors[st.b].t1 = t;
+            }
+        }
+    }
+    for (auto &st : p->steps) {
+        if (st.kernel != K_TC) continue;
+        for (int side = 0; side < 2; ++side) {
+            Planar &q = p->planars[side ? st.pb : st.pa];
+            q.t = st.t;  // last use
+            q.t0 = q.direct ? p->steps[p->tensors[q.tensor].producer].t : st.t - 2;
+        }
+    }
+    // invariant tensors read by the slice loop stay live through all batches
+    for (auto &st : p->steps)
+        if (st.dep) {
+            if (!p->tensors[st.a].dep) p->tensors[st.a].t1 = tend;
+            if (!p->tensors[st.b].dep) p->tensors[st.b].t1 = tend;
+        }
+    p->tensors[p->root].t1 = tend;
+
+    // The prologue's steps are small for the whole GPU: when all its tensors and split-K partials
+    // together are (512 MB), each gets memory of its own for the whole prologue, so that its graph can
+    // run independent branches of the tree at once (the 30-qubit annealed path's 150 launches:
+    // 1.85 -> 1.0 ms).
+    if (level == kBranches && p->opts.use_graph && !p->opts.profile && !p->exec[0].empty()) {
+        int64_t bytes = 0;
+        for (const auto &x : p->tensors)
+            if (!x.dep) bytes += (int64_t)8 << x.rank();
+        for (const auto &st : p->steps)
+            if (!st.dep && st.kernel == K_GEMM) {
+                const int sp = tn::gemm_simt_splits((int)st.M.size(), (int)st.N.size(),
+                                                    (int)st.K.size(), 1);
+                if (sp > 1) bytes += (int64_t)sp * ((int64_t)8 << (st.M.size() + st.N.size()));
+            }
+        p->prologue_branches = bytes <= ((int64_t)512 << 20);
+        if (p->prologue_branches) {
+            const int end = (int)p->exec[0].size();  // op 0 binds, 1 .. end are the steps
+            for (auto &x : p->tensors)
+                if (!x.dep) {
+                    x.t0 = 0;
+                    x.t1 = std::max(x.t1, end);
+                }
+        }
+    }
+}
+
+// No arrangement of `slices` slices takes less: the tensors of a step, tensor-core operands as planes.
+static int64_t least_bytes(const tn_plan_t *p, int64_t slices) {
+    int64_t most = 0;
+    for (const auto &st : p->steps) {
+        int64_t bytes = 0;
+        for (int x : {st.a, st.b, st.c}) {
+            const Tensor &t = p->tensors[x];
+            const bool tc = x != st.c && st.kernel == K_TC;
+            // a direct result is its reader's planes, 4 bytes per element at least
+            const int64_t size = tc ? p->planars[x == st.a ? st.pa : st.pb].bytes_per_slice
+                                    : (int64_t)(x == st.c && t.meta >= 0 ? 4 : 8) << t.rank();
+            bytes += size * (t.dep ? slices : 1);
+        }
+        most = std::max(most, bytes);
+    }
+    return most;
+}
+
 // host allocations of the planners may throw; nothing crosses the C ABI
 extern "C" tn_status tn_plan(const tn_network_t *net, int32_t path_len, const int32_t *path,
                              int32_t num_sliced, const int32_t *sliced_labels, tn_precision mode,
@@ -865,237 +1167,7 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
     }
     if (path_len == 0) p->tensors[p->root].order = p->root_open;
 
-    // 4. tensor-core operands get planar copies.  When the operand's producer is a GEMM
-    //    step of the slice loop (with whole 64 x 64 tiles to spare), that producer writes the
-    //    copy directly, with an exponent bounded from its own inputs' max-abs; otherwise a
-    //    conversion pass makes it from complex64 just before the step.
-    for (int s = 0; s < path_len; ++s) {
-        Step &st = p->steps[s];
-        if (!st.dep || st.kernel != K_TC) continue;
-        for (int side = 0; side < 2; ++side) {
-            Planar q;
-            q.tensor = side ? st.b : st.a;
-            q.planes = st.form == TN_GEMM_3M ? 3 : (st.form == kFormSplit ? 4 : 2);
-            if (st.tune_form) q.planes = 3;  // the tuner may pick 3M for this step
-            q.cap_planes = q.planes;
-            q.bytes_per_slice = (int64_t)((tf32_mode(mode) ? 4 : 2) * q.cap_planes)
-                                << p->tensors[q.tensor].rank();
-            const Tensor &X = p->tensors[q.tensor];
-            if (X.producer >= 0 && (st.form != kFormSplit || operand_dtype(mode) != 0)) {
-                // A producer's direct output takes its exponent from a bound (2 K max|a| max|b|)
-                // that can exceed the true maximum by many binades, which leaves the stored
-                // values low in FP16's range; single-pass operands keep their 11 significant
-                // bits there, but the lo planes of compensated FP16 operands would fall into the
-                // subnormals, so those are split from complex64 with their measured max-abs.
-                // BF16 and TF32 have FP32's exponents: hi and lo keep their bits at any scale.
-                // A CUDA-core producer writes directly only with whole 64 x 64 tiles, and then
-                // never splits K (its epilogue must hold final sums).
-                // A CUDA-core producer that would split K (judged at one slice in flight, its
-                // fewest tiles) writes complex64 instead: a long contraction over few tiles
-                // needs the split more than the saved conversion pass.
-                const Step &pr = p->steps[X.producer];
-                q.direct = pr.dep && (pr.kernel == K_TC || pr.kernel == K_STREAM ||
-                                      (pr.kernel == K_GEMM && pr.M.size() >= 6 &&
-                                       pr.N.size() >= 6 &&
-                                       tn::gemm_simt_splits((int)pr.M.size(), (int)pr.N.size(),
-                                                            (int)pr.K.size(), 1) == 1));
-            }
-            (side ? st.pb : st.pa) = (int)p->planars.size();
-            p->planars.push_back(q);
-        }
-    }
-    {
-        auto need_meta = [&](int ti) {
-            if (p->tensors[ti].meta < 0) p->tensors[ti].meta = p->nmeta++;
-        };
-        for (auto &q : p->planars) {
-            need_meta(q.tensor);
-            p->tensors[q.tensor].operand = true;
-        }
-        for (auto &q : p->planars)
-            if (q.direct) {
-                const Step &pr = p->steps[p->tensors[q.tensor].producer];
-                if (pr.kernel == K_GEMM || pr.kernel == K_STREAM)
-                    for (int x : {pr.a, pr.b}) {
-                        need_meta(x);
-                        if (q.planes != 4 && !tf32_mode(mode)) p->tensors[x].operand = true;
-                    }
-            }
-        // slice-independent blocks first: they are cleared once per call, the others per batch
-        {
-            int next = 0;
-            for (int dep = 0; dep < 2; ++dep) {
-                for (auto &x : p->tensors)
-                    if (x.meta >= 0 && x.dep == (dep == 1)) x.meta = next++;
-                if (dep == 0) p->nmeta_inv = next;
-            }
-        }
-        for (auto &q : p->planars) {
-            q.meta = p->tensors[q.tensor].meta;
-            if (q.direct) {
-                p->tensors[q.tensor].direct = true;
-                p->steps[p->tensors[q.tensor].producer].direct_planar = (int)(&q - &p->planars[0]);
-            }
-        }
-        // a tensor's max-abs is recorded by its producer's epilogue; leaves get an amax pass
-        for (auto &x : p->tensors)
-            if (x.meta >= 0 && x.producer >= 0) p->steps[x.producer].out_meta = x.meta;
-    }
-    // Launch order.  The small steps run many per launch (k_chain, k_chain_shm): just before a larger
-    // step that needs one of them, every small step whose operands exist by then joins one run,
-    // wherever the path has it, so a path whose small and large steps alternate still needs few
-    // launches.  The slice-independent prologue and the slice loop are ordered separately.
-    // Profile mode times every step on its own, in path order.
-    for (int cls = 0; cls < 2; ++cls) {
-        std::vector<int> todo;
-        for (int s = 0; s < path_len; ++s)
-            if (p->steps[s].dep == (cls == 1)) todo.push_back(s);
-        if (p->opts.profile) {
-            p->exec[cls] = todo;
-            continue;
-        }
-        auto rank_c = [&](const Step &st) { return p->tensors[st.c].rank(); };
-        auto tiny = [&](const Step &st) {
-            const int rc = rank_c(st), nk = (int)st.K.size();
-            return st.kernel == K_GENERIC && rc <= tn::kChainMaxRankC && nk <= tn::kChainMaxNk &&
-                   rc + nk <= tn::kChainMaxWork;
-        };
-        // In shared memory a run also takes streaming and GEMM steps of up to 2^16
-        // multiply-adds: a launch of their own costs 4-10 us, the block less than 1.  The sums
-        // are the same bits: one chain over k, or (GEMM, K > 16, too short to be split) blocks of
-        // 16 terms.
-        auto small_shm = [&](const Step &st) {
-            const int rc = rank_c(st), nk = (int)st.K.size();
-            return tiny(st) || ((st.kernel == K_STREAM || st.kernel == K_GEMM) && !st.thin_tc &&
-                                st.direct_planar < 0 && rc <= tn::kChainMaxRankC && nk <= 8 &&
-                                rc + nk <= 16);
-        };
-        // An outer product of 2^10 or more outputs that makes an operand (see Tensor), or with no
-        // other tiny step beside it in the path, rounds as k_generic_k1 does, the others as
-        // k_generic: the rule looks at path and precision only, so results do not depend on how
-        // steps share launches.
-        auto plain = [&](size_t i) {
-            return i < todo.size() && tiny(p->steps[todo[i]]) &&
-                   !p->tensors[p->steps[todo[i]].c].operand;
-        };
-        for (size_t i = 0; i < todo.size(); ++i) {
-            Step &st = p->steps[todo[i]];
-            st.fused_mul = st.K.empty() && rank_c(st) >= 10 &&
-                           (p->tensors[st.c].operand || !(plain(i - 1) || plain(i + 1)));
-        }
-        const size_t chains0 = p->chains.size();
-        auto schedule = [&](auto small) {
-            std::vector<char> done(path_len, 0);
-            for (int s = 0; s < path_len; ++s) done[s] = cls == 1 && !p->steps[s].dep;
-            auto ready = [&](const Step &st) {
-                const int pa = p->tensors[st.a].producer, pb = p->tensors[st.b].producer;
-                return (pa < 0 || done[pa]) && (pb < 0 || done[pb]);
-            };
-            auto run_small = [&]() {
-                Chain c;
-                for (int s : todo)  // path order, so an operand's producer comes before its reader
-                    if (!done[s] && small(p->steps[s]) && ready(p->steps[s])) {
-                        done[s] = 1;
-                        p->steps[s].chain = (int)p->chains.size();
-                        c.steps.push_back(s);
-                    }
-                if (c.steps.empty()) return;
-                p->steps[c.steps[0]].chain_head = true;
-                p->exec[cls].push_back(c.steps[0]);
-                p->chains.push_back(std::move(c));
-            };
-            for (int s : todo) {
-                if (small(p->steps[s])) continue;
-                if (!ready(p->steps[s])) run_small();
-                done[s] = 1;
-                p->exec[cls].push_back(s);
-            }
-            run_small();
-        };
-        schedule(small_shm);
-        bool fits = true;
-        for (size_t c = chains0; c < p->chains.size(); ++c)
-            for (const auto &part : chain_parts(p, p->chains[c]))
-                fits = fits && part.fits();
-        if (!fits) {  // the streaming and GEMM steps need the whole run in shared memory
-            for (int s : todo) {
-                p->steps[s].chain = -1;
-                p->steps[s].chain_head = false;
-            }
-            p->exec[cls].clear();
-            p->chains.resize(chains0);
-            schedule(tiny);
-        }
-    }
-    // op timeline: invariant leaves, invariant steps, sliced leaves, dependent steps (each
-    // tensor-core step preceded by its conversions; a run of chained steps is one op, so every
-    // tensor it touches is live at that op and no two of them share memory), accumulate
-    std::vector<Op> ops;
-    ops.push_back({0, -1});
-    for (int s : p->exec[0]) ops.push_back({1, s});
-    ops.push_back({2, -1});
-    for (int s : p->exec[1]) {
-        const Step &st = p->steps[s];
-        if (st.kernel == K_TC) {
-            ops.push_back({3, st.pa});
-            ops.push_back({3, st.pb});
-        }
-        ops.push_back({1, s});
-    }
-    ops.push_back({4, -1});
-    const int tend = (int)ops.size() - 1;
-    for (int t = 0; t < (int)ops.size(); ++t) {
-        const Op &op = ops[t];
-        if (op.kind == 0 || op.kind == 2) {
-            for (auto &x : p->tensors)
-                if (x.producer < 0 && x.dep == (op.kind == 2)) x.t0 = x.t1 = t;
-        } else if (op.kind == 1) {
-            const Step &head = p->steps[op.index];
-            const std::vector<int> one{op.index};
-            for (int k : head.chain_head ? p->chains[head.chain].steps : one) {
-                Step &st = p->steps[k];
-                st.t = t;
-                p->tensors[st.c].t0 = p->tensors[st.c].t1 = t;
-                p->tensors[st.a].t1 = t;
-                p->tensors[st.b].t1 = t;
-            }
-        }
-    }
-    for (auto &st : p->steps) {
-        if (st.kernel != K_TC) continue;
-        for (int side = 0; side < 2; ++side) {
-            Planar &q = p->planars[side ? st.pb : st.pa];
-            q.t = st.t;  // last use
-            q.t0 = q.direct ? p->steps[p->tensors[q.tensor].producer].t : st.t - 2;
-        }
-    }
-    // invariant tensors read by the slice loop stay live through all batches
-    for (auto &st : p->steps)
-        if (st.dep) {
-            if (!p->tensors[st.a].dep) p->tensors[st.a].t1 = tend;
-            if (!p->tensors[st.b].dep) p->tensors[st.b].t1 = tend;
-        }
-    p->tensors[p->root].t1 = tend;
-
-    // The prologue's steps are small for the whole GPU: when all its tensors together are (512 MB), each
-    // gets memory of its own for the whole prologue, so that its graph can run independent
-    // branches of the tree at once (the 30-qubit annealed path's 150 launches: 1.85 -> 1.0 ms).
-    if (p->opts.use_graph && !p->opts.profile && !p->exec[0].empty()) {
-        int64_t bytes = 0;
-        for (const auto &x : p->tensors)
-            if (!x.dep) bytes += (int64_t)8 << x.rank();
-        p->prologue_branches = bytes <= ((int64_t)512 << 20);
-        if (p->prologue_branches) {
-            const int end = (int)p->exec[0].size();  // op 0 binds, 1 .. end are the steps
-            for (auto &x : p->tensors)
-                if (!x.dep) {
-                    x.t0 = 0;
-                    x.t1 = std::max(x.t1, end);
-                }
-        }
-    }
-
-    // 5. slices per launch under the workspace limit
+    // 4. launch order and slices per launch under the workspace limit
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
         delete p;
@@ -1103,12 +1175,29 @@ static tn_status plan_impl(const tn_network_t *net, int32_t path_len, const int3
     }
     int64_t limit = p->opts.workspace_limit > 0 ? p->opts.workspace_limit
                                                 : (int64_t)((double)free_b * 0.6);
-    int64_t sb = p->num_slices;
-    if (p->opts.max_slices_in_flight > 0) sb = std::min(sb, p->opts.max_slices_in_flight);
-    sb = std::min<int64_t>(sb, 65535);
-    while (sb > 1 && layout_bytes(p, sb, false) > limit) sb = (sb + 1) / 2;
-    const int64_t need = layout_bytes(p, sb, true);
-    if (need > limit) {
+    int64_t most = p->num_slices;
+    if (p->opts.max_slices_in_flight > 0) most = std::min(most, p->opts.max_slices_in_flight);
+    most = std::min<int64_t>(most, 65535);
+    int64_t sb = 0;  // fits the limit so far, arranged as `chosen`
+    int chosen = kBranches, arranged = kBranches;
+    for (int level = kBranches; level <= kFrugal; ++level) {
+        if (level > kBranches) {
+            int64_t next = most;  // the least that would be more than sb
+            while (next > 1 && (next + 1) / 2 > sb) next = (next + 1) / 2;
+            if (least_bytes(p, next) > limit) break;
+            if (level == kMerged && !p->prologue_branches) continue;
+        }
+        arrange(p, arranged = level);
+        for (int64_t n = most; n > sb; n = n > 1 ? (n + 1) / 2 : 0)
+            if (layout_bytes(p, n, false) <= limit) {
+                sb = n;
+                chosen = level;
+            }
+        if (sb == most) break;
+    }
+    if (sb > 0 && arranged != chosen) arrange(p, chosen);
+    const int64_t need = layout_bytes(p, std::max<int64_t>(sb, 1), true);
+    if (sb == 0) {
         delete p;
         return fail(TN_ERR_OOM, "workspace needs %lld bytes for one slice, limit %lld",
                     (long long)need, (long long)limit);

@@ -84,3 +84,34 @@ def test_runs_of_small_steps_that_just_fit_shared_memory(fake, size):
     assert calls("launch") > 0
     plan.close(); net.close()
     """ % (labels, opens, path))
+
+
+# (rows, cols, cycles, open qubits, sliced bonds, mode): what one slice takes when the steps run in path
+# order, in bytes.  A plan may use more to save launches, but only where the workspace allows it.
+IN_PATH_ORDER = {(5, 5, 10, 6, 4, "c64"): 5081088, (5, 5, 10, 6, 4, "fp16_scaled"): 4016128,
+                 (3, 5, 11, 12, 0, "tf32"): 1599488, (4, 3, 6, 12, 0, "tf32"): 81920,
+                 (4, 5, 12, 10, 2, "split_tf32"): 489882624}
+
+
+@pytest.mark.parametrize("case", IN_PATH_ORDER, ids=str)
+def test_a_workspace_of_what_path_order_takes_is_enough(fake, case):
+    fake("""
+    rows, cols, cycles, opens, nsl, mode = %r
+    need, q = %d, rows * cols
+    net = W.build_network(W.random_circuit(rows, cols, cycles, 3), list(range(q - opens, q)),
+                          {i: 0 for i in range(q - opens)})
+    path = W.greedy_path(net.labels, net.open_labels)
+    cut = W.greedy_slices(net.labels, net.open_labels, path, nsl) if nsl else []
+    tnet = tn.Network.from_workload(net)
+    for graph in (False, True):
+        plan = tn.Plan(tnet, path, cut, mode=mode, use_graph=graph, max_slices_in_flight=1,
+                       workspace_limit=need)
+        assert plan.info()["workspace_bytes"] <= need
+        plan.close()
+        # and no slices in flight are lost to it
+        free = tn.Plan(tnet, path, cut, mode=mode, use_graph=False)
+        limit = free.info()["workspace_bytes"]
+        plan = tn.Plan(tnet, path, cut, mode=mode, use_graph=graph, workspace_limit=limit)
+        assert plan.info()["slices_in_flight"] == free.info()["slices_in_flight"]
+        plan.close(); free.close()
+    """ % (case, IN_PATH_ORDER[case]))
