@@ -2258,17 +2258,17 @@ const float2 *tn::plan_root(const tn_plan_t *p) {
     return reinterpret_cast<const float2 *>(p->arena) + p->tensors[p->root].off;
 }
 
-// Slice-independent leaves and steps, once per call.
-static tn_status run_prologue(tn_plan_t *p, cudaStream_t stream) {
+// Slice-independent leaves and steps, once per call.  captured: `stream` is lanes[0], being captured.
+static tn_status run_prologue(tn_plan_t *p, cudaStream_t stream, bool captured) {
     tn_status s = clear_amax(p, false, stream);
     if (s == TN_OK) s = bind_leaves(p, false, 0, 1, stream);
     if (s != TN_OK) return s;
-    if (!p->prologue_branches || stream != p->lanes[0]) {
+    if (!p->prologue_branches || !captured) {
         for (size_t i = 0; i < p->exec[0].size() && s == TN_OK; ++i)
             s = run_step(p, p->steps[p->exec[0][i]], 1, stream);
         return s;
     }
-    // being captured: a node per launch, named by its first step
+    // a node per launch, named by its first step
     tn::Branches br(p->lanes, p->steps.size());
     TN_CUDA(br.fork());
     for (int k : p->exec[0]) {
@@ -2296,7 +2296,7 @@ static tn_status run_prologue(tn_plan_t *p, cudaStream_t stream) {
 }
 
 // Replay `g` on `stream`.  The first time its work is launched directly, the second time it is
-// captured from body(stream) on a plan-owned stream: making a graph costs more than the launches
+// captured from body(stream, true) on a plan-owned stream: making a graph costs more than the launches
 // it saves once, so a plan used once never makes one (first pass over a new 12-qubit plan 158 ->
 // 111 us).
 template <class F>
@@ -2304,7 +2304,7 @@ static tn_status replay(tn_plan_t *p, Graph &g, cudaStream_t stream, F body) {
     // A graph of up to 4 launches costs more to launch than they do (a 2-launch one ~3 us more).
     if (!g.used || g.launches <= 4) {
         const int64_t l0 = p->launches;
-        const tn_status s = body(stream);
+        const tn_status s = body(stream, false);
         g.used = true;
         g.launches = p->launches - l0;
         return s;
@@ -2314,7 +2314,7 @@ static tn_status replay(tn_plan_t *p, Graph &g, cudaStream_t stream, F body) {
             if (!l) TN_CUDA(cudaStreamCreateWithFlags(&l, cudaStreamNonBlocking));
         const int64_t l0 = p->launches;
         TN_CUDA(cudaStreamBeginCapture(p->lanes[0], cudaStreamCaptureModeThreadLocal));
-        const tn_status s = body(p->lanes[0]);
+        const tn_status s = body(p->lanes[0], true);
         cudaGraph_t graph = nullptr;
         const cudaError_t e = cudaStreamEndCapture(p->lanes[0], &graph);
         g.launches = p->launches - l0;
@@ -2359,8 +2359,8 @@ static tn_status contract_range(tn_plan_t *p, int64_t slice_begin, int64_t slice
     tn_status s = TN_OK;
     if (graphs && (!p->opts.autotune || p->tuned) && slice_begin == 0 &&
         slice_end == p->num_slices && p->num_slices == p->sb) {
-        s = replay(p, p->g_call, stream, [&](cudaStream_t st) {
-            tn_status e = run_prologue(p, st);
+        s = replay(p, p->g_call, stream, [&](cudaStream_t st, bool captured) {
+            tn_status e = run_prologue(p, st, captured);
             if (e == TN_OK) e = bind_leaves(p, true, 0, p->sb, st);
             return e == TN_OK ? run_batch(p, p->sb, st) : e;
         });
@@ -2371,8 +2371,10 @@ static tn_status contract_range(tn_plan_t *p, int64_t slice_begin, int64_t slice
         const bool prologue = !p->exec[0].empty() || !p->bind_inv.empty() || !p->tiled_inv.empty();
         if (prologue)
             s = graphs ? replay(p, p->g_prologue, stream,
-                                [&](cudaStream_t st) { return run_prologue(p, st); })
-                       : run_prologue(p, stream);
+                                [&](cudaStream_t st, bool captured) {
+                                    return run_prologue(p, st, captured);
+                                })
+                       : run_prologue(p, stream, false);
         if (s != TN_OK) return s;
         for (int64_t s0 = slice_begin; s0 < slice_end; s0 += p->sb) {
             const int64_t ns = std::min(p->sb, slice_end - s0);
@@ -2391,7 +2393,7 @@ static tn_status contract_range(tn_plan_t *p, int64_t slice_begin, int64_t slice
                 p->tuned = true;
             } else if (graphs && ns == p->sb) {
                 s = replay(p, p->g_batch, stream,
-                           [&](cudaStream_t st) { return run_batch(p, p->sb, st); });
+                           [&](cudaStream_t st, bool) { return run_batch(p, p->sb, st); });
             } else {
                 s = run_batch(p, ns, stream);
             }

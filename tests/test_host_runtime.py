@@ -115,3 +115,25 @@ def test_a_workspace_of_what_path_order_takes_is_enough(fake, case):
         assert plan.info()["slices_in_flight"] == free.info()["slices_in_flight"]
         plan.close(); free.close()
     """ % (case, IN_PATH_ORDER[case]))
+
+
+def test_direct_launches_on_the_default_stream_take_no_branches(fake):
+    # branches of the prologue exist in a captured graph only; the default stream's handle is 0, as is
+    # a stream's that has not been made yet
+    fake("""
+    net = W.build_network(W.random_circuit(3, 4, 8, 3), list(range(6, 12)), {i: 0 for i in range(6)})
+    path = W.greedy_path(net.labels, net.open_labels)
+    cut = W.greedy_slices(net.labels, net.open_labels, path, 2)
+    tnet = tn.Network.from_workload(net)
+    for stream in (NULL, MINE):
+        plan = tn.Plan(tnet, path, cut, use_graph=True, max_slices_in_flight=1)
+        plan.contract_host(0, 1, stream=stream)
+        assert calls("cudaStreamWaitEvent") == 0 and calls("cudaEventRecord") == 0
+        plan.close()
+    # as a whole call, and again for work of up to 4 launches, which never becomes a graph
+    plan = tn.Plan(tnet, path, cut, use_graph=True)
+    plan.contract_host(stream=NULL)
+    assert calls("cudaStreamWaitEvent") == 0
+    plan.close()
+    tnet.close()
+    """)
