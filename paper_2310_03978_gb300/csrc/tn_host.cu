@@ -193,7 +193,7 @@ struct Chain {               // a run of small element-wise steps launched toget
 
 struct Graph {
     bool used = false;       // its work has run once, directly
-    cudaGraph_t graph = nullptr;
+    bool failed = false;     // it could not be made: its work is launched directly
     cudaGraphExec_t exec = nullptr;
     int64_t launches = 0;    // kernels inside one replay
 };
@@ -2309,23 +2309,14 @@ static tn_status replay(tn_plan_t *p, Graph &g, cudaStream_t stream, F body) {
         g.launches = p->launches - l0;
         return s;
     }
-    if (!g.exec) {
-        for (cudaStream_t &l : p->lanes)
-            if (!l) TN_CUDA(cudaStreamCreateWithFlags(&l, cudaStreamNonBlocking));
+    if (!g.exec && !g.failed) {
         const int64_t l0 = p->launches;
-        TN_CUDA(cudaStreamBeginCapture(p->lanes[0], cudaStreamCaptureModeThreadLocal));
-        const tn_status s = body(p->lanes[0], true);
-        cudaGraph_t graph = nullptr;
-        const cudaError_t e = cudaStreamEndCapture(p->lanes[0], &graph);
-        g.launches = p->launches - l0;
+        g.failed = !tn::capture_graph(p->lanes, &g.exec,
+                                      [&](cudaStream_t st) { return body(st, true); });
+        if (!g.failed) g.launches = p->launches - l0;
         p->launches = l0;
-        if (s != TN_OK || e != cudaSuccess) {
-            if (graph) cudaGraphDestroy(graph);
-            return s != TN_OK ? s : fail(TN_ERR_CUDA, "graph capture: %s", cudaGetErrorString(e));
-        }
-        g.graph = graph;
-        TN_CUDA(cudaGraphInstantiate(&g.exec, g.graph, 0));
     }
+    if (g.failed) return body(stream, false);
     TN_CUDA(cudaGraphLaunch(g.exec, stream));
     p->launches += g.launches;
     return TN_OK;
@@ -2490,7 +2481,6 @@ void tn_destroy(void *handle) {
         }
         for (Graph *g : {&p->g_prologue, &p->g_batch, &p->g_call}) {
             if (g->exec) cudaGraphExecDestroy(g->exec);
-            if (g->graph) cudaGraphDestroy(g->graph);
         }
         for (cudaStream_t l : p->lanes)
             if (l) cudaStreamDestroy(l);

@@ -492,6 +492,32 @@ private:
     int cur_ = 0, next_ = 0;
 };
 
+// Captures what body(lanes[0]) launches as an executable graph; the lanes are streams made here at
+// first use.  Where that cannot be done (no memory for the graph, say) nothing is left behind, no error
+// stays pending, and the caller launches the work itself.
+template <class Body>
+bool capture_graph(cudaStream_t *lanes, cudaGraphExec_t *exec, Body body) {
+    bool ok = true;
+    for (int i = 0; i < Branches::kLanes && ok; ++i)
+        if (!lanes[i])
+            ok = cudaStreamCreateWithFlags(&lanes[i], cudaStreamNonBlocking) == cudaSuccess;
+    cudaGraph_t graph = nullptr;
+    if (ok && cudaStreamBeginCapture(lanes[0], cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
+        ok = body(lanes[0]) == TN_OK;
+        ok = cudaStreamEndCapture(lanes[0], &graph) == cudaSuccess && ok;
+        ok = ok && cudaGraphInstantiate(exec, graph, 0) == cudaSuccess;
+        if (graph) cudaGraphDestroy(graph);
+    } else {
+        ok = false;
+    }
+    if (!ok) {
+        *exec = nullptr;
+        (void)cudaGetLastError();
+        clear_error();
+    }
+    return ok;
+}
+
 }  // namespace tn
 
 // A loaded network (tn_network_load): labels and offsets on the host, the complex128 data on the

@@ -115,7 +115,7 @@ struct tn_sparse_plan {
     // captured on.  It is made at the second call: making it costs more than one call's launches.
     bool called = false;
     cudaStream_t lanes[tn::Branches::kLanes] = {};
-    cudaGraph_t graph = nullptr;
+    bool graph_failed = false;  // it could not be made: calls launch directly
     cudaGraphExec_t graph_exec = nullptr;
     int64_t graph_launches = 0;
 };
@@ -128,7 +128,6 @@ void sparse_free(tn_sparse_plan_t *p) {
         if (sb.net) tn_destroy(sb.net);
     }
     if (p->graph_exec) cudaGraphExecDestroy(p->graph_exec);
-    if (p->graph) cudaGraphDestroy(p->graph);
     for (cudaStream_t st : p->lanes)
         if (st) cudaStreamDestroy(st);
     if (p->arena) cudaFree(p->arena);
@@ -603,7 +602,8 @@ tn_status sparse_run(tn_sparse_plan_t *p, cudaStream_t stream) {
 }
 
 // The same on the capturing stream lanes[0] and branches of it: every tensor has memory of its
-// own, so only the contraction tree orders the work.
+// own, so only the contraction tree orders the work.  One launch for ~110 and the steps of independent
+// branches at once, for the 24-qubit batch 5.3 -> 4.4 ms.
 tn_status sparse_capture(tn_sparse_plan_t *p) {
     tn::Branches br(p->lanes, p->ten.size());
     TN_CUDA(tn::launch_sparse_leaves(p->leaves_dev, (int32_t)p->leaves.size(), p->max_leaf_rank,
@@ -629,28 +629,6 @@ tn_status sparse_capture(tn_sparse_plan_t *p) {
     return TN_OK;
 }
 
-// One launch for ~110 and the steps of independent branches at once, for the 24-qubit batch
-// 5.3 -> 4.4 ms.
-tn_status sparse_make_graph(tn_sparse_plan_t *p) {
-    for (auto &st : p->lanes)
-        if (!st) TN_CUDA(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
-    const int64_t l0 = p->launches;
-    TN_CUDA(cudaStreamBeginCapture(p->lanes[0], cudaStreamCaptureModeThreadLocal));
-    tn_status s = sparse_capture(p);
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(p->lanes[0], &g);
-    p->graph_launches = p->launches - l0;
-    p->launches = l0;
-    if (s != TN_OK || e != cudaSuccess) {
-        if (g) cudaGraphDestroy(g);
-        return s != TN_OK ? s : fail(TN_ERR_CUDA, "sparse-state graph capture: %s",
-                                     cudaGetErrorString(e));
-    }
-    p->graph = g;
-    TN_CUDA(cudaGraphInstantiate(&p->graph_exec, p->graph, 0));
-    return TN_OK;
-}
-
 }  // namespace
 
 extern "C" {
@@ -668,15 +646,20 @@ tn_status tn_sparse_contract(tn_sparse_plan_t *p, void *amps_dev, void *stream_)
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     TN_CUDA(cudaStreamIsCapturing(stream, &capturing));
     tn_status s = TN_OK;
-    if (capturing != cudaStreamCaptureStatusNone || !p->called) {
+    if (p->called && capturing == cudaStreamCaptureStatusNone && !p->graph_exec &&
+        !p->graph_failed) {
+        const int64_t l0 = p->launches;
+        p->graph_failed = !tn::capture_graph(p->lanes, &p->graph_exec,
+                                             [&](cudaStream_t) { return sparse_capture(p); });
+        p->graph_launches = p->launches - l0;
+        p->launches = l0;
+    }
+    if (p->graph_exec && capturing == cudaStreamCaptureStatusNone) {
+        TN_CUDA(cudaGraphLaunch(p->graph_exec, stream));
+        p->launches += p->graph_launches;
+    } else {
         s = sparse_run(p, stream);
         p->called = true;
-    } else {
-        if (!p->graph_exec) s = sparse_make_graph(p);
-        if (s == TN_OK) {
-            TN_CUDA(cudaGraphLaunch(p->graph_exec, stream));
-            p->launches += p->graph_launches;
-        }
     }
     if (s != TN_OK) return s;
     TN_CUDA(tn::launch_sparse_amps(p->base[(size_t)p->root], p->sample_idx,

@@ -137,3 +137,42 @@ def test_direct_launches_on_the_default_stream_take_no_branches(fake):
     plan.close()
     tnet.close()
     """)
+
+
+@pytest.mark.parametrize("call", ["cudaGraphInstantiate", "cudaStreamBeginCapture",
+                                  "cudaStreamCreateWithFlags", "cudaEventCreateWithFlags"])
+def test_a_graph_that_cannot_be_made_leaves_the_direct_launches(fake, call):
+    fake("""
+    net = W.build_network(W.random_circuit(4, 5, 10, 3), list(range(12, 20)), {i: 0 for i in range(12)})
+    path = W.greedy_path(net.labels, net.open_labels)
+    cut = W.greedy_slices(net.labels, net.open_labels, path, 2)
+    tnet = tn.Network.from_workload(net)
+    amps = C.create_string_buffer(16 << 8)
+
+    def sparse():
+        plan = tn.SparsePlan(tnet, path, np.zeros((4, 8), np.uint8))
+        run = lambda: tn._check(L.tn_sparse_contract(plan.handle, amps, C.c_void_p(64)))
+        return plan, run, lambda: plan.info()["kernel_launches"]
+
+    def dense(flight):
+        plan = tn.Plan(tnet, path, cut, use_graph=True, max_slices_in_flight=flight)
+        run = lambda: plan.contract_host(stream=MINE)
+        return plan, run, lambda: plan.info()["kernel_launches"]
+
+    # one slice in flight: two graphs, of which the batch's has no branches and needs no events
+    for make in (sparse, lambda: dense(0), lambda: dense(1))[:2 if "%s" == "cudaEventCreateWithFlags" else 3]:
+        before = [L.fake_alive(k) for k in range(5)]
+        plan, run, launched = make()
+        L.fake_fail(b"%s", 0, 1000)
+        run()
+        first = launched()
+        for _ in range(2):
+            run()
+        L.fake_fail(b"%s", 0, 0)
+        run()
+        assert calls("cudaGraphLaunch") == 0 and launched() == 4 * first
+        assert L.fake_alive(2) == before[2] and L.fake_alive(3) == 0
+        plan.close()
+        assert [L.fake_alive(k) for k in range(5)] == before
+    tnet.close()
+    """ % (call, call, call))
