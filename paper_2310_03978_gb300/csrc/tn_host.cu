@@ -610,6 +610,7 @@ static void arrange(tn_plan_t *p, int level) {
     const tn_precision mode = p->mode;
     p->planars.clear();
     p->chains.clear();
+    for (auto &order : p->exec) order.clear();
     p->nmeta = p->nmeta_inv = 0;
     p->prologue_branches = false;
     for (auto &x : p->tensors) {
