@@ -2302,8 +2302,12 @@ static tn_status run_prologue(tn_plan_t *p, cudaStream_t stream, bool captured) 
 // 111 us).
 template <class F>
 static tn_status replay(tn_plan_t *p, Graph &g, cudaStream_t stream, F body) {
-    // A graph of up to 4 launches costs more to launch than they do (a 2-launch one ~3 us more).
-    if (!g.used || g.launches <= 4) {
+    // A graph of up to 4 launches costs more to launch than they do (a 2-launch one ~3 us more).  A
+    // caller that captures this stream gets the launches themselves: instantiating a graph meanwhile
+    // would invalidate the capture.
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    TN_CUDA(cudaStreamIsCapturing(stream, &capturing));
+    if (!g.used || g.launches <= 4 || capturing != cudaStreamCaptureStatusNone) {
         const int64_t l0 = p->launches;
         const tn_status s = body(stream, false);
         g.used = true;

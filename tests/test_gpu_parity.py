@@ -1441,3 +1441,36 @@ def test_plans_under_a_tight_workspace_give_the_same_amplitudes(tn, case):
             plan = None
     assert len(seen) > 1
     tnet.close()
+
+
+# A caller that captures its stream gets the launches, whatever the plan has run before.
+@pytest.mark.parametrize("calls", [0, 1, 2])
+@pytest.mark.parametrize("flight", [0, 1])
+def test_plans_with_graphs_under_a_callers_capture(tn, calls, flight):
+    net = W.build_network(W.random_circuit(4, 5, 10, 3), list(range(12, 20)),
+                          {q: 0 for q in range(12)})
+    path = W.greedy_path(net.labels, net.open_labels)
+    cut = W.greedy_slices(net.labels, net.open_labels, path, 2)
+    tnet = tn.Network.from_workload(net)
+    plan = tn.Plan(tnet, path, cut, max_slices_in_flight=flight, use_graph=True)
+    direct = tn.Plan(tnet, path, cut, max_slices_in_flight=flight)
+    ref = torch.zeros(256, dtype=torch.complex128, device="cuda")
+    direct.contract(ref)
+    amps = torch.zeros_like(ref)
+    for _ in range(calls):
+        plan.contract(amps)
+    torch.cuda.synchronize()
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        with torch.cuda.graph(graph, stream=stream):
+            plan.contract(amps, stream=stream)
+        amps.zero_()
+        graph.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(amps, ref)
+    amps.zero_()
+    plan.contract(amps)
+    assert torch.equal(amps, ref)
+    plan.close()
+    direct.close()
+    tnet.close()

@@ -176,3 +176,25 @@ def test_a_graph_that_cannot_be_made_leaves_the_direct_launches(fake, call):
         assert [L.fake_alive(k) for k in range(5)] == before
     tnet.close()
     """ % (call, call, call))
+
+
+def test_a_callers_capture_takes_the_launches_themselves(fake):
+    fake("""
+    net = W.build_network(W.random_circuit(4, 5, 10, 3), list(range(12, 20)), {i: 0 for i in range(12)})
+    path = W.greedy_path(net.labels, net.open_labels)
+    cut = W.greedy_slices(net.labels, net.open_labels, path, 2)
+    tnet = tn.Network.from_workload(net)
+    L.fake_capture.argtypes, made = [C.c_void_p], 0
+    for flight in (0, 1):
+        plan = tn.Plan(tnet, path, cut, use_graph=True, max_slices_in_flight=flight)
+        L.fake_capture(64)
+        for _ in range(3):
+            plan.contract_host(stream=MINE)
+        assert calls("cudaStreamBeginCapture") == made
+        L.fake_capture(0)
+        plan.contract_host(stream=MINE)  # used before: now a graph
+        assert calls("cudaStreamBeginCapture") > made
+        made = calls("cudaStreamBeginCapture")
+        plan.close()
+    tnet.close()
+    """)
