@@ -4,6 +4,8 @@
 #include <cuda_fp16.h>
 #include <cuda_bf16.h>
 
+#include <type_traits>
+
 #include "tn_internal.h"
 #include "tn_planar_out.cuh"
 
@@ -592,64 +594,128 @@ __global__ void __launch_bounds__(256, 4)
     }
 }
 
-// amps[x] += sum over slices s (in increasing order) of root[s][x], in FP64.  A thread takes two
-// amplitudes.  With one slice HBM bounds it (40 bytes per amplitude), with several the FP64 adds:
-// 2^24 amplitudes of one slice in 102 us (6.6 TB/s), 128 us when the root's values were widened and added
-// to zeros by the FP64 units too.
-__global__ void __launch_bounds__(256) k_accumulate(const float2 *root, int64_t sstride, int64_t n,
-                                                    int64_t slices, double2 *amps) {
+// amps[x] += sum over slices s (in increasing order) of root[s][x], in FP64.  One slice: a thread takes
+// two amplitudes and HBM bounds it (40 bytes per amplitude), 2^24 amplitudes in 102 us (6.6 TB/s),
+// 128 us when the root's values were widened and added to zeros by the FP64 units too.
+__global__ void __launch_bounds__(256) k_accumulate(const float2 *root, int64_t n, double2 *amps) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n >> 1);
          i += (int64_t)gridDim.x * blockDim.x) {
         double2 a = amps[2 * i], b = amps[2 * i + 1];
-#pragma unroll 4
-        for (int64_t s = 0; s < slices; ++s) {
-            const float4 v = reinterpret_cast<const float4 *>(root + s * sstride)[i];
-            a.x = add_widened(a.x, v.x);
-            a.y = add_widened(a.y, v.y);
-            b.x = add_widened(b.x, v.z);
-            b.y = add_widened(b.y, v.w);
-        }
+        const float4 v = reinterpret_cast<const float4 *>(root)[i];
+        a.x = add_widened(a.x, v.x);
+        a.y = add_widened(a.y, v.y);
+        b.x = add_widened(b.x, v.z);
+        b.y = add_widened(b.y, v.w);
         amps[2 * i] = a;
         amps[2 * i + 1] = b;
     }
-    if (n == 1 && blockIdx.x == 0 && threadIdx.x == 0) {
-        double2 a = amps[0];
-        for (int64_t s = 0; s < slices; ++s) {
-            const float2 v = root[s * sstride];
-            a.x = add_widened(a.x, v.x);
-            a.y = add_widened(a.y, v.y);
+}
+
+// Several slices: a thread takes PER consecutive amplitudes and reads AHEAD slices at once.  What bounds
+// it is the way to memory and back (few amplitudes), the FP64 adds or HBM (many).
+template <int PER, int AHEAD>
+__global__ void __launch_bounds__(256) k_accumulate_slices(const float2 *root, int64_t sstride,
+                                                           int64_t n, int64_t slices,
+                                                           double2 *amps) {
+    using V = typename std::conditional<PER == 2, float4, float2>::type;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n / PER;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        double2 a[PER];
+#pragma unroll
+        for (int q = 0; q < PER; ++q) a[q] = amps[PER * i + q];
+        for (int64_t s = 0; s < slices; s += AHEAD) {
+            V v[AHEAD];
+#pragma unroll
+            for (int j = 0; j < AHEAD; ++j)
+                if (s + j < slices)
+                    v[j] = reinterpret_cast<const V *>(root + (s + j) * sstride)[i];
+#pragma unroll
+            for (int j = 0; j < AHEAD; ++j)
+                if (s + j < slices) {
+                    a[0].x += widen(v[j].x);
+                    a[0].y += widen(v[j].y);
+                    if constexpr (PER == 2) {
+                        a[1].x += widen(v[j].z);
+                        a[1].y += widen(v[j].w);
+                    }
+                }
         }
-        amps[0] = a;
+#pragma unroll
+        for (int q = 0; q < PER; ++q) amps[PER * i + q] = a[q];
     }
 }
 
 // The same with sliced open labels (amplitude batches, Sec. 3.2 slicing applied to open
 // bonds): slice s0 + s adds its root into the block of amps that its bits for those labels (the
 // set bits of `open`) select.  Slices that differ in them write different amplitudes, so a thread
-// takes one root element of the first slice in flight of a block and walks that block's
-// slices in increasing order; 64 one-slice blocks of 64 amplitudes: 3 us, 36 us with a thread per
-// root element walking every slice.
-__global__ void k_accumulate_batched(const float2 *root, int64_t sstride, int64_t n,
-                                     int64_t slices, int64_t s0, const AccMap m, uint64_t open,
-                                     double2 *amps) {
-    const int64_t total = n * slices;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total;
+// takes one root element of one block and walks that block's slices in flight in increasing
+// order.
+//
+// The first id from s0 on whose open bits are o, and the next one with the same open bits; the others
+// count the slices of a block.  An id past the last one wraps to below s0.
+__device__ __forceinline__ uint64_t block_first(uint64_t s0, uint64_t open, uint64_t o) {
+    const uint64_t d = (s0 ^ o) & open;
+    if (d == 0) return s0;
+    const int q = 63 - __clzll((long long)d);  // below 40, the most sliced labels
+    const uint64_t hi = ~0ull << (q + 1);
+    if ((o >> q) & 1ull) return (s0 & hi) | (o & ~hi);
+    const uint64_t rest = ~open & hi;
+    return (((s0 | ~rest) + 1) & rest) | o;
+}
+__device__ __forceinline__ uint64_t block_next(uint64_t sig, uint64_t open) {
+    return (((sig | open) + 1) & ~open) | (sig & open);
+}
+
+// AHEAD: slices read at once.  The threads of a root element, 2^log2_g of them, share its blocks out.
+// These are numbered by the open bits that vary among the slices in flight (kByBlock, `vary`), or the
+// slices are, each a block of its own (kOwnBlock) or, with fewer slices than numbers of blocks, with the
+// first of each block going on (kFirstOfBlock).
+enum { kByBlock, kOwnBlock, kFirstOfBlock };
+template <int AHEAD>
+__global__ void __launch_bounds__(256)
+    k_accumulate_batched(const float2 *root, int64_t sstride, int log2_n, int64_t slices,
+                         int64_t s0_, const AccMap m, uint64_t open, uint64_t vary, int number,
+                         int log2_g, double2 *amps) {
+    const uint64_t s0 = (uint64_t)s0_, end = s0 + (uint64_t)slices;
+    const int64_t blocks = number == kByBlock ? 1ll << __popcll((long long)vary) : slices;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i >> (log2_n + log2_g) == 0;
          i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t x = i % n;
-        uint64_t sig = (uint64_t)(s0 + i / n);
-        const uint64_t rest = sig & ~open;  // counts the slices of one block
-        if (rest != 0 && (((rest - 1) & ~open) | (sig & open)) >= (uint64_t)s0)
-            continue;  // an earlier slice in flight belongs to the same block
-        uint64_t o = deposit((uint64_t)x, m.nroot, m.root_pos);
-        for (int j = 0; j < m.nb; ++j)
-            if ((sig >> m.bj[j]) & 1ull) o |= 1ull << m.bpos[j];
-        double2 a = amps[o];
-        for (; sig < (uint64_t)(s0 + slices); sig = (((sig | open) + 1) & ~open) | (sig & open)) {
-            const float2 v = root[(int64_t)(sig - (uint64_t)s0) * sstride + x];
-            a.x = add_widened(a.x, v.x);
-            a.y = add_widened(a.y, v.y);
+        const uint64_t x = (uint64_t)i & ((1ull << log2_n) - 1);
+        const uint64_t ox = deposit(x, m.nroot, m.root_pos);
+        for (int64_t g = i >> log2_n; g < blocks; g += 1ll << log2_g) {
+            uint64_t sig = s0 + (uint64_t)g;
+            if (number == kByBlock) {
+                uint64_t o = s0 & open & ~vary;
+                for (int j = 0, c = 0; j < m.nb; ++j)
+                    if ((vary >> m.bj[j]) & 1ull) o |= (((uint64_t)g >> c++) & 1ull) << m.bj[j];
+                sig = block_first(s0, open, o);
+                if (sig < s0 || sig >= end) continue;
+            } else if (number == kFirstOfBlock && block_first(s0, open, sig & open) != sig) {
+                continue;
+            }
+            uint64_t o = ox;
+            for (int j = 0; j < m.nb; ++j)
+                if ((sig >> m.bj[j]) & 1ull) o |= 1ull << m.bpos[j];
+            double2 a = amps[o];
+            while (sig < end) {
+                float2 v[AHEAD];
+                uint64_t t = sig;
+#pragma unroll
+                for (int j = 0; j < AHEAD; ++j)
+                    if (t < end) {
+                        v[j] = root[(int64_t)(t - s0) * sstride + (int64_t)x];
+                        t = block_next(t, open);
+                    }
+#pragma unroll
+                for (int j = 0; j < AHEAD; ++j)
+                    if (sig < end) {
+                        a.x += widen(v[j].x);
+                        a.y += widen(v[j].y);
+                        sig = block_next(sig, open);
+                    }
+            }
+            amps[o] = a;
         }
-        amps[o] = a;
     }
 }
 
@@ -951,17 +1017,46 @@ cudaError_t launch_bind_tiled(const BindTiled &b, const double2 *src, float2 *ar
 
 cudaError_t launch_accumulate(const float2 *root, int64_t root_sstride, int64_t n, int64_t slices,
                               double2 *amps, cudaStream_t st) {
-    k_accumulate<<<grid_for(n >> 1, 256), 256, 0, st>>>(root, root_sstride, n, slices, amps);
+    // 64 slices of 2^14 / 2^16 amplitudes 22 / 39 us, 4 of 2^20 34 us, 2 of 2^21 33 us: FP64 adds and
+    // their latency.  (Widened by the FP64 units, a slice after the other: 21 / 38, 33, 33.  Two
+    // amplitudes a thread and four slices at once: 59 for 64 slices of 2^16.)
+    if (slices == 1 && n > 1)
+        k_accumulate<<<grid_for(n >> 1, 256), 256, 0, st>>>(root, n, amps);
+    else if (n >= 1 << 18)
+        (slices <= 2 ? k_accumulate_slices<2, 2> : k_accumulate_slices<2, 4>)
+            <<<grid_for(n >> 1, 256), 256, 0, st>>>(root, root_sstride, n, slices, amps);
+    else
+        (slices <= 4 ? k_accumulate_slices<1, 4> : k_accumulate_slices<1, 16>)
+            <<<grid_for(n, 256), 256, 0, st>>>(root, root_sstride, n, slices, amps);
     return cudaGetLastError();
 }
 
 cudaError_t launch_accumulate_batched(const float2 *root, int64_t root_sstride, int64_t n,
                                       int64_t slices, int64_t s0, const AccMap &m,
                                       double2 *amps, cudaStream_t st) {
-    uint64_t open = 0;
+    if (slices <= 0) return cudaSuccess;
+    uint64_t open = 0, vary = (uint64_t)(s0 ^ (s0 + slices - 1));
     for (int j = 0; j < m.nb; ++j) open |= 1ull << m.bj[j];
-    k_accumulate_batched<<<grid_for(n * slices, 256), 256, 0, st>>>(root, root_sstride, n, slices,
-                                                                   s0, m, open, amps);
+    for (int j = 1; j < 64; j *= 2) vary |= vary >> j;  // every bit up to the highest that changes
+    // setting a thread up costs as much as a few slices, walking a block several at a time costs
+    // registers.  Against a thread per root element that walks every slice: 2^16 elements of 128
+    // slices, 1 / 6 / 7 of their labels open: 81 / 76 / 77 us (78 / 109 / 130); 2^20 of 4, both
+    // open: 39 (36); 2^12 of 256, two open: 26 (123).
+    const bool own = (vary & ~open) == 0;
+    vary &= open;
+    const int log2_n = __builtin_ctzll((uint64_t)n);
+    const int nb = __builtin_popcountll(vary);
+    const int number = own                                       ? kOwnBlock
+                       : nb < 62 && ((int64_t)1 << nb) <= slices ? kByBlock
+                                                                 : kFirstOfBlock;
+    const int64_t blocks = number == kByBlock ? (int64_t)1 << nb : slices;
+    int log2_g = 0;  // threads of a root element: as many as keep the GPU busy
+    while (((int64_t)1 << log2_g) < blocks && log2_n + log2_g < 19) ++log2_g;
+    auto kernel = own || (slices >> nb) <= 1 ? k_accumulate_batched<1>
+                  : (slices >> nb) <= 4 ? k_accumulate_batched<2>
+                                        : k_accumulate_batched<16>;
+    kernel<<<grid_for((int64_t)1 << (log2_n + log2_g), 256), 256, 0, st>>>(
+        root, root_sstride, log2_n, slices, s0, m, open, vary, number, log2_g, amps);
     return cudaGetLastError();
 }
 

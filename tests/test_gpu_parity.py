@@ -1474,3 +1474,33 @@ def test_plans_with_graphs_under_a_callers_capture(tn, calls, flight):
     plan.close()
     direct.close()
     tnet.close()
+
+
+# The sum over slices, bit for bit: few and many amplitudes, every batch length's remainder, sliced open
+# labels at any place of the slice id, ranges that start and end inside a block.  The slices' roots are
+# FP32 values themselves (the other tensor is 1), summed in slice order in FP64.
+@pytest.mark.parametrize("order,rank", [("bbbbb", 0), ("bbbbbb", 1), ("bbbb", 9), ("b", 18),
+                                        ("bb", 18), ("oob", 18), ("boobbob", 4), ("obbbbbo", 0),
+                                        ("bbbbooo", 10), ("ooobbbb", 6), ("oooooo", 13), ("o", 19)])
+def test_sums_over_slices_bit_for_bit(tn, order, rank):
+    rng = np.random.default_rng(len(order) + 10 * rank)
+    ns = len(order)
+    free, S = list(range(rank)), [100 + i for i in range(ns)]
+    A = crandn(rng, ns + rank).astype(np.complex64).astype(np.complex128)
+    bonds = [l for l, c in zip(S, order) if c == "b"]
+    opens = [int(x) for x in rng.permutation(free + [l for l in S if l not in bonds])]
+    net = tn.Network([A, np.ones((2,) * len(bonds), complex)], [S + free, bonds], opens)
+    plan = tn.Plan(net, [(0, 1)], S, max_slices_in_flight=64)
+    cut = [0, 3, (1 << ns) - 1, 1 << ns] if ns > 2 else [0, 1, 1 << ns]
+    got = torch.zeros(1 << len(opens), dtype=torch.complex128, device="cuda")
+    for lo, hi in zip(cut, cut[1:]):
+        plan.contract(got, lo, hi)
+    ref = np.zeros((2,) * len(opens), complex)
+    for s in range(1 << ns):  # bit j of the slice id belongs to the sliced label j
+        bit = {l: (s >> j) & 1 for j, l in enumerate(S)}
+        part = A[tuple(bit[l] for l in S)]  # axes: free
+        at = tuple(bit[l] if l in bit else slice(None) for l in opens)
+        ref[at] += np.transpose(part, [free.index(l) for l in opens if l in free])
+    assert np.array_equal(got.cpu().numpy().reshape(ref.shape), ref)
+    plan.close()
+    net.close()
