@@ -352,6 +352,9 @@ __device__ __forceinline__ void splitk_store(const GemmDesc &d, int64_t s, uint6
     d.C[s * d.sC + (int64_t)(deposit(m, d.lm, d.posC_m) | deposit(n, d.ln, d.posC_n))] = v;
 }
 
+// AHEAD: splits loaded at once, up to 16 (both are powers of two): 2^17 outputs of 32 splits 7.9 us,
+// 2^20 of 4 15.2.
+template <int AHEAD>
 __global__ void __launch_bounds__(256) k_splitk_reduce(GemmDesc d, int64_t slices) {
     const int64_t MN = 1ll << (d.lm + d.ln), s = blockIdx.y;
     float amx = 0.f;
@@ -359,11 +362,15 @@ __global__ void __launch_bounds__(256) k_splitk_reduce(GemmDesc d, int64_t slice
          e += (int64_t)gridDim.x * 256) {
         const float2 *P = d.partial + s * MN + e;
         float re = 0.f, im = 0.f;
-#pragma unroll 8
-        for (int z = 0; z < d.splits; ++z) {
-            const float2 v = P[(int64_t)z * slices * MN];
-            re += v.x;
-            im += v.y;
+        for (int z = 0; z < d.splits; z += AHEAD) {
+            float2 v[AHEAD];
+#pragma unroll
+            for (int j = 0; j < AHEAD; ++j) v[j] = P[(int64_t)(z + j) * slices * MN];
+#pragma unroll
+            for (int j = 0; j < AHEAD; ++j) {
+                re += v[j].x;
+                im += v[j].y;
+            }
         }
         splitk_store(d, s, (uint64_t)e, make_float2(re, im));
         amx = fmaxf(amx, fmaxf(fabsf(re), fabsf(im)));
@@ -378,11 +385,12 @@ __global__ void __launch_bounds__(256) k_splitk_reduce(GemmDesc d, int64_t slice
     }
 }
 
-// The same for 32 splits or more, which come with few outputs (at most ~19 tiles in all, see
-// gemm_simt_splits): one thread per output would wait for a few loads at a time, thousands of
-// splits long.  A block takes 16 outputs; its threads load 128 splits at once, one tile ahead, and
-// the first 16 add them in order from shared memory.
-constexpr int kDeepSplits = 32, kDeepCols = 16, kDeepRows = 128;
+// The same for many splits of few outputs (32 or more, at most 512 outputs per split): one thread per
+// output would wait for a few loads at a time, up to thousands of splits long.  A block takes 16
+// outputs; its threads load 128 splits at once, one tile ahead, and the first 16 add them in order from
+// shared memory.  32 outputs of 256 splits 3.7 us (15 us with a thread per output), 2^13 of 64 4.8
+// (17), 2^14 of 64 5.0 (6.7); past the line 2^16 of 32 took 10 us here, 5.0 with a thread per output.
+constexpr int kDeepSplits = 32, kDeepOutputs = 512, kDeepCols = 16, kDeepRows = 128;
 __global__ void __launch_bounds__(256) k_splitk_reduce_deep(GemmDesc d, int64_t slices) {
     constexpr int PER = kDeepRows * kDeepCols / 256;
     __shared__ float2 buf[2][kDeepRows][kDeepCols];
@@ -1057,14 +1065,18 @@ cudaError_t launch_gemm_simt(const GemmDesc &d, int64_t slices, cudaStream_t st)
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess || d.splits == 1) return e;
     const int64_t MN = 1ll << (d.lm + d.ln);
-    if (d.splits >= kDeepSplits) {
+    if (d.splits >= kDeepSplits && slices * MN <= (int64_t)kDeepOutputs * d.splits) {
         const int64_t blocks = (MN + kDeepCols - 1) / kDeepCols;
         k_splitk_reduce_deep<<<dim3((unsigned)blocks, (unsigned)slices), 256, 0, st>>>(d, slices);
     } else {
         int64_t blocks = (MN + 255) / 256;
         const int64_t most = (152 * 8 + slices - 1) / slices;
         if (blocks > most) blocks = most;
-        k_splitk_reduce<<<dim3((unsigned)blocks, (unsigned)slices), 256, 0, st>>>(d, slices);
+        auto kernel = d.splits >= 16   ? k_splitk_reduce<16>
+                      : d.splits >= 8 ? k_splitk_reduce<8>
+                      : d.splits >= 4 ? k_splitk_reduce<4>
+                                      : k_splitk_reduce<2>;
+        kernel<<<dim3((unsigned)blocks, (unsigned)slices), 256, 0, st>>>(d, slices);
     }
     return cudaGetLastError();
 }

@@ -1504,3 +1504,18 @@ def test_sums_over_slices_bit_for_bit(tn, order, rank):
     assert np.array_equal(got.cpu().numpy().reshape(ref.shape), ref)
     plan.close()
     net.close()
+
+
+# Split-K sums on both sides of the line between a thread per output and a block per 16, alone and
+# with two slices.
+@pytest.mark.parametrize("shape", [(9, 6, 13), (8, 6, 13), (9, 6, 14), (10, 6, 14), (4, 6, 15), (9, 9, 11)])
+@pytest.mark.parametrize("nsl", [0, 1])
+def test_split_k_sums_around_the_deep_kernels_line(tn, shape, nsl):
+    rng = np.random.default_rng(17 * sum(shape) + nsl)
+    (A, B), (la, lb), out = single_step(rng, *shape)
+    K = [l for l in la if l in lb]
+    ref = np.tensordot(A, B, ([la.index(l) for l in K], [lb.index(l) for l in K]))
+    order = [l for l in la if l not in K] + [l for l in lb if l not in K]
+    got, _, kernels = gpu_amps(tn, [A, B], [la, lb], out, [(0, 1)], K[:nsl])
+    assert kernels == ["gemm_simt"]
+    check(got, np.transpose(ref, [order.index(l) for l in out]), 1e-5)
