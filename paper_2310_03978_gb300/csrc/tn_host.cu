@@ -564,20 +564,19 @@ static bool made_in_run(const tn_plan_t *p, int id, int x) {
 }
 static std::vector<ChainPart> chain_parts(const tn_plan_t *p, const Chain &c) {
     const int id = p->steps[c.steps[0]].chain;
-    std::unordered_map<int, int> top, part, depth;  // per step: the step that reads its result, if
-                                                    // in the run; its part; its level
+    // per step: the step that reads its result, if in the run (-1: none); its part; its level
+    std::vector<int> top(p->steps.size(), -1), part(p->steps.size()), depth(p->steps.size());
     for (int k : c.steps)
         for (int x : {p->steps[k].a, p->steps[k].b})
             if (made_in_run(p, id, x)) top[p->tensors[x].producer] = k;
     std::vector<ChainPart> parts;
     for (size_t i = c.steps.size(); i-- > 0;) {  // readers before the steps they read
         const int k = c.steps[i];
-        const auto t = top.find(k);
-        if (t == top.end()) {
+        if (top[k] < 0) {
             part[k] = (int)parts.size();
             parts.emplace_back();
         } else {
-            part[k] = part[t->second];
+            part[k] = part[top[k]];
         }
     }
     for (int k : c.steps) {
@@ -719,15 +718,31 @@ static void arrange(tn_plan_t *p, int level) {
             return st.kernel == K_GENERIC && rc <= tn::kChainMaxRankC && nk <= tn::kChainMaxNk &&
                    rc + nk <= tn::kChainMaxWork;
         };
-        // In shared memory a run also takes streaming and GEMM steps of up to 2^16
-        // multiply-adds: a launch of their own costs 4-10 us, the block less than 1.  The sums
-        // are the same bits: one chain over k, or (GEMM, K > 16, too short to be split) blocks of
-        // 16 terms.
-        auto small_shm = [&](const Step &st) {
+        // In shared memory a run also takes streaming and GEMM steps of up to 2^16 multiply-adds.  The
+        // sums are the same bits: one chain over k, or (GEMM, K > 16, too short to be split) blocks of
+        // 16 terms.  One block then does what the step's own kernel gives the whole GPU; a step whose
+        // kernel would be faster by more than `slack` us is left alone.  Measured, in us: a multiply-add
+        // in the block 0.05e-3 (K <= 4), 0.12e-3 (8) and 0.25e-3 (from 16 on, where the rows of an
+        // operand meet in the same banks), a term of a sum 0.008 at least; the kernels 2 to 5 up to
+        // K = 2^4, 9 to 26 for a GEMM of K = 2^6 to 2^8, 28 for an element-wise sum of 2^10.
+        auto in_block = [&](const Step &st) {
+            const int nk = (int)st.K.size();
+            const double mac = nk <= 2 ? 0.05e-3 : (nk == 3 ? 0.12e-3 : 0.25e-3);
+            return std::max(std::ldexp(mac, rank_c(st) + nk), std::ldexp(0.008, nk));
+        };
+        auto in_kernel = [&](const Step &st) {
+            const int nk = std::min((int)st.K.size(), 10);
+            return st.kernel == K_GEMM     ? 3.5 + std::ldexp(0.09, nk)
+                   : st.kernel == K_STREAM ? 1.8 + std::ldexp(0.06, nk)
+                                           : 2.0 + std::ldexp(0.026, nk);
+        };
+        constexpr double kRunUs = 3.0;  // a run's launch, and its copies in and out per element
+        constexpr double kCopyUs = 0.45e-3;
+        auto absorbed = [&](const Step &st, double slack) {
             const int rc = rank_c(st), nk = (int)st.K.size();
-            return tiny(st) || ((st.kernel == K_STREAM || st.kernel == K_GEMM) && !st.thin_tc &&
-                                st.direct_planar < 0 && rc <= tn::kChainMaxRankC && nk <= 8 &&
-                                rc + nk <= 16);
+            return (st.kernel == K_STREAM || st.kernel == K_GEMM) && !st.thin_tc &&
+                   st.direct_planar < 0 && rc <= tn::kChainMaxRankC && nk <= 8 && rc + nk <= 16 &&
+                   in_block(st) <= in_kernel(st) + slack;
         };
         // An outer product of 2^10 or more outputs that makes an operand (see Tensor), or with no
         // other tiny step beside it in the path, rounds as k_generic_k1 does, the others as
@@ -743,7 +758,14 @@ static void arrange(tn_plan_t *p, int level) {
                            (p->tensors[st.c].operand || !(plain(i - 1) || plain(i + 1)));
         }
         const size_t chains0 = p->chains.size();
-        auto schedule = [&](auto small) {
+        auto schedule = [&](double slack) {
+            for (int s : todo) {
+                p->steps[s].chain = -1;
+                p->steps[s].chain_head = false;
+            }
+            p->exec[cls].clear();
+            p->chains.resize(chains0);
+            const auto small = [&](const Step &st) { return tiny(st) || absorbed(st, slack); };
             std::vector<char> done(path_len, 0);
             for (int s = 0; s < path_len; ++s) done[s] = cls == 1 && !p->steps[s].dep;
             auto ready = [&](const Step &st) {
@@ -759,8 +781,17 @@ static void arrange(tn_plan_t *p, int level) {
                         c.steps.push_back(s);
                     }
                 if (c.steps.empty()) return;
-                p->steps[c.steps[0]].chain_head = true;
+                Step &head = p->steps[c.steps[0]];
                 p->exec[cls].push_back(c.steps[0]);
+                // A step alone saves no launch, and its own kernel is mostly the faster one (2^7 x 2^5,
+                // K = 16: 25 us a call, 34 us as a run).  It rounds a product of 2^10 outputs in its
+                // own way.
+                if (c.steps.size() == 1 && in_kernel(head) <= kRunUs + in_block(head) &&
+                    (!head.K.empty() || rank_c(head) < 10 || head.fused_mul)) {
+                    head.chain = -1;
+                    return;
+                }
+                head.chain_head = true;
                 p->chains.push_back(std::move(c));
             };
             for (int s : todo) {
@@ -791,20 +822,63 @@ static void arrange(tn_plan_t *p, int level) {
             }
             continue;
         }
-        schedule(small_shm);
-        bool fits = true;
-        for (size_t c = chains0; c < p->chains.size(); ++c)
-            for (const auto &part : chain_parts(p, p->chains[c]))
-                fits = fits && part.fits();
-        if (!fits) {  // the streaming and GEMM steps need the whole run in shared memory
-            for (int s : todo) {
-                p->steps[s].chain = -1;
-                p->steps[s].chain_head = false;
+        // How much to absorb: each step also saves the gap before its launch (2 us from the host, next to
+        // none in a graph), and where it stands between small steps the launch and copies of a run.
+        // The slack with the least time in all is taken, by 5 % at least: the estimate is rough, and in
+        // the prologue's graph a run waits for the operands of all its steps.  Streaming and GEMM steps
+        // need their run in shared memory.
+        const int64_t flight = cls == 0 ? 1
+                               : p->opts.max_slices_in_flight > 0
+                                   ? std::min(p->num_slices, p->opts.max_slices_in_flight)
+                                   : p->num_slices;
+        auto cost = [&](double slack) {
+            const double gap = p->opts.use_graph ? 0.2 : 2.0;
+            double us = 0;
+            for (int s : p->exec[cls]) {
+                const Step &st = p->steps[s];
+                us += gap;
+                if (st.chain < 0) {
+                    us += in_kernel(st);
+                    continue;
+                }
+                double longest = 0;
+                for (const auto &part : chain_parts(p, p->chains[st.chain])) {
+                    double work = 0;
+                    bool any = false;
+                    for (int k : part.steps) {
+                        const Step &q = p->steps[k];
+                        if (absorbed(q, slack)) {
+                            any = true;
+                            work += in_block(q);
+                        }
+                        for (int x : {q.a, q.b})
+                            if (!made_in_run(p, st.chain, x))
+                                work += std::ldexp(kCopyUs, p->tensors[x].rank());
+                    }
+                    if (any && !part.fits()) return -1.0;
+                    // the part's last step makes what is read elsewhere
+                    work += std::ldexp(kCopyUs, rank_c(p->steps[part.steps.back()]));
+                    longest = std::max(longest, work);
+                }
+                us += kRunUs + longest * (double)((flight + 151) / 152);
             }
-            p->exec[cls].clear();
-            p->chains.resize(chains0);
-            schedule(tiny);
+            return us;
+        };
+        constexpr double kNone = -1e9;
+        double best = kNone, last = kNone, least = -1;
+        for (double slack : {kNone, 0.0, 6.0, 12.0}) {
+            if (slack > kNone && std::none_of(todo.begin(), todo.end(), [&](int s) {
+                    return absorbed(p->steps[s], slack) && !absorbed(p->steps[s], last);
+                }))
+                continue;
+            schedule(last = slack);
+            const double us = cost(slack);
+            if (us >= 0 && (least < 0 || us < 0.95 * least)) {
+                least = us;
+                best = slack;
+            }
         }
+        if (best != last) schedule(best);
     }
     // op timeline: invariant leaves, invariant steps, sliced leaves, dependent steps (each
     // tensor-core step preceded by its conversions; a run of chained steps is one op, so every

@@ -1411,7 +1411,7 @@ def test_runs_of_small_steps_at_the_shared_memory_limit(tn, ops):
 # Less workspace: without branches in the prologue, then in path order with planes made just before
 # their use.  The amplitudes stay the same bits.
 @pytest.mark.parametrize("case", [(5, 5, 10, 6, 4, "c64"), (5, 5, 10, 6, 4, "fp16_scaled"),
-                                  (3, 5, 11, 12, 0, "tf32"), (4, 3, 6, 12, 0, "tf32"),
+                                  (3, 5, 11, 12, 0, "tf32"), (4, 5, 10, 8, 2, "fp16_scaled"),
                                   (4, 5, 12, 10, 2, "split_tf32")], ids=str)
 def test_plans_under_a_tight_workspace_give_the_same_amplitudes(tn, case):
     rows, cols, cycles, opens, nsl, mode = case
@@ -1519,3 +1519,45 @@ def test_split_k_sums_around_the_deep_kernels_line(tn, shape, nsl):
     got, _, kernels = gpu_amps(tn, [A, B], [la, lb], out, [(0, 1)], K[:nsl])
     assert kernels == ["gemm_simt"]
     check(got, np.transpose(ref, [order.index(l) for l in out]), 1e-5)
+
+
+# Small streaming and GEMM steps give the same bits in a run as by their own kernels; which of the
+# two they take depends on the steps around them and on use_graph.
+@pytest.mark.parametrize("shapes", ["11.1.2 6.6.3", "6.6.2 7.5.3 5.7.4", "5.4.7 4.4.8", "10.2.3 6.5.5",
+                                    "3.4.8 6.6.4 8.4.3"])
+@pytest.mark.parametrize("nsl", [0, 2])
+def test_small_steps_give_the_same_bits_in_runs_and_alone(tn, shapes, nsl):
+    rng = np.random.default_rng(len(shapes) + nsl)
+    S, fresh, tensors, labels, path, wires = list(range(nsl)), 100, [], [], [], None
+    for shape in shapes.split():  # each step has a tensor that the one before it made, if any
+        m, n, k = (int(x) for x in shape.split("."))
+        if wires is None:
+            wires = [fresh + i for i in range(m + k)]
+            fresh += m + k
+            tensors.append(crandn(rng, m + k + nsl))
+            labels.append(S + wires)
+        have = len(wires)
+        K = [int(x) for x in rng.choice(wires, min(k, have), replace=False)]
+        N = [fresh + i for i in range(n)]
+        fresh += n
+        tensors.append(crandn(rng, len(K) + n + (nsl if len(labels) == 1 else 0), 2.0 ** -(k / 2)))
+        labels.append(K + N + (S if len(labels) == 1 else []))
+        path.append((0, len(labels) - 1))
+        wires = [w for w in wires if w not in K] + N
+        for g in range(len(wires) - 9):  # small steps between them, down to rank 9
+            tensors.append(crandn(rng, 1))
+            labels.append([wires.pop(0)])
+            path.append((0, len(labels) - 1))
+    net = tn.Network(tensors, labels, wires)
+    amps = {}
+    for graph, profile in ((True, False), (False, False), (False, True)):
+        plan = tn.Plan(net, path, S, use_graph=graph, profile=profile)
+        for _ in range(3):
+            a = torch.zeros(1 << len(wires), dtype=torch.complex128, device="cuda")
+            plan.contract(a)
+        amps[graph, profile] = a.cpu().numpy()
+        plan.close()
+    net.close()
+    check(amps[True, False], O.contract(tensors, labels, wires, path), TOL["c64"])
+    assert np.array_equal(amps[True, False], amps[False, False])
+    assert np.array_equal(amps[True, False], amps[False, True])
