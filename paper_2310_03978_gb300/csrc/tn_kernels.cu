@@ -470,15 +470,51 @@ __device__ __forceinline__ float narrow(double x) {
     const uint32_t up = (lo & 0x1fffffffu) + (m & 1u) > 0x10000000u;
     return __uint_as_float(sign | (m + up));
 }
-__device__ __forceinline__ double widen(float x) {
+__device__ __forceinline__ double widen_normal(float x) {
     const uint32_t u = __float_as_uint(x), sign = u & 0x80000000u, mag = u ^ sign;
-    if ((mag >> 23) - 1u > 253u && mag != 0) return (double)x;  // subnormal, infinite or NaN
-    return __hiloint2double((int)(sign | (mag ? (mag >> 3) + (896u << 20) : 0u)),
-                            (int)(u << 29));
+    return __hiloint2double((int)(sign | (mag ? (mag >> 3) + (896u << 20) : 0u)), (int)(u << 29));
 }
-// a + x; an amplitude that is still +0, as before its first slice, takes x as it is
-__device__ __forceinline__ double add_widened(double a, float x) {
-    return __double_as_longlong(a) != 0 ? a + widen(x) : widen(x == 0.f ? 0.f : x);
+__device__ __forceinline__ bool odd(float x) {  // subnormal, infinite or NaN
+    const uint32_t u = __float_as_uint(x) << 1;
+    return (u >> 24) - 1u > 253u && u != 0;
+}
+// N values under one test: with a branch for each, the adds that follow wait for one another (one
+// slice of 2^24 amplitudes onto others: 189 us).
+template <int N>
+__device__ __forceinline__ void widen(const float (&v)[N], double (&d)[N]) {
+    bool any = false;
+#pragma unroll
+    for (int i = 0; i < N; ++i) any = any || odd(v[i]);
+    if (any) {
+#pragma unroll
+        for (int i = 0; i < N; ++i) d[i] = (double)v[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) d[i] = widen_normal(v[i]);
+    }
+}
+// a += v for two amplitudes.  Amplitudes that are all still +0, as before their first slice, take v as
+// it is (-0 as +0) and need no FP64 unit.
+__device__ __forceinline__ void add_widened2(double2 &a, double2 &b, float4 v) {
+    double2 p, q;
+    if (odd(v.x) || odd(v.y) || odd(v.z) || odd(v.w)) {
+        p = make_double2((double)v.x, (double)v.y);
+        q = make_double2((double)v.z, (double)v.w);
+    } else {
+        p = make_double2(widen_normal(v.x), widen_normal(v.y));
+        q = make_double2(widen_normal(v.z), widen_normal(v.w));
+    }
+    const auto bits = [](double x) { return __double_as_longlong(x); };
+    if ((bits(a.x) | bits(a.y) | bits(b.x) | bits(b.y)) == 0) {
+        const auto plus = [&](double x) {
+            return __longlong_as_double(bits(x) == bits(-0.0) ? 0 : bits(x));
+        };
+        a = make_double2(plus(p.x), plus(p.y));
+        b = make_double2(plus(q.x), plus(q.y));
+    } else {
+        a = make_double2(a.x + p.x, a.y + p.y);
+        b = make_double2(b.x + q.x, b.y + q.y);
+    }
 }
 
 // Leaf binding: grid (item, slice, chunk); the blocks of one (item, slice) share its elements.
@@ -595,17 +631,14 @@ __global__ void __launch_bounds__(256, 4)
 }
 
 // amps[x] += sum over slices s (in increasing order) of root[s][x], in FP64.  One slice: a thread takes
-// two amplitudes and HBM bounds it (40 bytes per amplitude), 2^24 amplitudes in 102 us (6.6 TB/s),
-// 128 us when the root's values were widened and added to zeros by the FP64 units too.
+// two amplitudes and HBM bounds it (40 bytes per amplitude), 2^24 amplitudes in 97 us (6.9 TB/s),
+// added to others as to zeros; 128 us when the FP64 units widened the root's values too.
 __global__ void __launch_bounds__(256) k_accumulate(const float2 *root, int64_t n, double2 *amps) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < (n >> 1);
          i += (int64_t)gridDim.x * blockDim.x) {
         double2 a = amps[2 * i], b = amps[2 * i + 1];
         const float4 v = reinterpret_cast<const float4 *>(root)[i];
-        a.x = add_widened(a.x, v.x);
-        a.y = add_widened(a.y, v.y);
-        b.x = add_widened(b.x, v.z);
-        b.y = add_widened(b.y, v.w);
+        add_widened2(a, b, v);
         amps[2 * i] = a;
         amps[2 * i + 1] = b;
     }
@@ -624,21 +657,22 @@ __global__ void __launch_bounds__(256) k_accumulate_slices(const float2 *root, i
 #pragma unroll
         for (int q = 0; q < PER; ++q) a[q] = amps[PER * i + q];
         for (int64_t s = 0; s < slices; s += AHEAD) {
-            V v[AHEAD];
+            float v[2 * PER * AHEAD] = {};
+            double d[2 * PER * AHEAD];
 #pragma unroll
             for (int j = 0; j < AHEAD; ++j)
                 if (s + j < slices)
-                    v[j] = reinterpret_cast<const V *>(root + (s + j) * sstride)[i];
+                    *reinterpret_cast<V *>(v + 2 * PER * j) =
+                        reinterpret_cast<const V *>(root + (s + j) * sstride)[i];
+            widen(v, d);
 #pragma unroll
             for (int j = 0; j < AHEAD; ++j)
-                if (s + j < slices) {
-                    a[0].x += widen(v[j].x);
-                    a[0].y += widen(v[j].y);
-                    if constexpr (PER == 2) {
-                        a[1].x += widen(v[j].z);
-                        a[1].y += widen(v[j].w);
+                if (s + j < slices)
+#pragma unroll
+                    for (int q = 0; q < PER; ++q) {
+                        a[q].x += d[2 * (PER * j + q)];
+                        a[q].y += d[2 * (PER * j + q) + 1];
                     }
-                }
         }
 #pragma unroll
         for (int q = 0; q < PER; ++q) amps[PER * i + q] = a[q];
@@ -698,19 +732,23 @@ __global__ void __launch_bounds__(256)
                 if ((sig >> m.bj[j]) & 1ull) o |= 1ull << m.bpos[j];
             double2 a = amps[o];
             while (sig < end) {
-                float2 v[AHEAD];
+                float v[2 * AHEAD] = {};
+                double d[2 * AHEAD];
                 uint64_t t = sig;
 #pragma unroll
                 for (int j = 0; j < AHEAD; ++j)
                     if (t < end) {
-                        v[j] = root[(int64_t)(t - s0) * sstride + (int64_t)x];
+                        const float2 f = root[(int64_t)(t - s0) * sstride + (int64_t)x];
+                        v[2 * j] = f.x;
+                        v[2 * j + 1] = f.y;
                         t = block_next(t, open);
                     }
+                widen(v, d);
 #pragma unroll
                 for (int j = 0; j < AHEAD; ++j)
                     if (sig < end) {
-                        a.x += widen(v[j].x);
-                        a.y += widen(v[j].y);
+                        a.x += d[2 * j];
+                        a.y += d[2 * j + 1];
                         sig = block_next(sig, open);
                     }
             }
@@ -1017,16 +1055,15 @@ cudaError_t launch_bind_tiled(const BindTiled &b, const double2 *src, float2 *ar
 
 cudaError_t launch_accumulate(const float2 *root, int64_t root_sstride, int64_t n, int64_t slices,
                               double2 *amps, cudaStream_t st) {
-    // 64 slices of 2^14 / 2^16 amplitudes 22 / 39 us, 4 of 2^20 34 us, 2 of 2^21 33 us: FP64 adds and
-    // their latency.  (Widened by the FP64 units, a slice after the other: 21 / 38, 33, 33.  Two
-    // amplitudes a thread and four slices at once: 59 for 64 slices of 2^16.)
+    // 64 slices of 2^14 / 2^16 amplitudes 15 / 23 us, 4 of 2^20 and 2 of 2^21 19 us: FP64 adds and
+    // their latency, then HBM.  (Widened by the FP64 units, a slice after the other: 21 / 38, 33, 33.)
     if (slices == 1 && n > 1)
         k_accumulate<<<grid_for(n >> 1, 256), 256, 0, st>>>(root, n, amps);
     else if (n >= 1 << 18)
         (slices <= 2 ? k_accumulate_slices<2, 2> : k_accumulate_slices<2, 4>)
             <<<grid_for(n >> 1, 256), 256, 0, st>>>(root, root_sstride, n, slices, amps);
     else
-        (slices <= 4 ? k_accumulate_slices<1, 4> : k_accumulate_slices<1, 16>)
+        (slices <= 8 ? k_accumulate_slices<1, 4> : k_accumulate_slices<1, 16>)
             <<<grid_for(n, 256), 256, 0, st>>>(root, root_sstride, n, slices, amps);
     return cudaGetLastError();
 }
@@ -1040,8 +1077,8 @@ cudaError_t launch_accumulate_batched(const float2 *root, int64_t root_sstride, 
     for (int j = 1; j < 64; j *= 2) vary |= vary >> j;  // every bit up to the highest that changes
     // setting a thread up costs as much as a few slices, walking a block several at a time costs
     // registers.  Against a thread per root element that walks every slice: 2^16 elements of 128
-    // slices, 1 / 6 / 7 of their labels open: 81 / 76 / 77 us (78 / 109 / 130); 2^20 of 4, both
-    // open: 39 (36); 2^12 of 256, two open: 26 (123).
+    // slices, 1 / 6 / 7 of their labels open: 48 / 68 / 76 us (78 / 109 / 130); 2^20 of 4, both
+    // open: 37 (36); 2^12 of 256, two open: 19 (123).
     const bool own = (vary & ~open) == 0;
     vary &= open;
     const int log2_n = __builtin_ctzll((uint64_t)n);
