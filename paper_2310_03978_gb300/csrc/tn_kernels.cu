@@ -55,10 +55,10 @@ struct LowOffsets {
         return own.b | ((t & 1) ? bit8.b : 0) | ((t & 2) ? bit9.b : 0);
     }
 };
-// the offsets of the contracted index, up to 10 bits, in shared memory
-__device__ __forceinline__ void k_offsets(const GenericDesc &d, uint64_t *ka, uint64_t *kb) {
-    for (int k = threadIdx.x; k < (1 << d.nk); k += 256) {
-        const Offsets o = deposit2((uint32_t)k, d.nk, d.posA_k, d.posB_k);
+// the offsets of the contracted index's n lowest bits, up to 10, in shared memory
+__device__ __forceinline__ void k_offsets(const GenericDesc &d, int n, uint64_t *ka, uint64_t *kb) {
+    for (int k = threadIdx.x; k < (1 << n); k += 256) {
+        const Offsets o = deposit2((uint32_t)k, n, d.posA_k, d.posB_k);
         ka[k] = o.a;
         kb[k] = o.b;
     }
@@ -402,17 +402,17 @@ __global__ void k_sparse_leaves(const SparseLeafDesc *leaves) {
 // One sparse-state step, summing over the contracted dense bits in increasing order; the operand
 // entries are the configurations gA[c], gB[c] (the projections of c onto each operand's open
 // labels).  A block walks chunks of 2^LB consecutive outputs (see LowOffsets; chunks never leave a
-// configuration, those of less than 256 outputs go several at a time).  Bound by the
-// instructions per output: a deposit per output made the 2^24-output steps take 4 times as long.
+// configuration, those of less than 256 outputs go several at a time), and the sum 2^10 terms at a
+// time, whose offsets are in shared memory (one output of 2^20 terms: 1.7 ms, 13-19 ms with offsets
+// computed for every term).  Bound by the instructions per output: a deposit per output made the 2^24-output steps take 4 times as long.
 __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_t *gA,
                                                      const int32_t *gB, int64_t nconf) {
     __shared__ uint64_t koffA[1024], koffB[1024];
-    const int nk = d.nk;
-    const bool table = nk <= 10;
+    const int nk = d.nk, kb = nk < 10 ? nk : 10;
     const int lb = d.rank_c < 10 ? d.rank_c : 10;
     const LowOffsets low(d, lb);
     const HighOffsets high(d, lb);
-    if (table) k_offsets(d, koffA, koffB);
+    k_offsets(d, kb, koffA, koffB);
     __syncthreads();
     const int64_t K = 1ll << nk;
     const int64_t chunks = nconf << (d.rank_c - lb);
@@ -433,15 +433,19 @@ __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_
             const float2 *A = Ab + low.a(t);
             const float2 *B = Bb + low.b(t);
             float re = 0.f, im = 0.f;
+            for (int64_t k0 = 0; k0 < K; k0 += 1 << kb) {
+                const Offsets o = k0 ? deposit2((uint32_t)(k0 >> kb), nk - kb, d.posA_k + kb,
+                                                d.posB_k + kb)
+                                     : Offsets{0, 0};
+                const float2 *Ak = A + o.a, *Bk = B + o.b;
 #pragma unroll 4
-            for (int64_t k = 0; k < K; ++k) {
-                const uint64_t oa = table ? koffA[k] : deposit((uint64_t)k, nk, d.posA_k);
-                const uint64_t ob = table ? koffB[k] : deposit((uint64_t)k, nk, d.posB_k);
-                const float2 a = A[oa], b = B[ob];
-                re = fmaf(a.x, b.x, re);
-                re = fmaf(-a.y, b.y, re);
-                im = fmaf(a.x, b.y, im);
-                im = fmaf(a.y, b.x, im);
+                for (int k = 0; k < 1 << kb; ++k) {
+                    const float2 a = Ak[koffA[k]], b = Bk[koffB[k]];
+                    re = fmaf(a.x, b.x, re);
+                    re = fmaf(-a.y, b.y, re);
+                    im = fmaf(a.x, b.y, im);
+                    im = fmaf(a.y, b.x, im);
+                }
             }
             Cb[(t << 8) + j0] = make_float2(re, im);
         }

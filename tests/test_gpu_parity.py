@@ -1561,3 +1561,24 @@ def test_small_steps_give_the_same_bits_in_runs_and_alone(tn, shapes, nsl):
     check(amps[True, False], O.contract(tensors, labels, wires, path), TOL["c64"])
     assert np.array_equal(amps[True, False], amps[False, False])
     assert np.array_equal(amps[True, False], amps[False, True])
+
+
+# Long sparse-state contractions of few outputs, whose terms are numbered 2^10 at a time: less than that,
+# as many, and more, with a batch of samples and one.
+@pytest.mark.parametrize("m,n,k", [(0, 0, 9), (1, 2, 10), (0, 0, 11), (3, 1, 11), (2, 2, 13)])
+@pytest.mark.parametrize("ns", [1, 3])
+def test_sparse_state_long_contractions(tn, m, n, k, ns):
+    rng = np.random.default_rng(m + 10 * n + 100 * k + ns)
+    K, M, N = list(range(k)), [100 + i for i in range(m)], [200 + i for i in range(n)]
+    labels = [[int(x) for x in rng.permutation(K + M + [300])],
+              [int(x) for x in rng.permutation(K + N + [301, 302])], M + N + [303]]
+    tensors = [crandn(rng, len(ls), 2.0 ** (-len(ls) / 4)) for ls in labels]
+    opens, path = [300, 301, 302, 303], [(0, 1), (0, 2)]
+    smp = rng.integers(0, 2, (ns, 4), dtype=np.uint8)
+    got, _ = sparse_amps(tn, tensors, labels, opens, path, smp)
+    ref = O.contract_sparse(tensors, labels, opens, path, smp)
+    # FP32 rounding of a running sum of 2^k random terms: 2^-24 2^(k/2) / sqrt(2) of the root of the
+    # summed squares, in four standard deviations and with the other roundings 8 times that at most
+    scale = np.sqrt(O.contract_sparse([np.abs(x) ** 2 + 0j for x in tensors], labels, opens, path,
+                                      smp).real)
+    assert np.all(np.abs(got - ref) <= 8 * 2.0 ** (-24 + k / 2) * scale)
