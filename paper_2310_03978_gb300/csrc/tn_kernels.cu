@@ -404,17 +404,18 @@ __global__ void k_sparse_leaves(const SparseLeafDesc *leaves) {
 // labels).  A block walks chunks of 2^LB consecutive outputs (see LowOffsets; chunks never leave a
 // configuration, those of less than 256 outputs go several at a time), and the sum 2^10 terms at a
 // time, whose offsets are in shared memory (one output of 2^20 terms: 1.7 ms, 13-19 ms with offsets
-// computed for every term).  Bound by the instructions per output: a deposit per output made the 2^24-output steps take 4 times as long.
+// computed for every term; LONG, so that the many small steps don't load that code).  Bound by the
+// instructions per output: a deposit per output made the 2^24-output steps take 4 times as long.
+template <bool LONG>
 __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_t *gA,
                                                      const int32_t *gB, int64_t nconf) {
     __shared__ uint64_t koffA[1024], koffB[1024];
-    const int nk = d.nk, kb = nk < 10 ? nk : 10;
+    const int nk = d.nk, kb = LONG ? 10 : nk;
     const int lb = d.rank_c < 10 ? d.rank_c : 10;
     const LowOffsets low(d, lb);
     const HighOffsets high(d, lb);
     k_offsets(d, kb, koffA, koffB);
     __syncthreads();
-    const int64_t K = 1ll << nk;
     const int64_t chunks = nconf << (d.rank_c - lb);
     const int together = lb < 8 ? 256 >> lb : 1;  // chunks a block takes at once
     const int j0 = together > 1 ? threadIdx.x & ((1 << lb) - 1) : threadIdx.x;
@@ -433,11 +434,7 @@ __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_
             const float2 *A = Ab + low.a(t);
             const float2 *B = Bb + low.b(t);
             float re = 0.f, im = 0.f;
-            for (int64_t k0 = 0; k0 < K; k0 += 1 << kb) {
-                const Offsets o = k0 ? deposit2((uint32_t)(k0 >> kb), nk - kb, d.posA_k + kb,
-                                                d.posB_k + kb)
-                                     : Offsets{0, 0};
-                const float2 *Ak = A + o.a, *Bk = B + o.b;
+            auto sum = [&](const float2 *Ak, const float2 *Bk) {
 #pragma unroll 4
                 for (int k = 0; k < 1 << kb; ++k) {
                     const float2 a = Ak[koffA[k]], b = Bk[koffB[k]];
@@ -446,6 +443,14 @@ __global__ void __launch_bounds__(256) k_sparse_step(GenericDesc d, const int32_
                     im = fmaf(a.x, b.y, im);
                     im = fmaf(a.y, b.x, im);
                 }
+            };
+            if constexpr (LONG) {
+                for (int64_t k0 = 0; k0 < 1ll << (nk - kb); ++k0) {
+                    const Offsets o = deposit2((uint32_t)k0, nk - kb, d.posA_k + kb, d.posB_k + kb);
+                    sum(A + o.a, B + o.b);
+                }
+            } else {
+                sum(A, B);
             }
             Cb[(t << 8) + j0] = make_float2(re, im);
         }
@@ -1018,7 +1023,8 @@ cudaError_t launch_sparse_step(const GenericDesc &d, const int32_t *gA, const in
     const int64_t chunks = nconf << (d.rank_c - lb);
     int64_t blocks = lb < 8 ? (chunks + (256 >> lb) - 1) >> (8 - lb) : chunks;
     if (blocks > 152 * 8) blocks = 152 * 8;
-    k_sparse_step<<<(unsigned)blocks, 256, 0, st>>>(d, gA, gB, nconf);
+    (d.nk > 10 ? k_sparse_step<true> : k_sparse_step<false>)<<<(unsigned)blocks, 256, 0, st>>>(
+        d, gA, gB, nconf);
     return cudaGetLastError();
 }
 
