@@ -2,6 +2,7 @@
 object files linked against a stand-in for the CUDA runtime (fake_cudart.c), whose kernels do
 nothing.  Each test runs in a process of its own."""
 import os
+import re
 import shutil
 import subprocess
 import sys
@@ -198,3 +199,11 @@ def test_a_callers_capture_takes_the_launches_themselves(fake):
         plan.close()
     tnet.close()
     """)
+
+
+def test_a_change_of_any_included_header_rebuilds_the_library():
+    known = {os.path.basename(h) for h in B.headers()}
+    for name in os.listdir(B.CSRC):
+        with open(os.path.join(B.CSRC, name)) as f:
+            for header in re.findall(r'#include "([^"]+)"', f.read()):
+                assert os.path.basename(header) in known, "%s includes %s" % (name, header)
