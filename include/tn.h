@@ -427,7 +427,9 @@ tn_status tn_sparse_plan(const tn_network_t *net, int32_t path_len, const int32_
 /*
  * ADD the amplitudes of the samples into amps_dev (device complex128[num_samples], caller-owned
  * and caller-zeroed, entry i = sample i, repeated samples get the same value); all work on
- * `stream`.  Errors: TN_ERR_INVALID_ARG, TN_ERR_CUDA.
+ * `stream`.  The second call also makes a CUDA graph of the launches (0.1-0.5 ms on the host), which
+ * later calls replay; a call whose stream is being captured launches directly, as does every
+ * call when the graph cannot be made.  Errors: TN_ERR_INVALID_ARG, TN_ERR_CUDA.
  */
 tn_status tn_sparse_contract(tn_sparse_plan_t *plan, void *amps_dev, void *stream);
 

@@ -38,7 +38,7 @@ __device__ __forceinline__ int stage_off(const GemmDesc &d, int p) { return (1 <
 // BK is the K tile, 16.  ONE: a contraction of at most BK terms (8 or 16) in one tile: no second
 // set of sums and no loads ahead, so that four blocks fit an SM instead of two; these steps wait
 // for their loads and stores, not for the FMA units.  2^17 x 64, K = 4: 24 us, 40 us in the general
-// form (67 MB written: 10 us); 2^12 x 2^12, K = 8: 55 us, 76 us; K = 16: 77 us, 94 us.
+// form (67 MB written: 10 us); 2^12 x 2^12, K = 8: 55 us, 75 us; K = 16: 76 us, 96 us.
 template <int BK, bool ONE>
 __global__ void __launch_bounds__(256, ONE ? 4 : 2) k_gemm_simt(GemmDesc d, int64_t tiles_n) {
     constexpr int AS = 2 * 16 * (BM + 1), BS = 2 * 16 * (BN + 1);
@@ -443,13 +443,15 @@ __global__ void __launch_bounds__(256) k_splitk_reduce_deep(GemmDesc d, int64_t 
 // turn leave one block barrier per tile.  For longer K (KS = 0) a block
 // takes one tile and a thread reads its row 8 of K ahead, two 32-byte sectors that only it needs:
 // no barrier stands between the loads and the sums (2^13 x 8, K = 1024: 102 us, 199 us when
-// chunks of 16 were staged in shared memory; 2^17 x 16, K = 32: 26 us, 33 us).  A step whose small operand is A runs with the roles swapped (the complex
-// product commutes).  Each tile (256 x NT) is staged and written in C's order, 32 bytes per
+// chunks of 16 were staged in shared memory; 2^17 x 16, K = 32: 26 us, 33 us).  A step whose
+// small operand is A runs with the roles swapped (the complex product commutes).  Each tile (256 x NT) is staged and written in C's order, 32 bytes per
 // thread and store.  HBM should bound these steps, but the L1 / shared-memory pipe did (86% busy at
 // half the HBM rate): bank conflicts of the stage's reads (row stride NT + 1) and 16-byte accesses
-// that used half of each sector.  With the swizzle and 32-byte accesses 2^27 x 4 with K = 4
-// went from 2.73 to 2.53 ms (5.1 TB/s), 2^26 x 8 with K = 8 from 2.97 to 2.67 ms, and five steps of
-// 4 columns with planar results from 7.93 to 6.84 ms.
+// that used half of each sector.  With the swizzle and 32-byte accesses two
+// slices of 2^27 x 4 with K = 4 and FP16 planes as the result (12.9 GB) went from 2.73 to 2.53 ms
+// (5.1 TB/s), two of 2^26 x 8 with K = 8 (as many bytes) from 2.97 to 2.67 ms, and five steps of
+// 4 columns with planar results from 7.93 to 6.84 ms.  Complex64 results in the rows' own order:
+// 2^26 x 4 with K = 4 (4.3 GB) 0.63 ms (6.8 TB/s), 2^25 x 8 with K = 8 0.64 ms (0.86).
 constexpr int kThinRows = 256;
 // blocks per SM the launch bounds guarantee: rows of A are kept in registers (the walking form:
 // two tiles' worth), so 16 columns fit 2 blocks

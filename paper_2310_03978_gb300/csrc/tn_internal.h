@@ -285,7 +285,7 @@ cudaError_t launch_sparse_thin(const GenericDesc &d, int32_t ln, const int32_t *
 // amps[i] += root[idx[i]] for the n samples (complex128 accumulation)
 cudaError_t launch_sparse_amps(const float2 *root, const int32_t *idx, int64_t n, double2 *amps,
                                cudaStream_t st);
-// Set the chain kernels' shared-memory limit (once per device, outside any stream capture).
+// Set the chain kernels' shared-memory limit (by every plan, outside any stream capture).
 cudaError_t chain_prepare();
 // A run of small steps in shared memory: every slice is worked by `ngroups` independent blocks;
 // `elems`: the most complex64 a group's tensors and records take.
@@ -299,13 +299,14 @@ cudaError_t launch_chain_shm(const ChainGroup *groups, int32_t ngroups, const Ch
 cudaError_t launch_chain(const ChainItem *items, const int32_t *levels, int32_t nlevels,
                          float2 *arena, unsigned int *amax, int64_t sb, int64_t slices,
                          int32_t cluster, cudaStream_t st);
-// Set the CUDA-core kernels' shared-memory limits (once per device, outside any stream capture).
+// Set the CUDA-core kernels' shared-memory limits (by every plan, outside any stream capture).
 cudaError_t simt_prepare();
 cudaError_t launch_gemm_simt(const GemmDesc &d, int64_t slices, cudaStream_t st);
 int gemm_simt_splits(int lm, int ln, int lk, int64_t slices);
 // Thin steps on the CUDA cores: A is the operand with 2^lm >= 256 rows, B has 2^ln <= 16 rows,
-// 2 <= K <= 64; tile_bits = 8 + ln with tb_src / tb_pos sorted as for the tensor-core epilogue
-// (row bits tagged 128 | bit); complex64 output only.
+// 2 <= K <= 1024; tile_bits = 8 + ln with tb_src / tb_pos sorted as for the tensor-core epilogue,
+// tb_src as index bits of the stage (columns first), bank from stage_choose_banks; complex64 or
+// planar results.
 cudaError_t launch_gemm_thin(const GemmDesc &d, int64_t slices, cudaStream_t st);
 cudaError_t launch_bind(const BindItem *items_dev, int32_t n_items, const double2 *src,
                         float2 *arena, int64_t slice_begin, int64_t slices, int32_t max_rank,
@@ -377,7 +378,7 @@ struct TcGemmDesc {
     int8_t phi5[8];            //   the same for 4-byte staged elements (masks below 32)
 };
 bool tc_available();
-// Set the kernels' shared-memory limits (once per device, outside any stream capture).
+// Set the kernels' shared-memory limits (by every plan, outside any stream capture).
 cudaError_t tc_prepare();
 cudaError_t launch_gemm_tc(const TcGemmDesc &d, int64_t slices, cudaStream_t st);
 // Device status word of the tensor-core kernel (bit 0: a bounded wait timed out); cleared.

@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(256) k_generic(GenericDesc d, int64_t total) {
 // 2^26 x 2^2 outputs: 1.07 -> 0.50 ms (5.4 TB/s) against 8-byte stores in 1024-output chunks.
 template <int PER>
 __global__ void __launch_bounds__(256) k_generic_k1(GenericDesc d, int64_t total) {
-    constexpr int LB = PER == 1 ? 9 : (PER == 2 ? 10 : 12);
+    constexpr int LB = PER == 2 ? 10 : 12;
     static_assert((1 << LB) == 512 * PER, "outputs of a chunk");
     // bit 0 (the pair), then the thread's bits 1-8, then t's
     const Offsets own = deposit2(2 * threadIdx.x, 9, d.posA_c, d.posB_c);

@@ -112,7 +112,9 @@ struct tn_sparse_plan {
     double tcc = 0;
     int64_t arena_elems = 0, total_configs = 0, distinct = 0, launches = 0;
     // CUDA graph of everything but the addition into the caller's amplitudes, and the streams it is
-    // captured on.  It is made at the second call: making it costs more than one call's launches.
+    // captured on.  It is made at the second call, which takes longer for it (12 qubits, 64 samples: 0.63
+    // ms, then 0.86, then 0.25; 24 qubits, 4096 samples: 5.0, 5.5, 4.4): three calls are cheaper
+    // with it than without, one call never makes it.
     bool called = false;
     cudaStream_t lanes[tn::Branches::kLanes] = {};
     bool graph_failed = false;  // it could not be made: calls launch directly

@@ -1,8 +1,7 @@
 // Output stage of the tensor-core thin kernel (k_gemm_thin_tc): a tile of 128 rows and NT columns
 // of complex64, thread t of a drain group holding row t, is staged in shared memory and written
-// in the order of C's memory index, 8 consecutive elements of C per task.  (The CUDA-core thin kernel keeps a
-// padded stage, rows NT + 1 apart: the swizzle's extra address arithmetic and registers cost
-// it more than the bank conflicts it removes.)
+// in the order of C's memory index, 8 consecutive elements of C per task.  (The CUDA-core
+// kernels stage 256 rows under a swizzle of their own, stage_choose_banks.)
 //
 // Element (r, c) of the stage sits at r * NT + (c ^ phi(r)), phi(r) the XOR of d.phi[b] over the
 // set bits b of r (host: thin_choose_swizzle), so both the staging writes and the reads in C's
