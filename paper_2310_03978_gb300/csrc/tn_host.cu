@@ -2538,7 +2538,7 @@ void tn_destroy(void *handle) {
     const uint32_t magic = *reinterpret_cast<const uint32_t *>(handle);
     if (magic == kNetMagic) {
         auto *n = reinterpret_cast<tn_network *>(handle);
-        if (n->data) cudaFree(n->data);
+        if (n->data && n->own_data) cudaFree(n->data);
         n->magic = 0;
         delete n;
     } else if (magic == tn::kSparseMagic) {

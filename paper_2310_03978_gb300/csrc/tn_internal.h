@@ -531,4 +531,5 @@ struct tn_network {
     std::vector<int> open;
     int64_t total = 0;                     // complex128 elements
     double2 *data = nullptr;               // device copy
+    bool own_data = true;                  // false: another network's
 };

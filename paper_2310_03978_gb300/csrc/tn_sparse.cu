@@ -475,23 +475,15 @@ static tn_status sparse_plan_impl(const tn_network_t *net, int32_t path_len,
         sb.node = c;
         sb.net = new tn_network();
         sb.net->device = net->device;
+        // the subtree's leaves are read where they are, so that new data reach them
+        sb.net->data = net->data;
+        sb.net->own_data = false;
         for (int id : lv) {
             sb.net->labels.push_back(net->labels[id]);
-            sb.net->offset.push_back(sb.net->total);
-            sb.net->total += (int64_t)1 << net->labels[id].size();
+            sb.net->offset.push_back(net->offset[id]);
         }
         sb.net->open = p->ten[c].dense;
-        cudaError_t e = cudaMalloc(&sb.net->data, sizeof(double2) * (size_t)sb.net->total);
-        for (size_t q = 0; e == cudaSuccess && q < lv.size(); ++q)
-            e = cudaMemcpy(sb.net->data + sb.net->offset[q], net->data + net->offset[lv[q]],
-                           sizeof(double2) * ((size_t)1 << net->labels[lv[q]].size()),
-                           cudaMemcpyDeviceToDevice);
         p->subs.push_back(sb);  // owned by the plan from here on
-        if (e != cudaSuccess) {
-            sparse_free(p);
-            return fail(e == cudaErrorMemoryAllocation ? TN_ERR_OOM : TN_ERR_CUDA,
-                        "sparse-state dense subtree: %s", cudaGetErrorString(e));
-        }
         tn_status ps = tn_plan(sb.net, (int32_t)sub_steps.size(), lpath.data(), 0, nullptr, mode,
                                nullptr, &p->subs.back().plan);
         if (ps != TN_OK) {

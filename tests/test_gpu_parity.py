@@ -1582,3 +1582,23 @@ def test_sparse_state_long_contractions(tn, m, n, k, ns):
     scale = np.sqrt(O.contract_sparse([np.abs(x) ** 2 + 0j for x in tensors], labels, opens, path,
                                       smp).real)
     assert np.all(np.abs(got - ref) <= 8 * 2.0 ** (-24 + k / 2) * scale)
+
+
+# New numbers for a network reach a sparse-state plan made before them, its dense subtrees too.
+def test_sparse_state_follows_the_networks_data(tn):
+    circ, net, smp = W.sparse_state_workload(num_samples=64)
+    path, _, _ = tn.path_optimize(net.labels, net.open_labels,
+                                  W.greedy_path(net.labels, net.open_labels), seed=7,
+                                  sweeps=500, sweeps_final=0, t_start=0.03, t_end=0.001, chains=8)
+    tnet = tn.Network(net.tensors, net.labels, net.open_labels)
+    plan = tn.SparsePlan(tnet, path, smp)
+    assert plan.info()["dense_subtrees"] > 0
+    first = torch.zeros(len(smp), dtype=torch.complex128, device="cuda")
+    plan.contract(first)
+    tnet.set_data([np.conj(t) for t in net.tensors])
+    for _ in range(2):  # the graph's first use, and a replay
+        amps = torch.zeros_like(first)
+        plan.contract(amps)
+        check(amps.cpu().numpy(), np.conj(first.cpu().numpy()), TOL["c64"])
+    plan.close()
+    tnet.close()
