@@ -645,7 +645,9 @@ static void arrange(tn_plan_t *p, int level) {
                 // values low in FP16's range; single-pass operands keep their 11 significant
                 // bits there, but the lo planes of compensated FP16 operands would fall into the
                 // subnormals, so those are split from complex64 with their measured max-abs.
-                // BF16 and TF32 have FP32's exponents: hi and lo keep their bits at any scale.
+                // BF16 and TF32 have FP32's exponents: hi and lo keep their bits, and a product
+                // loses none in FP32 as long as the two operands' bounds exceed their maxima by
+                // no more than 2^120 in all.
                 // A CUDA-core producer writes directly only with whole 64 x 64 tiles, and then
                 // never splits K (its epilogue must hold final sums).
                 // A CUDA-core producer that would split K (judged at one slice in flight, its
