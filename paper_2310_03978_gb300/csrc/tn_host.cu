@@ -24,7 +24,6 @@
 #include <map>
 #include <new>
 #include <string>
-#include <unordered_map>
 #include <vector>
 
 #include "../../include/tn.h"
@@ -1521,7 +1520,7 @@ tn::GenericDesc make_generic_desc(const tn_plan_t *p, const Step &st, unsigned i
 std::vector<std::vector<int>> by_depth(const tn_plan_t *p, const std::vector<int> &steps) {
     const int id = p->steps[steps[0]].chain;
     std::vector<std::vector<int>> levels;
-    std::unordered_map<int, int> depth;
+    std::vector<int> depth(p->steps.size());
     for (int k : steps) {
         int d = 0;
         for (int x : {p->steps[k].a, p->steps[k].b})
@@ -1614,7 +1613,7 @@ tn::ChainGroup chain_group(const tn_plan_t *p, const std::vector<int> &steps,
                            std::vector<int32_t> &levels) {
     const int id = p->steps[steps[0]].chain;
     tn::ChainGroup g{};
-    std::unordered_map<int, int> shm;  // tensor -> offset
+    std::vector<int> shm(p->tensors.size());  // tensor -> offset
     auto take = [&](int x) {
         shm[x] = g.elems;
         g.elems += (int32_t)chain_elems(p->tensors[x]);
@@ -1628,7 +1627,7 @@ tn::ChainGroup chain_group(const tn_plan_t *p, const std::vector<int> &steps,
         c.lanes = (uint8_t)std::min(X.rank(), tn::kChainItemBits);
         for (uint32_t e = 0; e < (1u << X.rank()); e += tn::kChainItemLanes) {
             c.off = (uint16_t)e;
-            c.shm = (uint16_t)(shm.at(x) + (int)e);
+            c.shm = (uint16_t)(shm[x] + (int)e);
             copies.push_back(c);
         }
     };
@@ -1653,11 +1652,22 @@ tn::ChainGroup chain_group(const tn_plan_t *p, const std::vector<int> &steps,
         levels.push_back((int32_t)recs.size() - g.recs);
         for (int k : level) {
             const ChainStep cs(p, p->steps[k]);
-            const int a = shm.at(cs.ta), b = shm.at(cs.tb), c = shm.at(p->steps[k].c);
-            const std::vector<uint16_t> oa = cs.offsets(cs.in_a), ob = cs.offsets(cs.in_b);
-            for (uint32_t o = 0; o < (1u << cs.rc); ++o)
-                recs.push_back({(uint16_t)(a + oa[o]), (uint16_t)(b + ob[o]), (uint16_t)(c + o),
-                                (uint16_t)(cs.nk | cs.flags)});
+            const size_t at = recs.size();
+            recs.resize(at + ((size_t)1 << cs.rc));
+            // by output bit: the upper half's offsets are the lower half's plus the bit's
+            tn::ChainRec *out = recs.data() + at;
+            out[0] = {(uint16_t)shm[cs.ta], (uint16_t)shm[cs.tb], (uint16_t)shm[p->steps[k].c],
+                      (uint16_t)(cs.nk | cs.flags)};
+            uint32_t wa = 1u << cs.nk, wb = wa;
+            for (int i = 0; i < cs.rc; ++i) {
+                const uint32_t half = 1u << i, da = (cs.in_a >> i) & 1u ? wa : 0,
+                               db = (cs.in_b >> i) & 1u ? wb : 0;
+                for (uint32_t j = 0; j < half; ++j)
+                    out[half | j] = {(uint16_t)(out[j].a + da), (uint16_t)(out[j].b + db),
+                                     (uint16_t)(out[j].c + half), out[j].nk_flags};
+                wa <<= da != 0;
+                wb <<= db != 0;
+            }
         }
     }
     levels.push_back((int32_t)recs.size() - g.recs);
@@ -1711,29 +1721,45 @@ tn_status build_chains(tn_plan_t *p) {
         }
         c.first_group = (int64_t)groups.size();
         c.ngroups = (int)gs.size();
+        size_t more = 0;
+        for (const auto &g : gs) more += (size_t)g.recs + 1;
+        if (recs.capacity() < recs.size() + more) recs.reserve(2 * recs.size() + more);
         for (const auto &g : gs) {
             groups.push_back(chain_group(p, g.steps, copies, recs, levels));
             c.elems = std::max<int64_t>(c.elems, groups.back().elems + groups.back().n_recs);
         }
     }
-    auto bytes = [](const auto &v) { return sizeof(v[0]) * v.size(); };
-    std::vector<char> host;
-    auto add = [&](const auto &v) {  // 16-byte aligned: the sizes of what precedes are multiples
-        const size_t at = host.size();
-        host.resize(at + (bytes(v) + 15) / 16 * 16);
-        if (!v.empty()) memcpy(host.data() + at, v.data(), bytes(v));
-        return at;
+    // one allocation, 16-byte aligned parts; one copy while that is small, a copy each when packing
+    // them would cost more
+    struct Piece {
+        const void *src;
+        size_t bytes, at;
+    };
+    std::vector<Piece> pieces;
+    size_t total = 0;
+    auto add = [&](const auto &v) {
+        pieces.push_back({v.data(), sizeof(v[0]) * v.size(), total});
+        total += (pieces.back().bytes + 15) / 16 * 16;
+        return pieces.back().at;
     };
     const size_t oi = add(items), oc = add(copies), orr = add(recs), og = add(groups),
                  ol = add(levels);
     char *dev = nullptr;
-    TN_CUDA(cudaMalloc(&dev, host.size()));
+    TN_CUDA(cudaMalloc(&dev, total));
     p->chain_items = reinterpret_cast<tn::ChainItem *>(dev + oi);
     p->chain_copies = reinterpret_cast<tn::ChainCopy *>(dev + oc);
     p->chain_recs = reinterpret_cast<tn::ChainRec *>(dev + orr);
     p->chain_groups = reinterpret_cast<tn::ChainGroup *>(dev + og);
     p->chain_levels = reinterpret_cast<int32_t *>(dev + ol);
-    TN_CUDA(cudaMemcpy(dev, host.data(), host.size(), cudaMemcpyHostToDevice));
+    if (total <= (size_t)1 << 17) {
+        std::vector<char> host(total);
+        for (const Piece &x : pieces)
+            if (x.bytes) memcpy(host.data() + x.at, x.src, x.bytes);
+        TN_CUDA(cudaMemcpy(dev, host.data(), total, cudaMemcpyHostToDevice));
+        return TN_OK;
+    }
+    for (const Piece &x : pieces)
+        if (x.bytes) TN_CUDA(cudaMemcpy(dev + x.at, x.src, x.bytes, cudaMemcpyHostToDevice));
     return TN_OK;
 }
 
